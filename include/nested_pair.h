@@ -397,8 +397,8 @@ nt_status nt_debug_bounds_report(int32_t *out_h, int32_t reset);
 nt_status nt_debug_expire_wait(int32_t *status_d, int64_t limit_clocks, int32_t *observed_d, nt_stream stream);
 
 /* Testing aid: the bf16 pair-order attention uses two tensor-core kernels, one that holds a whole score row
- * on chip (samples of up to 224 tokens) and a key-blocked one (longer samples).  mode 1 sends every sample to
- * the key-blocked kernel, mode 0 restores the split by length.  Returns the previous mode. */
+ * on chip (samples of up to 224 tokens) and one that walks the keys in blocks (longer samples).  mode 1 sends every
+ * sample to the second kernel, mode 0 restores the split by length.  Returns the previous mode. */
 int32_t nt_attn_core_mode(int32_t mode);
 
 /* Testing aid: non-zero forces the shape-generic CUDA-core kernels even where a tensor-core

@@ -18,7 +18,7 @@ __device__ int g_nt_bounds[4] = {0, 0, 0, 0};
 
 std::atomic<long long> g_launches{0};
 int g_force_generic = 0;
-int g_kb_all = 0;   // testing aid (nt_attn_core_mode): the key-blocked attention core for every sample length
+int g_fr_all = 0;   // testing aid (nt_attn_core_mode): the register-fragment attention core for every sample length
 
 // ---- per-kernel event timing (off unless nt_profile_begin was called) ----------------------
 struct ProfRecord { const char* name; cudaEvent_t e0, e1; };
@@ -299,15 +299,15 @@ static nt_status attn_generic(const nt_layout* L, const Totals& tot, nt_order or
   const int Hd = H * d;
   const bool pair = order == NT_ORDER_PAIR_IJC;
   const bool tc = dt == NT_BF16 && !g_force_generic && pair && W->ln_gamma && tot.nmax < 60000;
-  const bool tc_in = tc && fast_attn_in_supported(c, H, d) && fast_attn_kb_supported(KB_MODE_PAIR_ROW, H, d, W->W_b != nullptr);   // bias goes out times sqrt(d)
+  const bool tc_in = tc && fast_attn_in_supported(c, H, d) && fast_attn_fr_supported(H, d);   // bias goes out times sqrt(d)
   const bool tc_out = tc && W->W_g && fast_attn_out_supported(c, H, d);   // recomputes the gate from z
   const bool tok_fast = dt == NT_BF16 && !g_force_generic && !pair && !W->W_b && c % 8 == 0 && c <= Hd && c <= 2048 &&
-                        fast_attn_kb_supported(KB_MODE_TOKEN, H, d, false) && fast_token_gemm_supported(c, Hd, Hd) &&
+                        fast_attn_fr_supported(H, d) && fast_token_gemm_supported(c, Hd, Hd) &&
                         fast_token_gemm_supported(Hd, c, 0);
-  // the key-blocked tcgen05 core takes every sample length (pair order: the samples beyond the whole-row core's reach)
+  // the register-fragment core takes every sample length (pair order: the samples beyond the whole-row core's reach)
   // (a bias must come from the tensor-core projection, which writes it in the units the cores expect)
-  const bool kb_pair = dt == NT_BF16 && !g_force_generic && pair && !col && tot.nmax < 60000 && (tc_in || !W->W_b) &&
-                       fast_attn_kb_supported(KB_MODE_PAIR_ROW, H, d, W->W_b != nullptr);
+  const bool fr_pair = dt == NT_BF16 && !g_force_generic && pair && !col && tot.nmax < 60000 && (tc_in || !W->W_b) &&
+                       fast_attn_fr_supported(H, d);
   AttnPrep aprep{};
   if (tc_in || tc_out) {
     nt_status r0 = W->prepared ? fast_attn_prep(W, c, H, d, const_cast<void*>(W->prepared), aprep, st, false)
@@ -335,7 +335,7 @@ static nt_status attn_generic(const nt_layout* L, const Totals& tot, nt_order or
       if ((r = fast_token_gemm(xh, rows, c, W->W_q, Hd, (char*)w.q + to, W->W_k, Hd, (char*)w.k + to, 0, 0, "tok_attn_in_qk", st)) != NT_OK) return r;
       if ((r = fast_token_gemm(xh, rows, c, W->W_v, Hd, (char*)w.v + to, W->W_g, W->W_g ? Hd : 0, W->W_g ? (char*)w.g + to : nullptr, 0, 0,
                                "tok_attn_in_vg", st)) != NT_OK) return r;
-      if ((r = fast_attn_core_kb(w.q, w.k, w.v, nullptr, w.o, H, d, KB_MODE_TOKEN, m, L->status_d, st)) != NT_OK) return r;
+      if ((r = fast_attn_core_fr(w.q, w.k, w.v, nullptr, w.o, H, d, FR_MODE_TOKEN, m, L->status_d, st)) != NT_OK) return r;
       if (W->W_g && (r = fast_gate_mul((char*)w.g + to, (char*)w.o + to, rows * Hd, st, "tok_attn_gate")) != NT_OK) return r;
       if ((r = fast_token_gemm((char*)w.o + to, rows, Hd, W->W_o, c, xr, nullptr, 0, nullptr, 0, 1, "tok_attn_out", st)) != NT_OK) return r;
       continue;
@@ -345,13 +345,13 @@ static nt_status attn_generic(const nt_layout* L, const Totals& tot, nt_order or
     pa.ln_g = W->ln_gamma; pa.ln_b = W->ln_beta; pa.eps = eps;
     pa.Nout = Hd; pa.act = ACT_NONE; pa.out_mode = O_STORE;
     // column-wise attention: the whole-row core gathers its (short) samples' bias tiles transposed itself; the
-    // key-blocked core wants the planes of the longer samples stored transposed
-    const bool kb_col = tc_in && col && fast_attn_kb_supported(KB_MODE_PAIR_COL, H, d, W->W_b != nullptr);
-    const int n_tc_col = (kb_col && !g_kb_all) ? fast_attn_tc_max_n(d, W->W_b != nullptr) : 0;
+    // register-fragment core wants the planes of the longer samples stored transposed
+    const bool fr_col = tc_in && col && fast_attn_fr_supported(H, d);
+    const int n_tc_col = (fr_col && !g_fr_all) ? fast_attn_tc_max_n(d, W->W_b != nullptr) : 0;
     if (tc_in) {
       // the gate buffer is free when the output stage recomputes the gate: it carries the z row statistics to it
       r = fast_attn_in(zx, aprep, eps, c, H, d, w.q, w.k, w.v, W->W_b ? w.bias : nullptr, m, L->status_d, st,
-                       tc_out ? (float2*)w.g : nullptr, kb_col ? n_tc_col : 0x7fffffff);
+                       tc_out ? (float2*)w.g : nullptr, fr_col ? n_tc_col : 0x7fffffff);
       if (r != NT_OK) return r;
     } else {
       pa.W1 = W->W_q; pa.out = w.q;
@@ -370,7 +370,7 @@ static nt_status attn_generic(const nt_layout* L, const Totals& tot, nt_order or
       pa.W1 = W->W_b; pa.Nout = H; pa.out = w.bias; pa.out_mode = O_CHANNEL_MAJOR;
       if ((r = launch_proj<T>(pa, m, st, "generic_attn_in_bias")) != NT_OK) return r;
     }
-    if (col && kb_col) {
+    if (col && fr_col) {
       bool any_short = false, any_long = false;
       for (int s = 0; s < m.B; ++s) {
         if (m.N[s] >= 1 && m.N[s] <= n_tc_col) any_short = true;
@@ -379,14 +379,14 @@ static nt_status attn_generic(const nt_layout* L, const Totals& tot, nt_order or
       r = NT_OK;
       if (any_short) r = fast_attn_core_tc(w.q, w.k, w.v, W->W_b ? w.bias : nullptr, w.o, H, d, m, n_tc_col, L->status_d, st, true);
       if (r == NT_OK && any_long)
-        r = fast_attn_core_kb(w.q, w.k, w.v, W->W_b ? w.bias : nullptr, w.o, H, d, KB_MODE_PAIR_COL, m, L->status_d, st, n_tc_col);
+        r = fast_attn_core_fr(w.q, w.k, w.v, W->W_b ? w.bias : nullptr, w.o, H, d, FR_MODE_PAIR_COL, m, L->status_d, st, n_tc_col);
     } else if (col) {
       // the shape-generic core (the bias is stored times sqrt(d) when the tensor-core projections wrote it)
       r = launch_attn_core<T>((const T*)w.q, (const T*)w.k, (const T*)w.v, W->W_b ? (const T*)w.bias : nullptr,
                               (T*)w.o, H, d, 2, m, st, 0, tc_in ? rsqrtf((float)d) : 1.0f);
-    } else if (kb_pair) {
-      // a score row of up to n_tc keys fits the whole-row core's accumulator; longer samples take the key-blocked core
-      int n_tc = g_kb_all ? 0 : fast_attn_tc_max_n(d, W->W_b != nullptr);
+    } else if (fr_pair) {
+      // a score row of up to n_tc keys fits the whole-row core's accumulator; longer samples take the register-fragment core
+      int n_tc = g_fr_all ? 0 : fast_attn_tc_max_n(d, W->W_b != nullptr);
       bool any_short = false, any_long = false;
       for (int s = 0; s < m.B; ++s) {
         if (m.N[s] >= 1 && m.N[s] <= n_tc) any_short = true;
@@ -395,7 +395,7 @@ static nt_status attn_generic(const nt_layout* L, const Totals& tot, nt_order or
       r = NT_OK;
       if (any_short) r = fast_attn_core_tc(w.q, w.k, w.v, W->W_b ? w.bias : nullptr, w.o, H, d, m, n_tc, L->status_d, st);
       if (r == NT_OK && any_long)
-        r = fast_attn_core_kb(w.q, w.k, w.v, W->W_b ? w.bias : nullptr, w.o, H, d, KB_MODE_PAIR_ROW, m, L->status_d, st, n_tc);
+        r = fast_attn_core_fr(w.q, w.k, w.v, W->W_b ? w.bias : nullptr, w.o, H, d, FR_MODE_PAIR_ROW, m, L->status_d, st, n_tc);
     }
     else
       r = launch_attn_core<T>((const T*)w.q, (const T*)w.k, (const T*)w.v, W->W_b ? (const T*)w.bias : nullptr,
@@ -455,7 +455,7 @@ static nt_status single_attn_impl(const nt_layout* L, const Totals& tot, int c_s
       if ((r = fast_token_gemm(xh, trows, c_s, W->W_q, Hd, (char*)w.q + to, W->W_k, Hd, (char*)w.k + to, 0, 0, "single_attn_in_qk", st)) != NT_OK) return r;
       if ((r = fast_token_gemm(xh, trows, c_s, W->W_v, Hd, (char*)w.v + to, W->W_g, Hd, (char*)w.g + to, 0, 0, "single_attn_in_vg", st)) != NT_OK) return r;
       if ((r = fast_single_bias(z, W->ln_z_gamma, W->ln_z_beta, W->W_b, eps, c_z, H, sqrtf((float)d), m, w.bias, st)) != NT_OK) return r;
-      if ((r = fast_attn_core_kb(w.q, w.k, w.v, w.bias, w.o, H, d, KB_MODE_TOKEN, m, L->status_d, st)) != NT_OK) return r;
+      if ((r = fast_attn_core_fr(w.q, w.k, w.v, w.bias, w.o, H, d, FR_MODE_TOKEN, m, L->status_d, st)) != NT_OK) return r;
       if ((r = fast_gate_mul((char*)w.g + to, (char*)w.o + to, trows * Hd, st)) != NT_OK) return r;
       if ((r = fast_token_gemm((char*)w.o + to, trows, Hd, W->W_o, c_s, xr, nullptr, 0, nullptr, 0, 1, "single_attn_out", st)) != NT_OK) return r;
       continue;
@@ -869,8 +869,8 @@ nt_status nt_debug_bounds_report(int32_t* out_h, int32_t reset) {
 }
 
 int32_t nt_attn_core_mode(int32_t mode) {
-  int32_t prev = g_kb_all;
-  g_kb_all = mode != 0;
+  int32_t prev = g_fr_all;
+  g_fr_all = mode != 0;
   return prev;
 }
 

@@ -64,13 +64,13 @@ int fast_attn_tc_max_n(int d, bool has_bias);
 nt_status fast_attn_core_tc(const void* q, const void* k, const void* v, const void* bias, void* o, int H, int d,
                             const BatchMeta& m, int n_max, int* status, cudaStream_t st, bool col = false);
 
-// key-blocked tcgen05 core for any sample length: pair order (rows = pair rows, one bias plane per (sample, head)
-// shared by all rows) or token order (rows = samples; the bias planes, if any, belong to the sample's own queries).
-// The bias comes stored times sqrt(d) (the units of q.k), as for the whole-row core.  Samples with N <= n_min are left
-// out (they belong to another kernel).
-enum { KB_MODE_PAIR_ROW = 0, KB_MODE_TOKEN = 1, KB_MODE_PAIR_COL = 2 };
-bool fast_attn_kb_supported(int mode, int H, int d, bool has_bias);
-nt_status fast_attn_core_kb(const void* q, const void* k, const void* v, const void* bias, void* o, int H, int d,
+// attention core with the softmax weights in register fragments (fast_attn_frag.cu): any sample length, d in {16, 32, 64},
+// pair order (rows or columns; one bias plane per (sample, head), stored times sqrt(d), for columns stored transposed)
+// or token order (rows = samples; the bias planes, if any, belong to the sample's own queries).  Samples with N <= n_min
+// are left out (they belong to another kernel).
+enum { FR_MODE_PAIR_ROW = 0, FR_MODE_TOKEN = 1, FR_MODE_PAIR_COL = 2 };
+bool fast_attn_fr_supported(int H, int d);
+nt_status fast_attn_core_fr(const void* q, const void* k, const void* v, const void* bias, void* o, int H, int d,
                             int mode, const BatchMeta& m, int* status, cudaStream_t st, int n_min = 0);
 
 // triangle contraction on tcgen05: a, b, t are three equally spaced channel-major buffers

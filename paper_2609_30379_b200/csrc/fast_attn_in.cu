@@ -248,7 +248,7 @@ __global__ void __launch_bounds__(AI_THREADS, 1) attn_in_kernel(const __grid_con
             const int N = p.N[s], ld = round_up8(N);
             const unsigned rr = (unsigned)(P - p.pair_off[s]);      // N^2 < 2^32 (N < 2^16 for this path)
             const unsigned i = rr / (unsigned)N, j = rr - i * (unsigned)N;
-            // (transposed planes: the key-blocked core reads a query's keys contiguously, and in column-wise attention
+            // (transposed planes: the register-fragment core reads a query's keys contiguously, and in column-wise attention
             // the bias of (query i, key k) is the plane's element [k][i])
             __nv_bfloat16* bp = p.bias + (long long)p.H * p.cm_off[s] + (N > p.bias_tr_above ? (long long)j * ld + i : (long long)i * ld + j);
             for (int h = 0; h < p.H; ++h)

@@ -597,7 +597,7 @@ __global__ void __launch_bounds__(256) single_bias_mma_kernel(const __nv_bfloat1
 
 bool fast_single_attn_supported(int c_s, int c_z, int H, int d) {
   const int Hd = H * d;
-  return c_s % 8 == 0 && c_s <= 2048 && c_z % 8 == 0 && c_z <= 1024 && H >= 1 && H <= SB_MAXH && fast_attn_kb_supported(KB_MODE_TOKEN, H, d, true) &&
+  return c_s % 8 == 0 && c_s <= 2048 && c_z % 8 == 0 && c_z <= 1024 && H >= 1 && H <= SB_MAXH && fast_attn_fr_supported(H, d) &&
          fast_token_gemm_supported(c_s, Hd, Hd) && fast_token_gemm_supported(Hd, c_s, 0);
 }
 

@@ -223,29 +223,20 @@ __device__ inline void umma_ts(unsigned d_tmem, unsigned a_tmem, unsigned long l
       "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}\n"
       ::"r"(d_tmem), "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate) : "memory");
 }
-// waits for the TMEM loads in flight; the destination registers pass through the statement so that no use of them
-// can be scheduled ahead of the wait
+// Waits for the TMEM loads in flight and then passes their destination registers through an empty statement, so that
+// no use of them can be scheduled ahead of the wait.  Two statements on purpose: the copies the compiler may make of
+// tied operands stand in front of the statement that ties them, and in front of the wait the loads have not landed.
+#define NT_TIE16(a)                                                                                                    \
+  asm volatile("" : "+r"(a[0]), "+r"(a[1]), "+r"(a[2]), "+r"(a[3]), "+r"(a[4]), "+r"(a[5]), "+r"(a[6]), "+r"(a[7]),   \
+                    "+r"(a[8]), "+r"(a[9]), "+r"(a[10]), "+r"(a[11]), "+r"(a[12]), "+r"(a[13]), "+r"(a[14]), "+r"(a[15])::"memory")
 __device__ inline void tmem_ld_wait16(unsigned (&a)[16]) {
-  asm volatile("tcgen05.wait::ld.sync.aligned;\n"
-               : "+r"(a[0]), "+r"(a[1]), "+r"(a[2]), "+r"(a[3]), "+r"(a[4]), "+r"(a[5]), "+r"(a[6]), "+r"(a[7]), "+r"(a[8]),
-                 "+r"(a[9]), "+r"(a[10]), "+r"(a[11]), "+r"(a[12]), "+r"(a[13]), "+r"(a[14]), "+r"(a[15])
-               :: "memory");
+  tmem_ld_wait();
+  NT_TIE16(a);
 }
-__device__ inline void tmem_ld_wait16_1(unsigned (&a)[16], unsigned& b) {
-  asm volatile("tcgen05.wait::ld.sync.aligned;\n"
-               : "+r"(a[0]), "+r"(a[1]), "+r"(a[2]), "+r"(a[3]), "+r"(a[4]), "+r"(a[5]), "+r"(a[6]), "+r"(a[7]), "+r"(a[8]),
-                 "+r"(a[9]), "+r"(a[10]), "+r"(a[11]), "+r"(a[12]), "+r"(a[13]), "+r"(a[14]), "+r"(a[15]), "+r"(b)
-               :: "memory");
-}
-// wait for the TMEM loads in flight; the two register sets are passed through the statement so that no use of
-// them can be scheduled ahead of the wait
 __device__ inline void tmem_ld_wait2(unsigned (&a)[16], unsigned (&b)[16]) {
-  asm volatile("tcgen05.wait::ld.sync.aligned;\n"
-               : "+r"(a[0]), "+r"(a[1]), "+r"(a[2]), "+r"(a[3]), "+r"(a[4]), "+r"(a[5]), "+r"(a[6]), "+r"(a[7]), "+r"(a[8]),
-                 "+r"(a[9]), "+r"(a[10]), "+r"(a[11]), "+r"(a[12]), "+r"(a[13]), "+r"(a[14]), "+r"(a[15]), "+r"(b[0]),
-                 "+r"(b[1]), "+r"(b[2]), "+r"(b[3]), "+r"(b[4]), "+r"(b[5]), "+r"(b[6]), "+r"(b[7]), "+r"(b[8]), "+r"(b[9]),
-                 "+r"(b[10]), "+r"(b[11]), "+r"(b[12]), "+r"(b[13]), "+r"(b[14]), "+r"(b[15])
-               :: "memory");
+  tmem_ld_wait();
+  NT_TIE16(a);
+  NT_TIE16(b);
 }
 
 // ---- MMA descriptors (bf16 operands, float accumulate)
