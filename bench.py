@@ -60,8 +60,7 @@ def kernel_work(cfg: wl.Config):
         # single-ragged special case: the attention works on the T1 token rows (c_z is the token width); one
         # exponential per (query, key, head) of every sample = sum N^2 per head
         R = T1
-        for n in ("q", "k", "v", "g"):
-            w[f"generic_attn_in_{n}"] = dict(bytes=R * (c_z + Hd) * e, flops=2 * R * c_z * Hd)
+        w["generic_attn_in"] = dict(bytes=R * (c_z + 4 * Hd) * e, flops=2 * R * c_z * 4 * Hd)
         w["generic_attn_core"] = w["attn_core"] = w["attn_core_tok"] = dict(bytes=R * 4 * Hd * e, flops=4 * T2 * Hd, exps=T2 * H)
         # token-side projections of the tensor-core path: q | k in one launch, v in another, the output projection
         w["tok_attn_in_qk"] = dict(bytes=R * (c_z + 2 * Hd) * e + 2 * Hd * c_z * e, flops=2 * R * c_z * 2 * Hd)
@@ -70,25 +69,21 @@ def kernel_work(cfg: wl.Config):
         w["generic_attn_out"] = w["attn_out"] = dict(bytes=R * (Hd + 2 * c_z) * e + c_z * Hd * e, flops=2 * R * Hd * c_z)
         w["segment_reduce"] = w["generic_segment_reduce"] = dict(bytes=R * c_z * e, flops=R * c_z)
         return w
-    tok = dict(bytes=T1 * c_s * e + c_z * c_s * e + T1 * c_z * 4, flops=2 * T1 * c_s * c_z)
-    w["tok_proj_u"] = w["tok_proj_v"] = tok
-    w["tok_proj"] = dict(bytes=T1 * c_s * e + 2 * c_z * c_s * e + 2 * T1 * c_z * 4, flops=4 * T1 * c_s * c_z)
+    w["generic_tok_proj"] = w["tok_proj"] = dict(bytes=T1 * c_s * e + 2 * c_z * c_s * e + 2 * T1 * c_z * 4, flops=4 * T1 * c_s * c_z)
     # per-token preparation of the broadcast: float rows read and written in place, two bf16 parts, squared norms
     w["broadcast_prep"] = dict(bytes=2 * T1 * (c_z * (4 + 4 + 2 + 2) + 4), flops=8 * T1 * c_z)
     bc = dict(bytes=T2 * c_z * e + 2 * T1 * c_z * 4, flops=8 * T2 * c_z)
     w["broadcast_ln"] = w["generic_broadcast_ln"] = bc
     # accumulated onto the state (persistent pair stream): the state is read as well as written
     w["broadcast_ln_add"] = w["generic_broadcast_ln_add"] = dict(bytes=2 * T2 * c_z * e + 2 * T1 * c_z * 4, flops=9 * T2 * c_z)
-    w["generic_tri_in_a"] = w["generic_tri_in_b"] = dict(bytes=T2 * (c_z + c_h) * e, flops=2 * T2 * c_z * 2 * c_h)
-    w["generic_tri_in_g"] = dict(bytes=2 * T2 * c_z * e, flops=2 * T2 * c_z * c_z)
+    # the shape-generic projections: a, b and the gate (q, k, v, gate and bias) from one read of the state
+    w["generic_tri_in"] = dict(bytes=T2 * (2 * c_z + 2 * c_h) * e, flops=2 * T2 * c_z * (4 * c_h + c_z))
     w["tri_in"] = dict(bytes=T2 * (c_z + 2 * c_h) * e, flops=2 * T2 * c_z * 4 * c_h)
     w["generic_tri_contract"] = w["tri_contract"] = dict(bytes=3 * T2 * c_h * e, flops=2 * N3 * c_h)
     w["generic_tri_contract_in"] = w["tri_contract_in"] = w["tri_contract"]      # incoming direction: same work
     w["generic_tri_out"] = dict(bytes=T2 * (c_h + 3 * c_z) * e, flops=2 * T2 * c_h * c_z)
     w["tri_out"] = dict(bytes=T2 * (c_h + 2 * c_z) * e, flops=2 * T2 * (c_h + c_z) * c_z)
-    for n in ("q", "k", "v", "g"):
-        w[f"generic_attn_in_{n}"] = dict(bytes=T2 * (c_z + Hd) * e, flops=2 * T2 * c_z * Hd)
-    w["generic_attn_in_bias"] = dict(bytes=T2 * (c_z + H) * e, flops=2 * T2 * c_z * H)
+    w["generic_attn_in"] = dict(bytes=T2 * (c_z + 4 * Hd + H) * e, flops=2 * T2 * c_z * (4 * Hd + H))
     w["attn_in"] = dict(bytes=T2 * (c_z + 3 * Hd + H) * e, flops=2 * T2 * c_z * (3 * Hd + H))   # q, k, v and the bias planes (the gate is recomputed by the output stage)
     # the softmax needs one exponential per (query, key, head): the special-function units retire 16 per clock and SM
     w["generic_attn_core"] = w["attn_core"] = dict(bytes=T2 * (4 * Hd + H) * e, flops=4 * N3 * Hd, exps=N3 * H)

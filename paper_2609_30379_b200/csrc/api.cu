@@ -205,16 +205,14 @@ static nt_status pair_broadcast_impl(const nt_layout* L, const Totals& tot, int 
   fill_meta(dummy, nullptr, 0, 0, 0, 0, 0);
   ProjArgs pa{};
   pa.A = x; pa.a_mode = A_ROWMAJOR; pa.row0 = 0; pa.rows = tot.T1; pa.K = c_s;
-  pa.W1 = W_a; pa.Nout = c_z; pa.act = ACT_NONE; pa.out = u; pa.out_mode = O_STORE; pa.out_f32 = 1;
+  pa.add(W_a, nullptr, c_z, ACT_NONE, u, O_STORE, 1);
+  pa.add(W_b, nullptr, c_z, ACT_NONE, v, O_STORE, 1);
   nt_status r;
   if (fast && fast_token_gemm_supported(c_s, c_z, c_z)) {
     r = fast_token_gemm(x, tot.T1, c_s, W_a, c_z, u, W_b, c_z, v, 1, 0, "tok_proj", st);
     if (r != NT_OK) return r;
   } else {
-    r = launch_proj<T>(pa, dummy, st, "tok_proj_u");
-    if (r != NT_OK) return r;
-    pa.W1 = W_b; pa.out = v;
-    r = launch_proj<T>(pa, dummy, st, "tok_proj_v");
+    r = launch_proj<T>(pa, dummy, st, "generic_tok_proj");
     if (r != NT_OK) return r;
   }
   if (fast && (r = fast_broadcast_prep(bp, tot.T1, tot.T1, g, c_z, st, "broadcast_prep")) != NT_OK) return r;
@@ -257,25 +255,19 @@ static nt_status tri_mul_generic(const nt_layout* L, const Totals& tot, int c_z,
       r = fast_tri_in(z, tprep, eps, c_z, c_h, w.a, w.b, m, L->status_d, st, (float2*)w.g);
       if (r != NT_OK) return r;
     } else {
-      pa.W1 = W->W_ag; pa.W2 = W->W_ap; pa.Nout = c_h; pa.out = w.a; pa.out_mode = O_CHANNEL_MAJOR;
-      r = launch_proj<T>(pa, m, st, "generic_tri_in_a");
-      if (r != NT_OK) return r;
-      pa.W1 = W->W_bg; pa.W2 = W->W_bp; pa.out = w.b;
-      r = launch_proj<T>(pa, m, st, "generic_tri_in_b");
-      if (r != NT_OK) return r;
-    }
-    const bool tc_out = tc && fast_tri_out_supported(c_z, c_h);   // recomputes the output gate from z
-    if (!tc_out) {
-      pa.W1 = W->W_g; pa.W2 = nullptr; pa.act = ACT_SIGMOID; pa.Nout = c_z; pa.out = w.g; pa.out_mode = O_STORE;
-      r = launch_proj<T>(pa, m, st, "generic_tri_in_g");
+      // a, b and the gate from the same normalised rows: one launch
+      pa.add(W->W_ag, W->W_ap, c_h, ACT_SIGMOID, w.a, O_CHANNEL_MAJOR);
+      pa.add(W->W_bg, W->W_bp, c_h, ACT_SIGMOID, w.b, O_CHANNEL_MAJOR);
+      pa.add(W->W_g, nullptr, c_z, ACT_SIGMOID, w.g, O_STORE);
+      r = launch_proj<T>(pa, m, st, "generic_tri_in");
       if (r != NT_OK) return r;
     }
-    if (tc && fast_contract_supported(c_h))
+    if (tc)
       r = fast_contract(w.a, (size_t)((char*)w.b - (char*)w.a), c_h, m, L->status_d, st, incoming);
     else
       r = launch_contract<T>((const T*)w.a, (const T*)w.b, (T*)w.t, c_h, m, st, incoming);
     if (r != NT_OK) return r;
-    if (tc_out) {
+    if (tc) {   // (recomputes the output gate from z)
       r = fast_tri_out(z, w.t, tprep, eps, c_z, c_h, m, L->status_d, st, (const float2*)w.g);
       if (r != NT_OK) return r;
       continue;
@@ -283,7 +275,8 @@ static nt_status tri_mul_generic(const nt_layout* L, const Totals& tot, int c_z,
     ProjArgs po{};
     po.A = w.t; po.a_mode = A_CHANNEL_MAJOR; po.row0 = row0; po.rows = rows; po.K = c_h;
     po.ln_g = W->ln_out_gamma; po.ln_b = W->ln_out_beta; po.eps = eps;
-    po.W1 = W->W_o; po.Nout = c_z; po.act = ACT_NONE; po.out = z; po.out_mode = O_ACCUM; po.gateO = w.g;
+    po.gateO = w.g;
+    po.add(W->W_o, nullptr, c_z, ACT_NONE, z, O_ACCUM);
     r = launch_proj<T>(po, m, st, "generic_tri_out");
     if (r != NT_OK) return r;
   }
@@ -343,7 +336,6 @@ static nt_status attn_generic(const nt_layout* L, const Totals& tot, nt_order or
     ProjArgs pa{};
     pa.A = zx; pa.a_mode = A_ROWMAJOR; pa.row0 = row0; pa.rows = rows; pa.K = c;
     pa.ln_g = W->ln_gamma; pa.ln_b = W->ln_beta; pa.eps = eps;
-    pa.Nout = Hd; pa.act = ACT_NONE; pa.out_mode = O_STORE;
     // column-wise attention: the whole-row core gathers its (short) samples' bias tiles transposed itself; the
     // register-fragment core wants the planes of the longer samples stored transposed
     const bool fr_col = tc_in && col && fast_attn_fr_supported(H, d);
@@ -354,22 +346,13 @@ static nt_status attn_generic(const nt_layout* L, const Totals& tot, nt_order or
                        tc_out ? (float2*)w.g : nullptr, fr_col ? n_tc_col : 0x7fffffff);
       if (r != NT_OK) return r;
     } else {
-      pa.W1 = W->W_q; pa.out = w.q;
-      if ((r = launch_proj<T>(pa, m, st, "generic_attn_in_q")) != NT_OK) return r;
-      pa.W1 = W->W_k; pa.out = w.k;
-      if ((r = launch_proj<T>(pa, m, st, "generic_attn_in_k")) != NT_OK) return r;
-      pa.W1 = W->W_v; pa.out = w.v;
-      if ((r = launch_proj<T>(pa, m, st, "generic_attn_in_v")) != NT_OK) return r;
+      pa.add(W->W_q, nullptr, Hd, ACT_NONE, w.q, O_STORE);
+      pa.add(W->W_k, nullptr, Hd, ACT_NONE, w.k, O_STORE);
+      pa.add(W->W_v, nullptr, Hd, ACT_NONE, w.v, O_STORE);
     }
-    if (W->W_g && !tc_out) {
-      pa.W1 = W->W_g; pa.out = w.g; pa.act = ACT_SIGMOID; pa.Nout = Hd; pa.out_mode = O_STORE;
-      if ((r = launch_proj<T>(pa, m, st, "generic_attn_in_g")) != NT_OK) return r;
-      pa.act = ACT_NONE;
-    }
-    if (W->W_b && !tc_in) {
-      pa.W1 = W->W_b; pa.Nout = H; pa.out = w.bias; pa.out_mode = O_CHANNEL_MAJOR;
-      if ((r = launch_proj<T>(pa, m, st, "generic_attn_in_bias")) != NT_OK) return r;
-    }
+    if (W->W_g && !tc_out) pa.add(W->W_g, nullptr, Hd, ACT_SIGMOID, w.g, O_STORE);
+    if (W->W_b && !tc_in) pa.add(W->W_b, nullptr, H, ACT_NONE, w.bias, O_CHANNEL_MAJOR);
+    if (pa.nseg && (r = launch_proj<T>(pa, m, st, "generic_attn_in")) != NT_OK) return r;
     if (col && fr_col) {
       bool any_short = false, any_long = false;
       for (int s = 0; s < m.B; ++s) {
@@ -383,7 +366,7 @@ static nt_status attn_generic(const nt_layout* L, const Totals& tot, nt_order or
     } else if (col) {
       // the shape-generic core (the bias is stored times sqrt(d) when the tensor-core projections wrote it)
       r = launch_attn_core<T>((const T*)w.q, (const T*)w.k, (const T*)w.v, W->W_b ? (const T*)w.bias : nullptr,
-                              (T*)w.o, H, d, 2, m, st, 0, tc_in ? rsqrtf((float)d) : 1.0f);
+                              (T*)w.o, H, d, 2, m, st, tc_in ? rsqrtf((float)d) : 1.0f);
     } else if (fr_pair) {
       // a score row of up to n_tc keys fits the whole-row core's accumulator; longer samples take the register-fragment core
       int n_tc = g_fr_all ? 0 : fast_attn_tc_max_n(d, W->W_b != nullptr);
@@ -422,7 +405,7 @@ static nt_status attn_generic(const nt_layout* L, const Totals& tot, nt_order or
     ProjArgs po{};
     po.A = w.o; po.a_mode = A_ROWMAJOR; po.row0 = row0; po.rows = rows; po.K = Hd;
     po.gateA = W->W_g ? w.g : nullptr;
-    po.W1 = W->W_o; po.Nout = c; po.act = ACT_NONE; po.out = zx; po.out_mode = O_ACCUM;
+    po.add(W->W_o, nullptr, c, ACT_NONE, zx, O_ACCUM);
     if ((r = launch_proj<T>(po, m, st, "generic_attn_out")) != NT_OK) return r;
   }
   return NT_OK;
@@ -463,26 +446,22 @@ static nt_status single_attn_impl(const nt_layout* L, const Totals& tot, int c_s
     ProjArgs pa{};
     pa.A = x; pa.a_mode = A_ROWMAJOR; pa.row0 = trow0; pa.rows = trows; pa.K = c_s;
     pa.ln_g = W->ln_gamma; pa.ln_b = W->ln_beta; pa.eps = eps;
-    pa.Nout = Hd; pa.act = ACT_NONE; pa.out_mode = O_STORE;
-    pa.W1 = W->W_q; pa.out = w.q;
-    if ((r = launch_proj<T>(pa, m, st, "single_attn_in_q")) != NT_OK) return r;
-    pa.W1 = W->W_k; pa.out = w.k;
-    if ((r = launch_proj<T>(pa, m, st, "single_attn_in_k")) != NT_OK) return r;
-    pa.W1 = W->W_v; pa.out = w.v;
-    if ((r = launch_proj<T>(pa, m, st, "single_attn_in_v")) != NT_OK) return r;
-    pa.W1 = W->W_g; pa.out = w.g; pa.act = ACT_SIGMOID;
-    if ((r = launch_proj<T>(pa, m, st, "single_attn_in_g")) != NT_OK) return r;
+    pa.add(W->W_q, nullptr, Hd, ACT_NONE, w.q, O_STORE);
+    pa.add(W->W_k, nullptr, Hd, ACT_NONE, w.k, O_STORE);
+    pa.add(W->W_v, nullptr, Hd, ACT_NONE, w.v, O_STORE);
+    pa.add(W->W_g, nullptr, Hd, ACT_SIGMOID, w.g, O_STORE);
+    if ((r = launch_proj<T>(pa, m, st, "generic_single_attn_in")) != NT_OK) return r;
     ProjArgs pb{};
     pb.A = z; pb.a_mode = A_ROWMAJOR; pb.row0 = prow0; pb.rows = prows; pb.K = c_z;
     pb.ln_g = W->ln_z_gamma; pb.ln_b = W->ln_z_beta; pb.eps = eps;
-    pb.W1 = W->W_b; pb.Nout = H; pb.act = ACT_NONE; pb.out = w.bias; pb.out_mode = O_CHANNEL_MAJOR;
+    pb.add(W->W_b, nullptr, H, ACT_NONE, w.bias, O_CHANNEL_MAJOR);
     if ((r = launch_proj<T>(pb, m, st, "single_attn_bias")) != NT_OK) return r;
     r = launch_attn_core<T>((const T*)w.q, (const T*)w.k, (const T*)w.v, (const T*)w.bias, (T*)w.o, H, d, 0, m, st);
     if (r != NT_OK) return r;
     ProjArgs po{};
     po.A = w.o; po.a_mode = A_ROWMAJOR; po.row0 = trow0; po.rows = trows; po.K = Hd;
     po.gateA = w.g;
-    po.W1 = W->W_o; po.Nout = c_s; po.act = ACT_NONE; po.out = x; po.out_mode = O_ACCUM;
+    po.add(W->W_o, nullptr, c_s, ACT_NONE, x, O_ACCUM);
     if ((r = launch_proj<T>(po, m, st, "single_attn_out")) != NT_OK) return r;
   }
   return NT_OK;
@@ -686,7 +665,7 @@ nt_status nt_token_update(nt_dtype dt, int32_t c_s, int32_t c_z, int64_t T1, con
   fill_meta(dummy, nullptr, 0, 0, 0, 0, 0);
   ProjArgs pa{};
   pa.A = mvals; pa.a_mode = A_ROWMAJOR; pa.row0 = 0; pa.rows = T1; pa.K = c_z;
-  pa.W1 = W_r; pa.Nout = c_s; pa.act = ACT_NONE; pa.out = x; pa.out_mode = O_ACCUM;
+  pa.add(W_r, nullptr, c_s, ACT_NONE, x, O_ACCUM);
   cudaStream_t st = (cudaStream_t)stream;
   if (dt == NT_F32) return launch_proj<float>(pa, dummy, st, "token_update");
   if (!g_force_generic && fast_token_gemm_supported(c_z, c_s, 0))
@@ -728,10 +707,10 @@ nt_status nt_pair_transition(nt_dtype dt, int32_t c, int32_t hidden, int64_t row
     ProjArgs pa{};
     pa.A = zr; pa.a_mode = A_ROWMAJOR; pa.row0 = 0; pa.rows = n; pa.K = c;
     pa.ln_g = W->ln_gamma; pa.ln_b = W->ln_beta; pa.eps = ln_eps;
-    pa.W1 = W->W_a; pa.W2 = W->W_b; pa.act = ACT_SILU; pa.Nout = hidden; pa.out = hbuf; pa.out_mode = O_STORE;
+    pa.add(W->W_a, W->W_b, hidden, ACT_SILU, hbuf, O_STORE);
     ProjArgs po{};
     po.A = hbuf; po.a_mode = A_ROWMAJOR; po.row0 = 0; po.rows = n; po.K = hidden;
-    po.W1 = W->W_2; po.Nout = c; po.act = ACT_NONE; po.out = zr; po.out_mode = O_ACCUM;
+    po.add(W->W_2, nullptr, c, ACT_NONE, zr, O_ACCUM);
     nt_status r = dt == NT_F32 ? launch_proj<float>(pa, dummy, st, "generic_transition_in")
                                : launch_proj<__nv_bfloat16>(pa, dummy, st, "generic_transition_in");
     if (r != NT_OK) return r;

@@ -1,156 +1,363 @@
 // Shape-generic CUDA-core kernels: tiled projection with LayerNorm / gate prologues and
-// row-major or channel-major epilogues, the per-(sample, channel) triangle contraction, the
-// gather + LayerNorm broadcast, an online-softmax attention core and the segmented reduction.
+// row-major or channel-major epilogues (several outputs of the same rows in one launch), the
+// per-(sample, channel) triangle contraction, the gather + LayerNorm broadcast, an online-softmax
+// attention core and the segmented reduction.
 #include "generic.cuh"
 
 namespace ntp {
 
+// four consecutive elements as floats
+__device__ inline float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
+__device__ inline float4 ld4(const __nv_bfloat16* p) {
+  const uint2 w = *reinterpret_cast<const uint2*>(p);
+  return make_float4(__uint_as_float(w.x << 16), __uint_as_float(w.x & 0xffff0000u), __uint_as_float(w.y << 16), __uint_as_float(w.y & 0xffff0000u));
+}
+__device__ inline void st4(float* p, float4 v) { *reinterpret_cast<float4*>(p) = v; }
+__device__ inline void st4(__nv_bfloat16* p, float4 v) {
+  __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y), hi = __floats2bfloat162_rn(v.z, v.w);
+  *reinterpret_cast<uint2*>(p) = make_uint2(*reinterpret_cast<unsigned*>(&lo), *reinterpret_cast<unsigned*>(&hi));
+}
+// elements k .. k + 3 of a row of K (zero past the end); vec: rows are aligned for four elements at a time
+template <typename T>
+__device__ inline float4 ld4_row(const T* row, int k, int K, bool vec) {
+  if (vec && k + 3 < K) return ld4(row + k);
+  float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (k < K) v.x = Cvt<T>::ld(row + k);
+  if (k + 1 < K) v.y = Cvt<T>::ld(row + k + 1);
+  if (k + 2 < K) v.z = Cvt<T>::ld(row + k + 2);
+  if (k + 3 < K) v.w = Cvt<T>::ld(row + k + 3);
+  return v;
+}
+
 // ------------------------------------------------------------------------------------------
-// projection
+// projection: 64 rows x 64 output columns at a time, K in panels of 32.  The column tiles of all outputs that share their
+// rows are one launch; a block takes one of them where there are few rows (the smallest states are latency and nothing
+// else) and all of them where the rows alone fill the GPU: the rows are then read and normalised once.  The row statistics
+// take one batch of loads for eight rows at a time (a row after the other they were sixteen dependent round trips to
+// memory, 10 of the kernel's 17 us on a 531-row state), the next panel is in registers while one is worked on, and
+// channel-major results leave through shared memory in runs of 64 positions.
 // ------------------------------------------------------------------------------------------
-constexpr int PBM = 64, PBN = 64, PBK = 16, PTHREADS = 256;
+constexpr int PBM = 64, PBN = 64, PBK = 32, PTHREADS = 256, PPITCH = PBM + 4;
+constexpr int PKA = 64;         // A tiles of up to this many columns stay in shared memory for all of a block's column tiles
+constexpr int PSMALL = 8;       // outputs of up to this many columns: one column per thread instead of a 4 x 4 patch
+constexpr int PLN_REGS = 4;     // a row of up to 32 * PLN_REGS elements stays in registers between the two passes
 
 __device__ inline float sigmoidf_acc(float x) { return 1.0f / (1.0f + expf(-x)); }
 
 template <typename T>
-__global__ void __launch_bounds__(PTHREADS) proj_kernel(ProjArgs a, BatchMeta m) {
-  __shared__ __align__(16) float As[PBK][PBM + 4];
-  __shared__ __align__(16) float W1s[PBK][PBN + 4];
-  __shared__ __align__(16) float W2s[PBK][PBN + 4];
+__global__ void __launch_bounds__(PTHREADS, 2) proj_kernel(ProjArgs a, BatchMeta m, int tiles, int tiles_per_block) {
+  __shared__ __align__(16) float As[PKA][PPITCH];
+  __shared__ __align__(16) float Ws[2][PBK][PPITCH];       // W1 | W2; afterwards the result tile of a channel-major output
   __shared__ float mu[PBM], rstd[PBM];
   __shared__ long long cmbase[PBM], inpl[PBM], plane[PBM];
 
   const int t = threadIdx.x;
   const long long r0 = a.row0 + (long long)blockIdx.x * PBM;
   const long long rend = a.row0 + a.rows;
-  const int n0 = blockIdx.y * PBN;
+  int sg = 0, n0 = 0;
+  const int tile0 = blockIdx.y * tiles_per_block, tile1 = min(tiles, tile0 + tiles_per_block);
+  for (int skip = tile0; skip > 0; --skip) {
+    n0 += PBN;
+    if (n0 >= a.seg[sg].Nout) { n0 = 0; ++sg; }
+  }
   const T* A = (const T*)a.A;
   const T* gA = (const T*)a.gateA;
+  const T* lng = (const T*)a.ln_g;
+  const T* lnb = (const T*)a.ln_b;
   const int K = a.K;
-  const bool need_cm = a.a_mode == A_CHANNEL_MAJOR || a.out_mode == O_CHANNEL_MAJOR;
+  const bool rowmajor = a.a_mode == A_ROWMAJOR, has_ln = lng != nullptr, resident = K <= PKA;
+  const bool avec = (K & 3) == 0 && (((uintptr_t)A | (uintptr_t)gA) & 15) == 0;
+  bool need_pos = !rowmajor;
+  for (int x = 0; x < a.nseg; ++x) need_pos |= a.seg[x].out_mode == O_CHANNEL_MAJOR;
 
-  if (t < PBM) {
-    long long p = r0 + t;
-    if (need_cm && p < rend) {
-      int s = find_sample(m.pair_off, m.B, p);
-      int N = m.N[s], ld = round_up8(N);
-      long long r = p - m.pair_off[s];
-      long long i = r / N, j = r - i * N;
+  if (need_pos && t < PBM) {
+    const long long p = r0 + t;
+    if (p < rend) {
+      const int s = find_sample(m.pair_off, m.B, p);
+      const int N = m.N[s], ld = round_up8(N);
+      const long long r = p - m.pair_off[s];
+      const long long i = r / N, j = r - i * N;
       cmbase[t] = m.cm_off[s];
       plane[t] = (long long)N * ld;
       inpl[t] = i * ld + j;
     }
   }
-  __syncthreads();
+  if (!rowmajor) __syncthreads();
 
-  auto loadA = [&](int rl, int k) -> float {
-    long long p = r0 + rl;
-    if (p >= rend || k >= K) return 0.f;
-    float v;
-    if (a.a_mode == A_ROWMAJOR) {
-      v = Cvt<T>::ld(A + p * K + k);
-      if (gA) v *= Cvt<T>::ld(gA + p * K + k);
-    } else {
-      v = Cvt<T>::ld(A + (long long)K * cmbase[rl] + (long long)k * plane[rl] + inpl[rl]);
+  if (has_ln && !rowmajor) {   // two-pass statistics of channel-major rows: lanes along the positions, four threads per row
+    float (*part)[PBM] = reinterpret_cast<float (*)[PBM]>(&As[0][0]);
+    const int rl = t & 63, pt = t >> 6;
+    const T* Ar = A + (r0 + rl < rend ? (long long)K * cmbase[rl] + inpl[rl] : 0);
+    const long long pl = r0 + rl < rend ? plane[rl] : 0;
+    float s = 0.f;
+#pragma unroll 8
+    for (int k = pt; k < K; k += 4) s += Cvt<T>::ld(Ar + k * pl);
+    part[pt][rl] = s;
+    __syncthreads();
+    const float mean = ((part[0][rl] + part[1][rl]) + (part[2][rl] + part[3][rl])) / (float)K;
+    float q = 0.f;
+#pragma unroll 8
+    for (int k = pt; k < K; k += 4) {
+      const float d = Cvt<T>::ld(Ar + k * pl) - mean;
+      q += d * d;
     }
-    return v;
-  };
-
-  const bool has_ln = a.ln_g != nullptr;
-  if (has_ln) {   // two-pass row statistics
+    part[4 + pt][rl] = q;
+    __syncthreads();
+    if (pt == 0) {
+      mu[rl] = mean;
+      rstd[rl] = rsqrtf(((part[4][rl] + part[5][rl]) + (part[6][rl] + part[7][rl])) / (float)K + a.eps);
+    }
+    __syncthreads();
+  } else if (has_ln) {   // two-pass statistics of row-major rows, eight rows per warp
     const int w = t >> 5, lane = t & 31;
-    for (int rl = w; rl < PBM; rl += PTHREADS / 32) {
-      float s = 0.f;
-      for (int k = lane; k < K; k += 32) s += loadA(rl, k);
+    constexpr int RW = PBM / (PTHREADS / 32);
+    auto at = [&](int rl, int k) -> float {
+      const long long p = r0 + rl;
+      if (p >= rend || k >= K) return 0.f;
+      return Cvt<T>::ld(A + p * K + k) * (gA ? Cvt<T>::ld(gA + p * K + k) : 1.f);
+    };
+    float keep[RW][PLN_REGS], s[RW], q[RW];
 #pragma unroll
-      for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-      const float mean = s / (float)K;
-      float q = 0.f;
-      for (int k = lane; k < K; k += 32) {
-        float dlt = loadA(rl, k) - mean;
-        q += dlt * dlt;
+    for (int x = 0; x < RW; ++x)
+#pragma unroll
+      for (int u = 0; u < PLN_REGS; ++u) keep[x][u] = at(w * RW + x, lane + 32 * u);
+#pragma unroll
+    for (int x = 0; x < RW; ++x) {
+      s[x] = (keep[x][0] + keep[x][1]) + (keep[x][2] + keep[x][3]);
+      for (int k = lane + 32 * PLN_REGS; k < K; k += 32) s[x] += at(w * RW + x, k);
+    }
+#pragma unroll
+    for (int o = 16; o; o >>= 1)
+#pragma unroll
+      for (int x = 0; x < RW; ++x) s[x] += __shfl_xor_sync(0xffffffffu, s[x], o);
+#pragma unroll
+    for (int x = 0; x < RW; ++x) {
+      s[x] /= (float)K;
+      q[x] = 0.f;
+#pragma unroll
+      for (int u = 0; u < PLN_REGS; ++u) {
+        const float d = lane + 32 * u < K ? keep[x][u] - s[x] : 0.f;
+        q[x] += d * d;
       }
+      for (int k = lane + 32 * PLN_REGS; k < K; k += 32) {
+        const float d = at(w * RW + x, k) - s[x];
+        q[x] += d * d;
+      }
+    }
 #pragma unroll
-      for (int o = 16; o; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
-      if (lane == 0) {
-        mu[rl] = mean;
-        rstd[rl] = rsqrtf(q / (float)K + a.eps);
+    for (int o = 16; o; o >>= 1)
+#pragma unroll
+      for (int x = 0; x < RW; ++x) q[x] += __shfl_xor_sync(0xffffffffu, q[x], o);
+    if (lane == 0) {
+#pragma unroll
+      for (int x = 0; x < RW; ++x) {
+        mu[w * RW + x] = s[x];
+        rstd[w * RW + x] = rsqrtf(q[x] / (float)K + a.eps);
       }
     }
     __syncthreads();
   }
 
-  const T* W1 = (const T*)a.W1;
-  const T* W2 = (const T*)a.W2;
-  const T* lng = (const T*)a.ln_g;
-  const T* lnb = (const T*)a.ln_b;
-  const int ty = t >> 4, tx = t & 15;
-  float acc1[4][4] = {}, acc2[4][4] = {};
-
-  for (int k0 = 0; k0 < K; k0 += PBK) {
+  // panel loads: thread -> (row, 4 + 4 elements of K) of A (row-major) and W; channel-major A: (position, 8 channels)
+  const int lr = t >> 2, lk = (t & 3) * 4;
+  const int cr = t & 63, ck = (t >> 6) * 8;
+  float4 ra[2], rw[2][2];
+  const T *W1 = nullptr, *W2 = nullptr;
+  int Nout = 0;
+  bool wvec = false;
+  auto open_tile = [&]() {            // (not every entry point asks for aligned weights)
+    W1 = (const T*)a.seg[sg].W1;
+    W2 = (const T*)a.seg[sg].W2;
+    Nout = a.seg[sg].Nout;
+    wvec = (K & 3) == 0 && (((uintptr_t)W1 | (uintptr_t)W2) & 15) == 0;
+  };
+  auto load_a = [&](int k0) {
+    if (rowmajor) {
+      const long long p = r0 + lr;
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      int rl, kk;
-      if (a.a_mode == A_ROWMAJOR) { rl = t >> 2; kk = (t & 3) * 4 + u; }
-      else { rl = t & 63; kk = (t >> 6) + 4 * u; }
-      const int k = k0 + kk;
-      float v = loadA(rl, k);
-      if (has_ln && k < K) v = (v - mu[rl]) * rstd[rl] * Cvt<T>::ld(lng + k) + Cvt<T>::ld(lnb + k);
-      As[kk][rl] = v;
-      const int nl = t >> 2, kw = (t & 3) * 4 + u, n = n0 + nl, k2 = k0 + kw;
-      const bool ok = n < a.Nout && k2 < K;
-      W1s[kw][nl] = ok ? Cvt<T>::ld(W1 + (long long)n * K + k2) : 0.f;
-      if (W2) W2s[kw][nl] = ok ? Cvt<T>::ld(W2 + (long long)n * K + k2) : 0.f;
+      for (int u = 0; u < 2; ++u) {
+        const int k = k0 + lk + 16 * u;
+        ra[u] = p < rend ? ld4_row(A + p * K, k, K, avec) : make_float4(0.f, 0.f, 0.f, 0.f);
+        if (gA && p < rend) {
+          const float4 gv = ld4_row(gA + p * K, k, K, avec);
+          ra[u] = make_float4(ra[u].x * gv.x, ra[u].y * gv.y, ra[u].z * gv.z, ra[u].w * gv.w);
+        }
+      }
+    } else {
+      float v[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int k = k0 + ck + u;
+        v[u] = r0 + cr < rend && k < K ? Cvt<T>::ld(A + (long long)K * cmbase[cr] + (long long)k * plane[cr] + inpl[cr]) : 0.f;
+      }
+      ra[0] = make_float4(v[0], v[1], v[2], v[3]);
+      ra[1] = make_float4(v[4], v[5], v[6], v[7]);
     }
-    __syncthreads();
+  };
+  auto load_w = [&](int k0) {
+    const int n = n0 + lr;
 #pragma unroll
-    for (int kk = 0; kk < PBK; ++kk) {
-      const float4 av = *reinterpret_cast<const float4*>(&As[kk][ty * 4]);
-      const float4 wv = *reinterpret_cast<const float4*>(&W1s[kk][tx * 4]);
-      const float ar[4] = {av.x, av.y, av.z, av.w};
-      const float wr[4] = {wv.x, wv.y, wv.z, wv.w};
+    for (int u = 0; u < 2; ++u) {
+      const int k = k0 + lk + 16 * u;
+      rw[0][u] = n < Nout ? ld4_row(W1 + (long long)n * K, k, K, wvec) : make_float4(0.f, 0.f, 0.f, 0.f);
+      if (W2) rw[1][u] = n < Nout ? ld4_row(W2 + (long long)n * K, k, K, wvec) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+  };
+  auto put_a = [&](int k0, int at) {
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const float av[4] = {ra[u].x, ra[u].y, ra[u].z, ra[u].w};
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const int row = rowmajor ? lr : cr, kk = rowmajor ? lk + 16 * u + e : ck + 4 * u + e, k = k0 + kk;
+        float v = av[e];
+        if (has_ln && k < K) v = (v - mu[row]) * rstd[row] * Cvt<T>::ld(lng + k) + Cvt<T>::ld(lnb + k);
+        As[at + kk][row] = v;
+      }
+    }
+  };
+  auto put_w = [&]() {
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const float w1[4] = {rw[0][u].x, rw[0][u].y, rw[0][u].z, rw[0][u].w};
+      const float w2[4] = {rw[1][u].x, rw[1][u].y, rw[1][u].z, rw[1][u].w};
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        Ws[0][lk + 16 * u + e][lr] = w1[e];
+        if (W2) Ws[1][lk + 16 * u + e][lr] = w2[e];
+      }
+    }
+  };
+  const int ty = t >> 4, tx = t & 15;
+  const T* gO = (const T*)a.gateO;
+  open_tile();
+  load_a(0);
+  load_w(0);
+  for (int tile = tile0; tile < tile1; ++tile) {
+    const ProjSeg g = a.seg[sg];
+    const bool small = g.Nout <= PSMALL && resident, gated = g.W2 != nullptr;
+    const int nt0 = n0;                      // first column of this tile (n0 moves on while the tile is worked on)
+    float acc1[4][4] = {}, acc2[4][4] = {};
+    for (int k0 = 0; k0 < K; k0 += PBK) {
+      const bool last = k0 + PBK >= K;
+      const int at = resident ? k0 : 0;
+      if (!resident || tile == tile0) put_a(k0, at);
+      put_w();
+      __syncthreads();
+      if (last && tile + 1 < tile1) {        // the next tile's first panel
+        n0 += PBN;
+        if (n0 >= g.Nout) { n0 = 0; ++sg; }
+        open_tile();
+        load_w(0);
+        if (!resident) load_a(0);
+      } else if (!last) {
+        load_w(k0 + PBK);
+        if (!resident || tile == tile0) load_a(k0 + PBK);
+      }
+      const int kmax = K - k0 < PBK ? K - k0 : PBK;
+      if (small) {                           // column t / 64 (and + 4) of row t % 64
+        for (int kk = 0; kk < kmax; ++kk) {
+          const float av = As[at + kk][t & 63];
+          acc1[0][0] = fmaf(av, Ws[0][kk][t >> 6], acc1[0][0]);
+          acc1[0][1] = fmaf(av, Ws[0][kk][(t >> 6) + 4], acc1[0][1]);
+          if (gated) {
+            acc2[0][0] = fmaf(av, Ws[1][kk][t >> 6], acc2[0][0]);
+            acc2[0][1] = fmaf(av, Ws[1][kk][(t >> 6) + 4], acc2[0][1]);
+          }
+        }
+      } else {
+#pragma unroll 8
+        for (int kk = 0; kk < kmax; ++kk) {
+          const float4 av = *reinterpret_cast<const float4*>(&As[at + kk][ty * 4]);
+          const float4 wv = *reinterpret_cast<const float4*>(&Ws[0][kk][tx * 4]);
+          const float ar[4] = {av.x, av.y, av.z, av.w};
+          const float wr[4] = {wv.x, wv.y, wv.z, wv.w};
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) acc1[i][j] = fmaf(ar[i], wr[j], acc1[i][j]);
+          if (gated) {
+            const float4 w2 = *reinterpret_cast<const float4*>(&Ws[1][kk][tx * 4]);
+            const float w2r[4] = {w2.x, w2.y, w2.z, w2.w};
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+              for (int j = 0; j < 4; ++j) acc2[i][j] = fmaf(ar[i], w2r[j], acc2[i][j]);
+          }
+        }
+      }
+      __syncthreads();
+    }
+    auto finish = [&](float x1, float x2) -> float {
+      if (gated) return (g.act == ACT_SILU ? x1 * sigmoidf_acc(x1) : sigmoidf_acc(x1)) * x2;
+      return g.act == ACT_SIGMOID ? sigmoidf_acc(x1) : x1;
+    };
+    auto store1 = [&](long long p, int n, float v) {
+      if (gO) v *= Cvt<T>::ld(gO + p * g.Nout + n);
+      if (g.out_f32) {
+        float* o = (float*)g.out + p * g.Nout + n;
+        *o = g.out_mode == O_ACCUM ? *o + v : v;
+      } else {
+        T* o = (T*)g.out + p * g.Nout + n;
+        Cvt<T>::st(o, g.out_mode == O_ACCUM ? v + Cvt<T>::ld(o) : v);
+      }
+    };
+    auto store_cm = [&](int rl, int n, float v) {
+      const long long at = (long long)g.Nout * cmbase[rl] + (long long)n * plane[rl] + inpl[rl];
+      if (NT_IN(at, (long long)g.Nout * m.cm_off[m.B], NT_SITE_PROJ_OUT)) Cvt<T>::st((T*)g.out + at, v);
+    };
+    if (small) {
+      const int rl = t & 63;
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const int n = (t >> 6) + 4 * u;
+        if (n >= g.Nout || r0 + rl >= rend || !NT_IN(r0 + rl, a.row0 + a.rows, NT_SITE_PROJ_OUT)) continue;
+        const float v = finish(acc1[0][u], acc2[0][u]);
+        if (g.out_mode == O_CHANNEL_MAJOR) store_cm(rl, n, v);
+        else store1(r0 + rl, n, v);
+      }
+    } else if (g.out_mode == O_CHANNEL_MAJOR) {      // through shared memory: a warp writes 32 consecutive positions of a channel
+      float (*Cs)[PPITCH] = Ws[0];                   // [64 channels][positions]: Ws[0] and Ws[1] are one array of 64 rows
 #pragma unroll
       for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc1[i][j] = fmaf(ar[i], wr[j], acc1[i][j]);
-      if (W2) {
-        const float4 w2 = *reinterpret_cast<const float4*>(&W2s[kk][tx * 4]);
-        const float w2r[4] = {w2.x, w2.y, w2.z, w2.w};
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-          for (int j = 0; j < 4; ++j) acc2[i][j] = fmaf(ar[i], w2r[j], acc2[i][j]);
+        for (int j = 0; j < 4; ++j) Cs[tx * 4 + j][ty * 4 + i] = finish(acc1[i][j], acc2[i][j]);
+      __syncthreads();
+      for (int idx = t; idx < PBM * PBN; idx += PTHREADS) {
+        const int n = nt0 + (idx >> 6), rl = idx & 63;
+        if (n < g.Nout && r0 + rl < rend) store_cm(rl, n, Cs[idx >> 6][rl]);
       }
-    }
-    __syncthreads();
-  }
-
-  const T* gO = (const T*)a.gateO;
+      __syncthreads();
+    } else {
+      const bool ovec = (g.Nout & 3) == 0 && ((uintptr_t)g.out & 15) == 0;
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int rl = ty * 4 + i;
-    const long long p = r0 + rl;
-    if (p >= rend) continue;
+      for (int i = 0; i < 4; ++i) {
+        const long long p = r0 + ty * 4 + i;
+        const int n = nt0 + tx * 4;
+        if (p >= rend || !NT_IN(p, a.row0 + a.rows, NT_SITE_PROJ_OUT) || n >= g.Nout) continue;
+        float v[4];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int n = n0 + tx * 4 + j;
-      if (n >= a.Nout) continue;
-      float v = acc1[i][j];
-      if (W2) v = (a.act == ACT_SILU ? v * sigmoidf_acc(v) : sigmoidf_acc(v)) * acc2[i][j];
-      else if (a.act == ACT_SIGMOID) v = sigmoidf_acc(v);
-      if (gO) v *= Cvt<T>::ld(gO + p * a.Nout + n);
-      if (a.out_mode == O_CHANNEL_MAJOR) {
-        const long long idx = (long long)a.Nout * cmbase[rl] + (long long)n * plane[rl] + inpl[rl];
-        if (NT_IN(idx, (long long)a.Nout * m.cm_off[m.B], NT_SITE_PROJ_OUT)) Cvt<T>::st((T*)a.out + idx, v);
-      } else if (!NT_IN(p, a.row0 + a.rows, NT_SITE_PROJ_OUT)) {
-        // checked build: a row outside [row0, row0 + rows) was recorded and is not written
-      } else if (a.out_f32) {
-        float* o = (float*)a.out + p * a.Nout + n;
-        *o = (a.out_mode == O_ACCUM) ? *o + v : v;
-      } else {
-        T* o = (T*)a.out + p * a.Nout + n;
-        if (a.out_mode == O_ACCUM) v += Cvt<T>::ld(o);
-        Cvt<T>::st(o, v);
+        for (int j = 0; j < 4; ++j) v[j] = finish(acc1[i][j], acc2[i][j]);
+        if (ovec) {                                  // (n is a multiple of 4: the four columns exist)
+          if (gO) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) v[j] *= Cvt<T>::ld(gO + p * g.Nout + n + j);
+          }
+          float4 r = make_float4(v[0], v[1], v[2], v[3]);
+          if (g.out_f32) {
+            float* o = (float*)g.out + p * g.Nout + n;
+            if (g.out_mode == O_ACCUM) { const float4 b = ld4(o); r = make_float4(r.x + b.x, r.y + b.y, r.z + b.z, r.w + b.w); }
+            st4(o, r);
+          } else {
+            T* o = (T*)g.out + p * g.Nout + n;
+            if (g.out_mode == O_ACCUM) { const float4 b = ld4(o); r = make_float4(r.x + b.x, r.y + b.y, r.z + b.z, r.w + b.w); }
+            st4(o, r);
+          }
+        } else {
+#pragma unroll
+          for (int j = 0; j < 4; ++j)
+            if (n + j < g.Nout) store1(p, n + j, v[j]);
+        }
       }
     }
   }
@@ -158,13 +365,18 @@ __global__ void __launch_bounds__(PTHREADS) proj_kernel(ProjArgs a, BatchMeta m)
 
 template <typename T>
 nt_status launch_proj(const ProjArgs& a, const BatchMeta& m, cudaStream_t st, const char* name) {
-  if (a.rows <= 0 || a.Nout <= 0) return NT_OK;
+  long long tiles = 0;
+  for (int s = 0; s < a.nseg; ++s) tiles += (a.seg[s].Nout + PBN - 1) / PBN;
+  if (a.rows <= 0 || tiles <= 0) return NT_OK;
   long long bx = (a.rows + PBM - 1) / PBM;
-  if (bx > 0x7FFFFFFFll) return NT_ERR_UNSUPPORTED;
-  dim3 grid((unsigned)bx, (unsigned)((a.Nout + PBN - 1) / PBN));
+  if (bx > 0x7FFFFFFFll || tiles > 65535) return NT_ERR_UNSUPPORTED;
   {
     LaunchScope ls(name, st);
-    proj_kernel<T><<<grid, PTHREADS, 0, st>>>(a, m);
+    // one column tile per block while that leaves SMs without a block, all of them once the rows alone fill the GPU
+    const long long want = 2 * sm_count();
+    const long long split = bx >= want ? 1 : bx * tiles <= want ? tiles : (want + bx - 1) / bx;
+    const int tpb = (int)((tiles + split - 1) / split);
+    proj_kernel<T><<<dim3((unsigned)bx, (unsigned)((tiles + tpb - 1) / tpb)), PTHREADS, 0, st>>>(a, m, (int)tiles, tpb);
   }
   return cuda_ok();
 }
@@ -174,8 +386,10 @@ template nt_status launch_proj<__nv_bfloat16>(const ProjArgs&, const BatchMeta&,
 // ------------------------------------------------------------------------------------------
 // triangle contraction  t[c][i][j] = sum_k a[c][i][k] b[c][j][k]   (outgoing)
 //                       t[c][i][j] = sum_k a[c][k][i] b[c][k][j]   (incoming)
+// 64 x 64 tiles; the operands arrive four elements at a time (rows start on multiples of 8 elements) and the next panel is
+// in registers while one is worked on.
 // ------------------------------------------------------------------------------------------
-constexpr int CT = 64, CK = 16;
+constexpr int CT = 64, CK = 32;
 
 template <typename T>
 __global__ void __launch_bounds__(256) contract_kernel(const T* __restrict__ a, const T* __restrict__ b,
@@ -199,20 +413,53 @@ __global__ void __launch_bounds__(256) contract_kernel(const T* __restrict__ a, 
   const T* Ap = a + base;
   const T* Bp = b + base;
   const int t = threadIdx.x, ty = t >> 4, tx = t & 15;
+  // outgoing: thread -> (row t / 4, 4 + 4 elements of k); incoming: (k t / 16 and + 16, 4 elements of the row)
+  const int lr = t >> 2, lk = (t & 3) * 4, ik = t >> 4, ir = (t & 15) * 4;
+  float4 ra[2], rb[2];
+  const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+  auto clip = [](float4 v, int left) {      // elements from `left` on are padding
+    if (left < 4) v.w = 0.f;
+    if (left < 3) v.z = 0.f;
+    if (left < 2) v.y = 0.f;
+    if (left < 1) v.x = 0.f;
+    return v;
+  };
+  auto load = [&](int k0) {
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      if (incoming) {
+        const int k = k0 + ik + 16 * u;
+        ra[u] = k < N && i0 + ir < N ? clip(ld4(Ap + (long long)k * ld + i0 + ir), N - i0 - ir) : zero;
+        rb[u] = k < N && j0 + ir < N ? clip(ld4(Bp + (long long)k * ld + j0 + ir), N - j0 - ir) : zero;
+      } else {
+        const int k = k0 + lk + 16 * u;
+        ra[u] = k < N && i0 + lr < N ? clip(ld4(Ap + (long long)(i0 + lr) * ld + k), N - k) : zero;
+        rb[u] = k < N && j0 + lr < N ? clip(ld4(Bp + (long long)(j0 + lr) * ld + k), N - k) : zero;
+      }
+    }
+  };
   float acc[4][4] = {};
+  load(0);
   for (int k0 = 0; k0 < N; k0 += CK) {
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int rl = t >> 2, kk = (t & 3) * 4 + u, k = k0 + kk;
-      const int i = i0 + rl, j = j0 + rl;
-      const long long ia = incoming ? (long long)k * ld + i : (long long)i * ld + k;
-      const long long ib = incoming ? (long long)k * ld + j : (long long)j * ld + k;
-      As[kk][rl] = (i < N && k < N) ? Cvt<T>::ld(Ap + ia) : 0.f;
-      Bs[kk][rl] = (j < N && k < N) ? Cvt<T>::ld(Bp + ib) : 0.f;
+    for (int u = 0; u < 2; ++u) {
+      if (incoming) {
+        *reinterpret_cast<float4*>(&As[ik + 16 * u][ir]) = ra[u];
+        *reinterpret_cast<float4*>(&Bs[ik + 16 * u][ir]) = rb[u];
+      } else {
+        const float av[4] = {ra[u].x, ra[u].y, ra[u].z, ra[u].w}, bv[4] = {rb[u].x, rb[u].y, rb[u].z, rb[u].w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          As[lk + 16 * u + e][lr] = av[e];
+          Bs[lk + 16 * u + e][lr] = bv[e];
+        }
+      }
     }
     __syncthreads();
-#pragma unroll
-    for (int kk = 0; kk < CK; ++kk) {
+    if (k0 + CK < N) load(k0 + CK);
+    const int kmax = N - k0 < CK ? N - k0 : CK;
+#pragma unroll 8
+    for (int kk = 0; kk < kmax; ++kk) {
       const float4 av = *reinterpret_cast<const float4*>(&As[kk][ty * 4]);
       const float4 bv = *reinterpret_cast<const float4*>(&Bs[kk][tx * 4]);
       const float ar[4] = {av.x, av.y, av.z, av.w};
@@ -226,13 +473,12 @@ __global__ void __launch_bounds__(256) contract_kernel(const T* __restrict__ a, 
   }
   T* Tp = tout + base;
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int ii = i0 + ty * 4 + i, jj = j0 + tx * 4 + j;
-      if (ii < N && jj < N && NT_IN(base + (long long)ii * ld + jj, (long long)C * m.cm_off[m.B], NT_SITE_CONTRACT_OUT))
-        Cvt<T>::st(Tp + (long long)ii * ld + jj, acc[i][j]);
-    }
+  for (int i = 0; i < 4; ++i) {
+    const int ii = i0 + ty * 4 + i, jj = j0 + tx * 4;
+    // (jj < N and ld a multiple of 8: the four columns lie inside the row, padding included)
+    if (ii < N && jj < N && NT_IN(base + (long long)ii * ld + jj, (long long)C * m.cm_off[m.B], NT_SITE_CONTRACT_OUT))
+      st4(Tp + (long long)ii * ld + jj, make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]));
+  }
 }
 
 template <typename T>
@@ -255,21 +501,53 @@ template nt_status launch_contract<__nv_bfloat16>(const __nv_bfloat16*, const __
                                                   const BatchMeta&, cudaStream_t, bool);
 
 // ------------------------------------------------------------------------------------------
-// broadcast + LayerNorm (generic widths): one warp per packed position
+// broadcast + LayerNorm (generic widths).  L = 4 .. 32 lanes per packed position, four channels per lane (L = 0: a warp
+// per position, one channel per lane and step, for widths that are not a multiple of 4 or beyond 128).
 // ------------------------------------------------------------------------------------------
-template <typename T>
+template <typename T, int L>
 __global__ void __launch_bounds__(256) broadcast_ln_kernel(const float* __restrict__ u, const float* __restrict__ v,
                                                           const T* __restrict__ gamma, const T* __restrict__ beta,
                                                           float eps, int c_z, T* __restrict__ z, BatchMeta m, int accumulate) {
-  const int lane = threadIdx.x & 31;
-  const long long p = m.pair_off[0] + (long long)blockIdx.x * 8 + (threadIdx.x >> 5);
-  if (p >= m.pair_off[m.B]) return;
-  const int s = find_sample(m.pair_off, m.B, p);
-  const int N = m.N[s];
-  const long long r = p - m.pair_off[s];
+  constexpr int W = L ? L : 32;
+  const int lane = threadIdx.x % W;
+  const long long p = m.pair_off[0] + (long long)blockIdx.x * (256 / W) + threadIdx.x / W;
+  const bool live = p < m.pair_off[m.B];
+  const int s = live ? find_sample(m.pair_off, m.B, p) : 0;
+  const unsigned N = live ? (unsigned)m.N[s] : 1u;
+  const long long r = live ? p - m.pair_off[s] : 0;
   const long long i = r / N, j = r - i * N;
-  const float* ur = u + (m.tok_off[s] + i) * c_z;
-  const float* vr = v + (m.tok_off[s] + j) * c_z;
+  const float* ur = u + (live ? m.tok_off[s] + i : 0) * c_z;
+  const float* vr = v + (live ? m.tok_off[s] + j : 0) * c_z;
+  T* zr = z + p * c_z;
+  const bool ok = live && NT_IN(m.tok_off[s] + i, m.tok_off[m.B], NT_SITE_BROADCAST_OUT) && NT_IN(m.tok_off[s] + j, m.tok_off[m.B], NT_SITE_BROADCAST_OUT);
+  if (L) {
+    const int c = lane * 4;
+    const bool has = ok && c < c_z;
+    float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (has) {
+      const float4 uu = ld4(ur + c), vv = ld4(vr + c);
+      x = make_float4(uu.x + vv.x, uu.y + vv.y, uu.z + vv.z, uu.w + vv.w);
+    }
+    float sum = (x.x + x.y) + (x.z + x.w);
+#pragma unroll
+    for (int o = W / 2; o; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    const float mean = sum / (float)c_z;
+    const float4 d = make_float4(x.x - mean, x.y - mean, x.z - mean, x.w - mean);
+    float q = has ? (d.x * d.x + d.y * d.y) + (d.z * d.z + d.w * d.w) : 0.f;
+#pragma unroll
+    for (int o = W / 2; o; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
+    if (!has) return;
+    const float rs = rsqrtf(q / (float)c_z + eps);
+    const float4 g = ld4(gamma + c), be = ld4(beta + c);
+    float4 y = make_float4(d.x * rs * g.x + be.x, d.y * rs * g.y + be.y, d.z * rs * g.z + be.z, d.w * rs * g.w + be.w);
+    if (accumulate) {
+      const float4 b = ld4(zr + c);
+      y = make_float4(y.x + b.x, y.y + b.y, y.z + b.z, y.w + b.w);
+    }
+    st4(zr + c, y);
+    return;
+  }
+  if (!ok) return;      // (a whole warp)
   float sum = 0.f;
   for (int c = lane; c < c_z; c += 32) sum += ur[c] + vr[c];
 #pragma unroll
@@ -283,10 +561,15 @@ __global__ void __launch_bounds__(256) broadcast_ln_kernel(const float* __restri
 #pragma unroll
   for (int o = 16; o; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
   const float rs = rsqrtf(q / (float)c_z + eps);
-  T* zr = z + p * c_z;
-  if (!NT_IN(m.tok_off[s] + i, m.tok_off[m.B], NT_SITE_BROADCAST_OUT) || !NT_IN(m.tok_off[s] + j, m.tok_off[m.B], NT_SITE_BROADCAST_OUT)) return;
   for (int c = lane; c < c_z; c += 32)
     Cvt<T>::st(zr + c, (ur[c] + vr[c] - mean) * rs * Cvt<T>::ld(gamma + c) + Cvt<T>::ld(beta + c) + (accumulate ? Cvt<T>::ld(zr + c) : 0.f));
+}
+
+template <typename T, int L>
+static void run_broadcast_ln(const float* u, const float* v, const T* gamma, const T* beta, float eps, int c_z, T* z,
+                             const BatchMeta& m, cudaStream_t st, bool accumulate, long long npos) {
+  const int per = 256 / (L ? L : 32);
+  broadcast_ln_kernel<T, L><<<(unsigned)((npos + per - 1) / per), 256, 0, st>>>(u, v, gamma, beta, eps, c_z, z, m, accumulate ? 1 : 0);
 }
 
 template <typename T>
@@ -294,11 +577,16 @@ nt_status launch_broadcast_ln(const float* u, const float* v, const T* gamma, co
                               T* z, const BatchMeta& m, cudaStream_t st, bool accumulate) {
   long long npos = m.pair_off[m.B] - m.pair_off[0];
   if (npos <= 0) return NT_OK;
-  long long blocks = (npos + 7) / 8;
-  if (blocks > 0x7FFFFFFFll) return NT_ERR_UNSUPPORTED;
+  if (npos / 8 + 1 > 0x7FFFFFFFll) return NT_ERR_UNSUPPORTED;
+  // four elements at a time need aligned gamma / beta (the entry points ask 16 bytes of the other arrays only)
+  const bool vec = c_z % 4 == 0 && c_z <= 128 && (((uintptr_t)gamma | (uintptr_t)beta) & 15) == 0;
   {
     LaunchScope ls(accumulate ? "generic_broadcast_ln_add" : "generic_broadcast_ln", st);
-    broadcast_ln_kernel<T><<<(unsigned)blocks, 256, 0, st>>>(u, v, gamma, beta, eps, c_z, z, m, accumulate ? 1 : 0);
+    if (!vec) run_broadcast_ln<T, 0>(u, v, gamma, beta, eps, c_z, z, m, st, accumulate, npos);
+    else if (c_z <= 16) run_broadcast_ln<T, 4>(u, v, gamma, beta, eps, c_z, z, m, st, accumulate, npos);
+    else if (c_z <= 32) run_broadcast_ln<T, 8>(u, v, gamma, beta, eps, c_z, z, m, st, accumulate, npos);
+    else if (c_z <= 64) run_broadcast_ln<T, 16>(u, v, gamma, beta, eps, c_z, z, m, st, accumulate, npos);
+    else run_broadcast_ln<T, 32>(u, v, gamma, beta, eps, c_z, z, m, st, accumulate, npos);
   }
   return cuda_ok();
 }
@@ -309,25 +597,32 @@ template nt_status launch_broadcast_ln<__nv_bfloat16>(const float*, const float*
                                                       const BatchMeta&, cudaStream_t, bool);
 
 // ------------------------------------------------------------------------------------------
-// attention core: one warp per (attention row, head, query); lanes over keys; online softmax.
+// attention core: a block per (attention row, head, block of queries), keys in chunks of 32 staged in shared memory and
+// read by broadcast; LP lanes share a query (DC channels each, LP = 1 up to head dim 32) and keep its q, its accumulator
+// and the running maximum and sum in registers; eight scores are taken between two looks at the maximum.  (One warp per
+// query with the lanes over the keys read K with a stride of H d elements and V once per key and query: 1215 us for
+// lengths 24-110 with 4 heads of 16 in float, 55 now.)
 // pair_order: 0 = token segments, 1 = pair rows (queries and keys run along j of row i), 2 = pair columns (queries
 // and keys run along the first index of column i; the bias of (query, key) is bias[key][query]).
 // ------------------------------------------------------------------------------------------
-constexpr int AQB = 8;      // queries (warps) per block
-constexpr int AD_MAX = 128; // head dim limit of the generic core
+constexpr int AT = 64;        // threads
+constexpr int AKC = 32;       // keys per chunk
+constexpr int AKS = 8;        // keys per softmax step
+constexpr int AD_MAX = 128;   // head dim limit of the generic core
 
-template <typename T>
-__global__ void __launch_bounds__(AQB * 32) attn_core_kernel(const T* __restrict__ q, const T* __restrict__ k,
-                                                            const T* __restrict__ v, const T* __restrict__ bias,
-                                                            T* __restrict__ o, int H, int d, int pair_order,
-                                                            BatchMeta m, int skip_max_n, float bias_scale) {
-  __shared__ float qs[AQB][AD_MAX];
+template <typename T, int DC, int LP>
+__global__ void __launch_bounds__(AT) attn_core_kernel(const T* __restrict__ q, const T* __restrict__ k,
+                                                       const T* __restrict__ v, const T* __restrict__ bias,
+                                                       T* __restrict__ o, int H, int d, int pair_order,
+                                                       BatchMeta m, float bias_scale) {
+  constexpr int DP = DC * LP, QB = AT / LP;
+  __shared__ __align__(16) float Ks[AKC][DP], Vs[AKC][DP];
   long long w = blockIdx.x;
   int s = 0, N = 0, nqb = 0;
   for (; s < m.B; ++s) {
     N = m.N[s];
-    nqb = (N + AQB - 1) / AQB;
-    long long cnt = N <= skip_max_n ? 0 : (long long)(pair_order ? N : (N > 0 ? 1 : 0)) * H * nqb;
+    nqb = (N + QB - 1) / QB;
+    const long long cnt = (long long)(pair_order ? N : (N > 0 ? 1 : 0)) * H * nqb;
     if (w < cnt) break;
     w -= cnt;
   }
@@ -337,84 +632,137 @@ __global__ void __launch_bounds__(AQB * 32) attn_core_kernel(const T* __restrict
   const long long i = w / ((long long)nqb * H);
   const long long base = pair_order == 1 ? m.pair_off[s] + i * N : pair_order == 2 ? m.pair_off[s] + i : m.tok_off[s];
   const long long step = pair_order == 2 ? N : 1;          // packed rows between consecutive queries / keys
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int j = jb * AQB + warp;
-  const int Hd = H * d;
-  const bool active = j < N;
-  if (active)
-    for (int e = lane; e < d; e += 32) qs[warp][e] = Cvt<T>::ld(q + (base + j * step) * Hd + h * d + e);
-  __syncwarp();
-  if (!active) return;
+  const int t = threadIdx.x, part = t % LP;
+  const int j = jb * QB + t / LP;
+  const bool active = j < N, vec = (d & 3) == 0;
+  const bool warp_live = jb * QB + (t & ~31) / LP < N;
+  const long long Hd = (long long)H * d;
+  const int c0 = part * DC;                                // this lane's channels
+  float2 qv[DC / 2], acc[DC / 2];                          // channel pairs: two products per instruction
+#pragma unroll
+  for (int e = 0; e < DC / 2; e += 2) {
+    const float4 x = active ? ld4_row(q + (base + j * step) * Hd + h * d, c0 + 2 * e, d, vec) : make_float4(0.f, 0.f, 0.f, 0.f);
+    qv[e] = make_float2(x.x, x.y);
+    qv[e + 1] = make_float2(x.z, x.w);
+    acc[e] = acc[e + 1] = make_float2(0.f, 0.f);
+  }
   const int ld = round_up8(N);
-  const T* brow = bias ? bias + (long long)H * m.cm_off[s] + (long long)h * N * ld + (pair_order == 2 ? (long long)j : (long long)j * ld) : nullptr;
-  const long long bstep = pair_order == 2 ? ld : 1;
+  const T* plane = bias ? bias + (long long)H * m.cm_off[s] + (long long)h * N * ld : nullptr;
   const float scale = rsqrtf((float)d);
   float mrun = -INFINITY, lrun = 0.f;
-  float oacc[AD_MAX / 32] = {};
-  const int ne = (d + 31) / 32;
-  for (int c0 = 0; c0 < N; c0 += 32) {
-    const int kk = c0 + lane;
-    float sc = -INFINITY;
-    if (kk < N) {
-      const T* kr = k + (base + kk * step) * Hd + h * d;
-      float dot = 0.f;
-      for (int e = 0; e < d; ++e) dot = fmaf(qs[warp][e], Cvt<T>::ld(kr + e), dot);
-      sc = dot * scale;
-      if (brow) sc += Cvt<T>::ld(brow + kk * bstep) * bias_scale;
+  for (int k0 = 0; k0 < N; k0 += AKC) {
+    if (k0) __syncthreads();
+    for (int idx = t; idx < AKC * (DP / 4); idx += AT) {
+      const int r = idx / (DP / 4), c = (idx - r * (DP / 4)) * 4;
+      const bool in = k0 + r < N;
+      const long long at = (base + (in ? k0 + r : 0) * step) * Hd + h * d;
+      const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+      *reinterpret_cast<float4*>(&Ks[r][c]) = in ? ld4_row(k + at, c, d, vec) : zero;
+      *reinterpret_cast<float4*>(&Vs[r][c]) = in ? ld4_row(v + at, c, d, vec) : zero;
     }
-    float cmax = sc;
+    __syncthreads();
+    if (!warp_live) continue;
+    const int lim = min(AKC, N - k0);
+    for (int kk = 0; kk < lim; kk += AKS) {
+      float sc[AKS], b[AKS];
 #pragma unroll
-    for (int of = 16; of; of >>= 1) cmax = fmaxf(cmax, __shfl_xor_sync(0xffffffffu, cmax, of));
-    const float mnew = fmaxf(mrun, cmax);
-    const float corr = expf(mrun - mnew);   // first chunk: exp(-inf) = 0
-    const float pr = (kk < N) ? expf(sc - mnew) : 0.f;
-    float psum = pr;
+      for (int x = 0; x < AKS; ++x) b[x] = 0.f;
+      if (plane && active) {
+        if (pair_order == 2) {
 #pragma unroll
-    for (int of = 16; of; of >>= 1) psum += __shfl_xor_sync(0xffffffffu, psum, of);
-    lrun = lrun * corr + psum;
-    mrun = mnew;
-    for (int u = 0; u < ne; ++u) oacc[u] *= corr;
-    const int lim = min(32, N - c0);
-    for (int k2 = 0; k2 < lim; ++k2) {
-      const float pk = __shfl_sync(0xffffffffu, pr, k2);
-      const T* vr = v + (base + (c0 + k2) * step) * Hd + h * d;
-      for (int u = 0; u < ne; ++u) {
-        const int e = u * 32 + lane;
-        if (e < d) oacc[u] = fmaf(pk, Cvt<T>::ld(vr + e), oacc[u]);
+          for (int x = 0; x < AKS; ++x) b[x] = k0 + kk + x < N ? Cvt<T>::ld(plane + (long long)(k0 + kk + x) * ld + j) : 0.f;
+        } else {      // (pad columns of a row are readable and masked below)
+          const float4 b0 = ld4(plane + (long long)j * ld + k0 + kk), b1 = ld4(plane + (long long)j * ld + k0 + kk + 4);
+          b[0] = b0.x; b[1] = b0.y; b[2] = b0.z; b[3] = b0.w; b[4] = b1.x; b[5] = b1.y; b[6] = b1.z; b[7] = b1.w;
+        }
+      }
+      float mx = -INFINITY;
+#pragma unroll
+      for (int x = 0; x < AKS; ++x) {
+        float2 d2[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+#pragma unroll
+        for (int e = 0; e < DC / 2; e += 2) {
+          const float4 kv = *reinterpret_cast<const float4*>(&Ks[kk + x][c0 + 2 * e]);
+          d2[0] = __ffma2_rn(qv[e], make_float2(kv.x, kv.y), d2[0]);
+          d2[1] = __ffma2_rn(qv[e + 1], make_float2(kv.z, kv.w), d2[1]);
+        }
+        float dot = (d2[0].x + d2[0].y) + (d2[1].x + d2[1].y);
+#pragma unroll
+        for (int of = 1; of < LP; of <<= 1) dot += __shfl_xor_sync(0xffffffffu, dot, of);
+        sc[x] = kk + x < lim ? dot * scale + b[x] * bias_scale : -INFINITY;
+        mx = fmaxf(mx, sc[x]);
+      }
+      const float mnew = fmaxf(mrun, mx);                 // (a step has at least one key: finite)
+      const float corr = expf(mrun - mnew);               // first step: exp(-inf) = 0
+      float sum = 0.f;
+#pragma unroll
+      for (int x = 0; x < AKS; ++x) {
+        sc[x] = expf(sc[x] - mnew);
+        sum += sc[x];
+      }
+      lrun = lrun * corr + sum;
+      mrun = mnew;
+      const float2 corr2 = make_float2(corr, corr);
+#pragma unroll
+      for (int e = 0; e < DC / 2; e += 2) {
+        float2 y0 = __fmul2_rn(acc[e], corr2), y1 = __fmul2_rn(acc[e + 1], corr2);
+#pragma unroll
+        for (int x = 0; x < AKS; ++x) {
+          const float4 vv = *reinterpret_cast<const float4*>(&Vs[kk + x][c0 + 2 * e]);
+          const float2 p2 = make_float2(sc[x], sc[x]);
+          y0 = __ffma2_rn(p2, make_float2(vv.x, vv.y), y0);
+          y1 = __ffma2_rn(p2, make_float2(vv.z, vv.w), y1);
+        }
+        acc[e] = y0;
+        acc[e + 1] = y1;
       }
     }
   }
+  if (!active || !NT_IN(base + j * step, pair_order ? m.pair_off[m.B] : m.tok_off[m.B], NT_SITE_ATTN_OUT)) return;
   const float inv = 1.0f / lrun;
-  for (int u = 0; u < ne; ++u) {
-    const int e = u * 32 + lane;
-    if (e < d && NT_IN(base + j * step, pair_order ? m.pair_off[m.B] : m.tok_off[m.B], NT_SITE_ATTN_OUT))
-      Cvt<T>::st(o + (base + j * step) * Hd + h * d + e, oacc[u] * inv);
+  T* orow = o + (base + j * step) * Hd + h * d;
+#pragma unroll
+  for (int e = 0; e < DC / 2; e += 2) {
+    const int c = c0 + 2 * e;
+    const float r[4] = {acc[e].x * inv, acc[e].y * inv, acc[e + 1].x * inv, acc[e + 1].y * inv};
+    if (vec && c < d) {
+      st4(orow + c, make_float4(r[0], r[1], r[2], r[3]));
+    } else {
+#pragma unroll
+      for (int x = 0; x < 4; ++x)
+        if (c + x < d) Cvt<T>::st(orow + c + x, r[x]);
+    }
   }
 }
 
 template <typename T>
 nt_status launch_attn_core(const T* q, const T* k, const T* v, const T* bias, T* o, int H, int d, int pair_order,
-                           const BatchMeta& m, cudaStream_t st, int skip_max_n, float bias_scale) {
+                           const BatchMeta& m, cudaStream_t st, float bias_scale) {
   if (d > AD_MAX) return NT_ERR_UNSUPPORTED;
+  const int lp = d <= 32 ? 1 : d <= 64 ? 2 : 4, qb = AT / lp;
   long long blocks = 0;
   for (int s = 0; s < m.B; ++s) {
-    long long N = m.N[s], nqb = (N + AQB - 1) / AQB;
-    if (N <= skip_max_n) continue;
+    const long long N = m.N[s], nqb = (N + qb - 1) / qb;
     blocks += (pair_order ? N : (N > 0 ? 1 : 0)) * H * nqb;
   }
   if (blocks == 0) return NT_OK;
   if (blocks > 0x7FFFFFFFll) return NT_ERR_UNSUPPORTED;
   {
     LaunchScope ls(pair_order == 2 ? "generic_attn_core_col" : "generic_attn_core", st);
-    attn_core_kernel<T><<<(unsigned)blocks, AQB * 32, 0, st>>>(q, k, v, bias, o, H, d, pair_order, m, skip_max_n, bias_scale);
+    const unsigned g = (unsigned)blocks;
+    if (d <= 8) attn_core_kernel<T, 8, 1><<<g, AT, 0, st>>>(q, k, v, bias, o, H, d, pair_order, m, bias_scale);
+    else if (d <= 16) attn_core_kernel<T, 16, 1><<<g, AT, 0, st>>>(q, k, v, bias, o, H, d, pair_order, m, bias_scale);
+    else if (d <= 32) attn_core_kernel<T, 32, 1><<<g, AT, 0, st>>>(q, k, v, bias, o, H, d, pair_order, m, bias_scale);
+    else if (d <= 64) attn_core_kernel<T, 32, 2><<<g, AT, 0, st>>>(q, k, v, bias, o, H, d, pair_order, m, bias_scale);
+    else attn_core_kernel<T, 32, 4><<<g, AT, 0, st>>>(q, k, v, bias, o, H, d, pair_order, m, bias_scale);
   }
   return cuda_ok();
 }
 template nt_status launch_attn_core<float>(const float*, const float*, const float*, const float*, float*, int, int,
-                                           int, const BatchMeta&, cudaStream_t, int, float);
+                                           int, const BatchMeta&, cudaStream_t, float);
 template nt_status launch_attn_core<__nv_bfloat16>(const __nv_bfloat16*, const __nv_bfloat16*, const __nv_bfloat16*,
                                                    const __nv_bfloat16*, __nv_bfloat16*, int, int, int,
-                                                   const BatchMeta&, cudaStream_t, int, float);
+                                                   const BatchMeta&, cudaStream_t, float);
 
 // ------------------------------------------------------------------------------------------
 // segmented reduction (generic widths): one block per group
@@ -431,6 +779,7 @@ __global__ void __launch_bounds__(256) segment_reduce_kernel(const T* __restrict
   if (C >= 256) {
     for (int c = t; c < C; c += 256) {
       float acc = 0.f;
+#pragma unroll 8
       for (long long r = lo; r < hi; ++r) acc += Cvt<T>::ld(v + r * C + c);
       Cvt<T>::st(out + g * C + c, acc * sc);
     }
@@ -439,8 +788,10 @@ __global__ void __launch_bounds__(256) segment_reduce_kernel(const T* __restrict
   const int RS = 256 / C;
   const int ch = t % C, slot = t / C;
   float acc = 0.f;
-  if (slot < RS)
+  if (slot < RS) {
+#pragma unroll 8
     for (long long r = lo + slot; r < hi; r += RS) acc += Cvt<T>::ld(v + r * C + ch);
+  }
   part[t] = acc;
   __syncthreads();
   if (t < C) {

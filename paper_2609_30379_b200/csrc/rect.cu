@@ -166,10 +166,12 @@ static nt_status rect_broadcast_impl(nt_dtype dt, int B, const int64_t* ln, cons
     if ((r = fast_token_gemm(y, t1m, c_s, W_b, c_z, v, nullptr, 0, nullptr, 1, 0, "rect_tok_proj_v", st)) != NT_OK) return r;
   } else {
     ProjArgs pa{};
-    pa.a_mode = A_ROWMAJOR; pa.row0 = 0; pa.K = c_s; pa.Nout = c_z; pa.act = ACT_NONE; pa.out_mode = O_STORE; pa.out_f32 = 1;
-    pa.A = x; pa.rows = t1n; pa.W1 = W_a; pa.out = u;
+    pa.a_mode = A_ROWMAJOR; pa.row0 = 0; pa.K = c_s;
+    pa.A = x; pa.rows = t1n;
+    pa.add(W_a, nullptr, c_z, ACT_NONE, u, O_STORE, 1);
     if (t1n > 0 && (r = launch_proj<T>(pa, dummy, st, "rect_tok_proj_u")) != NT_OK) return r;
-    pa.A = y; pa.rows = t1m; pa.W1 = W_b; pa.out = v;
+    pa.A = y; pa.rows = t1m; pa.nseg = 0;
+    pa.add(W_b, nullptr, c_z, ACT_NONE, v, O_STORE, 1);
     if (t1m > 0 && (r = launch_proj<T>(pa, dummy, st, "rect_tok_proj_v")) != NT_OK) return r;
   }
   if (fast && (r = fast_broadcast_prep(bp, t1n, t1m, g, c_z, st, "rect_broadcast_prep")) != NT_OK) return r;
