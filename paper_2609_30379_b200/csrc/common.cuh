@@ -91,6 +91,36 @@ struct LaunchScope {
   int slot;
 };
 
+// Launch with programmatic stream serialisation: the kernel may be set up while its predecessor in the stream drains, and
+// waits for it in pdl_begin, which every kernel of the library calls before it touches global memory.  (2.4 -> 1.9 us of
+// host time per launch, and the launch latency, barrier set-up and TMEM allocation of a small kernel run in the shadow of
+// the one before.)
+template <typename... KArgs, typename... Args>
+inline void launch_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+#ifdef __CUDACC__
+// Every thread: waits until the kernels before this one in the stream are complete and their writes visible.  A grid that
+// leaves SMs free lets its successor in at once (the successor then waits in its own pdl_begin); a grid that fills the GPU
+// does not: the successor's blocks could only sit beside it (2.37 -> 2.41 ms for the near-uniform stack when they did).
+// Loads before this point, and loads the compiler may move there (const __restrict__, __ldg), must not read what an
+// earlier kernel wrote.
+__device__ inline void pdl_begin() {
+  if (gridDim.x * gridDim.y < 128) asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+  asm volatile("griddepcontrol.wait;\n" ::: "memory");
+}
+#endif
+
 // Reports the pending CUDA error (and where it was seen) on stderr and maps it to NT_ERR_CUDA.
 nt_status cuda_fail(const char* where);
 

@@ -403,6 +403,7 @@ __global__ void __launch_bounds__(128 + 128 * NT, 1) attn_fr_kernel(const __grid
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  pdl_begin();
   const unsigned tmem_base = __shfl_sync(0xffffffffu, tmem_base_s, 0);
   AbortCtx ab{p.status, &abort_flag};
   const unsigned nstage = (unsigned)p.nstage;
@@ -726,7 +727,7 @@ static nt_status launch_attn_fr(AttnFrParams& p, int n_min, cudaStream_t st) {
   const unsigned grid = (unsigned)(items < sms ? items : sms);
   {
     LaunchScope ls(p.mode == FR_MODE_TOKEN ? "attn_core_tok" : p.mode == FR_MODE_PAIR_COL ? "attn_core_col" : "attn_core", st);
-    attn_fr_kernel<D, HAS_BIAS, NT><<<grid, 128 + 128 * NT, fr_smem_bytes(D, HAS_BIAS, p.nstage), st>>>(p);
+    launch_kernel(attn_fr_kernel<D, HAS_BIAS, NT>, grid, 128 + 128 * NT, fr_smem_bytes(D, HAS_BIAS, p.nstage), st, p);
   }
   return cuda_ok("attention launch");
 }

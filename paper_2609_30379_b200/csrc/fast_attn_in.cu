@@ -90,6 +90,7 @@ __global__ void __launch_bounds__(AI_THREADS, 1) attn_in_kernel(const __grid_con
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  pdl_begin();
   const unsigned tmem_base = tmem_base_s;
   AbortCtx ab{p.status, &abort_flag};
   const long long ntiles = (p.rows + 127) / 128;
@@ -346,7 +347,7 @@ nt_status fast_attn_in(const void* z, const AttnPrep& ap, float eps, int c, int 
     const unsigned grid = (unsigned)(ntiles < sm_count() ? ntiles : sm_count());
     {
       LaunchScope ls("attn_in", st);
-      attn_in_kernel<<<grid, AI_THREADS, smem, st>>>(p);
+      launch_kernel(attn_in_kernel, grid, AI_THREADS, smem, st, p);
     }
     if (cudaPeekAtLastError() != cudaSuccess) return cuda_fail("attn_in launch");
   }

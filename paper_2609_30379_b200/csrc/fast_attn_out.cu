@@ -92,6 +92,7 @@ __global__ void __launch_bounds__(AO_THREADS, 1) attn_out_kernel(const __grid_co
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  pdl_begin();
   const unsigned tmem_base = tmem_base_s;
   AbortCtx ab{p.status, &abort_flag};
   const long long ntiles = (p.rows + 127) / 128;
@@ -160,7 +161,7 @@ __global__ void __launch_bounds__(AO_THREADS, 1) attn_out_kernel(const __grid_co
     unsigned phase = 0;
     for (long long t = blockIdx.x; t < ntiles; t += gridDim.x) {
       if (p.zstats) {                       // the input projection normalised the same rows: take its statistics
-        const float2 zst = t * 128 + row < p.rows ? __ldg(p.zstats + t * 128 + row) : make_float2(0.f, 1.f);
+        const float2 zst = t * 128 + row < p.rows ? *(p.zstats + t * 128 + row) : make_float2(0.f, 1.f);
         mbar_wait(&afull[stage], phase, ab);
         sStats[stage][row] = zst;
         __syncwarp();
@@ -335,9 +336,10 @@ __global__ void __launch_bounds__(AO_THREADS, 1) attn_out_kernel(const __grid_co
 // Adds the partial column sums of every pair row (= token row g of the group) in ascending position order.  Group
 // mt of 32 positions keeps the sum of the row that holds its first position in slot 0 and of the row that starts
 // inside it in slot 1.
-__global__ void __launch_bounds__(128) segment_partials_kernel(const float* __restrict__ partial, BatchMeta m,
+__global__ void __launch_bounds__(128) segment_partials_kernel(const float* partial, BatchMeta m,
                                                                long long P0, int C, int mean,
-                                                               __nv_bfloat16* __restrict__ out) {
+                                                               __nv_bfloat16* out) {
+  pdl_begin();
   const long long g = m.tok_off[0] + blockIdx.x;
   const int s = find_sample(m.tok_off, m.B, g);
   const long long N = m.N[s];
@@ -375,7 +377,7 @@ nt_status fast_segment_partials(const float* partial, const BatchMeta& m, int C,
   if (G > 0x7FFFFFFFll) return NT_ERR_UNSUPPORTED;
   {
     LaunchScope ls("segment_partials", st);
-    segment_partials_kernel<<<(unsigned)G, 128, 0, st>>>(partial, m, m.pair_off[0], C, mean, (__nv_bfloat16*)out);
+    launch_kernel(segment_partials_kernel, (unsigned)G, 128, 0, st, partial, m, m.pair_off[0], C, mean, (__nv_bfloat16*)out);
   }
   return cuda_ok();
 }
@@ -440,7 +442,7 @@ nt_status fast_attn_out(void* z, const void* o, const void* W_o, const AttnPrep&
   const unsigned grid = (unsigned)(ntiles < sm_count() ? ntiles : sm_count());
   {
     LaunchScope ls("attn_out", st);
-    attn_out_kernel<<<grid, AO_THREADS, smem, st>>>(p);
+    launch_kernel(attn_out_kernel, grid, AO_THREADS, smem, st, p);
   }
   if (cudaPeekAtLastError() != cudaSuccess) return cuda_fail("attn_out launch");
   return NT_OK;

@@ -135,6 +135,7 @@ __global__ void __launch_bounds__(TCA_THREADS, 1) attn_tc_kernel(const __grid_co
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  pdl_begin();
   const unsigned tmem_base = tmem_base_s;
   AbortCtx ab{p.status, &abort_flag};
   const float sc2 = rsqrtf((float)D) * TCA_LOG2E;
@@ -518,7 +519,7 @@ static nt_status launch_attn_tc(const __nv_bfloat16* q, const __nv_bfloat16* k, 
   const unsigned grid = (unsigned)(total < sm_count() ? total : sm_count());
   {
     LaunchScope ls(COL ? "attn_core_col" : "attn_core", st);
-    attn_tc_kernel<D, COL><<<grid, TCA_THREADS, smem, st>>>(p);
+    launch_kernel(attn_tc_kernel<D, COL>, grid, TCA_THREADS, smem, st, p);
   }
   return cuda_ok("attention tc launch");
 }

@@ -52,7 +52,8 @@ __device__ inline void bl_cp4(void* dst, const void* src) {
 // ------------------------------------------------------------------------------------------
 template <int C>
 __global__ void __launch_bounds__(256) broadcast_prep_kernel(BcastPrepared p, long long rows_u, long long rows_v,
-                                                             const __nv_bfloat16* __restrict__ gamma) {
+                                                             const __nv_bfloat16* gamma) {
+  pdl_begin();
   constexpr int FPL = C > 128 ? C / 128 : 1;       // 16-byte pieces per lane
   constexpr int RPI = C < 128 ? 128 / C : 1;       // rows per warp
   constexpr int LR = 32 / RPI;                     // lanes per row
@@ -135,10 +136,11 @@ __device__ inline void bl_stage(const BcastPrepared& p, bool col_side, long long
 
 template <int C, bool ACC>       // ACC: z += the broadcast (persistent pair stream) instead of z = the broadcast
 __global__ void __launch_bounds__(256, BL_OCC) broadcast_ln_moments_kernel(BcastPrepared p,
-                                                                           const __nv_bfloat16* __restrict__ gamma,
-                                                                           const __nv_bfloat16* __restrict__ beta,
-                                                                           float eps, __nv_bfloat16* __restrict__ z,
+                                                                           const __nv_bfloat16* gamma,
+                                                                           const __nv_bfloat16* beta,
+                                                                           float eps, __nv_bfloat16* z,
                                                                            BcastGeom m, long long n_cols) {
+  pdl_begin();
   constexpr int LP = C / 16;                       // lanes per position in the streaming loop
   constexpr int PPW = 32 / LP;                     // positions per warp-wide instruction
   constexpr int VS = C / 4 + 1;                    // float row pitch in 16-byte pieces
@@ -324,9 +326,9 @@ nt_status fast_broadcast_prep(const BcastPrepared& p, long long rows_u, long lon
   const unsigned blocks = (unsigned)((rows + rpb - 1) / rpb);
   const __nv_bfloat16* g = (const __nv_bfloat16*)gamma;
   LaunchScope ls(scope, st);
-  if (c_z == 64) broadcast_prep_kernel<64><<<blocks, 256, 0, st>>>(p, rows_u, rows_v, g);
-  else if (c_z == 128) broadcast_prep_kernel<128><<<blocks, 256, 0, st>>>(p, rows_u, rows_v, g);
-  else broadcast_prep_kernel<256><<<blocks, 256, 0, st>>>(p, rows_u, rows_v, g);
+  if (c_z == 64) launch_kernel(broadcast_prep_kernel<64>, blocks, 256, 0, st, p, rows_u, rows_v, g);
+  else if (c_z == 128) launch_kernel(broadcast_prep_kernel<128>, blocks, 256, 0, st, p, rows_u, rows_v, g);
+  else launch_kernel(broadcast_prep_kernel<256>, blocks, 256, 0, st, p, rows_u, rows_v, g);
   return cuda_ok();
 }
 
@@ -355,7 +357,7 @@ static nt_status bl_launch(const BcastPrepared& p, const __nv_bfloat16* g, const
   const long long cap = (long long)sm_count() * BL_OCC;
   if (blocks > cap) blocks = cap;
   LaunchScope ls(scope, st);
-  broadcast_ln_moments_kernel<C, ACC><<<(unsigned)blocks, 256, smem, st>>>(p, g, b, eps, z, m, items);
+  launch_kernel(broadcast_ln_moments_kernel<C, ACC>, (unsigned)blocks, 256, smem, st, p, g, b, eps, z, m, items);
   return NT_OK;
 }
 

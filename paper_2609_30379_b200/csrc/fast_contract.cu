@@ -79,6 +79,7 @@ __global__ void __launch_bounds__(CT_THREADS, 1) tri_contract_kernel(const __gri
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  pdl_begin();
   const unsigned tmem_base = tmem_base_s;
   AbortCtx ab{p.status, &abort_flag};
   const long long njobs = p.job_off[p.B];
@@ -262,8 +263,8 @@ nt_status fast_contract(const void* a, size_t buf_stride_bytes, int C, const Bat
     const unsigned grid = (unsigned)(njobs < sm_count() ? njobs : sm_count());
     {
       LaunchScope ls(incoming ? "tri_contract_in" : "tri_contract", st);
-      if (incoming) tri_contract_kernel<true><<<grid, CT_THREADS, CT_SMEM, st>>>(p);
-      else tri_contract_kernel<false><<<grid, CT_THREADS, CT_SMEM, st>>>(p);
+      if (incoming) launch_kernel(tri_contract_kernel<true>, grid, CT_THREADS, CT_SMEM, st, p);
+      else launch_kernel(tri_contract_kernel<false>, grid, CT_THREADS, CT_SMEM, st, p);
     }
     if (cudaPeekAtLastError() != cudaSuccess) return cuda_fail("tensor-core kernel launch");
   }

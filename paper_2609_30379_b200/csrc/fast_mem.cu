@@ -13,10 +13,11 @@ constexpr int SR_THREADS = 128;
 constexpr int SR_UNROLL = 4;
 constexpr int SR_CHUNK = 128;     // channels per block
 
-__global__ void __launch_bounds__(SR_THREADS) segment_reduce_fast_kernel(const __nv_bfloat16* __restrict__ v,
-                                                                        __nv_bfloat16* __restrict__ out,
-                                                                        const int64_t* __restrict__ splits, int C,
+__global__ void __launch_bounds__(SR_THREADS) segment_reduce_fast_kernel(const __nv_bfloat16* v,
+                                                                        __nv_bfloat16* out,
+                                                                        const int64_t* splits, int C,
                                                                         int mean) {
+  pdl_begin();
   extern __shared__ float part[];   // [RS][Cc]
   // a block reduces one group over a chunk of up to 128 channels (blockIdx.y): wide rows keep several row slots
   const int CV = C >> 3;                                  // 16-byte vectors per row
@@ -35,7 +36,7 @@ __global__ void __launch_bounds__(SR_THREADS) segment_reduce_fast_kernel(const _
     for (; r + (long long)(SR_UNROLL - 1) * RS < hi; r += (long long)SR_UNROLL * RS) {
       uint4 d[SR_UNROLL];
 #pragma unroll
-      for (int uu = 0; uu < SR_UNROLL; ++uu) d[uu] = __ldg(base + (r + (long long)uu * RS) * CV);
+      for (int uu = 0; uu < SR_UNROLL; ++uu) d[uu] = *(base + (r + (long long)uu * RS) * CV);
 #pragma unroll
       for (int uu = 0; uu < SR_UNROLL; ++uu) {
         const unsigned w[4] = {d[uu].x, d[uu].y, d[uu].z, d[uu].w};
@@ -47,7 +48,7 @@ __global__ void __launch_bounds__(SR_THREADS) segment_reduce_fast_kernel(const _
       }
     }
     for (; r < hi; r += RS) {
-      const uint4 d = __ldg(base + r * CV);
+      const uint4 d = *(base + r * CV);
       const unsigned w[4] = {d.x, d.y, d.z, d.w};
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
@@ -78,7 +79,7 @@ nt_status fast_segment_reduce(const void* v, void* out, const int64_t* splits, l
   const dim3 grid((unsigned)G, (unsigned)((C + SR_CHUNK - 1) / SR_CHUNK));
   {
     LaunchScope ls("segment_reduce", st);
-    segment_reduce_fast_kernel<<<grid, SR_THREADS, smem, st>>>((const __nv_bfloat16*)v, (__nv_bfloat16*)out,
+    launch_kernel(segment_reduce_fast_kernel, grid, SR_THREADS, smem, st, (const __nv_bfloat16*)v, (__nv_bfloat16*)out,
                                                                      splits, C, mean);
   }
   return cuda_ok();
@@ -106,6 +107,7 @@ struct TokGemmArgs {
 };
 
 __global__ void __launch_bounds__(256) token_gemm_kernel(TokGemmArgs a) {
+  pdl_begin();
   extern __shared__ __align__(16) unsigned char tg_smem[];
   const int K = a.K, ldk = K + 8;
   __nv_bfloat16* As = reinterpret_cast<__nv_bfloat16*>(tg_smem);
@@ -179,6 +181,7 @@ __device__ inline void tg_mma(float (&c)[4], const unsigned (&a)[4], unsigned b0
 }
 
 __global__ void __launch_bounds__(256) token_gemm_mma_kernel(TokGemmArgs a) {
+  pdl_begin();
   extern __shared__ __align__(16) unsigned char tg_smem[];
   const int K = a.K, ldk = K + 8;                      // row pitch 16 bytes off a multiple of 128: conflict-free ldmatrix
   __nv_bfloat16* As = reinterpret_cast<__nv_bfloat16*>(tg_smem);
@@ -272,7 +275,7 @@ nt_status fast_token_gemm(const void* A, long long rows, int K, const void* W0, 
       dim3 grid64((unsigned)bx64, (unsigned)((N0 + N1) / 64));
       {
         LaunchScope ls(name, st);
-        token_gemm_mma_kernel<<<grid64, 256, smem64, st>>>(a);
+        launch_kernel(token_gemm_mma_kernel, grid64, 256, smem64, st, a);
       }
       return cuda_ok(name);
     }
@@ -292,7 +295,7 @@ nt_status fast_token_gemm(const void* A, long long rows, int K, const void* W0, 
   dim3 grid((unsigned)bx, (unsigned)((N0 + N1) / 32));
   {
     LaunchScope ls(name, st);
-    token_gemm_kernel<<<grid, 256, smem, st>>>(a);
+    launch_kernel(token_gemm_kernel, grid, 256, smem, st, a);
   }
   return cuda_ok(name);
 }
@@ -305,9 +308,10 @@ nt_status fast_token_gemm(const void* A, long long rows, int K, const void* W0, 
 namespace ntp {
 
 // LayerNorm of token rows, bf16 in / bf16 out: one warp per row, 16-byte loads.
-__global__ void __launch_bounds__(256) ln_rows_kernel(const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __restrict__ gamma,
-                                                      const __nv_bfloat16* __restrict__ beta, float eps, int C, long long rows,
-                                                      __nv_bfloat16* __restrict__ out) {
+__global__ void __launch_bounds__(256) ln_rows_kernel(const __nv_bfloat16* x, const __nv_bfloat16* gamma,
+                                                      const __nv_bfloat16* beta, float eps, int C, long long rows,
+                                                      __nv_bfloat16* out) {
+  pdl_begin();
   const long long r = (long long)blockIdx.x * 8 + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (r >= rows) return;
@@ -356,7 +360,8 @@ __global__ void __launch_bounds__(256) ln_rows_kernel(const __nv_bfloat16* __res
 }
 
 // o <- sigmoid(g) * o, elementwise on bf16 (eight elements per thread)
-__global__ void __launch_bounds__(256) gate_mul_kernel(const __nv_bfloat16* __restrict__ g, __nv_bfloat16* __restrict__ o, long long n8) {
+__global__ void __launch_bounds__(256) gate_mul_kernel(const __nv_bfloat16* g, __nv_bfloat16* o, long long n8) {
+  pdl_begin();
   const long long i = (long long)blockIdx.x * 256 + threadIdx.x;
   if (i >= n8) return;
   const uint4 gv = *reinterpret_cast<const uint4*>(g + i * 8);
@@ -380,10 +385,11 @@ __global__ void __launch_bounds__(256) gate_mul_kernel(const __nv_bfloat16* __re
 // warp writes each head's 32 values as one run.
 constexpr int SB_MAXH = 8;
 template <int HT>      // heads the arithmetic runs over (H <= HT; rows H .. HT - 1 of the weight table are zeros)
-__global__ void __launch_bounds__(256) single_bias_kernel(const __nv_bfloat16* __restrict__ z, const __nv_bfloat16* __restrict__ gamma,
-                                                          const __nv_bfloat16* __restrict__ beta, const __nv_bfloat16* __restrict__ Wb,
+__global__ void __launch_bounds__(256) single_bias_kernel(const __nv_bfloat16* z, const __nv_bfloat16* gamma,
+                                                          const __nv_bfloat16* beta, const __nv_bfloat16* Wb,
                                                           float eps, int C, int H, float scale, BatchMeta m,
-                                                          __nv_bfloat16* __restrict__ bias) {
+                                                          __nv_bfloat16* bias) {
+  pdl_begin();
   extern __shared__ float sbw[];            // [HT][C] folded weights, then c0[HT], c1[HT]
   float* c0 = sbw + HT * C;
   float* c1 = c0 + SB_MAXH;
@@ -501,10 +507,11 @@ __device__ inline void mma_bf16_16816(float (&c)[4], const unsigned (&a)[4], uns
 }
 
 template <int NK>
-__global__ void __launch_bounds__(256) single_bias_mma_kernel(const __nv_bfloat16* __restrict__ z, const __nv_bfloat16* __restrict__ gamma,
-                                                              const __nv_bfloat16* __restrict__ beta, const __nv_bfloat16* __restrict__ Wb,
+__global__ void __launch_bounds__(256) single_bias_mma_kernel(const __nv_bfloat16* z, const __nv_bfloat16* gamma,
+                                                              const __nv_bfloat16* beta, const __nv_bfloat16* Wb,
                                                               float eps, int H, float scale, BatchMeta m,
-                                                              __nv_bfloat16* __restrict__ bias) {
+                                                              __nv_bfloat16* bias) {
+  pdl_begin();
   constexpr int C = 16 * NK;
   __shared__ __nv_bfloat16 sW[4][C];        // W' rounded to bf16 (rows H .. 3 zero)
   __shared__ float c0[4], c1[4];
@@ -606,7 +613,7 @@ nt_status fast_ln_rows(const void* x, const void* g, const void* b, float eps, i
   if (rows <= 0) return NT_OK;
   {
     LaunchScope ls(name, st);
-    ln_rows_kernel<<<(unsigned)((rows + 7) / 8), 256, 0, st>>>((const __nv_bfloat16*)x, (const __nv_bfloat16*)g, (const __nv_bfloat16*)b, eps, C,
+    launch_kernel(ln_rows_kernel, (unsigned)((rows + 7) / 8), 256, 0, st, (const __nv_bfloat16*)x, (const __nv_bfloat16*)g, (const __nv_bfloat16*)b, eps, C,
                                                                rows, (__nv_bfloat16*)out);
   }
   return cuda_ok("single attention LayerNorm launch");
@@ -617,7 +624,7 @@ nt_status fast_gate_mul(const void* g, void* o, long long n, cudaStream_t st, co
   const long long n8 = n / 8;
   {
     LaunchScope ls(name, st);
-    gate_mul_kernel<<<(unsigned)((n8 + 255) / 256), 256, 0, st>>>((const __nv_bfloat16*)g, (__nv_bfloat16*)o, n8);
+    launch_kernel(gate_mul_kernel, (unsigned)((n8 + 255) / 256), 256, 0, st, (const __nv_bfloat16*)g, (__nv_bfloat16*)o, n8);
   }
   return cuda_ok("single attention gate launch");
 }
@@ -635,10 +642,10 @@ nt_status fast_single_bias(const void* z, const void* g, const void* b, const vo
     {
       LaunchScope ls("single_attn_bias", st);
       if (C == 128)
-        single_bias_mma_kernel<8><<<gridm, 256, 0, st>>>((const __nv_bfloat16*)z, (const __nv_bfloat16*)g, (const __nv_bfloat16*)b,
+        launch_kernel(single_bias_mma_kernel<8>, gridm, 256, 0, st, (const __nv_bfloat16*)z, (const __nv_bfloat16*)g, (const __nv_bfloat16*)b,
                                                          (const __nv_bfloat16*)Wb, eps, H, scale, m, (__nv_bfloat16*)bias);
       else
-        single_bias_mma_kernel<4><<<gridm, 256, 0, st>>>((const __nv_bfloat16*)z, (const __nv_bfloat16*)g, (const __nv_bfloat16*)b,
+        launch_kernel(single_bias_mma_kernel<4>, gridm, 256, 0, st, (const __nv_bfloat16*)z, (const __nv_bfloat16*)g, (const __nv_bfloat16*)b,
                                                          (const __nv_bfloat16*)Wb, eps, H, scale, m, (__nv_bfloat16*)bias);
     }
     return cuda_ok("single attention bias launch");
@@ -648,10 +655,10 @@ nt_status fast_single_bias(const void* z, const void* g, const void* b, const vo
   {
     LaunchScope ls("single_attn_bias", st);
     if (HT == 4)
-      single_bias_kernel<4><<<grid, 256, smem, st>>>((const __nv_bfloat16*)z, (const __nv_bfloat16*)g, (const __nv_bfloat16*)b,
+      launch_kernel(single_bias_kernel<4>, grid, 256, smem, st, (const __nv_bfloat16*)z, (const __nv_bfloat16*)g, (const __nv_bfloat16*)b,
                                                      (const __nv_bfloat16*)Wb, eps, C, H, scale, m, (__nv_bfloat16*)bias);
     else
-      single_bias_kernel<8><<<grid, 256, smem, st>>>((const __nv_bfloat16*)z, (const __nv_bfloat16*)g, (const __nv_bfloat16*)b,
+      launch_kernel(single_bias_kernel<8>, grid, 256, smem, st, (const __nv_bfloat16*)z, (const __nv_bfloat16*)g, (const __nv_bfloat16*)b,
                                                      (const __nv_bfloat16*)Wb, eps, C, H, scale, m, (__nv_bfloat16*)bias);
   }
   return cuda_ok("single attention bias launch");

@@ -23,6 +23,7 @@ struct PrepJob {
 struct PrepArgs { PrepJob job[2]; int njobs; };
 
 __global__ void __launch_bounds__(256) ln_fold_prep_kernel(PrepArgs a) {
+  pdl_begin();
   int n = blockIdx.x * 8 + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   int j = 0;
@@ -128,7 +129,7 @@ static nt_status run_prep(const PrepArgs& a, cudaStream_t st) {
   for (int j = 0; j < a.njobs; ++j) total += a.job[j].total;
   {
     LaunchScope ls("weight_prep", st);
-    ln_fold_prep_kernel<<<(total + 7) / 8, 256, 0, st>>>(a);
+    launch_kernel(ln_fold_prep_kernel, (total + 7) / 8, 256, 0, st, a);
   }
   return cuda_ok("weight_prep launch");
 }

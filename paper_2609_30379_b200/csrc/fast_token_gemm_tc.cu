@@ -57,6 +57,7 @@ __global__ void __launch_bounds__(TG_THREADS, 1) token_gemm_tc_kernel(const __gr
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  pdl_begin();
   const unsigned tmem_base = tmem_base_s;
   AbortCtx ab{p.status, &abort_flag};
   const int ncol = p.ntile[0] + p.ntile[1];
@@ -214,7 +215,7 @@ static nt_status launch_tg(TokGemmTcParams& p, const char* name, cudaStream_t st
   const int sms = sm_count();
   {
     LaunchScope ls(name, st);
-    token_gemm_tc_kernel<BN><<<(unsigned)(njobs < sms ? njobs : sms), TG_THREADS, smem, st>>>(p);
+    launch_kernel(token_gemm_tc_kernel<BN>, (unsigned)(njobs < sms ? njobs : sms), TG_THREADS, smem, st, p);
   }
   return cuda_ok(name);
 }

@@ -125,6 +125,7 @@ __global__ void __launch_bounds__(TR_THREADS, 1) transition_kernel(const __grid_
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  pdl_begin();
   const unsigned tmem_base = tmem_base_s;
   AbortCtx ab{p.status, &abort_flag};
   const long long ntiles = (p.rows + 127) / 128;
@@ -400,7 +401,7 @@ nt_status fast_transition(void* z, const nt_transition_weights* W, float eps, in
   const unsigned grid = (unsigned)(npairs < sm_count() ? npairs : sm_count());
   {
     LaunchScope ls("transition", st);
-    transition_kernel<<<grid, TR_THREADS, smem, st>>>(p);
+    launch_kernel(transition_kernel, grid, TR_THREADS, smem, st, p);
   }
   return cuda_ok("transition launch");
 }

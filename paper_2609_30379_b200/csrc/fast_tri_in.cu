@@ -115,6 +115,7 @@ __global__ void __launch_bounds__(TI_THREADS, 1) tri_in_kernel(const __grid_cons
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  pdl_begin();
   const unsigned tmem_base = tmem_base_s;
   AbortCtx ab{p.status, &abort_flag};
   const long long nchunks = p.chunk_off[p.B];
@@ -419,7 +420,7 @@ nt_status fast_tri_in(const void* z, const TriPrep& tp, float eps, int c_z, int 
     const unsigned grid = (unsigned)(ntiles < sm_count() ? ntiles : sm_count());
     {
       LaunchScope ls("tri_in", st);
-      tri_in_kernel<<<grid, TI_THREADS, smem, st>>>(p);
+      launch_kernel(tri_in_kernel, grid, TI_THREADS, smem, st, p);
     }
     if (cudaPeekAtLastError() != cudaSuccess) return cuda_fail("tri_in launch");
   }

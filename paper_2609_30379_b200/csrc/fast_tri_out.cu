@@ -115,6 +115,7 @@ __global__ void __launch_bounds__(TO_THREADS, 1) tri_out_kernel(const __grid_con
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  pdl_begin();
   const unsigned tmem_base = tmem_base_s;
   AbortCtx ab{p.status, &abort_flag};
   const long long nchunks = p.chunk_off[p.B];
@@ -204,7 +205,7 @@ __global__ void __launch_bounds__(TO_THREADS, 1) tri_out_kernel(const __grid_con
         if (to_decode(p, 2 * t + q, s_, i_, j_)) {
           eps_t = p.eps / ((float)p.N[s_] * (float)p.N[s_]);
           const int j = j_ + (row & 63);
-          if (p.zstats && j < p.N[s_]) zst = __ldg(p.zstats + p.pos_off[s_] + (long long)i_ * p.N[s_] + j);
+          if (p.zstats && j < p.N[s_]) zst = *(p.zstats + p.pos_off[s_] + (long long)i_ * p.N[s_] + j);
         }
       }
       mbar_wait(&tfullb[stage], phase, ab);
@@ -451,7 +452,7 @@ nt_status fast_tri_out(void* z, const void* t, const TriPrep& tp, float eps, int
     const unsigned grid = (unsigned)(ntiles < sm_count() ? ntiles : sm_count());
     {
       LaunchScope ls("tri_out", st);
-      tri_out_kernel<<<grid, TO_THREADS, smem, st>>>(p);
+      launch_kernel(tri_out_kernel, grid, TO_THREADS, smem, st, p);
     }
     if (cudaPeekAtLastError() != cudaSuccess) return cuda_fail("tri_out launch");
   }

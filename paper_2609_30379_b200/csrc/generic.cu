@@ -46,6 +46,7 @@ __device__ inline float sigmoidf_acc(float x) { return 1.0f / (1.0f + expf(-x));
 
 template <typename T>
 __global__ void __launch_bounds__(PTHREADS, 2) proj_kernel(ProjArgs a, BatchMeta m, int tiles, int tiles_per_block) {
+  pdl_begin();
   __shared__ __align__(16) float As[PKA][PPITCH];
   __shared__ __align__(16) float Ws[2][PBK][PPITCH];       // W1 | W2; afterwards the result tile of a channel-major output
   __shared__ float mu[PBM], rstd[PBM];
@@ -376,7 +377,7 @@ nt_status launch_proj(const ProjArgs& a, const BatchMeta& m, cudaStream_t st, co
     const long long want = 2 * sm_count();
     const long long split = bx >= want ? 1 : bx * tiles <= want ? tiles : (want + bx - 1) / bx;
     const int tpb = (int)((tiles + split - 1) / split);
-    proj_kernel<T><<<dim3((unsigned)bx, (unsigned)((tiles + tpb - 1) / tpb)), PTHREADS, 0, st>>>(a, m, (int)tiles, tpb);
+    launch_kernel(proj_kernel<T>, dim3((unsigned)bx, (unsigned)((tiles + tpb - 1) / tpb)), PTHREADS, 0, st, a, m, (int)tiles, tpb);
   }
   return cuda_ok();
 }
@@ -392,8 +393,9 @@ template nt_status launch_proj<__nv_bfloat16>(const ProjArgs&, const BatchMeta&,
 constexpr int CT = 64, CK = 32;
 
 template <typename T>
-__global__ void __launch_bounds__(256) contract_kernel(const T* __restrict__ a, const T* __restrict__ b,
-                                                      T* __restrict__ tout, int C, BatchMeta m, int incoming) {
+__global__ void __launch_bounds__(256) contract_kernel(const T* a, const T* b,
+                                                      T* tout, int C, BatchMeta m, int incoming) {
+  pdl_begin();
   __shared__ __align__(16) float As[CK][CT + 4];
   __shared__ __align__(16) float Bs[CK][CT + 4];
   long long w = blockIdx.x;
@@ -492,7 +494,7 @@ nt_status launch_contract(const T* a, const T* b, T* t, int C, const BatchMeta& 
   if (tiles > 0x7FFFFFFFll) return NT_ERR_UNSUPPORTED;
   {
     LaunchScope ls(incoming ? "generic_tri_contract_in" : "generic_tri_contract", st);
-    contract_kernel<T><<<(unsigned)tiles, 256, 0, st>>>(a, b, t, C, m, incoming ? 1 : 0);
+    launch_kernel(contract_kernel<T>, (unsigned)tiles, 256, 0, st, a, b, t, C, m, incoming ? 1 : 0);
   }
   return cuda_ok();
 }
@@ -505,9 +507,10 @@ template nt_status launch_contract<__nv_bfloat16>(const __nv_bfloat16*, const __
 // per position, one channel per lane and step, for widths that are not a multiple of 4 or beyond 128).
 // ------------------------------------------------------------------------------------------
 template <typename T, int L>
-__global__ void __launch_bounds__(256) broadcast_ln_kernel(const float* __restrict__ u, const float* __restrict__ v,
-                                                          const T* __restrict__ gamma, const T* __restrict__ beta,
-                                                          float eps, int c_z, T* __restrict__ z, BatchMeta m, int accumulate) {
+__global__ void __launch_bounds__(256) broadcast_ln_kernel(const float* u, const float* v,
+                                                          const T* gamma, const T* beta,
+                                                          float eps, int c_z, T* z, BatchMeta m, int accumulate) {
+  pdl_begin();
   constexpr int W = L ? L : 32;
   const int lane = threadIdx.x % W;
   const long long p = m.pair_off[0] + (long long)blockIdx.x * (256 / W) + threadIdx.x / W;
@@ -569,7 +572,7 @@ template <typename T, int L>
 static void run_broadcast_ln(const float* u, const float* v, const T* gamma, const T* beta, float eps, int c_z, T* z,
                              const BatchMeta& m, cudaStream_t st, bool accumulate, long long npos) {
   const int per = 256 / (L ? L : 32);
-  broadcast_ln_kernel<T, L><<<(unsigned)((npos + per - 1) / per), 256, 0, st>>>(u, v, gamma, beta, eps, c_z, z, m, accumulate ? 1 : 0);
+  launch_kernel(broadcast_ln_kernel<T, L>, (unsigned)((npos + per - 1) / per), 256, 0, st, u, v, gamma, beta, eps, c_z, z, m, accumulate ? 1 : 0);
 }
 
 template <typename T>
@@ -611,10 +614,11 @@ constexpr int AKS = 8;        // keys per softmax step
 constexpr int AD_MAX = 128;   // head dim limit of the generic core
 
 template <typename T, int DC, int LP>
-__global__ void __launch_bounds__(AT) attn_core_kernel(const T* __restrict__ q, const T* __restrict__ k,
-                                                       const T* __restrict__ v, const T* __restrict__ bias,
-                                                       T* __restrict__ o, int H, int d, int pair_order,
+__global__ void __launch_bounds__(AT) attn_core_kernel(const T* q, const T* k,
+                                                       const T* v, const T* bias,
+                                                       T* o, int H, int d, int pair_order,
                                                        BatchMeta m, float bias_scale) {
+  pdl_begin();
   constexpr int DP = DC * LP, QB = AT / LP;
   __shared__ __align__(16) float Ks[AKC][DP], Vs[AKC][DP];
   long long w = blockIdx.x;
@@ -750,11 +754,11 @@ nt_status launch_attn_core(const T* q, const T* k, const T* v, const T* bias, T*
   {
     LaunchScope ls(pair_order == 2 ? "generic_attn_core_col" : "generic_attn_core", st);
     const unsigned g = (unsigned)blocks;
-    if (d <= 8) attn_core_kernel<T, 8, 1><<<g, AT, 0, st>>>(q, k, v, bias, o, H, d, pair_order, m, bias_scale);
-    else if (d <= 16) attn_core_kernel<T, 16, 1><<<g, AT, 0, st>>>(q, k, v, bias, o, H, d, pair_order, m, bias_scale);
-    else if (d <= 32) attn_core_kernel<T, 32, 1><<<g, AT, 0, st>>>(q, k, v, bias, o, H, d, pair_order, m, bias_scale);
-    else if (d <= 64) attn_core_kernel<T, 32, 2><<<g, AT, 0, st>>>(q, k, v, bias, o, H, d, pair_order, m, bias_scale);
-    else attn_core_kernel<T, 32, 4><<<g, AT, 0, st>>>(q, k, v, bias, o, H, d, pair_order, m, bias_scale);
+    if (d <= 8) launch_kernel(attn_core_kernel<T, 8, 1>, g, AT, 0, st, q, k, v, bias, o, H, d, pair_order, m, bias_scale);
+    else if (d <= 16) launch_kernel(attn_core_kernel<T, 16, 1>, g, AT, 0, st, q, k, v, bias, o, H, d, pair_order, m, bias_scale);
+    else if (d <= 32) launch_kernel(attn_core_kernel<T, 32, 1>, g, AT, 0, st, q, k, v, bias, o, H, d, pair_order, m, bias_scale);
+    else if (d <= 64) launch_kernel(attn_core_kernel<T, 32, 2>, g, AT, 0, st, q, k, v, bias, o, H, d, pair_order, m, bias_scale);
+    else launch_kernel(attn_core_kernel<T, 32, 4>, g, AT, 0, st, q, k, v, bias, o, H, d, pair_order, m, bias_scale);
   }
   return cuda_ok();
 }
@@ -768,8 +772,9 @@ template nt_status launch_attn_core<__nv_bfloat16>(const __nv_bfloat16*, const _
 // segmented reduction (generic widths): one block per group
 // ------------------------------------------------------------------------------------------
 template <typename T>
-__global__ void __launch_bounds__(256) segment_reduce_kernel(const T* __restrict__ v, T* __restrict__ out,
-                                                            const int64_t* __restrict__ splits, int C, int mean) {
+__global__ void __launch_bounds__(256) segment_reduce_kernel(const T* v, T* out,
+                                                            const int64_t* splits, int C, int mean) {
+  pdl_begin();
   __shared__ float part[256];
   const long long g = blockIdx.x;
   const long long lo = splits[g], hi = splits[g + 1];
@@ -808,7 +813,7 @@ nt_status launch_segment_reduce(const T* v, T* out, const int64_t* splits, long 
   if (G > 0x7FFFFFFFll) return NT_ERR_UNSUPPORTED;
   {
     LaunchScope ls("generic_segment_reduce", st);
-    segment_reduce_kernel<T><<<(unsigned)G, 256, 0, st>>>(v, out, splits, C, mean);
+    launch_kernel(segment_reduce_kernel<T>, (unsigned)G, 256, 0, st, v, out, splits, C, mean);
   }
   return cuda_ok();
 }

@@ -8,11 +8,13 @@ namespace ntp {
 constexpr int SCAN_THREADS = 1024;
 
 __global__ void __launch_bounds__(SCAN_THREADS)
-scan_lengths_kernel(const int64_t* __restrict__ len, int B, long long T1, long long T2,
-                    int64_t* __restrict__ tok_off, int64_t* __restrict__ pair_off, int32_t* status) {
+scan_lengths_kernel(const int64_t* len, int B, long long T1, long long T2,
+                    int64_t* tok_off, int64_t* pair_off, int32_t* status) {
+  pdl_begin();
   __shared__ long long s1[SCAN_THREADS], s2[SCAN_THREADS];
   const int t = threadIdx.x;
-  const int per = (B + SCAN_THREADS - 1) / SCAN_THREADS;
+  const int nthreads = blockDim.x;
+  const int per = (B + nthreads - 1) / nthreads;
   const int lo = min(B, t * per), hi = min(B, lo + per);
   long long a = 0, b = 0;
   bool neg = false;
@@ -25,7 +27,7 @@ scan_lengths_kernel(const int64_t* __restrict__ len, int B, long long T1, long l
   s1[t] = a;
   s2[t] = b;
   __syncthreads();
-  for (int off = 1; off < SCAN_THREADS; off <<= 1) {   // inclusive Hillis-Steele scan
+  for (int off = 1; off < nthreads; off <<= 1) {   // inclusive Hillis-Steele scan
     long long va = 0, vb = 0;
     if (t >= off) { va = s1[t - off]; vb = s2[t - off]; }
     __syncthreads();
@@ -41,7 +43,7 @@ scan_lengths_kernel(const int64_t* __restrict__ len, int B, long long T1, long l
     ea += n;
     eb += n * n;
   }
-  if (t == SCAN_THREADS - 1) {
+  if (t == nthreads - 1) {
     tok_off[B] = s1[t];
     pair_off[B] = s2[t];
     if ((s1[t] != T1 || s2[t] != T2) && status) atomicCAS(status, 0, (int)NT_ERR_INCONSISTENT);
@@ -58,9 +60,10 @@ __device__ inline int search_global(const int64_t* off, int B, long long p) {
   return lo;
 }
 
-__global__ void row_splits_kernel(const int64_t* __restrict__ len, const int64_t* __restrict__ tok_off,
-                                  const int64_t* __restrict__ pair_off, int B, long long T1, long long T2,
-                                  int64_t* __restrict__ row_splits) {
+__global__ void row_splits_kernel(const int64_t* len, const int64_t* tok_off,
+                                  const int64_t* pair_off, int B, long long T1, long long T2,
+                                  int64_t* row_splits) {
+  pdl_begin();
   if (tok_off[B] != T1 || pair_off[B] != T2) return;   // inconsistent totals: flagged by the scan
   long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t > T1) return;
@@ -74,10 +77,11 @@ constexpr int DEC_PER_THREAD = 4;
 constexpr int DEC_SMEM_B = 2048;
 
 __global__ void __launch_bounds__(DEC_THREADS)
-decode_kernel(const int64_t* __restrict__ len, const int64_t* __restrict__ tok_off,
-              const int64_t* __restrict__ pair_off, int B, long long T1, long long T2,
-              int32_t* __restrict__ ps, int32_t* __restrict__ pi, int32_t* __restrict__ pj,
-              int64_t* __restrict__ grow, int64_t* __restrict__ gcol) {
+decode_kernel(const int64_t* len, const int64_t* tok_off,
+              const int64_t* pair_off, int B, long long T1, long long T2,
+              int32_t* ps, int32_t* pi, int32_t* pj,
+              int64_t* grow, int64_t* gcol) {
+  pdl_begin();
   if (tok_off[B] != T1 || pair_off[B] != T2) return;
   __shared__ long long so[DEC_SMEM_B + 1];
   const bool in_smem = B <= DEC_SMEM_B;
@@ -146,12 +150,14 @@ extern "C" nt_status nt_offsets_build(const int64_t* lengths_d, int32_t B, int64
 
   {
     LaunchScope ls("offsets_scan", stream);
-    scan_lengths_kernel<<<1, SCAN_THREADS, 0, stream>>>(lengths_d, B, T1, T2, tok_off_d, pair_off_d, status_d);
+    // (a warp's worth of threads for each 32 samples: the scan is one pass of log2(threads) barriers)
+    const unsigned threads = B >= SCAN_THREADS ? SCAN_THREADS : B < 32 ? 32u : (unsigned)((B + 31) / 32 * 32);
+    launch_kernel(scan_lengths_kernel, 1, threads, 0, stream, lengths_d, B, T1, T2, tok_off_d, pair_off_d, status_d);
   }
   if (row_splits_d) {
     long long n = T1 + 1;
     LaunchScope ls("offsets_row_splits", stream);
-    row_splits_kernel<<<(unsigned)((n + 255) / 256), 256, 0, stream>>>(lengths_d, tok_off_d, pair_off_d, B, T1, T2,
+    launch_kernel(row_splits_kernel, (unsigned)((n + 255) / 256), 256, 0, stream, lengths_d, tok_off_d, pair_off_d, B, T1, T2,
                                                                       row_splits_d);
   }
   if ((want_pos || want_gather) && T2 > 0) {
@@ -159,7 +165,7 @@ extern "C" nt_status nt_offsets_build(const int64_t* lengths_d, int32_t B, int64
     long long blocks = (T2 + per_block - 1) / per_block;
     if (blocks > 0x7FFFFFFFll) return NT_ERR_UNSUPPORTED;
     LaunchScope ls("offsets_decode", stream);
-    decode_kernel<<<(unsigned)blocks, DEC_THREADS, 0, stream>>>(lengths_d, tok_off_d, pair_off_d, B, T1, T2,
+    launch_kernel(decode_kernel, (unsigned)blocks, DEC_THREADS, 0, stream, lengths_d, tok_off_d, pair_off_d, B, T1, T2,
                                                                pos_sample_d, pos_i_d, pos_j_d, gather_rows_d,
                                                                gather_cols_d);
   }

@@ -15,9 +15,10 @@ namespace ntp {
 constexpr int RS_THREADS = 1024;
 
 __global__ void __launch_bounds__(RS_THREADS)
-rect_scan_kernel(const int64_t* __restrict__ ln, const int64_t* __restrict__ lm, int B, long long T1n, long long T1m,
-                 long long T2, int64_t* __restrict__ tokn_off, int64_t* __restrict__ tokm_off,
-                 int64_t* __restrict__ pair_off, int32_t* status) {
+rect_scan_kernel(const int64_t* ln, const int64_t* lm, int B, long long T1n, long long T1m,
+                 long long T2, int64_t* tokn_off, int64_t* tokm_off,
+                 int64_t* pair_off, int32_t* status) {
+  pdl_begin();
   __shared__ long long s1[RS_THREADS], s2[RS_THREADS], s3[RS_THREADS];
   const int t = threadIdx.x;
   const int per = (B + RS_THREADS - 1) / RS_THREADS;
@@ -72,9 +73,10 @@ __device__ inline int rect_search(const int64_t* off, int B, long long p) {   //
   return lo;
 }
 
-__global__ void rect_row_splits_kernel(const int64_t* __restrict__ lm, const int64_t* __restrict__ tokn_off,
-                                       const int64_t* __restrict__ pair_off, int B, long long T1n, long long T2,
-                                       int64_t* __restrict__ row_splits) {
+__global__ void rect_row_splits_kernel(const int64_t* lm, const int64_t* tokn_off,
+                                       const int64_t* pair_off, int B, long long T1n, long long T2,
+                                       int64_t* row_splits) {
+  pdl_begin();
   if (tokn_off[B] != T1n || pair_off[B] != T2) return;   // inconsistent totals: flagged by the scan
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t > T1n) return;
@@ -84,8 +86,9 @@ __global__ void rect_row_splits_kernel(const int64_t* __restrict__ lm, const int
 }
 
 __global__ void __launch_bounds__(256)
-rect_decode_kernel(const int64_t* __restrict__ lm, const int64_t* __restrict__ pair_off, int B, long long T2,
-                   int32_t* __restrict__ ps, int32_t* __restrict__ pi, int32_t* __restrict__ pj) {
+rect_decode_kernel(const int64_t* lm, const int64_t* pair_off, int B, long long T2,
+                   int32_t* ps, int32_t* pi, int32_t* pj) {
+  pdl_begin();
   if (pair_off[B] != T2) return;
   const long long p = (long long)blockIdx.x * 256 + threadIdx.x;
   if (p >= T2) return;
@@ -106,9 +109,10 @@ struct RectMeta {
 
 // Shape-generic form: one warp per packed cell (any c_z, float or bf16).
 template <typename T>
-__global__ void __launch_bounds__(256) rect_broadcast_ln_kernel(const float* __restrict__ u, const float* __restrict__ v,
-                                                               const T* __restrict__ gamma, const T* __restrict__ beta,
-                                                               float eps, int c_z, T* __restrict__ z, RectMeta m) {
+__global__ void __launch_bounds__(256) rect_broadcast_ln_kernel(const float* u, const float* v,
+                                                               const T* gamma, const T* beta,
+                                                               float eps, int c_z, T* z, RectMeta m) {
+  pdl_begin();
   const int lane = threadIdx.x & 31;
   const long long p = m.pair_off[0] + (long long)blockIdx.x * 8 + (threadIdx.x >> 5);
   if (p >= m.pair_off[m.B]) return;
@@ -204,7 +208,7 @@ static nt_status rect_broadcast_impl(nt_dtype dt, int B, const int64_t* ln, cons
       const long long blocks = (cells + 7) / 8;
       if (blocks > 0x7FFFFFFFll) return NT_ERR_UNSUPPORTED;
       LaunchScope ls("generic_rect_broadcast_ln", st);
-      rect_broadcast_ln_kernel<T><<<(unsigned)blocks, 256, 0, st>>>(u, v, (const T*)g, (const T*)b, eps, c_z, (T*)z, m);
+      launch_kernel(rect_broadcast_ln_kernel<T>, (unsigned)blocks, 256, 0, st, u, v, (const T*)g, (const T*)b, eps, c_z, (T*)z, m);
     }
     if (cudaPeekAtLastError() != cudaSuccess) return cuda_fail("rectangular broadcast launch");
   }
@@ -229,20 +233,20 @@ nt_status nt_rect_offsets_build(const int64_t* lengths_n_d, const int64_t* lengt
   if (want_pos && !(pos_sample_d && pos_i_d && pos_j_d)) return NT_ERR_INVALID_ARG;
   {
     LaunchScope ls("rect_offsets_scan", stream);
-    rect_scan_kernel<<<1, RS_THREADS, 0, stream>>>(lengths_n_d, lengths_m_d, B, T1n, T1m, T2, tokn_off_d, tokm_off_d, pair_off_d,
+    launch_kernel(rect_scan_kernel, 1, RS_THREADS, 0, stream, lengths_n_d, lengths_m_d, B, T1n, T1m, T2, tokn_off_d, tokm_off_d, pair_off_d,
                                                    status_d);
   }
   if (row_splits_d) {
     const long long n = T1n + 1;
     LaunchScope ls("rect_offsets_row_splits", stream);
-    rect_row_splits_kernel<<<(unsigned)((n + 255) / 256), 256, 0, stream>>>(lengths_m_d, tokn_off_d, pair_off_d, B, T1n, T2,
+    launch_kernel(rect_row_splits_kernel, (unsigned)((n + 255) / 256), 256, 0, stream, lengths_m_d, tokn_off_d, pair_off_d, B, T1n, T2,
                                                                            row_splits_d);
   }
   if (want_pos && T2 > 0) {
     const long long blocks = (T2 + 255) / 256;
     if (blocks > 0x7FFFFFFFll) return NT_ERR_UNSUPPORTED;
     LaunchScope ls("rect_offsets_decode", stream);
-    rect_decode_kernel<<<(unsigned)blocks, 256, 0, stream>>>(lengths_m_d, pair_off_d, B, T2, pos_sample_d, pos_i_d, pos_j_d);
+    launch_kernel(rect_decode_kernel, (unsigned)blocks, 256, 0, stream, lengths_m_d, pair_off_d, B, T2, pos_sample_d, pos_i_d, pos_j_d);
   }
   return cuda_ok();
 }

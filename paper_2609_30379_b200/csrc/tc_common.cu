@@ -53,6 +53,7 @@ bool make_tmap_bf16(CUtensorMap* map, const void* base, int rank, const unsigned
 // at, with a limit of a few thousand clocks.  The warp records NT_ERR_TIMEOUT in the status word, raises the CTA's
 // abort flag and the kernel ends normally: exactly what a kernel does when one of its waits runs out.
 __global__ void expire_wait_kernel(int* status, long long limit_clocks, int* observed) {
+  pdl_begin();
   __shared__ __align__(8) unsigned long long bar;
   __shared__ int abort_flag;
   if (threadIdx.x == 0) {
@@ -73,7 +74,7 @@ __global__ void expire_wait_kernel(int* status, long long limit_clocks, int* obs
 nt_status launch_expire_wait(int* status, long long limit_clocks, int* observed, cudaStream_t st) {
   {
     LaunchScope ls("debug_expire_wait", st);
-    expire_wait_kernel<<<1, 64, 0, st>>>(status, limit_clocks, observed);
+    launch_kernel(expire_wait_kernel, 1, 64, 0, st, status, limit_clocks, observed);
   }
   return cuda_ok("expire wait launch");
 }

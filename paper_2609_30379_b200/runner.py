@@ -107,7 +107,7 @@ class PairStack:
         """forward(x) through a graph captured the first time this stack sees the current lengths and this x buffer,
         and replayed afterwards: the kernel arguments carry the batch's offsets by value, so a captured step is valid
         for one length signature; another signature (Layout.rebuild with other lengths) captures again."""
-        key = (tuple(int(v) for v in self.L.lengths_h), x.data_ptr())
+        key = (self.L.lengths_h.tobytes(), x.data_ptr())
         cache = self.__dict__.setdefault("_graphs", {})
         if key not in cache:
             keep = x.clone()
