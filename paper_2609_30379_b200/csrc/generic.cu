@@ -32,74 +32,83 @@ __device__ inline float4 ld4_row(const T* row, int k, int K, bool vec) {
 // ------------------------------------------------------------------------------------------
 // projection: 64 rows x 64 output columns at a time, K in panels of 32.  The column tiles of all outputs that share their
 // rows are one launch; a block takes one of them where there are few rows (the smallest states are latency and nothing
-// else) and all of them where the rows alone fill the GPU: the rows are then read and normalised once.  The row statistics
-// take one batch of loads for eight rows at a time (a row after the other they were sixteen dependent round trips to
-// memory, 10 of the kernel's 17 us on a 531-row state), the next panel is in registers while one is worked on, and
-// channel-major results leave through shared memory in runs of 64 positions.
+// else) and all of them where the rows alone fill the GPU: the rows are then read and normalised once.  Rows of up to 64
+// elements are normalised in shared memory, the next panel is in registers while one is worked on, and results leave
+// through shared memory in a rolled loop.  The loops are rolled on purpose: on a state of 531 rows a fully unrolled
+// kernel spent its time fetching instructions (17 us a launch for 1500 to 2200 instructions per warp, two thirds of the
+// stalls "no instruction").  VEC: rows of A and W can be read four elements at a time.
 // ------------------------------------------------------------------------------------------
 constexpr int PBM = 64, PBN = 64, PBK = 32, PTHREADS = 256, PPITCH = PBM + 4;
 constexpr int PKA = 64;         // A tiles of up to this many columns stay in shared memory for all of a block's column tiles
 constexpr int PSMALL = 8;       // outputs of up to this many columns: one column per thread instead of a 4 x 4 patch
-constexpr int PLN_REGS = 4;     // a row of up to 32 * PLN_REGS elements stays in registers between the two passes
+constexpr int PTILE = 64 * PPITCH;
+constexpr size_t PSMEM = (size_t)3 * PTILE * sizeof(float);    // A tile | W1 and W2 panels (results later) | gated values
 
 __device__ inline float sigmoidf_acc(float x) { return 1.0f / (1.0f + expf(-x)); }
 
-template <typename T>
-__global__ void __launch_bounds__(PTHREADS, 2) proj_kernel(ProjArgs a, BatchMeta m, int tiles, int tiles_per_block) {
+template <typename T, bool VEC>
+__device__ inline float4 ld4_k(const T* row, int k, int K) {
+  if (VEC) return k < K ? ld4(row + k) : make_float4(0.f, 0.f, 0.f, 0.f);
+  return ld4_row(row, k, K, false);
+}
+
+template <typename T, bool VEC>
+__global__ void __launch_bounds__(PTHREADS, 3) proj_kernel(const __grid_constant__ ProjArgs a, const __grid_constant__ BatchMeta m,
+                                                           int tiles, int tiles_per_block) {
   pdl_begin();
-  __shared__ __align__(16) float As[PKA][PPITCH];
-  __shared__ __align__(16) float Ws[2][PBK][PPITCH];       // W1 | W2; afterwards the result tile of a channel-major output
+  extern __shared__ __align__(16) float psmem[];
+  float* As = psmem;                           // [k][row]
+  float* Ws = psmem + PTILE;                   // W1 [32][column] | W2 [32][column]; afterwards the result tile
+  float* Gs = psmem + 2 * PTILE;               // the second factor of a gated result
   __shared__ float mu[PBM], rstd[PBM];
   __shared__ long long cmbase[PBM], inpl[PBM], plane[PBM];
 
   const int t = threadIdx.x;
   const long long r0 = a.row0 + (long long)blockIdx.x * PBM;
-  const long long rend = a.row0 + a.rows;
+  const int rows = (int)min((long long)PBM, a.row0 + a.rows - r0);
   int sg = 0, n0 = 0;
   const int tile0 = blockIdx.y * tiles_per_block, tile1 = min(tiles, tile0 + tiles_per_block);
   for (int skip = tile0; skip > 0; --skip) {
     n0 += PBN;
     if (n0 >= a.seg[sg].Nout) { n0 = 0; ++sg; }
   }
-  const T* A = (const T*)a.A;
-  const T* gA = (const T*)a.gateA;
+  const T* A = (const T*)a.A + (a.a_mode == A_ROWMAJOR ? r0 * a.K : 0);
+  const T* gA = a.gateA ? (const T*)a.gateA + r0 * a.K : nullptr;
   const T* lng = (const T*)a.ln_g;
   const T* lnb = (const T*)a.ln_b;
   const int K = a.K;
   const bool rowmajor = a.a_mode == A_ROWMAJOR, has_ln = lng != nullptr, resident = K <= PKA;
-  const bool avec = (K & 3) == 0 && (((uintptr_t)A | (uintptr_t)gA) & 15) == 0;
-  bool need_pos = !rowmajor;
-  for (int x = 0; x < a.nseg; ++x) need_pos |= a.seg[x].out_mode == O_CHANNEL_MAJOR;
 
-  if (need_pos && t < PBM) {
+  if (a.need_pos && t < rows) {                // where the block's positions lie in channel-major buffers
     const long long p = r0 + t;
-    if (p < rend) {
-      const int s = find_sample(m.pair_off, m.B, p);
-      const int N = m.N[s], ld = round_up8(N);
-      const long long r = p - m.pair_off[s];
-      const long long i = r / N, j = r - i * N;
-      cmbase[t] = m.cm_off[s];
-      plane[t] = (long long)N * ld;
-      inpl[t] = i * ld + j;
-    }
+    const int s = find_sample(m.pair_off, m.B, p);
+    const int N = m.N[s], ld = round_up8(N);
+    const unsigned long long r = (unsigned long long)(p - m.pair_off[s]);
+    unsigned long long i;
+    if (r >> 32) i = r / (unsigned)N;
+    else i = (unsigned)r / (unsigned)N;
+    cmbase[t] = m.cm_off[s];
+    plane[t] = (long long)N * ld;
+    inpl[t] = (long long)i * ld + (long long)(r - i * N);
   }
   if (!rowmajor) __syncthreads();
 
-  if (has_ln && !rowmajor) {   // two-pass statistics of channel-major rows: lanes along the positions, four threads per row
-    float (*part)[PBM] = reinterpret_cast<float (*)[PBM]>(&As[0][0]);
-    const int rl = t & 63, pt = t >> 6;
-    const T* Ar = A + (r0 + rl < rend ? (long long)K * cmbase[rl] + inpl[rl] : 0);
-    const long long pl = r0 + rl < rend ? plane[rl] : 0;
-    float s = 0.f;
-#pragma unroll 8
-    for (int k = pt; k < K; k += 4) s += Cvt<T>::ld(Ar + k * pl);
+  if (has_ln && !resident) {                   // two-pass row statistics from memory
+    float (*part)[PBM] = reinterpret_cast<float (*)[PBM]>(As);
+    const int rl = rowmajor ? t >> 2 : t & 63, pt = rowmajor ? t & 3 : t >> 6;      // four threads per row
+    const bool in = rl < rows;
+    const T* Ar = rowmajor ? A + (in ? (long long)rl * K : 0) : A + (in ? (long long)K * cmbase[rl] + inpl[rl] : 0);
+    const T* Gr = gA ? gA + (in ? (long long)rl * K : 0) : nullptr;
+    const long long step = rowmajor ? 1 : in ? plane[rl] : 0;
+    float s = 0.f, q = 0.f;
+#pragma unroll 4
+    for (int k = pt; k < K; k += 4) s += Cvt<T>::ld(Ar + k * step) * (Gr ? Cvt<T>::ld(Gr + k) : 1.f);
     part[pt][rl] = s;
     __syncthreads();
     const float mean = ((part[0][rl] + part[1][rl]) + (part[2][rl] + part[3][rl])) / (float)K;
-    float q = 0.f;
-#pragma unroll 8
+#pragma unroll 4
     for (int k = pt; k < K; k += 4) {
-      const float d = Cvt<T>::ld(Ar + k * pl) - mean;
+      const float d = Cvt<T>::ld(Ar + k * step) * (Gr ? Cvt<T>::ld(Gr + k) : 1.f) - mean;
       q += d * d;
     }
     part[4 + pt][rl] = q;
@@ -109,102 +118,46 @@ __global__ void __launch_bounds__(PTHREADS, 2) proj_kernel(ProjArgs a, BatchMeta
       rstd[rl] = rsqrtf(((part[4][rl] + part[5][rl]) + (part[6][rl] + part[7][rl])) / (float)K + a.eps);
     }
     __syncthreads();
-  } else if (has_ln) {   // two-pass statistics of row-major rows, eight rows per warp
-    const int w = t >> 5, lane = t & 31;
-    constexpr int RW = PBM / (PTHREADS / 32);
-    auto at = [&](int rl, int k) -> float {
-      const long long p = r0 + rl;
-      if (p >= rend || k >= K) return 0.f;
-      return Cvt<T>::ld(A + p * K + k) * (gA ? Cvt<T>::ld(gA + p * K + k) : 1.f);
-    };
-    float keep[RW][PLN_REGS], s[RW], q[RW];
-#pragma unroll
-    for (int x = 0; x < RW; ++x)
-#pragma unroll
-      for (int u = 0; u < PLN_REGS; ++u) keep[x][u] = at(w * RW + x, lane + 32 * u);
-#pragma unroll
-    for (int x = 0; x < RW; ++x) {
-      s[x] = (keep[x][0] + keep[x][1]) + (keep[x][2] + keep[x][3]);
-      for (int k = lane + 32 * PLN_REGS; k < K; k += 32) s[x] += at(w * RW + x, k);
-    }
-#pragma unroll
-    for (int o = 16; o; o >>= 1)
-#pragma unroll
-      for (int x = 0; x < RW; ++x) s[x] += __shfl_xor_sync(0xffffffffu, s[x], o);
-#pragma unroll
-    for (int x = 0; x < RW; ++x) {
-      s[x] /= (float)K;
-      q[x] = 0.f;
-#pragma unroll
-      for (int u = 0; u < PLN_REGS; ++u) {
-        const float d = lane + 32 * u < K ? keep[x][u] - s[x] : 0.f;
-        q[x] += d * d;
-      }
-      for (int k = lane + 32 * PLN_REGS; k < K; k += 32) {
-        const float d = at(w * RW + x, k) - s[x];
-        q[x] += d * d;
-      }
-    }
-#pragma unroll
-    for (int o = 16; o; o >>= 1)
-#pragma unroll
-      for (int x = 0; x < RW; ++x) q[x] += __shfl_xor_sync(0xffffffffu, q[x], o);
-    if (lane == 0) {
-#pragma unroll
-      for (int x = 0; x < RW; ++x) {
-        mu[w * RW + x] = s[x];
-        rstd[w * RW + x] = rsqrtf(q[x] / (float)K + a.eps);
-      }
-    }
-    __syncthreads();
   }
 
   // panel loads: thread -> (row, 4 + 4 elements of K) of A (row-major) and W; channel-major A: (position, 8 channels)
   const int lr = t >> 2, lk = (t & 3) * 4;
   const int cr = t & 63, ck = (t >> 6) * 8;
   float4 ra[2], rw[2][2];
-  const T *W1 = nullptr, *W2 = nullptr;
-  int Nout = 0;
-  bool wvec = false;
-  auto open_tile = [&]() {            // (not every entry point asks for aligned weights)
-    W1 = (const T*)a.seg[sg].W1;
-    W2 = (const T*)a.seg[sg].W2;
-    Nout = a.seg[sg].Nout;
-    wvec = (K & 3) == 0 && (((uintptr_t)W1 | (uintptr_t)W2) & 15) == 0;
-  };
+  const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
   auto load_a = [&](int k0) {
     if (rowmajor) {
-      const long long p = r0 + lr;
 #pragma unroll
       for (int u = 0; u < 2; ++u) {
         const int k = k0 + lk + 16 * u;
-        ra[u] = p < rend ? ld4_row(A + p * K, k, K, avec) : make_float4(0.f, 0.f, 0.f, 0.f);
-        if (gA && p < rend) {
-          const float4 gv = ld4_row(gA + p * K, k, K, avec);
+        ra[u] = lr < rows ? ld4_k<T, VEC>(A + (long long)lr * K, k, K) : zero;
+        if (gA && lr < rows) {
+          const float4 gv = ld4_k<T, VEC>(gA + (long long)lr * K, k, K);
           ra[u] = make_float4(ra[u].x * gv.x, ra[u].y * gv.y, ra[u].z * gv.z, ra[u].w * gv.w);
         }
       }
     } else {
       float v[8];
+      const T* Ar = A + (cr < rows ? (long long)K * cmbase[cr] + inpl[cr] : 0);
+      const long long pl = cr < rows ? plane[cr] : 0;
 #pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int k = k0 + ck + u;
-        v[u] = r0 + cr < rend && k < K ? Cvt<T>::ld(A + (long long)K * cmbase[cr] + (long long)k * plane[cr] + inpl[cr]) : 0.f;
-      }
+      for (int u = 0; u < 8; ++u) v[u] = cr < rows && k0 + ck + u < K ? Cvt<T>::ld(Ar + (k0 + ck + u) * pl) : 0.f;
       ra[0] = make_float4(v[0], v[1], v[2], v[3]);
       ra[1] = make_float4(v[4], v[5], v[6], v[7]);
     }
   };
   auto load_w = [&](int k0) {
     const int n = n0 + lr;
+    const T* w1 = (const T*)a.seg[sg].W1 + (long long)n * K;
+    const T* w2 = (const T*)a.seg[sg].W2 + (long long)n * K;
+    const bool in = n < a.seg[sg].Nout, two = a.seg[sg].W2 != nullptr;
 #pragma unroll
     for (int u = 0; u < 2; ++u) {
-      const int k = k0 + lk + 16 * u;
-      rw[0][u] = n < Nout ? ld4_row(W1 + (long long)n * K, k, K, wvec) : make_float4(0.f, 0.f, 0.f, 0.f);
-      if (W2) rw[1][u] = n < Nout ? ld4_row(W2 + (long long)n * K, k, K, wvec) : make_float4(0.f, 0.f, 0.f, 0.f);
+      rw[0][u] = in ? ld4_k<T, VEC>(w1, k0 + lk + 16 * u, K) : zero;
+      rw[1][u] = in && two ? ld4_k<T, VEC>(w2, k0 + lk + 16 * u, K) : zero;
     }
   };
-  auto put_a = [&](int k0, int at) {
+  auto put_a = [&](int k0, int at, bool ln) {
 #pragma unroll
     for (int u = 0; u < 2; ++u) {
       const float av[4] = {ra[u].x, ra[u].y, ra[u].z, ra[u].w};
@@ -212,65 +165,94 @@ __global__ void __launch_bounds__(PTHREADS, 2) proj_kernel(ProjArgs a, BatchMeta
       for (int e = 0; e < 4; ++e) {
         const int row = rowmajor ? lr : cr, kk = rowmajor ? lk + 16 * u + e : ck + 4 * u + e, k = k0 + kk;
         float v = av[e];
-        if (has_ln && k < K) v = (v - mu[row]) * rstd[row] * Cvt<T>::ld(lng + k) + Cvt<T>::ld(lnb + k);
-        As[at + kk][row] = v;
+        if (ln && k < K) v = (v - mu[row]) * rstd[row] * Cvt<T>::ld(lng + k) + Cvt<T>::ld(lnb + k);
+        As[(at + kk) * PPITCH + row] = v;
       }
     }
   };
-  auto put_w = [&]() {
+  auto put_w = [&](bool two) {
 #pragma unroll
     for (int u = 0; u < 2; ++u) {
       const float w1[4] = {rw[0][u].x, rw[0][u].y, rw[0][u].z, rw[0][u].w};
       const float w2[4] = {rw[1][u].x, rw[1][u].y, rw[1][u].z, rw[1][u].w};
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
-        Ws[0][lk + 16 * u + e][lr] = w1[e];
-        if (W2) Ws[1][lk + 16 * u + e][lr] = w2[e];
+        Ws[(lk + 16 * u + e) * PPITCH + lr] = w1[e];
+        if (two) Ws[(PBK + lk + 16 * u + e) * PPITCH + lr] = w2[e];
       }
     }
   };
-  const int ty = t >> 4, tx = t & 15;
-  const T* gO = (const T*)a.gateO;
-  open_tile();
   load_a(0);
   load_w(0);
+  if (resident) {                              // the whole A tile; its LayerNorm in shared memory, four threads per row
+    put_a(0, 0, false);
+    if (K > PBK) {
+      load_a(PBK);
+      put_a(PBK, PBK, false);
+    }
+    __syncthreads();
+    if (has_ln) {
+      const int rl = t >> 2, pt = t & 3;
+      float s = 0.f, q = 0.f;
+#pragma unroll 4
+      for (int k = pt; k < K; k += 4) s += As[k * PPITCH + rl];
+      s += __shfl_xor_sync(0xffffffffu, s, 1);
+      s += __shfl_xor_sync(0xffffffffu, s, 2);
+      const float mean = s / (float)K;
+#pragma unroll 4
+      for (int k = pt; k < K; k += 4) {
+        const float d = As[k * PPITCH + rl] - mean;
+        q += d * d;
+      }
+      q += __shfl_xor_sync(0xffffffffu, q, 1);
+      q += __shfl_xor_sync(0xffffffffu, q, 2);
+      const float rs = rsqrtf(q / (float)K + a.eps);
+#pragma unroll 4
+      for (int k = pt; k < K; k += 4) As[k * PPITCH + rl] = (As[k * PPITCH + rl] - mean) * rs * Cvt<T>::ld(lng + k) + Cvt<T>::ld(lnb + k);
+    }
+  }
+  const int ty = t >> 4, tx = t & 15;
+  const T* gO = (const T*)a.gateO;
+#pragma unroll 1
   for (int tile = tile0; tile < tile1; ++tile) {
     const ProjSeg g = a.seg[sg];
     const bool small = g.Nout <= PSMALL && resident, gated = g.W2 != nullptr;
     const int nt0 = n0;                      // first column of this tile (n0 moves on while the tile is worked on)
     float acc1[4][4] = {}, acc2[4][4] = {};
+#pragma unroll 1
     for (int k0 = 0; k0 < K; k0 += PBK) {
       const bool last = k0 + PBK >= K;
-      const int at = resident ? k0 : 0;
-      if (!resident || tile == tile0) put_a(k0, at);
-      put_w();
+      if (!resident) put_a(k0, 0, has_ln);
+      put_w(gated);
       __syncthreads();
       if (last && tile + 1 < tile1) {        // the next tile's first panel
         n0 += PBN;
         if (n0 >= g.Nout) { n0 = 0; ++sg; }
-        open_tile();
         load_w(0);
         if (!resident) load_a(0);
       } else if (!last) {
         load_w(k0 + PBK);
-        if (!resident || tile == tile0) load_a(k0 + PBK);
+        if (!resident) load_a(k0 + PBK);
       }
-      const int kmax = K - k0 < PBK ? K - k0 : PBK;
+      const int kmax = (min(K - k0, PBK) + 3) & ~3;      // (the panels are zero beyond K)
+      const float* Ak = As + (resident ? k0 : 0) * PPITCH;
       if (small) {                           // column t / 64 (and + 4) of row t % 64
-        for (int kk = 0; kk < kmax; ++kk) {
-          const float av = As[at + kk][t & 63];
-          acc1[0][0] = fmaf(av, Ws[0][kk][t >> 6], acc1[0][0]);
-          acc1[0][1] = fmaf(av, Ws[0][kk][(t >> 6) + 4], acc1[0][1]);
+        const float *ap = Ak + (t & 63), *wp = Ws + (t >> 6);
+#pragma unroll 4
+        for (int kk = 0; kk < kmax; ++kk, ap += PPITCH, wp += PPITCH) {
+          acc1[0][0] = fmaf(*ap, wp[0], acc1[0][0]);
+          acc1[0][1] = fmaf(*ap, wp[4], acc1[0][1]);
           if (gated) {
-            acc2[0][0] = fmaf(av, Ws[1][kk][t >> 6], acc2[0][0]);
-            acc2[0][1] = fmaf(av, Ws[1][kk][(t >> 6) + 4], acc2[0][1]);
+            acc2[0][0] = fmaf(*ap, wp[PBK * PPITCH], acc2[0][0]);
+            acc2[0][1] = fmaf(*ap, wp[PBK * PPITCH + 4], acc2[0][1]);
           }
         }
       } else {
-#pragma unroll 8
-        for (int kk = 0; kk < kmax; ++kk) {
-          const float4 av = *reinterpret_cast<const float4*>(&As[at + kk][ty * 4]);
-          const float4 wv = *reinterpret_cast<const float4*>(&Ws[0][kk][tx * 4]);
+        const float *ap = Ak + ty * 4, *wp = Ws + tx * 4;
+#pragma unroll 4
+        for (int kk = 0; kk < kmax; ++kk, ap += PPITCH, wp += PPITCH) {
+          const float4 av = *reinterpret_cast<const float4*>(ap);
+          const float4 wv = *reinterpret_cast<const float4*>(wp);
           const float ar[4] = {av.x, av.y, av.z, av.w};
           const float wr[4] = {wv.x, wv.y, wv.z, wv.w};
 #pragma unroll
@@ -278,7 +260,7 @@ __global__ void __launch_bounds__(PTHREADS, 2) proj_kernel(ProjArgs a, BatchMeta
 #pragma unroll
             for (int j = 0; j < 4; ++j) acc1[i][j] = fmaf(ar[i], wr[j], acc1[i][j]);
           if (gated) {
-            const float4 w2 = *reinterpret_cast<const float4*>(&Ws[1][kk][tx * 4]);
+            const float4 w2 = *reinterpret_cast<const float4*>(wp + PBK * PPITCH);
             const float w2r[4] = {w2.x, w2.y, w2.z, w2.w};
 #pragma unroll
             for (int i = 0; i < 4; ++i)
@@ -289,11 +271,41 @@ __global__ void __launch_bounds__(PTHREADS, 2) proj_kernel(ProjArgs a, BatchMeta
       }
       __syncthreads();
     }
-    auto finish = [&](float x1, float x2) -> float {
-      if (gated) return (g.act == ACT_SILU ? x1 * sigmoidf_acc(x1) : sigmoidf_acc(x1)) * x2;
-      return g.act == ACT_SIGMOID ? sigmoidf_acc(x1) : x1;
-    };
-    auto store1 = [&](long long p, int n, float v) {
+    // results to shared memory, the faster index of the output innermost, then out in order
+    const bool cm = g.out_mode == O_CHANNEL_MAJOR;
+    const int si = cm ? 1 : PPITCH, sj = cm ? PPITCH : 1;      // step of a row / of a column
+    if (small) {
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        Ws[(t & 63) * si + ((t >> 6) + 4 * u) * sj] = acc1[0][u];
+        if (gated) Gs[(t & 63) * si + ((t >> 6) + 4 * u) * sj] = acc2[0][u];
+      }
+    } else {
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          Ws[(ty * 4 + i) * si + (tx * 4 + j) * sj] = acc1[i][j];
+          if (gated) Gs[(ty * 4 + i) * si + (tx * 4 + j) * sj] = acc2[i][j];
+        }
+    }
+    __syncthreads();
+    const int ncol = min(PBN, g.Nout - nt0);
+    const int total = cm ? ncol * PBM : rows * PBN;
+#pragma unroll 2
+    for (int idx = t; idx < total; idx += PTHREADS) {
+      const int hi = idx >> 6, lo = idx & 63, rl = cm ? lo : hi, n = nt0 + (cm ? hi : lo);
+      if (rl >= rows || n >= g.Nout) continue;
+      const long long p = r0 + rl;
+      float v = Ws[hi * PPITCH + lo];
+      if (gated) v = (g.act == ACT_SILU ? v * sigmoidf_acc(v) : sigmoidf_acc(v)) * Gs[hi * PPITCH + lo];
+      else if (g.act == ACT_SIGMOID) v = sigmoidf_acc(v);
+      if (cm) {
+        const long long at = (long long)g.Nout * cmbase[rl] + (long long)n * plane[rl] + inpl[rl];
+        if (NT_IN(at, (long long)g.Nout * m.cm_off[m.B], NT_SITE_PROJ_OUT)) Cvt<T>::st((T*)g.out + at, v);
+        continue;
+      }
+      if (!NT_IN(p, a.row0 + a.rows, NT_SITE_PROJ_OUT)) continue;
       if (gO) v *= Cvt<T>::ld(gO + p * g.Nout + n);
       if (g.out_f32) {
         float* o = (float*)g.out + p * g.Nout + n;
@@ -302,84 +314,51 @@ __global__ void __launch_bounds__(PTHREADS, 2) proj_kernel(ProjArgs a, BatchMeta
         T* o = (T*)g.out + p * g.Nout + n;
         Cvt<T>::st(o, g.out_mode == O_ACCUM ? v + Cvt<T>::ld(o) : v);
       }
-    };
-    auto store_cm = [&](int rl, int n, float v) {
-      const long long at = (long long)g.Nout * cmbase[rl] + (long long)n * plane[rl] + inpl[rl];
-      if (NT_IN(at, (long long)g.Nout * m.cm_off[m.B], NT_SITE_PROJ_OUT)) Cvt<T>::st((T*)g.out + at, v);
-    };
-    if (small) {
-      const int rl = t & 63;
-#pragma unroll
-      for (int u = 0; u < 2; ++u) {
-        const int n = (t >> 6) + 4 * u;
-        if (n >= g.Nout || r0 + rl >= rend || !NT_IN(r0 + rl, a.row0 + a.rows, NT_SITE_PROJ_OUT)) continue;
-        const float v = finish(acc1[0][u], acc2[0][u]);
-        if (g.out_mode == O_CHANNEL_MAJOR) store_cm(rl, n, v);
-        else store1(r0 + rl, n, v);
-      }
-    } else if (g.out_mode == O_CHANNEL_MAJOR) {      // through shared memory: a warp writes 32 consecutive positions of a channel
-      float (*Cs)[PPITCH] = Ws[0];                   // [64 channels][positions]: Ws[0] and Ws[1] are one array of 64 rows
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) Cs[tx * 4 + j][ty * 4 + i] = finish(acc1[i][j], acc2[i][j]);
-      __syncthreads();
-      for (int idx = t; idx < PBM * PBN; idx += PTHREADS) {
-        const int n = nt0 + (idx >> 6), rl = idx & 63;
-        if (n < g.Nout && r0 + rl < rend) store_cm(rl, n, Cs[idx >> 6][rl]);
-      }
-      __syncthreads();
-    } else {
-      const bool ovec = (g.Nout & 3) == 0 && ((uintptr_t)g.out & 15) == 0;
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const long long p = r0 + ty * 4 + i;
-        const int n = nt0 + tx * 4;
-        if (p >= rend || !NT_IN(p, a.row0 + a.rows, NT_SITE_PROJ_OUT) || n >= g.Nout) continue;
-        float v[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) v[j] = finish(acc1[i][j], acc2[i][j]);
-        if (ovec) {                                  // (n is a multiple of 4: the four columns exist)
-          if (gO) {
-#pragma unroll
-            for (int j = 0; j < 4; ++j) v[j] *= Cvt<T>::ld(gO + p * g.Nout + n + j);
-          }
-          float4 r = make_float4(v[0], v[1], v[2], v[3]);
-          if (g.out_f32) {
-            float* o = (float*)g.out + p * g.Nout + n;
-            if (g.out_mode == O_ACCUM) { const float4 b = ld4(o); r = make_float4(r.x + b.x, r.y + b.y, r.z + b.z, r.w + b.w); }
-            st4(o, r);
-          } else {
-            T* o = (T*)g.out + p * g.Nout + n;
-            if (g.out_mode == O_ACCUM) { const float4 b = ld4(o); r = make_float4(r.x + b.x, r.y + b.y, r.z + b.z, r.w + b.w); }
-            st4(o, r);
-          }
-        } else {
-#pragma unroll
-          for (int j = 0; j < 4; ++j)
-            if (n + j < g.Nout) store1(p, n + j, v[j]);
-        }
-      }
     }
+    __syncthreads();
   }
 }
 
+template <typename T, bool VEC>
+static nt_status run_proj(const ProjArgs& a, const BatchMeta& m, dim3 grid, int tiles, int tpb, cudaStream_t st) {
+  static bool attr_set[64] = {};
+  int dev = 0;
+  cudaGetDevice(&dev);
+  if (!attr_set[dev & 63]) {
+    if (cudaFuncSetAttribute(proj_kernel<T, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PSMEM) != cudaSuccess)
+      return cuda_fail("projection smem attribute");
+    attr_set[dev & 63] = true;
+  }
+  launch_kernel(proj_kernel<T, VEC>, grid, PTHREADS, PSMEM, st, a, m, tiles, tpb);
+  return NT_OK;
+}
+
 template <typename T>
-nt_status launch_proj(const ProjArgs& a, const BatchMeta& m, cudaStream_t st, const char* name) {
+nt_status launch_proj(const ProjArgs& args, const BatchMeta& m, cudaStream_t st, const char* name) {
+  ProjArgs a = args;
   long long tiles = 0;
-  for (int s = 0; s < a.nseg; ++s) tiles += (a.seg[s].Nout + PBN - 1) / PBN;
+  uintptr_t low = (uintptr_t)a.A | (uintptr_t)a.gateA;
+  a.need_pos = a.a_mode != A_ROWMAJOR;
+  for (int s = 0; s < a.nseg; ++s) {
+    tiles += (a.seg[s].Nout + PBN - 1) / PBN;
+    low |= (uintptr_t)a.seg[s].W1 | (uintptr_t)a.seg[s].W2;
+    if (a.seg[s].out_mode == O_CHANNEL_MAJOR) a.need_pos = 1;
+  }
   if (a.rows <= 0 || tiles <= 0) return NT_OK;
   long long bx = (a.rows + PBM - 1) / PBM;
   if (bx > 0x7FFFFFFFll || tiles > 65535) return NT_ERR_UNSUPPORTED;
+  // one column tile per block while that leaves SMs without a block, all of them once the rows alone fill the GPU
+  const long long want = 2 * sm_count();
+  const long long split = bx >= want ? 1 : bx * tiles <= want ? tiles : (want + bx - 1) / bx;
+  const int tpb = (int)((tiles + split - 1) / split);
+  const dim3 grid((unsigned)bx, (unsigned)((tiles + tpb - 1) / tpb));
+  const bool vec = (a.K & 3) == 0 && (low & 15) == 0;      // (not every entry point asks for aligned weights)
+  nt_status r;
   {
     LaunchScope ls(name, st);
-    // one column tile per block while that leaves SMs without a block, all of them once the rows alone fill the GPU
-    const long long want = 2 * sm_count();
-    const long long split = bx >= want ? 1 : bx * tiles <= want ? tiles : (want + bx - 1) / bx;
-    const int tpb = (int)((tiles + split - 1) / split);
-    launch_kernel(proj_kernel<T>, dim3((unsigned)bx, (unsigned)((tiles + tpb - 1) / tpb)), PTHREADS, 0, st, a, m, (int)tiles, tpb);
+    r = vec ? run_proj<T, true>(a, m, grid, (int)tiles, tpb, st) : run_proj<T, false>(a, m, grid, (int)tiles, tpb, st);
   }
-  return cuda_ok();
+  return r != NT_OK ? r : cuda_ok();
 }
 template nt_status launch_proj<float>(const ProjArgs&, const BatchMeta&, cudaStream_t, const char*);
 template nt_status launch_proj<__nv_bfloat16>(const ProjArgs&, const BatchMeta&, cudaStream_t, const char*);

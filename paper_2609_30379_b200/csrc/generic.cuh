@@ -32,6 +32,7 @@ struct ProjArgs {
   const void* ln_b;
   float eps;
   const void* gateO;    // nullable: row-major [.., Nout]; value *= gateO before store/accumulate
+  int need_pos;         // set by launch_proj: some buffer is channel-major
   int nseg;
   ProjSeg seg[PROJ_MAXSEG];
   void add(const void* W1, const void* W2, int Nout, int act, void* out, int out_mode, int out_f32 = 0) {
