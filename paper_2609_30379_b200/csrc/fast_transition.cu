@@ -18,8 +18,8 @@
 // ((-mean_hi, -mean_lo, -mean_hi) per row against (c1_hi, c1_hi, c1_lo) per weight row), rstd and c0 are applied in
 // the gate stage; the z tile itself is only converted bf16 -> fp16 (exact), because it is also the residual.
 // The state tiles are double buffered per tile of the pair: the next pair loads and converts while this one computes.
-// Roles: warp 0 producer (weights ring, state tiles), warps 1 and 14 MMA issuers of tile 0 and tile 1 (converged, one
-// elected lane), warps 2-5 converters (one row per thread), warps 6-9 / 10-13 gate and output stage of tile 0 / 1.
+// Roles: warp 0 producer (weights ring, state tiles), warps 1 and 22 MMA issuers of tile 0 and tile 1 (converged, one
+// elected lane), warps 2-5 converters (one row per thread), warps 6-21 gate and output stage: two groups of four per tile.
 // All waits are bounded.
 #include <cstring>
 
@@ -30,7 +30,9 @@ namespace ntp {
 
 constexpr int TR_CHUNK = 32;                 // hidden units per chunk
 constexpr int TR_WST = 3;                    // weight ring stages
-constexpr int TR_THREADS = 64 + 128 + 256 + 32;
+constexpr int TR_GATE_WARPS = 16;             // two groups of four per tile: even and odd chunks
+constexpr int TR_ISSUER1 = 6 + TR_GATE_WARPS; // warp that issues tile 1's MMAs
+constexpr int TR_THREADS = 32 * (TR_ISSUER1 + 1);
 
 struct TransParams {
   CUtensorMap zmap;      // state {c, rows}, box {64, 128} (loads)
@@ -100,14 +102,14 @@ __global__ void __launch_bounds__(TR_THREADS, 1) transition_kernel(const __grid_
     abort_flag = 0;
     for (int s = 0; s < 4; ++s) {
       mbar_init(&zfull[s], 1);
-      mbar_init(&zempty[s], 4);
+      mbar_init(&zempty[s], 8);
       mbar_init(&zconv[s], 4);
       mbar_init(&gvfull[s], 1);
       mbar_init(&hfull[s], 4);
     }
     for (int s = 0; s < 2; ++s) {
       mbar_init(&ofull[s], 1);
-      mbar_init(&oempty[s], 4);
+      mbar_init(&oempty[s], 8);
     }
     for (int s = 0; s < TR_WST; ++s) {
       mbar_init(&w1full[s], 1);
@@ -176,7 +178,7 @@ __global__ void __launch_bounds__(TR_THREADS, 1) transition_kernel(const __grid_
       if (++q == nchunk) { q = 0; ++pass; }
       if (++st == TR_WST) { st = 0; ph ^= 1; }
     }
-  } else if (warp == 1 || warp == 14) {
+  } else if (warp == 1 || warp == TR_ISSUER1) {
     // ------------------------------------------------------------------ MMA issuer of tile r (whole warp, one elected lane)
     // Order: GEMM 1 of chunk 0; then per chunk g: GEMM 1 of chunk g + 1 (other accumulator buffer), GEMM 2 of chunk g.
     const int r = warp == 1 ? 0 : 1;
@@ -257,60 +259,70 @@ __global__ void __launch_bounds__(TR_THREADS, 1) transition_kernel(const __grid_
         if (lane == 0) mbar_arrive(&zconv[zb]);
       }
     }
-  } else if (warp < 14) {
-    // ------------------------------------------------------------------ gate stage and output stage: warps 6-9 own
-    // tile 0 of the pair, warps 10-13 tile 1; a warp covers 32 rows (its TMEM lane quarter) and all columns
-    const int quarter = warp & 3, r = (warp - 6) >> 2;
+  } else {
+    // ------------------------------------------------------------------ gate stage and output stage: eight warps per tile
+    // of the pair, in two groups that take the even and the odd chunks (one accumulator buffer each); a warp covers 32 rows
+    // (its TMEM lane quarter).  A chunk is a chain of TMEM read, 32 units of arithmetic, TMEM write and two barrier hops,
+    // about 2500 clocks for a warp alone: with one group per tile that chain was the kernel's period.
+    const int quarter = warp & 3, r = ((warp - 6) >> 2) & 1, b = (warp - 6) >> 3;
     const int row = quarter * 32 + lane;
     const unsigned t_lane = tmem_base + ((unsigned)(quarter * 32) << 16);
+    const unsigned t_gv = t_lane + r * 128 + b * 64;
+    const int cpg = c / 2;                                   // output channels of this group
     unsigned g = 0;
     for (int pass = 0; pass < npass; ++pass) {
       const int zb = r * 2 + (pass & 1);
       float rstd = 0.f;
+      bool have = false;
       for (int q = 0; q < nchunk; ++q, ++g) {
-        const unsigned t_gv = t_lane + r * 128 + (g & 1) * 64;
-        mbar_wait(&gvfull[r * 2 + (g & 1)], (g >> 1) & 1, ab);   // GEMM 1 has run, so the converters' statistics are published
+        if ((int)(g & 1) != b) continue;
+        mbar_wait(&gvfull[r * 2 + b], (g >> 1) & 1, ab);     // GEMM 1 has run, so the converters' statistics are published
         tc_fence_after();
-        if (q == 0) rstd = sRstd[zb][row];
-        unsigned rg[32], rv[32];
-        tmem_ld32(t_gv, rg);
-        tmem_ld32(t_gv + 32, rv);
-        tmem_ld_wait();
-        const float4* cg = reinterpret_cast<const float4*>(sC0 + q * TR_CHUNK);
-        const float4* cv = reinterpret_cast<const float4*>(sC0 + hidden + q * TR_CHUNK);
-        unsigned w[16];
+        if (!have) rstd = sRstd[zb][row];
+        have = true;
 #pragma unroll
-        for (int e = 0; e < 8; ++e) {
-          const float4 kg = cg[e], kv = cv[e];
-          const float g0 = fmaf(rstd, __uint_as_float(rg[4 * e]), kg.x), g1 = fmaf(rstd, __uint_as_float(rg[4 * e + 1]), kg.y);
-          const float g2 = fmaf(rstd, __uint_as_float(rg[4 * e + 2]), kg.z), g3 = fmaf(rstd, __uint_as_float(rg[4 * e + 3]), kg.w);
-          const float v0 = fmaf(rstd, __uint_as_float(rv[4 * e]), kv.x), v1 = fmaf(rstd, __uint_as_float(rv[4 * e + 1]), kv.y);
-          const float v2 = fmaf(rstd, __uint_as_float(rv[4 * e + 2]), kv.z), v3 = fmaf(rstd, __uint_as_float(rv[4 * e + 3]), kv.w);
-          // g arrives halved: silu(2 g') = g' tanh(g') + g'
-          const float h0 = fmaf(g0, tr_tanh(g0), g0) * v0, h1 = fmaf(g1, tr_tanh(g1), g1) * v1;
-          const float h2 = fmaf(g2, tr_tanh(g2), g2) * v2, h3 = fmaf(g3, tr_tanh(g3), g3) * v3;
-          __nv_bfloat162 ha = __floats2bfloat162_rn(h0, h1), hb = __floats2bfloat162_rn(h2, h3);
-          w[2 * e] = *reinterpret_cast<unsigned*>(&ha);
-          w[2 * e + 1] = *reinterpret_cast<unsigned*>(&hb);
+        for (int half = 0; half < 2; ++half) {               // 16 units at a time: fewer registers, room for 16 warps
+          unsigned rg[16], rv[16];
+          tmem_ld16(t_gv + half * 16, rg);
+          tmem_ld16(t_gv + 32 + half * 16, rv);
+          tmem_ld_wait2(rg, rv);
+          const float4* cg = reinterpret_cast<const float4*>(sC0 + q * TR_CHUNK + half * 16);
+          const float4* cv = reinterpret_cast<const float4*>(sC0 + hidden + q * TR_CHUNK + half * 16);
+          unsigned w[8];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const float4 kg = cg[e], kv = cv[e];
+            const float2 r2 = make_float2(rstd, rstd);
+            const float2 ga = __ffma2_rn(r2, make_float2(__uint_as_float(rg[4 * e]), __uint_as_float(rg[4 * e + 1])), make_float2(kg.x, kg.y));
+            const float2 gb = __ffma2_rn(r2, make_float2(__uint_as_float(rg[4 * e + 2]), __uint_as_float(rg[4 * e + 3])), make_float2(kg.z, kg.w));
+            const float2 va = __ffma2_rn(r2, make_float2(__uint_as_float(rv[4 * e]), __uint_as_float(rv[4 * e + 1])), make_float2(kv.x, kv.y));
+            const float2 vb = __ffma2_rn(r2, make_float2(__uint_as_float(rv[4 * e + 2]), __uint_as_float(rv[4 * e + 3])), make_float2(kv.z, kv.w));
+            // g arrives halved: silu(2 g') = g' tanh(g') + g'
+            const float2 ha = __fmul2_rn(__ffma2_rn(ga, make_float2(tr_tanh(ga.x), tr_tanh(ga.y)), ga), va);
+            const float2 hb = __fmul2_rn(__ffma2_rn(gb, make_float2(tr_tanh(gb.x), tr_tanh(gb.y)), gb), vb);
+            __nv_bfloat162 pa = __floats2bfloat162_rn(ha.x, ha.y), pb = __floats2bfloat162_rn(hb.x, hb.y);
+            w[2 * e] = *reinterpret_cast<unsigned*>(&pa);
+            w[2 * e + 1] = *reinterpret_cast<unsigned*>(&pb);
+          }
+          tmem_st8(t_gv + half * 8, w);       // over gate columns that are already in registers
         }
-        tmem_st16(t_gv, w);               // over gate columns that are already in registers
         tmem_st_wait();
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive(&hfull[r * 2 + (g & 1)]);
+        if (lane == 0) mbar_arrive(&hfull[r * 2 + b]);
       }
-      // ---- output stage: out + z through the z tile, then one TMA store per 64-channel slab
+      // ---- output stage: out + z through the z tile, half of the channels per group, then one TMA store per 64-channel slab
       const long long t = 2 * ((long long)blockIdx.x + (long long)pass * gridDim.x) + r;
       mbar_wait(&ofull[r], pass & 1, ab);
       tc_fence_after();
       unsigned char* zt = sZ + zb * z_stage;
-      for (int c0 = 0; c0 < c; c0 += 32) {
-        unsigned rr[32];
-        tmem_ld32(t_lane + 256 + r * 128 + c0, rr);
-        tmem_ld_wait();
+      for (int c0 = b * cpg; c0 < (b + 1) * cpg; c0 += 16) {
+        unsigned rr[16];
+        tmem_ld16(t_lane + 256 + r * 128 + c0, rr);
+        tmem_ld_wait16(rr);
         unsigned char* zp = zt + (c0 >> 6) * slab;
 #pragma unroll
-        for (int ch = 0; ch < 4; ++ch) {
+        for (int ch = 0; ch < 2; ++ch) {
           uint4* ptr = reinterpret_cast<uint4*>(zp + sw128_off(row, ((c0 & 63) >> 3) + ch));
           const uint4 v = *ptr;
           unsigned wz[4] = {v.x, v.y, v.z, v.w};
@@ -327,11 +339,13 @@ __global__ void __launch_bounds__(TR_THREADS, 1) transition_kernel(const __grid_
       __syncwarp();
       if (lane == 0) mbar_arrive(&oempty[r]);
       fence_proxy_async_smem();
-      __syncwarp();
+      // two slabs: each group stores its own; one slab: the two warps of a lane quarter share it and the first stores
+      if (nslab == 1) named_bar_sync(1 + r * 4 + quarter, 64);
+      else __syncwarp();
       if (lane == 0) {
         const long long r0 = t * 128 + quarter * 32;
-        if (r0 < p.rows)
-          for (int sl = 0; sl < nslab; ++sl) tma_store_2d(&p.zsmap, zt + sl * slab + quarter * 32 * 128, sl * 64, (int)r0);
+        if (r0 < p.rows && (nslab == 2 || b == 0))
+          tma_store_2d(&p.zsmap, zt + (nslab == 2 ? b : 0) * slab + quarter * 32 * 128, (nslab == 2 ? b : 0) * 64, (int)r0);
         tma_store_commit();
         tma_store_wait_read0();
         mbar_arrive(&zempty[zb]);
