@@ -91,13 +91,14 @@ __global__ void __launch_bounds__(256) ln_fold_prep_kernel(PrepArgs a) {
     J.c01[n] = make_float2(c0, c1);
     if (J.aug) {
       // Extra K columns that make the MMA itself apply the LayerNorm correction: against activation columns
-      // (m_hi, m_lo, m_hi, 1, 1) with m = -mean * rstd they contribute m * c1 + c0 (hi/lo split keeps ~22 bits).
+      // (m_hi, m_lo, m_hi, 1, 1) with m = -mean * rstd they contribute m * c1 + c0 (hi/lo split keeps ~22 bits).  The
+      // columns 5 and 6 serve a reader that has c0 times a factor split into three fp16 parts instead of c0 times 1.
       const __half c1h = __float2half_rn(c1), c1l = __float2half_rn(c1 - __half2float(c1h));
       const __half c0h = __float2half_rn(c0), c0l = __float2half_rn(c0 - __half2float(c0h));
       const __half z = __float2half_rn(0.f);
       __half* r0 = J.aug + (long long)n * 8;
       __half* r1 = J.aug + ((long long)J.total + n) * 8;
-      r0[0] = c1h; r0[1] = c1h; r0[2] = c1l; r0[3] = c0h; r0[4] = c0l; r0[5] = z; r0[6] = z; r0[7] = z;
+      r0[0] = c1h; r0[1] = c1h; r0[2] = c1l; r0[3] = c0h; r0[4] = c0l; r0[5] = c0h; r0[6] = __float2half_rn(__half2float(c0h) * (1.f / 4096.f)); r0[7] = z;
       for (int e = 0; e < 8; ++e) r1[e] = z;
     }
   }
