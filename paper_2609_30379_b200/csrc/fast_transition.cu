@@ -22,8 +22,8 @@
 // (c1_hi, c1_hi, c1_lo, c0_hi, c0_lo, c0_hi, c0_hi / 4096, 0) per weight row, so that rstd times the accumulator is
 // the normalised projection; the z tile itself is only converted bf16 -> fp16 (exact), because it is also the residual.
 // The state tiles are double buffered per tile of the pair: the next pair loads and converts while this one computes.
-// Roles: warp 0 producer (W_1 ring, state tiles), warp 23 producer (W_2 ring), warps 1 and 22 MMA issuers of tile 0 and 1
-// (converged, one elected lane), warps 2-5 converters (one row per thread), warps 6-21 gate and output stage: two groups
+// Roles: warp 0 producer (W_1 ring, state tiles), warp 22 producer (W_2 ring), warp 1 MMA issuer (converged, one
+// elected lane), warps 2-5 converters (one row per thread), warps 6-21 gate and output stage: two groups
 // of four per tile.  All waits are bounded.
 #include <cstring>
 
@@ -36,8 +36,7 @@ constexpr int TR_HALF = 32;                   // hidden units per half: one gate
 constexpr int TR_CHUNK = 2 * TR_HALF;         // hidden units per GEMM 1
 constexpr int TR_WST = 2;                     // stages of either weight ring: W_1 by chunk, W_2 by half
 constexpr int TR_GATE_WARPS = 16;             // two groups of four per tile: first and second half of a chunk
-constexpr int TR_ISSUER1 = 6 + TR_GATE_WARPS; // warp that issues tile 1's MMAs
-constexpr int TR_W2PROD = TR_ISSUER1 + 1;     // warp that loads W_2
+constexpr int TR_W2PROD = 6 + TR_GATE_WARPS;  // warp that loads W_2
 constexpr int TR_THREADS = 32 * (TR_W2PROD + 1);
 constexpr int TR_SMEM_MAX = 224 * 1024;       // dynamic; c = 128 needs 228352 bytes
 
@@ -95,9 +94,9 @@ __global__ void __launch_bounds__(TR_THREADS, 1) transition_kernel(const __grid_
   unsigned long long* zempty = bars + 4;    // [4] the tile's stores have read the buffer
   unsigned long long* zconv = bars + 8;     // [4]
   unsigned long long* w1full = bars + 12;   // [2]
-  unsigned long long* w1empty = bars + 14;  // [2] count 2: one arrival per issuer
+  unsigned long long* w1empty = bars + 14;  // [2] both tiles' GEMM 1s have read the stage
   unsigned long long* w2full = bars + 16;   // [2]
-  unsigned long long* w2empty = bars + 18;  // [2] count 2
+  unsigned long long* w2empty = bars + 18;  // [2]
   unsigned long long* ofull = bars + 20;    // [2] output accumulator of a tile is complete
   unsigned long long* oempty = bars + 22;   // [2]
   unsigned long long* gvfull = bars + 24;   // [2] gate | value accumulators of a tile complete
@@ -119,9 +118,9 @@ __global__ void __launch_bounds__(TR_THREADS, 1) transition_kernel(const __grid_
     }
     for (int s = 0; s < TR_WST; ++s) {
       mbar_init(&w1full[s], 1);
-      mbar_init(&w1empty[s], 2);
+      mbar_init(&w1empty[s], 1);
       mbar_init(&w2full[s], 1);
-      mbar_init(&w2empty[s], 2);
+      mbar_init(&w2empty[s], 1);
     }
     mbar_fence_init();
   }
@@ -189,65 +188,88 @@ __global__ void __launch_bounds__(TR_THREADS, 1) transition_kernel(const __grid_
           if (++st == TR_WST) { st = 0; ph ^= 1; }
         }
     }
-  } else if (warp == 1 || warp == TR_ISSUER1) {
-    // ------------------------------------------------------------------ MMA issuer of tile r (whole warp, one elected lane)
-    const int r = warp == 1 ? 0 : 1;
+  } else if (warp == 1) {
+    // ------------------------------------------------------------------ MMA issuer (whole warp, one elected lane)
+    // One issuer for both tiles, in the order GEMM 2 and the next GEMM 1 of tile 0, then of tile 1: the tensor pipe takes
+    // MMAs as they are issued, so that tile 1's follow tile 0's as a block and one tile's gate stage lies under the
+    // other's MMAs.  An issuer per tile interleaves them: both GEMM 1s end together and both gate stages run together.
     const unsigned idesc1 = idesc_f16(128, 2 * TR_CHUNK, 0, 0, FMT_F16, FMT_F16);   // rows x 2 x (32 gate | 32 value)
     const unsigned idesc2 = idesc_f16(128, c, 0, 0, FMT_BF16, FMT_BF16);            // rows x c, A = hidden slice (TMEM)
     const unsigned zero_addr = smem_u32(sZero);
-    const unsigned d_gv = tmem_base + r * 128;
-    const unsigned d_out = tmem_base + 256 + r * 128;
-    unsigned st1 = 0, ph1 = 0, st2 = 0, ph2 = 0, phh = 0;      // ring positions, phase of hfull
-    for (int pass = 0; pass < npass; ++pass) {
-      const int zb = r * 2 + (pass & 1);
+    const int total = npass * nchunk;                      // chunks of this CTA
+    int q1 = 0, pass1 = 0, q2 = 0, pass2 = 0;              // chunk and pair of the next GEMM 1 / GEMM 2
+    unsigned st1 = 0, ph1 = 0, st2 = 0, ph2 = 0;           // their ring positions
+    auto gemm1 = [&](int r) {
+      const int zb = r * 2 + (pass1 & 1);
+      const unsigned d_gv = tmem_base + r * 128;
+      if (q1 == 0) mbar_wait(&zconv[zb], (pass1 >> 1) & 1, ab);
+      mbar_wait(&w1full[st1], ph1, ab);
+      tc_fence_after();
+      const unsigned w_addr = smem_u32(sW1 + st1 * w1_stage);
+      const unsigned long long w1_desc = desc_kmajor_sw128(w_addr);
+      const unsigned wx_addr = w_addr + w1_bytes;
+      const unsigned long long wx_desc = desc_kmajor_nosw(wx_addr, zero_addr - wx_addr, 128);
       const unsigned long long z_desc = desc_kmajor_sw128(smem_u32(sZ + zb * z_stage));
       const unsigned zx_addr = smem_u32(sZx + zb * 2048);
       const unsigned long long zx_desc = desc_kmajor_nosw(zx_addr, zero_addr - zx_addr, 128);
-      mbar_wait(&zconv[zb], (pass >> 1) & 1, ab);
-      for (int q = 0; q < nchunk; ++q) {
-        mbar_wait(&w1full[st1], ph1, ab);
-        tc_fence_after();
-        const unsigned w_addr = smem_u32(sW1 + st1 * w1_stage);
-        const unsigned long long w1_desc = desc_kmajor_sw128(w_addr);
-        const unsigned wx_addr = w_addr + w1_bytes;
-        const unsigned long long wx_desc = desc_kmajor_nosw(wx_addr, zero_addr - wx_addr, 128);
 #pragma unroll
-        for (int sl = 0; sl < 2; ++sl)
-          if (sl < nslab) {
+      for (int sl = 0; sl < 2; ++sl)
+        if (sl < nslab) {
 #pragma unroll
-            for (int k4 = 0; k4 < 4; ++k4)
-              if (elect_one())
-                umma_bf16(d_gv, z_desc + (sl * (slab >> 4) + k4 * 2), w1_desc + (sl * (slab >> 4) + k4 * 2), idesc1, (sl | k4) != 0);
-          }
-        if (elect_one()) {
-          umma_bf16(d_gv, zx_desc, wx_desc, idesc1, 1);   // mean and offset
-          tc_commit(&gvfull[r]);
-          tc_commit(&w1empty[st1]);
+          for (int k4 = 0; k4 < 4; ++k4)
+            if (elect_one())
+              umma_bf16(d_gv, z_desc + (sl * (slab >> 4) + k4 * 2), w1_desc + (sl * (slab >> 4) + k4 * 2), idesc1, (sl | k4) != 0);
         }
-        __syncwarp();
-        if (++st1 == TR_WST) { st1 = 0; ph1 ^= 1; }
-        if (q == 0) mbar_wait(&oempty[r], (pass & 1) ^ 1, ab);
-#pragma unroll
-        for (int b = 0; b < 2; ++b) {
-          mbar_wait(&hfull[r * 2 + b], phh, ab);           // also for a half that is not there: it paces the gate warps
-          if (2 * q + b < nhalf) {
-            mbar_wait(&w2full[st2], ph2, ab);
-            tc_fence_after();
-            const unsigned long long w2_desc = tr_desc_sw64(smem_u32(sW2 + st2 * w2_bytes));
-#pragma unroll
-            for (int ks = 0; ks < 2; ++ks)
-              if (elect_one()) umma_ts(d_out, d_gv + b * 64 + ks * 8, w2_desc + ks * 2, idesc2, (q | b | ks) != 0);
-            if (elect_one()) {
-              tc_commit(&w2empty[st2]);
-              if (2 * q + b == nhalf - 1) tc_commit(&ofull[r]);
-            }
-            __syncwarp();
-            if (++st2 == TR_WST) { st2 = 0; ph2 ^= 1; }
-          }
-        }
-        phh ^= 1;
+      if (elect_one()) {
+        umma_bf16(d_gv, zx_desc, wx_desc, idesc1, 1);   // mean and offset
+        tc_commit(&gvfull[r]);
+        if (r == 1) tc_commit(&w1empty[st1]);
       }
+      __syncwarp();
+      if (r == 1) {
+        if (++q1 == nchunk) { q1 = 0; ++pass1; }
+        if (++st1 == TR_WST) { st1 = 0; ph1 ^= 1; }
+      }
+    };
+    auto gemm2 = [&](int r, unsigned phh) {
+      const unsigned d_gv = tmem_base + r * 128;
+      const unsigned d_out = tmem_base + 256 + r * 128;
+      unsigned st = st2, ph = ph2;
+      if (q2 == 0) mbar_wait(&oempty[r], (pass2 & 1) ^ 1, ab);
+#pragma unroll
+      for (int b = 0; b < 2; ++b) {
+        mbar_wait(&hfull[r * 2 + b], phh, ab);           // also for a half that is not there: it paces the gate warps
+        if (2 * q2 + b < nhalf) {
+          mbar_wait(&w2full[st], ph, ab);
+          tc_fence_after();
+          const unsigned long long w2_desc = tr_desc_sw64(smem_u32(sW2 + st * w2_bytes));
+#pragma unroll
+          for (int ks = 0; ks < 2; ++ks)
+            if (elect_one()) umma_ts(d_out, d_gv + b * 64 + ks * 8, w2_desc + ks * 2, idesc2, (q2 | b | ks) != 0);
+          if (elect_one()) {
+            if (r == 1) tc_commit(&w2empty[st]);
+            if (2 * q2 + b == nhalf - 1) tc_commit(&ofull[r]);
+          }
+          __syncwarp();
+          if (++st == TR_WST) { st = 0; ph ^= 1; }
+        }
+      }
+      if (r == 1) {
+        st2 = st;
+        ph2 = ph;
+        if (++q2 == nchunk) { q2 = 0; ++pass2; }
+      }
+    };
+    if (total > 0) {
+      gemm1(0);
+      gemm1(1);
     }
+    for (int g = 0; g < total; ++g)
+#pragma unroll
+      for (int r = 0; r < 2; ++r) {
+        gemm2(r, g & 1);
+        if (g + 1 < total) gemm1(r);
+      }
   } else if (warp < 6) {
     // ------------------------------------------------------------------ converters (4 warps, one row per thread)
     const int row = (warp - 2) * 32 + lane;
