@@ -71,7 +71,7 @@ __device__ inline unsigned long long tr_desc_sw64(unsigned saddr) {
 
 __global__ void __launch_bounds__(TR_THREADS, 1) transition_kernel(const __grid_constant__ TransParams p) {
   extern __shared__ unsigned char smem_raw[];
-  __shared__ __align__(8) unsigned long long bars[30];
+  __shared__ __align__(8) unsigned long long bars[28];
   __shared__ float sRstd[4][128];
   __shared__ unsigned tmem_base_s;
   __shared__ int abort_flag;
@@ -100,7 +100,7 @@ __global__ void __launch_bounds__(TR_THREADS, 1) transition_kernel(const __grid_
   unsigned long long* ofull = bars + 20;    // [2] output accumulator of a tile is complete
   unsigned long long* oempty = bars + 22;   // [2]
   unsigned long long* gvfull = bars + 24;   // [2] gate | value accumulators of a tile complete
-  unsigned long long* hfull = bars + 26;    // [4] index tile * 2 + half: hidden slice stored over them
+  unsigned long long* hfull = bars + 26;    // [2] hidden slices of a tile stored over them
 
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;   // warp-uniform for the compiler too
   if (threadIdx.x == 0) {
@@ -109,10 +109,10 @@ __global__ void __launch_bounds__(TR_THREADS, 1) transition_kernel(const __grid_
       mbar_init(&zfull[s], 1);
       mbar_init(&zempty[s], 8);
       mbar_init(&zconv[s], 4);
-      mbar_init(&hfull[s], 4);
     }
     for (int s = 0; s < 2; ++s) {
       mbar_init(&gvfull[s], 1);
+      mbar_init(&hfull[s], 8);
       mbar_init(&ofull[s], 1);
       mbar_init(&oempty[s], 8);
     }
@@ -132,7 +132,7 @@ __global__ void __launch_bounds__(TR_THREADS, 1) transition_kernel(const __grid_
   __syncthreads();
   tc_fence_after();
   pdl_begin();
-  const unsigned tmem_base = tmem_base_s;
+  const unsigned tmem_base = __shfl_sync(0xffffffffu, tmem_base_s, 0);
   AbortCtx ab{p.status, &abort_flag};
   const long long ntiles = (p.rows + 127) / 128;
   const long long npairs = (ntiles + 1) / 2;
@@ -203,7 +203,7 @@ __global__ void __launch_bounds__(TR_THREADS, 1) transition_kernel(const __grid_
       const int zb = r * 2 + (pass1 & 1);
       const unsigned d_gv = tmem_base + r * 128;
       if (q1 == 0) mbar_wait(&zconv[zb], (pass1 >> 1) & 1, ab);
-      mbar_wait(&w1full[st1], ph1, ab);
+      if (r == 0) mbar_wait(&w1full[st1], ph1, ab);    // tile 1 follows on the same stage
       tc_fence_after();
       const unsigned w_addr = smem_u32(sW1 + st1 * w1_stage);
       const unsigned long long w1_desc = desc_kmajor_sw128(w_addr);
@@ -236,24 +236,25 @@ __global__ void __launch_bounds__(TR_THREADS, 1) transition_kernel(const __grid_
       const unsigned d_out = tmem_base + 256 + r * 128;
       unsigned st = st2, ph = ph2;
       if (q2 == 0) mbar_wait(&oempty[r], (pass2 & 1) ^ 1, ab);
+      mbar_wait(&hfull[r], phh, ab);
+      tc_fence_after();
 #pragma unroll
-      for (int b = 0; b < 2; ++b) {
-        mbar_wait(&hfull[r * 2 + b], phh, ab);           // also for a half that is not there: it paces the gate warps
+      for (int b = 0; b < 2; ++b)
         if (2 * q2 + b < nhalf) {
-          mbar_wait(&w2full[st], ph, ab);
-          tc_fence_after();
+          if (r == 0) mbar_wait(&w2full[st], ph, ab);
           const unsigned long long w2_desc = tr_desc_sw64(smem_u32(sW2 + st * w2_bytes));
 #pragma unroll
           for (int ks = 0; ks < 2; ++ks)
             if (elect_one()) umma_ts(d_out, d_gv + b * 64 + ks * 8, w2_desc + ks * 2, idesc2, (q2 | b | ks) != 0);
-          if (elect_one()) {
-            if (r == 1) tc_commit(&w2empty[st]);
-            if (2 * q2 + b == nhalf - 1) tc_commit(&ofull[r]);
+          if (r == 1) {
+            if (elect_one()) tc_commit(&w2empty[st]);
           }
-          __syncwarp();
           if (++st == TR_WST) { st = 0; ph ^= 1; }
         }
+      if (q2 == nchunk - 1) {
+        if (elect_one()) tc_commit(&ofull[r]);
       }
+      __syncwarp();
       if (r == 1) {
         st2 = st;
         ph2 = ph;
@@ -319,7 +320,7 @@ __global__ void __launch_bounds__(TR_THREADS, 1) transition_kernel(const __grid_
         mbar_wait(&gvfull[r], phg, ab);                      // GEMM 1 has run, so the converters' statistics are published
         phg ^= 1;
         if (2 * q + b >= nhalf) {
-          if (lane == 0) mbar_arrive(&hfull[r * 2 + b]);
+          if (lane == 0) mbar_arrive(&hfull[r]);           // a half that is not there
           continue;
         }
         tc_fence_after();
@@ -350,7 +351,7 @@ __global__ void __launch_bounds__(TR_THREADS, 1) transition_kernel(const __grid_
         tmem_st_wait();
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive(&hfull[r * 2 + b]);
+        if (lane == 0) mbar_arrive(&hfull[r]);
         if (q == 0) give_back();
       }
       // ---- output stage: out + z through the z tile, half of the channels per group, then one TMA store per 64-channel slab
