@@ -214,12 +214,7 @@ __global__ void __launch_bounds__(TR_THREADS, 1) transition_kernel(const __grid_
       const unsigned long long zx_desc = desc_kmajor_nosw(zx_addr, zero_addr - zx_addr, 128);
 #pragma unroll
       for (int sl = 0; sl < 2; ++sl)
-        if (sl < nslab) {
-#pragma unroll
-          for (int k4 = 0; k4 < 4; ++k4)
-            if (elect_one())
-              umma_bf16(d_gv, z_desc + (sl * (slab >> 4) + k4 * 2), w1_desc + (sl * (slab >> 4) + k4 * 2), idesc1, (sl | k4) != 0);
-        }
+        if (sl < nslab) umma_k4(d_gv, z_desc + sl * (slab >> 4), w1_desc + sl * (slab >> 4), idesc1, sl);
       if (elect_one()) {
         umma_bf16(d_gv, zx_desc, wx_desc, idesc1, 1);   // mean and offset
         tc_commit(&gvfull[r]);
