@@ -64,6 +64,36 @@ __device__ inline void tca_cp_async16(void* smem, const void* gmem, bool valid) 
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(sa), "l"(gmem), "r"(sz));
 }
 
+// 16, 32 or 64 consecutive columns of this thread's row, landed: load and wait are one statement, so the compiler can neither use
+// nor copy the registers in between, and ties no registers afterwards.
+__device__ inline void tca_ld(unsigned t, unsigned (&a)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n\t"
+      "tcgen05.wait::ld.sync.aligned;\n"
+      : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3]), "=r"(a[4]), "=r"(a[5]), "=r"(a[6]), "=r"(a[7]), "=r"(a[8]), "=r"(a[9]), "=r"(a[10]), "=r"(a[11]), "=r"(a[12]), "=r"(a[13]), "=r"(a[14]), "=r"(a[15]) : "r"(t) : "memory");
+}
+__device__ inline void tca_ld(unsigned t, unsigned (&a)[16], unsigned (&b)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%32];\n\t"
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%33];\n\t"
+      "tcgen05.wait::ld.sync.aligned;\n"
+      : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3]), "=r"(a[4]), "=r"(a[5]), "=r"(a[6]), "=r"(a[7]), "=r"(a[8]), "=r"(a[9]), "=r"(a[10]), "=r"(a[11]), "=r"(a[12]), "=r"(a[13]), "=r"(a[14]), "=r"(a[15]),
+        "=r"(b[0]), "=r"(b[1]), "=r"(b[2]), "=r"(b[3]), "=r"(b[4]), "=r"(b[5]), "=r"(b[6]), "=r"(b[7]), "=r"(b[8]), "=r"(b[9]), "=r"(b[10]), "=r"(b[11]), "=r"(b[12]), "=r"(b[13]), "=r"(b[14]), "=r"(b[15]) : "r"(t), "r"(t + 16) : "memory");
+}
+__device__ inline void tca_ld(unsigned t, unsigned (&a)[16], unsigned (&b)[16], unsigned (&c)[16], unsigned (&d)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%64];\n\t"
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%65];\n\t"
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%32,%33,%34,%35,%36,%37,%38,%39,%40,%41,%42,%43,%44,%45,%46,%47}, [%66];\n\t"
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%48,%49,%50,%51,%52,%53,%54,%55,%56,%57,%58,%59,%60,%61,%62,%63}, [%67];\n\t"
+      "tcgen05.wait::ld.sync.aligned;\n"
+      : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3]), "=r"(a[4]), "=r"(a[5]), "=r"(a[6]), "=r"(a[7]), "=r"(a[8]), "=r"(a[9]), "=r"(a[10]), "=r"(a[11]), "=r"(a[12]), "=r"(a[13]), "=r"(a[14]), "=r"(a[15]),
+        "=r"(b[0]), "=r"(b[1]), "=r"(b[2]), "=r"(b[3]), "=r"(b[4]), "=r"(b[5]), "=r"(b[6]), "=r"(b[7]), "=r"(b[8]), "=r"(b[9]), "=r"(b[10]), "=r"(b[11]), "=r"(b[12]), "=r"(b[13]), "=r"(b[14]), "=r"(b[15]),
+        "=r"(c[0]), "=r"(c[1]), "=r"(c[2]), "=r"(c[3]), "=r"(c[4]), "=r"(c[5]), "=r"(c[6]), "=r"(c[7]), "=r"(c[8]), "=r"(c[9]), "=r"(c[10]), "=r"(c[11]), "=r"(c[12]), "=r"(c[13]), "=r"(c[14]), "=r"(c[15]),
+        "=r"(d[0]), "=r"(d[1]), "=r"(d[2]), "=r"(d[3]), "=r"(d[4]), "=r"(d[5]), "=r"(d[6]), "=r"(d[7]), "=r"(d[8]), "=r"(d[9]), "=r"(d[10]), "=r"(d[11]), "=r"(d[12]), "=r"(d[13]), "=r"(d[14]), "=r"(d[15])
+      : "r"(t), "r"(t + 16), "r"(t + 32), "r"(t + 48) : "memory");
+}
+
 __device__ inline float tca_exp2(float x) {
   float y;
   asm("ex2.approx.ftz.f32 %0, %1;\n" : "=f"(y) : "f"(x));
@@ -118,7 +148,7 @@ __global__ void __launch_bounds__(TCA_THREADS, 1) attn_tc_kernel(const __grid_co
 
   const BatchMeta& m = p.m;
   const int H = p.H, Hd = H * D;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;   // warp-uniform for the compiler too
   if (threadIdx.x == 0) {
     abort_flag = 0;
     for (int s = 0; s < 12; ++s) mbar_init(&bars[s], 1);
@@ -136,7 +166,7 @@ __global__ void __launch_bounds__(TCA_THREADS, 1) attn_tc_kernel(const __grid_co
   __syncthreads();
   tc_fence_after();
   pdl_begin();
-  const unsigned tmem_base = tmem_base_s;
+  const unsigned tmem_base = __shfl_sync(0xffffffffu, tmem_base_s, 0);
   AbortCtx ab{p.status, &abort_flag};
   const float sc2 = rsqrtf((float)D) * TCA_LOG2E;
   const bool has_bias = p.bias != nullptr;
@@ -327,27 +357,19 @@ __global__ void __launch_bounds__(TCA_THREADS, 1) attn_tc_kernel(const __grid_co
 #pragma unroll 1
           for (; g + 4 <= ge; g += 4) {
             unsigned rc[16], rd[16];
-            tmem_ld16(t_row + g * 16, ra);
-            tmem_ld16(t_row + g * 16 + 16, rb);
-            tmem_ld16(t_row + g * 16 + 32, rc);
-            tmem_ld16(t_row + g * 16 + 48, rd);
-            tmem_ld_wait2(ra, rb);
-            tmem_ld_wait2(rc, rd);
+            tca_ld(t_row + g * 16, ra, rb, rc, rd);
 #pragma unroll
             for (int e = 0; e < 16; ++e)
               m4[e & 3] = tca_max3(tca_max3(m4[e & 3], __uint_as_float(ra[e]), __uint_as_float(rb[e])), __uint_as_float(rc[e]), __uint_as_float(rd[e]));
           }
 #pragma unroll 1
           for (; g + 2 <= ge; g += 2) {
-            tmem_ld16(t_row + g * 16, ra);
-            tmem_ld16(t_row + g * 16 + 16, rb);
-            tmem_ld_wait2(ra, rb);
+            tca_ld(t_row + g * 16, ra, rb);
 #pragma unroll
             for (int e = 0; e < 16; ++e) m4[e & 3] = tca_max3(m4[e & 3], __uint_as_float(ra[e]), __uint_as_float(rb[e]));
           }
           if (g < ge) {
-            tmem_ld16(t_row + g * 16, ra);
-            tmem_ld_wait16(ra);
+            tca_ld(t_row + g * 16, ra);
 #pragma unroll
             for (int e = 0; e < 16; ++e) m4[e & 3] = fmaxf(m4[e & 3], __uint_as_float(ra[e]));
           }
@@ -382,22 +404,18 @@ __global__ void __launch_bounds__(TCA_THREADS, 1) attn_tc_kernel(const __grid_co
           };
           int g = gb;
           if ((g & 1) && g < ge) {
-            tmem_ld16(t_row + g * 16, ra);
-            tmem_ld_wait16(ra);
+            tca_ld(t_row + g * 16, ra);
             pass2(g, ra);
             ++g;
           }
 #pragma unroll 1
           for (; g + 2 <= ge; g += 2) {
-            tmem_ld16(t_row + g * 16, ra);
-            tmem_ld16(t_row + g * 16 + 16, rb);
-            tmem_ld_wait2(ra, rb);
+            tca_ld(t_row + g * 16, ra, rb);
             pass2(g, ra);
             pass2(g + 1, rb);
           }
           if (g < ge) {
-            tmem_ld16(t_row + g * 16, ra);
-            tmem_ld_wait16(ra);
+            tca_ld(t_row + g * 16, ra);
             pass2(g, ra);
           }
           lsum = (l2[0].x + l2[0].y) + (l2[1].x + l2[1].y);
@@ -413,17 +431,23 @@ __global__ void __launch_bounds__(TCA_THREADS, 1) attn_tc_kernel(const __grid_co
         tc_fence_after();
         if (warp_live && (D >= 32 || hf == 0)) {
           constexpr int CPT = D >= 32 ? D / 2 : D;                 // output channels per thread (16)
-          tmem_ld16(t_row + TCA_O_COL + hf * CPT, ra);
           const float inv = 1.0f / (xm[256 + row] + xm[256 + 128 + row]);
-          tmem_ld_wait16(ra);
+          tca_ld(t_row + TCA_O_COL + hf * CPT, ra);
           const long long orow = COL ? (long long)j * N + i : (long long)i * N + j;
           if (j < N && NT_IN(row_base + orow, m.pair_off[m.B] - p.row0, NT_SITE_ROW_ATTN_OUT)) {
             __nv_bfloat16* op = p.o + (p.row0 + row_base + orow) * Hd + h * D + hf * CPT;
             unsigned w[8];
 #pragma unroll
             for (int e = 0; e < 8; ++e) w[e] = tca_pack(__uint_as_float(ra[2 * e]) * inv, __uint_as_float(ra[2 * e + 1]) * inv);
-            *reinterpret_cast<uint4*>(op) = make_uint4(w[0], w[1], w[2], w[3]);
-            *reinterpret_cast<uint4*>(op + 8) = make_uint4(w[4], w[5], w[6], w[7]);
+            // One 32-byte store where the address allows it (callers' buffers may be aligned to 16 bytes only): a thread's 16
+            // channels are one sector, which two 16-byte stores each write in part (206 -> 198 us at eight samples of 215).
+            if (((unsigned long long)p.o & 31) == 0) {
+              asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};\n" ::"l"(op), "r"(w[0]), "r"(w[1]), "r"(w[2]),
+                           "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7]) : "memory");
+            } else {
+              *reinterpret_cast<uint4*>(op) = make_uint4(w[0], w[1], w[2], w[3]);
+              *reinterpret_cast<uint4*>(op + 8) = make_uint4(w[4], w[5], w[6], w[7]);
+            }
           }
         }
       }
