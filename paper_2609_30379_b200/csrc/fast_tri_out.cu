@@ -22,7 +22,9 @@
 
 namespace ntp {
 
-constexpr int TO_THREADS = 64 + 128 + 256;   // producer, MMA, 4 converter warps, 8 epilogue warps
+constexpr int TO_EPI = 16;                              // epilogue warps
+constexpr int TO_STORE = 6 + TO_EPI;                    // the warp that stores finished tiles
+constexpr int TO_THREADS = 32 * (TO_STORE + 1);         // producer, MMA, 4 statistics warps, epilogue, store
 constexpr int TO_MAXB = 12;
 
 struct TriOutParams {
@@ -61,7 +63,7 @@ __device__ inline float to_tanh(float x) {
 
 __global__ void __launch_bounds__(TO_THREADS, 1) tri_out_kernel(const __grid_constant__ TriOutParams p) {
   extern __shared__ unsigned char smem_raw[];
-  __shared__ __align__(8) unsigned long long bars[17];
+  __shared__ __align__(8) unsigned long long bars[19];
   __shared__ float4 sStats[2][128];        // per z stage and position: (rstd_t / 2, rstd_z / 2, -mean_t rstd_t / 2, -mean_z rstd_z / 2)
   __shared__ unsigned tmem_base_s;
   __shared__ int abort_flag;
@@ -89,17 +91,19 @@ __global__ void __launch_bounds__(TO_THREADS, 1) tri_out_kernel(const __grid_con
   unsigned long long* tempty = bars + 10;   // [2]
   unsigned long long* sconv = bars + 12;    // [2] statistics published
   unsigned long long* wfull = bars + 14;
+  unsigned long long* zdone = bars + 15;    // [2] the new z is in the tile
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;   // warp-uniform for the compiler too
   if (threadIdx.x == 0) {
     abort_flag = 0;
     for (int s = 0; s < 2; ++s) {
       mbar_init(&tfullb[s], 1);
       mbar_init(&tfree[s], 1 + 4);                   // MMA commit + the four statistics warps
       mbar_init(&zfullb[s], 1);
-      mbar_init(&zfree[s], 1 + 4 + 4 * (p.c_z / 64)); // MMA commit + the statistics warps + the storing epilogue lanes
+      mbar_init(&zfree[s], 1 + 4 + 1);               // MMA commit + the statistics warps + the store warp
       mbar_init(&tfull[s], 1);
-      mbar_init(&tempty[s], 8);
+      mbar_init(&tempty[s], TO_EPI);
+      mbar_init(&zdone[s], TO_EPI);
       mbar_init(&sconv[s], 4);
     }
     mbar_init(wfull, 1);
@@ -116,7 +120,7 @@ __global__ void __launch_bounds__(TO_THREADS, 1) tri_out_kernel(const __grid_con
   __syncthreads();
   tc_fence_after();
   pdl_begin();
-  const unsigned tmem_base = tmem_base_s;
+  const unsigned tmem_base = __shfl_sync(0xffffffffu, tmem_base_s, 0);
   AbortCtx ab{p.status, &abort_flag};
   const long long nchunks = p.chunk_off[p.B];
   const long long ntiles = (nchunks + 1) / 2;
@@ -291,32 +295,32 @@ __global__ void __launch_bounds__(TO_THREADS, 1) tri_out_kernel(const __grid_con
       }
       if (++stage == 2) { stage = 0; phase ^= 1; }
     }
-  } else if (warp >= 6) {
-    // ------------------------------------------------------------------ epilogue (8 warps)
+  } else if (warp < TO_STORE) {
+    // ------------------------------------------------------------------ epilogue (16 warps: four per TMEM lane quarter, a
+    // quarter of the channels each).  With 8 warps that also stored, this stage was the kernel's period: 2560 clocks of
+    // arithmetic and 1770 of waiting for the store engine per tile of 128 positions, against 4950 for the tile.
     const int quarter = warp & 3;
-    const int half = (warp - 6) >> 2;
+    const int part = (warp - 6) >> 2;
     const int row = quarter * 32 + lane;           // position inside the tile
     int stage = 0;
-    unsigned phase = 0, tph[2] = {0, 0};
-    long long n = 0;
-    for (long long t = blockIdx.x; t < ntiles; t += gridDim.x, ++n) {
-      const int buf = (int)(n & 1);
+    unsigned phase = 0;
+    for (long long t = blockIdx.x; t < ntiles; t += gridDim.x) {
       unsigned char* zrow = sZ + stage * z_stage;
       mbar_wait(&sconv[stage], phase, ab);
       const float4 stt = sStats[stage][row];
       const float trh = stt.x, zrh = stt.y, tmh = stt.z, zmh = stt.w;
-      mbar_wait(&tfull[buf], tph[buf], ab);
-      tph[buf] ^= 1;
+      mbar_wait(&tfull[stage], phase, ab);         // accumulator buffers and z stages advance together
       tc_fence_after();
-      const unsigned taddr = tmem_base + ((unsigned)(quarter * 32) << 16) + buf * 256;
-      for (int c0 = half * (c_z / 2); c0 < (half + 1) * (c_z / 2); c0 += 32) {
-        unsigned r1[32], r2[32];
-        tmem_ld32(taddr + c0, r1);
-        tmem_ld32(taddr + c_z + c0, r2);
-        tmem_ld_wait();
+      const unsigned taddr = tmem_base + ((unsigned)(quarter * 32) << 16) + stage * 256;
+#pragma unroll 1
+      for (int c0 = part * (c_z / 4); c0 < (part + 1) * (c_z / 4); c0 += 16) {
+        unsigned r1[16], r2[16];
+        tmem_ld16(taddr + c0, r1);
+        tmem_ld16(taddr + c_z + c0, r2);
+        tmem_ld_wait2(r1, r2);
         unsigned char* zp = zrow + (c0 >> 6) * z_slab;
 #pragma unroll
-        for (int ch = 0; ch < 4; ++ch) {
+        for (int ch = 0; ch < 2; ++ch) {
           const int chunk16 = ((c0 & 63) >> 3) + ch;
           uint4* ptr = reinterpret_cast<uint4*>(zp + sw128_off(row, chunk16));
           uint4 v = *ptr;
@@ -352,26 +356,31 @@ __global__ void __launch_bounds__(TO_THREADS, 1) tri_out_kernel(const __grid_con
         }
       }
       tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&tempty[buf]);
-      // every warp stores its own 32 positions x 64 channels as soon as it has written them (c_z = 64: the two
-      // warps of a lane quarter share the slab and meet at a barrier of their own)
       fence_proxy_async_smem();
-      if (zslab == 1) named_bar_sync(2 + quarter, 64);
-      else __syncwarp();
-      if (lane == 0 && (zslab == 2 || half == 0)) {
-        const int qq = quarter >> 1, sub = quarter & 1;
-        int s, i, j0;
-        if (to_decode(p, 2 * t + qq, s, i, j0) && j0 + sub * 32 < p.N[s])
-          tma_store_4d(&p.zmap[s], zrow + (zslab == 2 ? half : 0) * z_slab + (qq * 64 + sub * 32) * 128, (zslab == 2 ? half : 0) * 64,
-                       j0 + sub * 32, i, 0);
-        tma_store_commit();
-        tma_store_wait_read0();
-        mbar_arrive(&zfree[stage]);
+      __syncwarp();
+      if (lane == 0) {
+        mbar_arrive(&tempty[stage]);
+        mbar_arrive(&zdone[stage]);
       }
       if (++stage == 2) { stage = 0; phase ^= 1; }
     }
-    if (lane == 0) tma_store_wait_all0();
+  } else {
+    // ------------------------------------------------------------------ store: lane l takes 32 positions of a 64-channel slab
+    int stage = 0;
+    unsigned phase = 0;
+    for (long long t = blockIdx.x; t < ntiles; t += gridDim.x) {
+      const int quarter = lane & 3, sl = lane >> 2, sub = quarter & 1;
+      int s, i, j0;
+      const bool any = sl < zslab && to_decode(p, 2 * t + (quarter >> 1), s, i, j0) && j0 + sub * 32 < p.N[s];
+      mbar_wait(&zdone[stage], phase, ab);
+      if (any) tma_store_4d(&p.zmap[s], sZ + stage * z_stage + sl * z_slab + quarter * 32 * 128, sl * 64, j0 + sub * 32, i, 0);
+      tma_store_commit();
+      tma_store_wait_read0();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&zfree[stage]);
+      if (++stage == 2) { stage = 0; phase ^= 1; }
+    }
+    tma_store_wait_all0();
   }
   tc_fence_before();
   __syncthreads();
