@@ -7,9 +7,14 @@
 // [T2, c_z] buffer.  Both LayerNorms are folded into the weights (W' = W gamma; W_o' fp16 against the
 // fp16 t, W_g' bf16 against the bf16 state itself), so NOTHING has to touch the tiles between the TMA
 // load and the MMA: the MMAs start as soon as the tiles land, four warps take the row statistics of t
-// and z from the same tiles meanwhile, and the epilogue applies them:
-//   o / 2 = (rstd_t / 2) (acc_o - mean_t c1_o) + c0_o / 2,  g / 2 = (rstd_z / 2) (acc_g - mean_z c1_g) + c0_g / 2,
-//   z += (tanh(g / 2) + 1) (o / 2)        with c1 = sum_k W'[n][k], c0 = sum_k W[n][k] beta[k].
+// and z from the same tiles meanwhile and write them as one more K step of either product (ln_aug_row), and the epilogue is
+//   z += (tanh(g / 2) + 1) (o / 2),  o / 2 = (rstd_t / 2) acc_o,  g / 2 = (rstd_z / 2) acc_g.
+// Bound: the life of a z stage -- load, statistics, epilogue, store -- with room for two of them beside the weights.
+// Tables of the LayerNorm constants in the epilogue (four 16-byte reads per four channels and warp) were two fifths of
+// the shared-memory traffic, which is why the constants travel through the tensor cores instead.
+// Measured at eight samples of about 215 positions: 76.4 us with eight storing epilogue warps, 72.4 us with sixteen and a
+// store warp, 70.3 us without the tables.  (Without statistics and arithmetic it takes 62 us.  Storing from registers, 78 us,
+// and eight statistics warps, 73 us, were slower.)
 //
 // A tile is two 64-position chunks (s, i, j0).  The t chunks and the z tile travel through rings of
 // their own: a t stage is free once the MMAs and the statistics have read it, a z stage only after the
@@ -64,7 +69,7 @@ __device__ inline float to_tanh(float x) {
 __global__ void __launch_bounds__(TO_THREADS, 1) tri_out_kernel(const __grid_constant__ TriOutParams p) {
   extern __shared__ unsigned char smem_raw[];
   __shared__ __align__(8) unsigned long long bars[19];
-  __shared__ float4 sStats[2][128];        // per z stage and position: (rstd_t / 2, rstd_z / 2, -mean_t rstd_t / 2, -mean_z rstd_z / 2)
+  __shared__ float2 sStats[2][128];        // per z stage and position: (rstd_t / 2, rstd_z / 2)
   __shared__ unsigned tmem_base_s;
   __shared__ int abort_flag;
   unsigned char* smem = smem_raw + ((1024 - (smem_u32(smem_raw) & 1023)) & 1023);
@@ -79,10 +84,9 @@ __global__ void __launch_bounds__(TO_THREADS, 1) tri_out_kernel(const __grid_con
   unsigned char* sWg = sWo + wo_bytes;
   unsigned char* sT = sWg + wg_bytes;                        // 2 stages of the two t chunks
   unsigned char* sZ = sT + 2 * t_stage;                      // 2 stages of the z tile
-  float* sCo = reinterpret_cast<float*>(sZ + 2 * z_stage);   // c0 of W_o / 2 per channel
-  float* sCg = sCo + c_z;                                    // c0 of W_g / 2
-  float* sKo = sCg + c_z;                                    // c1 of W_o
-  float* sKg = sKo + c_z;                                    // c1 of W_g
+  unsigned char* sAx = sZ + 2 * z_stage;                     // [2 stages][t | z][128][8] fp16: augmentation columns 0-7 of the rows
+  unsigned char* sBx = sAx + 4 * 2048;                       // [W_o | W_g][c_z][8] fp16: augmentation columns 0-7 of the weights
+  unsigned char* sZero = sBx + 2 * c_z * 16;                 // [128][8] zeros: augmentation columns 8-15 of all of them
   unsigned long long* tfullb = bars;        // [2] t chunks landed
   unsigned long long* tfree = bars + 2;     // [2] MMAs and statistics have read them
   unsigned long long* zfullb = bars + 4;    // [2] z tile landed
@@ -110,16 +114,17 @@ __global__ void __launch_bounds__(TO_THREADS, 1) tri_out_kernel(const __grid_con
     mbar_fence_init();
   }
   if (warp == 1) tmem_alloc(&tmem_base_s, 512);
-  for (int n = threadIdx.x; n < c_z; n += TO_THREADS) {
-    sCo[n] = 0.5f * p.c01o[n].x;
-    sCg[n] = 0.5f * p.c01g[n].x;
-    sKo[n] = p.c01o[n].y;
-    sKg[n] = p.c01g[n].y;
-  }
+  for (int n = threadIdx.x; n < 128; n += TO_THREADS) *reinterpret_cast<uint4*>(sZero + n * 16) = make_uint4(0, 0, 0, 0);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   pdl_begin();
+  for (int n = threadIdx.x; n < 2 * c_z; n += TO_THREADS) {
+    const float2 k = n < c_z ? p.c01o[n] : p.c01g[n - c_z];
+    *reinterpret_cast<uint4*>(sBx + n * 16) = ln_aug_weight(k.x, k.y);
+  }
+  fence_proxy_async_smem();
+  __syncthreads();
   const unsigned tmem_base = __shfl_sync(0xffffffffu, tmem_base_s, 0);
   AbortCtx ab{p.status, &abort_flag};
   const long long nchunks = p.chunk_off[p.B];
@@ -164,6 +169,7 @@ __global__ void __launch_bounds__(TO_THREADS, 1) tri_out_kernel(const __grid_con
     unsigned n = 0;
     const unsigned idesc_t = idesc_f16(128, c_z, 1, 0, FMT_F16, FMT_F16);     // A = t (fp16, MN-major), W_o' fp16
     const unsigned idesc_z = idesc_f16(128, c_z, 0, 0, FMT_BF16, FMT_BF16);   // A = the bf16 z tile, W_g' bf16
+    const unsigned idesc_x = idesc_f16(128, c_z, 0, 0, FMT_F16, FMT_F16);     // augmentation step
     const unsigned long long wo_desc = desc_kmajor_sw128(smem_u32(sWo)), wg_desc = desc_kmajor_sw128(smem_u32(sWg));
     const unsigned wo16 = (unsigned)wo_slab >> 4, wg16 = (unsigned)wg_slab >> 4, z16 = (unsigned)z_slab >> 4;
     for (long long t = blockIdx.x; t < ntiles; t += gridDim.x, ++n) {
@@ -184,9 +190,14 @@ __global__ void __launch_bounds__(TO_THREADS, 1) tri_out_kernel(const __grid_con
       tc_fence_after();
       const unsigned long long z_desc = desc_kmajor_sw128(smem_u32(sZ + stage * z_stage));
 #pragma unroll
-      for (int ks = 0; ks < 8; ++ks)
-        if (ks < c_z / 16 && elect_one())
-          umma_bf16(d2, z_desc + ((ks >> 2) * z16 + (ks & 3) * 2), wg_desc + ((ks >> 2) * wg16 + (ks & 3) * 2), idesc_z, ks != 0);
+      for (int sl = 0; sl < 2; ++sl)
+        if (sl < zslab) umma_k4(d2, z_desc + sl * z16, wg_desc + sl * wg16, idesc_z, sl);
+      mbar_wait(&sconv[stage], phase, ab);                 // the rows' augmentation columns are written
+      tc_fence_after();
+      const unsigned ax = smem_u32(sAx + stage * 4096), bx = smem_u32(sBx), zero = smem_u32(sZero);
+      if (elect_one()) umma_bf16(d1, desc_kmajor_nosw(ax, zero - ax, 128), desc_kmajor_nosw(bx, zero - bx, 128), idesc_x, 1);
+      if (elect_one())
+        umma_bf16(d2, desc_kmajor_nosw(ax + 2048, zero - ax - 2048, 128), desc_kmajor_nosw(bx + c_z * 16, zero - bx - c_z * 16, 128), idesc_x, 1);
       if (elect_one()) {
         tc_commit(&tfull[buf]);
         tc_commit(&zfree[stage]);
@@ -264,7 +275,7 @@ __global__ void __launch_bounds__(TO_THREADS, 1) tri_out_kernel(const __grid_con
       if (lane == 0) mbar_arrive(&tfree[stage]);
       // t arrives scaled by 1 / N_s (see the contraction); LayerNorm is scale-free once eps is scaled alike
       const float tmean = ts / (float)c_h;
-      const float trstd = rsqrtf(fmaxf(tq / (float)c_h - tmean * tmean, 0.f) + eps_t);
+      const float tve = fmaxf(tq / (float)c_h - tmean * tmean, 0.f) + eps_t, trstd = rsqrtf(tve);
       // z row: statistics of the bf16 tile (read only)
       mbar_wait(&zfullb[stage], phase, ab);
       float zs = 0.f, zq = 0.f;
@@ -287,7 +298,11 @@ __global__ void __launch_bounds__(TO_THREADS, 1) tri_out_kernel(const __grid_con
       }
       const float zmean = p.zstats ? zst.x : zs / (float)c_z;
       const float zrstd = p.zstats ? zst.y : rsqrtf(fmaxf(zq / (float)c_z - zmean * zmean, 0.f) + p.eps);
-      sStats[stage][row] = make_float4(0.5f * trstd, 0.5f * zrstd, -0.5f * trstd * tmean, -0.5f * zrstd * zmean);
+      // (the z tile has landed, so the MMAs that read this stage's columns for the tile before are complete)
+      *reinterpret_cast<uint4*>(sAx + stage * 4096 + row * 16) = ln_aug_row(tmean, tve * trstd);
+      *reinterpret_cast<uint4*>(sAx + stage * 4096 + 2048 + row * 16) = ln_aug_row(zmean, 1.f / zrstd);
+      sStats[stage][row] = make_float2(0.5f * trstd, 0.5f * zrstd);
+      fence_proxy_async_smem();
       __syncwarp();
       if (lane == 0) {
         mbar_arrive(&sconv[stage]);
@@ -306,11 +321,10 @@ __global__ void __launch_bounds__(TO_THREADS, 1) tri_out_kernel(const __grid_con
     unsigned phase = 0;
     for (long long t = blockIdx.x; t < ntiles; t += gridDim.x) {
       unsigned char* zrow = sZ + stage * z_stage;
-      mbar_wait(&sconv[stage], phase, ab);
-      const float4 stt = sStats[stage][row];
-      const float trh = stt.x, zrh = stt.y, tmh = stt.z, zmh = stt.w;
-      mbar_wait(&tfull[stage], phase, ab);         // accumulator buffers and z stages advance together
+      mbar_wait(&tfull[stage], phase, ab);         // accumulator buffers and z stages advance together; the MMAs waited for the statistics
       tc_fence_after();
+      const float2 stt = sStats[stage][row];
+      const float2 tr2 = make_float2(stt.x, stt.x), zr2 = make_float2(stt.y, stt.y);
       const unsigned taddr = tmem_base + ((unsigned)(quarter * 32) << 16) + stage * 256;
 #pragma unroll 1
       for (int c0 = part * (c_z / 4); c0 < (part + 1) * (c_z / 4); c0 += 16) {
@@ -325,28 +339,12 @@ __global__ void __launch_bounds__(TO_THREADS, 1) tri_out_kernel(const __grid_con
           uint4* ptr = reinterpret_cast<uint4*>(zp + sw128_off(row, chunk16));
           uint4 v = *ptr;
           unsigned w[4] = {v.x, v.y, v.z, v.w};
-          const int cb = c0 + ch * 8;
-          const float4 co0 = *reinterpret_cast<const float4*>(sCo + cb), co1 = *reinterpret_cast<const float4*>(sCo + cb + 4);
-          const float4 cg0 = *reinterpret_cast<const float4*>(sCg + cb), cg1 = *reinterpret_cast<const float4*>(sCg + cb + 4);
-          const float4 ko0 = *reinterpret_cast<const float4*>(sKo + cb), ko1 = *reinterpret_cast<const float4*>(sKo + cb + 4);
-          const float4 kg0 = *reinterpret_cast<const float4*>(sKg + cb), kg1 = *reinterpret_cast<const float4*>(sKg + cb + 4);
-          // per channel: c0 / 2 - mean rstd c1 / 2, the part of the LayerNorm that does not depend on the accumulator
-          // (everything on packed float pairs: half the issue slots)
-          const float2 tm2 = make_float2(tmh, tmh), zm2 = make_float2(zmh, zmh), tr2 = make_float2(trh, trh), zr2 = make_float2(zrh, zrh);
-          const float2 bo[4] = {__ffma2_rn(tm2, make_float2(ko0.x, ko0.y), make_float2(co0.x, co0.y)),
-                                __ffma2_rn(tm2, make_float2(ko0.z, ko0.w), make_float2(co0.z, co0.w)),
-                                __ffma2_rn(tm2, make_float2(ko1.x, ko1.y), make_float2(co1.x, co1.y)),
-                                __ffma2_rn(tm2, make_float2(ko1.z, ko1.w), make_float2(co1.z, co1.w))};
-          const float2 bg[4] = {__ffma2_rn(zm2, make_float2(kg0.x, kg0.y), make_float2(cg0.x, cg0.y)),
-                                __ffma2_rn(zm2, make_float2(kg0.z, kg0.w), make_float2(cg0.z, cg0.w)),
-                                __ffma2_rn(zm2, make_float2(kg1.x, kg1.y), make_float2(cg1.x, cg1.y)),
-                                __ffma2_rn(zm2, make_float2(kg1.z, kg1.w), make_float2(cg1.z, cg1.w))};
 #pragma unroll
           for (int e = 0; e < 4; ++e) {
             const int n0 = ch * 8 + e * 2;
             const float2 z2 = make_float2(__uint_as_float(w[e] << 16), __uint_as_float(w[e] & 0xffff0000u));   // the bf16 state
-            const float2 oh = __ffma2_rn(tr2, make_float2(__uint_as_float(r1[n0]), __uint_as_float(r1[n0 + 1])), bo[e]);
-            const float2 ta = __ffma2_rn(zr2, make_float2(__uint_as_float(r2[n0]), __uint_as_float(r2[n0 + 1])), bg[e]);
+            const float2 oh = __fmul2_rn(tr2, make_float2(__uint_as_float(r1[n0]), __uint_as_float(r1[n0 + 1])));
+            const float2 ta = __fmul2_rn(zr2, make_float2(__uint_as_float(r2[n0]), __uint_as_float(r2[n0 + 1])));
             const float2 th = make_float2(to_tanh(ta.x), to_tanh(ta.y));
             const float2 res = __fadd2_rn(__ffma2_rn(oh, th, oh), z2);
             __nv_bfloat162 hh = __floats2bfloat162_rn(res.x, res.y);
@@ -399,7 +397,7 @@ nt_status fast_tri_out(void* z, const void* t, const TriPrep& tp, float eps, int
   const float2* c01g = (const float2*)tp.c01g;
   const int zslab = c_z / 64, hslab = c_h / 64;
   const size_t smem = (size_t)hslab * c_z * 128 + (size_t)zslab * c_z * 128 +
-                      2 * ((size_t)2 * c_h * 128 + (size_t)zslab * 128 * 128) + 4 * c_z * 4 + 1024;
+                      2 * ((size_t)2 * c_h * 128 + (size_t)zslab * 128 * 128) + 5 * 2048 + 2 * (size_t)c_z * 16 + 1024;
   // the attribute belongs to a (kernel, device) pair: one flag per device
   static bool attr_set_dev[64] = {};
   int attr_dev = 0;

@@ -369,6 +369,27 @@ __device__ inline void convert_row_bf16_to_f16(unsigned char* tile, int nslab, i
   sq = (q4[0] + q4[1]) + (q4[2] + q4[3]);
 }
 
+// LayerNorm folded into the MMA for a tile that stays as it is.  One more K step adds s c0 - mean c1 to the raw product,
+// s = 1 / rstd, so that rstd times the accumulator is the normalised projection and a reader of the accumulator needs no
+// tables.  Both sides are split into fp16 parts: the row side is (-m_hi, -m_lo, -m_hi, s_hi, s_hi, s_lo, 4096 s_rest,
+// -4096 m_rest), the weight side (c1_hi, c1_hi, c1_lo, c0_hi, c0_lo, c0_hi, c0_hi / 4096, c1_hi / 4096).
+__device__ inline uint4 ln_aug_row(float mean, float s) {
+  s = fminf(s, 65504.f);                              // above that the tile's own fp16 values have overflowed
+  const __half mh = __float2half_rn(-mean), sh = __float2half_rn(s);
+  const float m1 = -mean - __half2float(mh), s1 = s - __half2float(sh);
+  const __half ml = __float2half_rn(m1), sl = __float2half_rn(s1);
+  const __half mr = __float2half_rn((m1 - __half2float(ml)) * 4096.f), sr = __float2half_rn((s1 - __half2float(sl)) * 4096.f);
+  __half2 a[4] = {__halves2half2(mh, ml), __halves2half2(mh, sh), __halves2half2(sh, sl), __halves2half2(sr, mr)};
+  return *reinterpret_cast<const uint4*>(a);
+}
+__device__ inline uint4 ln_aug_weight(float c0, float c1) {
+  const __half c1h = __float2half_rn(c1), c1l = __float2half_rn(c1 - __half2float(c1h));
+  const __half c0h = __float2half_rn(c0), c0l = __float2half_rn(c0 - __half2float(c0h));
+  const __half c0s = __float2half_rn(__half2float(c0h) * (1.f / 4096.f)), c1s = __float2half_rn(__half2float(c1h) * (1.f / 4096.f));
+  __half2 a[4] = {__halves2half2(c1h, c1h), __halves2half2(c1l, c0h), __halves2half2(c0l, c0h), __halves2half2(c0s, c1s)};
+  return *reinterpret_cast<const uint4*>(a);
+}
+
 // LayerNorm folded into the MMA, activation side.  Two threads per tile row (hf = 0 / 1), each owning four of the
 // eight 16-byte chunks of every 64-channel slab of a K-major 128-byte-swizzled bf16 tile: the row is rewritten in
 // place as fp16 scaled by its rstd, and hf = 0 writes the row's augmentation columns (m_hi, m_lo, m_hi, 1, 1, 0, 0, 0),
