@@ -1,11 +1,14 @@
 // Attention output stage on tcgen05 (bf16, float accumulate), in place on the pair state:
 //   z += (sigmoid(LN(z) W_g^T) * o) W_o^T
 // The gate is recomputed from z here (LayerNorm folded into W_g: W_g' = bf16(W_g gamma) meets the bf16 state
-// directly, the row statistics are taken beside the MMA and applied in the epilogue) instead of
-// being written by the input projection.  Per 128-position tile: TMA brings the z tile and the o
-// tile; the MMA warp computes the gate pre-activation into TMEM as soon as they land; the epilogue warps turn it
-// into sigmoid(.) * o, written back over the o tile in shared memory; the MMA warp multiplies that by
-// W_o; the epilogue adds the residual into the z tile and TMA-stores it.
+// directly, the row statistics are taken beside the MMA and enter it as one more K step, ln_aug_row) instead of
+// being written by the input projection.  Per 128-position tile: TMA brings the z tile and the o tile; the gate MMAs
+// run as soon as they land; eight gate warps turn the result into sigmoid(.) * o, written back over the o tile in
+// shared memory; the output MMAs multiply that by W_o; eight output warps add the residual into the z tile, and a
+// warp of its own stores it.
+// Bound: the life of a tile -- load, gate MMA, gate warps, output MMA, output warps, store -- with room for two of them
+// beside the weights.  With one group of warps for both stages, the two tiles' lives did not overlap at all.
+// Measured at eight samples of about 215 positions: 79 us with one group of eight warps, 66 us so.
 //
 // Optional fused reduction (the mean over j that follows the attention in the block): while the finished tile is
 // still in shared memory the epilogue threads add up its columns per group of 32 positions, split at the one pair
@@ -19,7 +22,9 @@
 
 namespace ntp {
 
-constexpr int AO_THREADS = 64 + 128 + 256;   // producer, MMA, 4 statistics warps, 8 epilogue warps
+// producer, gate MMAs, 4 statistics warps, 8 gate warps, 8 output warps, store, output MMAs
+constexpr int AO_GATE = 6, AO_OUT = 14, AO_STORE = 22, AO_MMA2 = 23;
+constexpr int AO_THREADS = 32 * 24;
 
 struct AttnOutParams {
   CUtensorMap zmap;              // {c, rows}, box {64, 128}: load and store
@@ -45,8 +50,8 @@ __device__ inline float ao_tanh(float x) {
 
 __global__ void __launch_bounds__(AO_THREADS, 1) attn_out_kernel(const __grid_constant__ AttnOutParams p) {
   extern __shared__ unsigned char smem_raw[];
-  __shared__ __align__(8) unsigned long long bars[15];
-  __shared__ float2 sStats[2][128];        // per stage: (mean, rstd) of every z row
+  __shared__ __align__(8) unsigned long long bars[17];
+  __shared__ float sStats[2][128];         // per stage: rstd / 2 of every z row
   __shared__ unsigned tmem_base_s;
   __shared__ int abort_flag;
   unsigned char* smem = smem_raw + ((1024 - (smem_u32(smem_raw) & 1023)) & 1023);
@@ -58,8 +63,9 @@ __global__ void __launch_bounds__(AO_THREADS, 1) attn_out_kernel(const __grid_co
   unsigned char* sWg = smem;                          // zslab slabs of [Hd rows][64]
   unsigned char* sWo = sWg + zslab * wg_slab;         // oslab slabs of [c rows][64]
   unsigned char* sSt = sWo + oslab * wo_slab;         // 2 stages: z slabs then o slabs
-  float* sC0 = reinterpret_cast<float*>(sSt + 2 * stage_bytes);   // c0 / 2 per gate channel
-  float* sC1 = sC0 + Hd;                                          // c1 per gate channel
+  unsigned char* sAx = sSt + 2 * stage_bytes;         // [2 stages][128][8] fp16: augmentation columns 0-7 of the rows
+  unsigned char* sBx = sAx + 2 * 2048;                // [Hd][8] fp16: augmentation columns 0-7 of W_g
+  unsigned char* sZero = sBx + Hd * 16;               // [128][8] zeros: augmentation columns 8-15 of either
   unsigned long long* afull = bars;        // [2]
   unsigned long long* aempty = bars + 2;   // [2]
   unsigned long long* gfull = bars + 4;    // [2]
@@ -68,86 +74,106 @@ __global__ void __launch_bounds__(AO_THREADS, 1) attn_out_kernel(const __grid_co
   unsigned long long* tempty = bars + 10;  // [2]
   unsigned long long* wfull = bars + 12;
   unsigned long long* aconv = bars + 13;   // [2]
+  unsigned long long* zdone = bars + 15;   // [2] the new z is in the tile
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;   // warp-uniform for the compiler too
   if (threadIdx.x == 0) {
     abort_flag = 0;
     for (int s = 0; s < 2; ++s) {
       mbar_init(&afull[s], 1);
-      mbar_init(&aempty[s], p.partial ? 2 + 8 : 2);   // + the epilogue warps that read the tile for the column sums
+      mbar_init(&aempty[s], p.partial ? 2 + 8 : 2);   // output MMAs, store, + the output warps that read the tile for the column sums
       mbar_init(&gfull[s], 1);
       mbar_init(&ogated[s], 8);
       mbar_init(&ofull[s], 1);
       mbar_init(&tempty[s], 8);
       mbar_init(&aconv[s], 4);
+      mbar_init(&zdone[s], 8);
     }
     mbar_init(wfull, 1);
     mbar_fence_init();
   }
   if (warp == 1) tmem_alloc(&tmem_base_s, 512);
-  for (int n = threadIdx.x; n < Hd; n += AO_THREADS) {
-    sC0[n] = 0.5f * p.c01g[n].x;
-    sC1[n] = p.c01g[n].y;
-  }
+  for (int n = threadIdx.x; n < 128; n += AO_THREADS) *reinterpret_cast<uint4*>(sZero + n * 16) = make_uint4(0, 0, 0, 0);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   pdl_begin();
-  const unsigned tmem_base = tmem_base_s;
+  for (int n = threadIdx.x; n < Hd; n += AO_THREADS) {
+    const float2 k = p.c01g[n];
+    *reinterpret_cast<uint4*>(sBx + n * 16) = ln_aug_weight(k.x, k.y);
+  }
+  fence_proxy_async_smem();
+  __syncthreads();
+  const unsigned tmem_base = __shfl_sync(0xffffffffu, tmem_base_s, 0);
   AbortCtx ab{p.status, &abort_flag};
   const long long ntiles = (p.rows + 127) / 128;
 
-  if (warp == 0 && lane == 0) {
+  if (warp == 0) {
     // ------------------------------------------------------------------ producer
-    mbar_expect_tx(wfull, zslab * wg_slab + oslab * wo_slab);
-    for (int sl = 0; sl < zslab; ++sl) tma_load_2d(sWg + sl * wg_slab, &p.wgmap, wfull, sl * 64, 0);
-    for (int sl = 0; sl < oslab; ++sl) tma_load_2d(sWo + sl * wo_slab, &p.womap, wfull, sl * 64, 0);
-    int stage = 0;
-    unsigned phase = 0;
-    for (long long t = blockIdx.x; t < ntiles; t += gridDim.x) {
-      mbar_wait(&aempty[stage], phase ^ 1, ab);
-      mbar_expect_tx(&afull[stage], stage_bytes);
-      unsigned char* st = sSt + stage * stage_bytes;
-      for (int sl = 0; sl < zslab; ++sl) tma_load_2d(st + sl * slab, &p.zmap, &afull[stage], sl * 64, (int)(t * 128));
-      for (int sl = 0; sl < oslab; ++sl)
-        tma_load_2d(st + (zslab + sl) * slab, &p.omap, &afull[stage], sl * 64, (int)(t * 128));
-      if (++stage == 2) { stage = 0; phase ^= 1; }
+    if (lane == 0) {
+      mbar_expect_tx(wfull, zslab * wg_slab + oslab * wo_slab);
+      for (int sl = 0; sl < zslab; ++sl) tma_load_2d(sWg + sl * wg_slab, &p.wgmap, wfull, sl * 64, 0);
+      for (int sl = 0; sl < oslab; ++sl) tma_load_2d(sWo + sl * wo_slab, &p.womap, wfull, sl * 64, 0);
+      int stage = 0;
+      unsigned phase = 0;
+      for (long long t = blockIdx.x; t < ntiles; t += gridDim.x) {
+        mbar_wait(&aempty[stage], phase ^ 1, ab);
+        mbar_expect_tx(&afull[stage], stage_bytes);
+        unsigned char* st = sSt + stage * stage_bytes;
+        for (int sl = 0; sl < zslab; ++sl) tma_load_2d(st + sl * slab, &p.zmap, &afull[stage], sl * 64, (int)(t * 128));
+        for (int sl = 0; sl < oslab; ++sl)
+          tma_load_2d(st + (zslab + sl) * slab, &p.omap, &afull[stage], sl * 64, (int)(t * 128));
+        if (++stage == 2) { stage = 0; phase ^= 1; }
+      }
     }
   } else if (warp == 1) {
-    // ------------------------------------------------------------------ MMA issuer (whole warp, one elected lane issues)
+    // ------------------------------------------------------------------ gate MMAs (whole warp, one elected lane issues)
     mbar_wait(wfull, 0, ab);
     int stage = 0;
-    unsigned phase = 0, tph0 = 0, tph1 = 0, gph0 = 0, gph1 = 0;
-    unsigned n = 0;
+    unsigned phase = 0;
     const unsigned idesc_g = idesc_f16(128, Hd, 0, 0, FMT_BF16, FMT_BF16);  // the bf16 z tile, folded W_g bf16
-    const unsigned idesc_o = idesc_f16(128, c, 0, 0, FMT_BF16, FMT_BF16);   // gated o bf16, W_o as given (bf16)
-    const unsigned long long wg_desc = desc_kmajor_sw128(smem_u32(sWg)), wo_desc = desc_kmajor_sw128(smem_u32(sWo));
-    const unsigned slab16 = (unsigned)slab >> 4, wg16 = (unsigned)wg_slab >> 4, wo16 = (unsigned)wo_slab >> 4;
-    for (long long t = blockIdx.x; t < ntiles; t += gridDim.x, ++n) {
-      const unsigned buf = n & 1;
-      if (buf == 0) { mbar_wait(&tempty[0], tph0 ^ 1, ab); tph0 ^= 1; }
-      else { mbar_wait(&tempty[1], tph1 ^ 1, ab); tph1 ^= 1; }
+    const unsigned idesc_x = idesc_f16(128, Hd, 0, 0, FMT_F16, FMT_F16);    // augmentation step
+    const unsigned long long wg_desc = desc_kmajor_sw128(smem_u32(sWg));
+    const unsigned slab16 = (unsigned)slab >> 4, wg16 = (unsigned)wg_slab >> 4;
+    const unsigned bx = smem_u32(sBx), zero = smem_u32(sZero);
+    for (long long t = blockIdx.x; t < ntiles; t += gridDim.x) {
+      mbar_wait(&tempty[stage], phase ^ 1, ab);              // accumulators and stages advance together
       mbar_wait(&afull[stage], phase, ab);
       tc_fence_after();
       const unsigned long long st_desc = desc_kmajor_sw128(smem_u32(sSt + stage * stage_bytes));
-      const unsigned dg = tmem_base + buf * 256, dout = dg + Hd;
+      const unsigned dg = tmem_base + stage * 256;
 #pragma unroll
-      for (int ks = 0; ks < 8; ++ks)
-        if (ks < c / 16 && elect_one())
-          umma_bf16(dg, st_desc + ((ks >> 2) * slab16 + (ks & 3) * 2), wg_desc + ((ks >> 2) * wg16 + (ks & 3) * 2), idesc_g, ks != 0);
-      if (elect_one()) tc_commit(&gfull[buf]);
-      __syncwarp();
-      // gated o tile written back by the epilogue warps
-      if (buf == 0) { mbar_wait(&ogated[0], gph0, ab); gph0 ^= 1; }
-      else { mbar_wait(&ogated[1], gph1, ab); gph1 ^= 1; }
+      for (int sl = 0; sl < 2; ++sl)
+        if (sl < zslab) umma_k4(dg, st_desc + sl * slab16, wg_desc + sl * wg16, idesc_g, sl);
+      mbar_wait(&aconv[stage], phase, ab);                   // the rows' augmentation columns are written
       tc_fence_after();
-#pragma unroll
-      for (int ks = 0; ks < 8; ++ks)
-        if (ks < Hd / 16 && elect_one())
-          umma_bf16(dout, st_desc + ((zslab + (ks >> 2)) * slab16 + (ks & 3) * 2), wo_desc + ((ks >> 2) * wo16 + (ks & 3) * 2),
-                    idesc_o, ks != 0);
+      const unsigned ax = smem_u32(sAx + stage * 2048);
       if (elect_one()) {
-        tc_commit(&ofull[buf]);
+        umma_bf16(dg, desc_kmajor_nosw(ax, zero - ax, 128), desc_kmajor_nosw(bx, zero - bx, 128), idesc_x, 1);
+        tc_commit(&gfull[stage]);
+      }
+      __syncwarp();
+      if (++stage == 2) { stage = 0; phase ^= 1; }
+    }
+  } else if (warp == AO_MMA2) {
+    // ------------------------------------------------------------------ output MMAs: an issuer of their own, so that they
+    // never wait for the next tile's load and its gate MMAs never for this tile's gate warps
+    mbar_wait(wfull, 0, ab);
+    int stage = 0;
+    unsigned phase = 0;
+    const unsigned idesc_o = idesc_f16(128, c, 0, 0, FMT_BF16, FMT_BF16);   // gated o bf16, W_o as given (bf16)
+    const unsigned long long wo_desc = desc_kmajor_sw128(smem_u32(sWo));
+    const unsigned slab16 = (unsigned)slab >> 4, wo16 = (unsigned)wo_slab >> 4;
+    for (long long t = blockIdx.x; t < ntiles; t += gridDim.x) {
+      mbar_wait(&ogated[stage], phase, ab);
+      tc_fence_after();
+      const unsigned long long o_desc = desc_kmajor_sw128(smem_u32(sSt + stage * stage_bytes + zslab * slab));
+      const unsigned dout = tmem_base + stage * 256 + Hd;
+#pragma unroll
+      for (int sl = 0; sl < 2; ++sl)
+        if (sl < oslab) umma_k4(dout, o_desc + sl * slab16, wo_desc + sl * wo16, idesc_o, sl);
+      if (elect_one()) {
+        tc_commit(&ofull[stage]);
         tc_commit(&aempty[stage]);
       }
       __syncwarp();
@@ -163,7 +189,9 @@ __global__ void __launch_bounds__(AO_THREADS, 1) attn_out_kernel(const __grid_co
       if (p.zstats) {                       // the input projection normalised the same rows: take its statistics
         const float2 zst = t * 128 + row < p.rows ? *(p.zstats + t * 128 + row) : make_float2(0.f, 1.f);
         mbar_wait(&afull[stage], phase, ab);
-        sStats[stage][row] = zst;
+        *reinterpret_cast<uint4*>(sAx + stage * 2048 + row * 16) = ln_aug_row(zst.x, 1.f / zst.y);
+        sStats[stage][row] = 0.5f * zst.y;
+        fence_proxy_async_smem();
         __syncwarp();
         if (lane == 0) mbar_arrive(&aconv[stage]);
         if (++stage == 2) { stage = 0; phase ^= 1; }
@@ -185,32 +213,31 @@ __global__ void __launch_bounds__(AO_THREADS, 1) attn_out_kernel(const __grid_co
       }
       const float sum = (s4[0] + s4[1]) + (s4[2] + s4[3]), sq = (q4[0] + q4[1]) + (q4[2] + q4[3]);
       const float mean = sum / (float)c;
-      sStats[stage][row] = make_float2(mean, rsqrtf(fmaxf(sq / (float)c - mean * mean, 0.f) + p.eps));
+      const float ve = fmaxf(sq / (float)c - mean * mean, 0.f) + p.eps, rstd = rsqrtf(ve);
+      *reinterpret_cast<uint4*>(sAx + stage * 2048 + row * 16) = ln_aug_row(mean, ve * rstd);
+      sStats[stage][row] = 0.5f * rstd;
+      fence_proxy_async_smem();
       __syncwarp();
       if (lane == 0) mbar_arrive(&aconv[stage]);
       if (++stage == 2) { stage = 0; phase ^= 1; }
     }
-  } else if (warp >= 6) {
-    // ------------------------------------------------------------------ epilogue (8 warps)
+  } else if (warp < AO_OUT) {
+    // ------------------------------------------------------------------ gate warps: o <- sigmoid(gate) * o, in place in shared memory
     const int quarter = warp & 3;
-    const int half = (warp - 6) >> 2;
+    const int half = (warp - AO_GATE) >> 2;
     const int row = quarter * 32 + lane;
-    const int ep_tid = threadIdx.x - 192;
     int stage = 0;
-    unsigned gph[2] = {0, 0}, oph[2] = {0, 0};
-    long long n = 0;
-    for (long long t = blockIdx.x; t < ntiles; t += gridDim.x, ++n) {
-      const int buf = (int)(n & 1);
+    unsigned phase = 0;
+    for (long long t = blockIdx.x; t < ntiles; t += gridDim.x) {
       unsigned char* st = sSt + stage * stage_bytes;
-      // ---- phase 1: o <- sigmoid(gate) * o, in place in shared memory
-      mbar_wait(&aconv[stage], (unsigned)((n >> 1) & 1), ab);   // the row statistics are published
-      mbar_wait(&gfull[buf], gph[buf], ab);
-      gph[buf] ^= 1;
+      mbar_wait(&gfull[stage], phase, ab);
+      mbar_wait(&aconv[stage], phase, ab);   // (long complete: orders the read of what the statistics warps left)
       tc_fence_after();
-      // sigmoid(x) = tanh(x / 2) / 2 + 1 / 2 with x / 2 = (rstd / 2) acc + (c0 / 2 - mean (rstd / 2) c1), on packed float pairs
-      const float rh = 0.5f * sStats[stage][row].y, mh = -sStats[stage][row].x * rh;
-      const float2 rh2 = make_float2(rh, rh), mh2 = make_float2(mh, mh), half2 = make_float2(0.5f, 0.5f);
-      const unsigned taddr = tmem_base + ((unsigned)(quarter * 32) << 16) + buf * 256;
+      // sigmoid(x) o = tanh(x / 2) (o / 2) + o / 2 with x / 2 = (rstd / 2) acc, on packed float pairs
+      const float rh = sStats[stage][row];
+      const float2 rh2 = make_float2(rh, rh), half2 = make_float2(0.5f, 0.5f);
+      const unsigned taddr = tmem_base + ((unsigned)(quarter * 32) << 16) + stage * 256;
+#pragma unroll 1
       for (int c0 = half * (Hd / 2); c0 < (half + 1) * (Hd / 2); c0 += 32) {
         unsigned r[32];
         tmem_ld32(taddr + c0, r);
@@ -224,10 +251,9 @@ __global__ void __launch_bounds__(AO_THREADS, 1) attn_out_kernel(const __grid_co
 #pragma unroll
           for (int e = 0; e < 4; ++e) {
             const int n0 = ch * 8 + e * 2;
-            const float2 k0 = *reinterpret_cast<const float2*>(sC0 + c0 + n0), k1 = *reinterpret_cast<const float2*>(sC1 + c0 + n0);
-            const float2 xh = __ffma2_rn(rh2, make_float2(__uint_as_float(r[n0]), __uint_as_float(r[n0 + 1])), __ffma2_rn(mh2, k1, k0));
-            const float2 g = __ffma2_rn(half2, make_float2(ao_tanh(xh.x), ao_tanh(xh.y)), half2);
-            const float2 go = __fmul2_rn(g, make_float2(__uint_as_float(w[e] << 16), __uint_as_float(w[e] & 0xffff0000u)));
+            const float2 xh = __fmul2_rn(rh2, make_float2(__uint_as_float(r[n0]), __uint_as_float(r[n0 + 1])));
+            const float2 oh = __fmul2_rn(half2, make_float2(__uint_as_float(w[e] << 16), __uint_as_float(w[e] & 0xffff0000u)));
+            const float2 go = __ffma2_rn(make_float2(ao_tanh(xh.x), ao_tanh(xh.y)), oh, oh);
             __nv_bfloat162 hh = __floats2bfloat162_rn(go.x, go.y);
             w[e] = *reinterpret_cast<unsigned*>(&hh);
           }
@@ -237,11 +263,23 @@ __global__ void __launch_bounds__(AO_THREADS, 1) attn_out_kernel(const __grid_co
       tc_fence_before();
       fence_proxy_async_smem();
       __syncwarp();
-      if (lane == 0) mbar_arrive(&ogated[buf]);
-      // ---- phase 2: z += (gated o) W_o^T, in place in the z tile, then store
-      mbar_wait(&ofull[buf], oph[buf], ab);
-      oph[buf] ^= 1;
+      if (lane == 0) mbar_arrive(&ogated[stage]);
+      if (++stage == 2) { stage = 0; phase ^= 1; }
+    }
+  } else if (warp < AO_STORE) {
+    // ------------------------------------------------------------------ output warps: z += (gated o) W_o^T, in place in the z tile
+    const int quarter = warp & 3;
+    const int half = (warp - AO_OUT) >> 2;
+    const int row = quarter * 32 + lane;
+    const int ep_tid = threadIdx.x - AO_OUT * 32;
+    int stage = 0;
+    unsigned phase = 0;
+    for (long long t = blockIdx.x; t < ntiles; t += gridDim.x) {
+      unsigned char* st = sSt + stage * stage_bytes;
+      const unsigned taddr = tmem_base + ((unsigned)(quarter * 32) << 16) + stage * 256;
+      mbar_wait(&ofull[stage], phase, ab);
       tc_fence_after();
+#pragma unroll 1
       for (int c0 = half * (c / 2); c0 < (half + 1) * (c / 2); c0 += 32) {
         unsigned r[32];
         tmem_ld32(taddr + Hd + c0, r);
@@ -264,15 +302,14 @@ __global__ void __launch_bounds__(AO_THREADS, 1) attn_out_kernel(const __grid_co
         }
       }
       tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&tempty[buf]);
       fence_proxy_async_smem();
-      named_bar_sync(1, 256);
-      if (ep_tid == 0) {
-        for (int sl = 0; sl < zslab; ++sl) tma_store_2d(&p.zmap, st + sl * slab, sl * 64, (int)(t * 128));
-        tma_store_commit();
+      __syncwarp();
+      if (lane == 0) {
+        mbar_arrive(&tempty[stage]);
+        mbar_arrive(&zdone[stage]);
       }
       if (p.partial) {
+        named_bar_sync(1, 256);
         // thread = (channel pair, quarter of the tile): column sums of 32 positions, split at the pair row boundary
         const int cp = ep_tid & 63, q = ep_tid >> 6;
         const long long p0 = t * 128 + q * 32;
@@ -318,13 +355,22 @@ __global__ void __launch_bounds__(AO_THREADS, 1) attn_out_kernel(const __grid_co
         __syncwarp();
         if (lane == 0) mbar_arrive(&aempty[stage]);      // this warp has read what it needs of the tile
       }
-      if (ep_tid == 0) {
-        tma_store_wait_read0();
-        mbar_arrive(&aempty[stage]);
-      }
-      if (++stage == 2) stage = 0;
+      if (++stage == 2) { stage = 0; phase ^= 1; }
     }
-    if (ep_tid == 0) tma_store_wait_all0();
+  } else if (warp == AO_STORE) {
+    // ------------------------------------------------------------------ store: lane l takes slab l
+    int stage = 0;
+    unsigned phase = 0;
+    for (long long t = blockIdx.x; t < ntiles; t += gridDim.x) {
+      mbar_wait(&zdone[stage], phase, ab);
+      if (lane < zslab) tma_store_2d(&p.zmap, sSt + stage * stage_bytes + lane * slab, lane * 64, (int)(t * 128));
+      tma_store_commit();
+      tma_store_wait_read0();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&aempty[stage]);
+      if (++stage == 2) { stage = 0; phase ^= 1; }
+    }
+    tma_store_wait_all0();
   }
   tc_fence_before();
   __syncthreads();
@@ -396,7 +442,7 @@ nt_status fast_attn_out(void* z, const void* o, const void* W_o, const AttnPrep&
   const float2* c01g = (const float2*)ap.c01g;
   const int zslab = c / 64, oslab = Hd / 64;
   const size_t smem = (size_t)zslab * Hd * 128 + (size_t)oslab * c * 128 + 2 * (size_t)(zslab + oslab) * 128 * 128 +
-                      (size_t)Hd * 8 + 1024;
+                      3 * 2048 + (size_t)Hd * 16 + 1024;
   // the attribute belongs to a (kernel, device) pair: one flag per device
   static bool attr_set_dev[64] = {};
   int attr_dev = 0;
