@@ -94,7 +94,7 @@ __global__ void __launch_bounds__(TI_THREADS, 1) tri_in_kernel(const __grid_cons
   unsigned long long* wfull = bars + 8;
   unsigned long long* aconv = bars + 9;    // [2] tile normalised / converted, augmentation written
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;   // warp-uniform for the compiler too
   if (threadIdx.x == 0) {
     abort_flag = 0;
     for (int s = 0; s < 2; ++s) {
@@ -116,7 +116,7 @@ __global__ void __launch_bounds__(TI_THREADS, 1) tri_in_kernel(const __grid_cons
   __syncthreads();
   tc_fence_after();
   pdl_begin();
-  const unsigned tmem_base = tmem_base_s;
+  const unsigned tmem_base = __shfl_sync(0xffffffffu, tmem_base_s, 0);
   AbortCtx ab{p.status, &abort_flag};
   const long long nchunks = p.chunk_off[p.B];
   const long long ntiles = (nchunks + 3) / 4;
@@ -182,13 +182,7 @@ __global__ void __launch_bounds__(TI_THREADS, 1) tri_in_kernel(const __grid_cons
           const unsigned d_tmem = tmem_base + buf * 256 + part * 128;
 #pragma unroll
           for (int sl = 0; sl < 2; ++sl) {
-            if (sl < nslab) {
-#pragma unroll
-              for (int k4 = 0; k4 < 4; ++k4)
-                if (elect_one())
-                  umma_bf16(d_tmem, w_desc + (sl * w_slab16 + row16 + k4 * 2), z_desc + (sl * z_slab16 + k4 * 2), idesc,
-                            (sl | k4) != 0);
-            }
+            if (sl < nslab) umma_k4(d_tmem, w_desc + (sl * w_slab16 + row16), z_desc + sl * z_slab16, idesc, sl);
           }
           // augmentation K step: c1 / c0 columns against the (-mean rstd, 1) columns (16-byte rows)
           const unsigned wxa = wx_addr + (unsigned)(u * 256 + part * 128) * 16;
@@ -295,7 +289,7 @@ __global__ void __launch_bounds__(TI_THREADS, 1) tri_in_kernel(const __grid_cons
         // four steps of 16 positions; the TMEM loads of step k + 1 are in flight while step k is computed.  A step's
         // 32 channels x 16 positions go through a 1 KB staging tile and out with one TMA store (runs of 32 bytes per
         // channel row, clipped at the row end), which keeps the scattered writes off the load / store units.
-        unsigned rg[2][16], rv[2][16];
+        unsigned rg[2][16], rv[2][16], w[2][8];
         tmem_ld16(taddr, rg[0]);
         tmem_ld16(taddr + 128, rv[0]);
 #pragma unroll
@@ -306,7 +300,6 @@ __global__ void __launch_bounds__(TI_THREADS, 1) tri_in_kernel(const __grid_cons
             tmem_ld16(taddr + 128 + (k + 1) * 16, rv[(k + 1) & 1]);
           }
           const int4 info = tinfo[tn & 7][half * 2 + (k >> 1)];
-          unsigned w[8];
 #pragma unroll
           for (int e = 0; e < 8; ++e) {
             // the gate and value weight rows were folded times 1/2, so with g' = g / 2, v' = v / 2:
@@ -316,21 +309,23 @@ __global__ void __launch_bounds__(TI_THREADS, 1) tri_in_kernel(const __grid_cons
             const float v1 = fmaf(h1, tanh_fast(__uint_as_float(rg[k & 1][2 * e + 1])), h1);
             __half2 h = __floats2half2_rn(v0, v1);          // overflow gives inf, clamped below
             h = __hmax2(__hmin2(h, hmax2), hmin2);
-            w[e] = *reinterpret_cast<unsigned*>(&h);
+            w[k & 1][e] = *reinterpret_cast<unsigned*>(&h);
           }
           // a chunk (two steps, 32 positions) is staged as 32 channel rows of 64 bytes and leaves with one TMA store:
           // the store engine's cost is per row, so rows should be as long as the tile geometry allows
-          if ((k & 1) == 0) {
-            if (lane == 0) tma_store_wait_read0();          // the previous chunk's store has read the staging tile
-            __syncwarp();
-          }
-          // 64-byte swizzle of the store map: the 16-byte pieces of a row are XOR-ed with the row's bits 1-2, so eight
-          // lanes cover all banks
-          unsigned char* rowp = stg0 + lane * 64;
-          const int sw = (lane >> 1) & 3;
-          *reinterpret_cast<uint4*>(rowp + ((((k & 1) * 2) ^ sw) << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
-          *reinterpret_cast<uint4*>(rowp + ((((k & 1) * 2 + 1) ^ sw) << 4)) = make_uint4(w[4], w[5], w[6], w[7]);
           if (k & 1) {
+            // The store of the chunk before has had two steps of arithmetic to read the staging tile.  (Waiting after the first
+            // step: 83.3 us per launch at eight samples of about 215 positions, 76.9 so.)
+            if (lane == 0) tma_store_wait_read0();
+            __syncwarp();
+            // 64-byte swizzle of the store map: the 16-byte pieces of a row are XOR-ed with the row's bits 1-2, so eight
+            // lanes cover all banks
+            unsigned char* rowp = stg0 + lane * 64;
+            const int sw = (lane >> 1) & 3;
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+              *reinterpret_cast<uint4*>(rowp + ((e ^ sw) << 4)) =
+                  make_uint4(w[e >> 1][(e & 1) * 4], w[e >> 1][(e & 1) * 4 + 1], w[e >> 1][(e & 1) * 4 + 2], w[e >> 1][(e & 1) * 4 + 3]);
             fence_proxy_async_smem();
             __syncwarp();
             if (lane == 0 && info.w) {
