@@ -148,10 +148,7 @@ __global__ void __launch_bounds__(AI_THREADS, 1) attn_in_kernel(const __grid_con
 #pragma unroll
         for (int sl = 0; sl < 2; ++sl)
           if (sl < nslab) {
-#pragma unroll
-            for (int k4 = 0; k4 < 4; ++k4)
-              if (elect_one())
-                umma_bf16(d_tmem, a_desc + (sl * a16 + k4 * 2), w_desc + (sl * w16 + row16 + k4 * 2), idesc, (sl | k4) != 0);
+            umma_k4(d_tmem, a_desc + sl * a16, w_desc + (sl * w16 + row16), idesc, sl);
           }
         // augmentation K step: (-mean rstd, 1) columns against the c1 / c0 columns (16-byte rows)
         if (elect_one()) umma_bf16(d_tmem, ax_desc, wx_desc + (unsigned)u_row[u], idesc, 1);
@@ -183,10 +180,8 @@ __global__ void __launch_bounds__(AI_THREADS, 1) attn_in_kernel(const __grid_con
     const int quarter = warp & 3;
     const int half = (warp - AI_EPI_WARP0) >> 2;
     const int row = quarter * 32 + lane;
-    const int ep_tid = threadIdx.x - 32 * AI_EPI_WARP0;
     const int cpw = Hd / 2;                         // channels of one output handled by this warp
-    int stage = 0;
-    unsigned phase = 0, tph[2] = {0, 0};
+    unsigned tph[2] = {0, 0};
     long long unit = 0;
     bool store_pending = false;
     for (long long t = blockIdx.x; t < ntiles; t += gridDim.x) {
@@ -204,28 +199,41 @@ __global__ void __launch_bounds__(AI_THREADS, 1) attn_in_kernel(const __grid_con
             // warps of a lane quarter share the slab and meet at a barrier of their own), so no store waits for the
             // other warps and only the warp's own previous store has to have read its corner of the panels.
             const bool storer = lane == 0 && (npanel == 2 || half == 0);
+            // The output before has the time of this one's loads and conversions to leave the panels.  (Waiting first: 83 us
+            // per launch at eight samples of about 215 positions, 77 so; line stores from registers instead of the copy engine: 86.)
+            unsigned w[32];
+#pragma unroll
+            for (int ci = 0; ci < 2; ++ci)
+              if (ci * 32 < cpw) {
+                unsigned r[32];
+                tmem_ld32(taddr + oi * Hd + half * cpw + ci * 32, r);
+                tmem_ld_wait();
+#pragma unroll
+                for (int e = 0; e < 16; ++e) {
+                  __nv_bfloat162 hh = __floats2bfloat162_rn(__uint_as_float(r[2 * e]), __uint_as_float(r[2 * e + 1]));
+                  w[ci * 16 + e] = *reinterpret_cast<unsigned*>(&hh);
+                }
+              }
+            if (oi == nout - 1) {                           // the accumulator has been read
+              tc_fence_before();
+              __syncwarp();
+              if (lane == 0) mbar_arrive(&tempty[buf]);
+            }
             if (store_pending) {
               if (storer) tma_store_wait_read0();
               if (npanel == 1) named_bar_sync(2 + quarter, 64);
               else __syncwarp();
             }
-            for (int c0 = half * cpw; c0 < (half + 1) * cpw; c0 += 32) {
-              unsigned r[32];
-              tmem_ld32(taddr + oi * Hd + c0, r);
-              tmem_ld_wait();
-              unsigned char* panel = sOut + (c0 >> 6) * a_slab;
 #pragma unroll
-              for (int ch = 0; ch < 4; ++ch) {
-                unsigned w[4];
+            for (int ci = 0; ci < 2; ++ci)
+              if (ci * 32 < cpw) {
+                const int c0 = half * cpw + ci * 32;
+                unsigned char* panel = sOut + (c0 >> 6) * a_slab;
 #pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                  const int n0 = ch * 8 + e * 2;
-                  __nv_bfloat162 hh = __floats2bfloat162_rn(__uint_as_float(r[n0]), __uint_as_float(r[n0 + 1]));
-                  w[e] = *reinterpret_cast<unsigned*>(&hh);
-                }
-                *reinterpret_cast<uint4*>(panel + sw128_off(row, ((c0 & 63) >> 3) + ch)) = make_uint4(w[0], w[1], w[2], w[3]);
+                for (int ch = 0; ch < 4; ++ch)
+                  *reinterpret_cast<uint4*>(panel + sw128_off(row, ((c0 & 63) >> 3) + ch)) =
+                      make_uint4(w[ci * 16 + ch * 4], w[ci * 16 + ch * 4 + 1], w[ci * 16 + ch * 4 + 2], w[ci * 16 + ch * 4 + 3]);
               }
-            }
             fence_proxy_async_smem();
             if (npanel == 1) named_bar_sync(2 + quarter, 64);
             else __syncwarp();
@@ -239,9 +247,9 @@ __global__ void __launch_bounds__(AI_THREADS, 1) attn_in_kernel(const __grid_con
           }
         } else if (half == 0) {
           // bias: H values per position, written head-major / channel-major
-          unsigned r[32];
-          tmem_ld32(taddr, r);
-          tmem_ld_wait();
+          unsigned r[16];
+          tmem_ld16(taddr, r);
+          tmem_ld_wait16(r);
           const long long P = t * 128 + row;
           if (P < p.rows) {
             int s = 0;
@@ -252,16 +260,18 @@ __global__ void __launch_bounds__(AI_THREADS, 1) attn_in_kernel(const __grid_con
             // (transposed planes: the register-fragment core reads a query's keys contiguously, and in column-wise attention
             // the bias of (query i, key k) is the plane's element [k][i])
             __nv_bfloat16* bp = p.bias + (long long)p.H * p.cm_off[s] + (N > p.bias_tr_above ? (long long)j * ld + i : (long long)i * ld + j);
-            for (int h = 0; h < p.H; ++h)
-              if (NT_IN((bp - p.bias) + (long long)h * N * ld, p.bias_elems, NT_SITE_ATTN_IN_BIAS))
+#pragma unroll
+            for (int h = 0; h < 16; ++h)
+              if (h < p.H && NT_IN((bp - p.bias) + (long long)h * N * ld, p.bias_elems, NT_SITE_ATTN_IN_BIAS))
                 bp[(long long)h * N * ld] = __float2bfloat16_rn(__uint_as_float(r[h]));
           }
         }
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&tempty[buf]);
+        if (u == 2) {
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&tempty[buf]);
+        }
       }
-      if (++stage == 2) { stage = 0; phase ^= 1; }
     }
     if (lane == 0) tma_store_wait_all0();
   }
