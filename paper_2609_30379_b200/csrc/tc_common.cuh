@@ -275,7 +275,7 @@ __device__ inline unsigned long long desc_kmajor_nosw(unsigned saddr, unsigned l
   return d;
 }
 // instruction descriptor of kind::f16: D = f32, M x N tile, operand majors (0 = K-major, 1 = MN-major)
-// and per-operand 16-bit formats (FMT_F16 or FMT_BF16; the two operands may differ)
+// and the 16-bit format, FMT_F16 or FMT_BF16, the same for both operands
 constexpr int FMT_F16 = 0, FMT_BF16 = 1;
 __device__ inline unsigned idesc_f16(int M, int N, int a_mn_major, int b_mn_major, int a_fmt, int b_fmt) {
   return (1u << 4) | ((unsigned)a_fmt << 7) | ((unsigned)b_fmt << 10) | ((unsigned)a_mn_major << 15) |
