@@ -62,9 +62,8 @@ def kernel_work(cfg: wl.Config):
         R = T1
         w["generic_attn_in"] = dict(bytes=R * (c_z + 4 * Hd) * e, flops=2 * R * c_z * 4 * Hd)
         w["generic_attn_core"] = w["attn_core"] = w["attn_core_tok"] = dict(bytes=R * 4 * Hd * e, flops=4 * T2 * Hd, exps=T2 * H)
-        # token-side projections of the tensor-core path: q | k in one launch, v in another, the output projection
-        w["tok_attn_in_qk"] = dict(bytes=R * (c_z + 2 * Hd) * e + 2 * Hd * c_z * e, flops=2 * R * c_z * 2 * Hd)
-        w["tok_attn_in_vg"] = dict(bytes=R * (c_z + Hd) * e + Hd * c_z * e, flops=2 * R * c_z * Hd)
+        # token-side projections of the tensor-core path: q | k | v in one launch, the output projection
+        w["tok_attn_in"] = dict(bytes=R * (c_z + 3 * Hd) * e + 3 * Hd * c_z * e, flops=2 * R * c_z * 3 * Hd)
         w["tok_attn_out"] = dict(bytes=R * (Hd + 2 * c_z) * e + c_z * Hd * e, flops=2 * R * Hd * c_z)
         w["generic_attn_out"] = w["attn_out"] = dict(bytes=R * (Hd + 2 * c_z) * e + c_z * Hd * e, flops=2 * R * Hd * c_z)
         w["segment_reduce"] = w["generic_segment_reduce"] = dict(bytes=R * c_z * e, flops=R * c_z)

@@ -209,7 +209,8 @@ static nt_status pair_broadcast_impl(const nt_layout* L, const Totals& tot, int 
   pa.add(W_b, nullptr, c_z, ACT_NONE, v, O_STORE, 1);
   nt_status r;
   if (fast && fast_token_gemm_supported(c_s, c_z, c_z)) {
-    r = fast_token_gemm(x, tot.T1, c_s, W_a, c_z, u, W_b, c_z, v, 1, 0, "tok_proj", st);
+    const TokSeg seg[2] = {{x, tot.T1, W_a, c_z, u}, {x, tot.T1, W_b, c_z, v}};
+    r = fast_token_gemm(seg, 2, c_s, 1, 0, "tok_proj", st);
     if (r != NT_OK) return r;
   } else {
     r = launch_proj<T>(pa, dummy, st, "generic_tok_proj");
@@ -316,7 +317,7 @@ static nt_status attn_generic(const nt_layout* L, const Totals& tot, nt_order or
     nt_status r;
     if (tok_fast) {
       // token order: the rows are T1 tokens, so the projections are small GEMMs on mma.sync tiles around the
-      // segmented core: LayerNorm once into the (not yet written) o buffer, q | k and v | g in two launches that share
+      // segmented core: LayerNorm once into the (not yet written) o buffer, q | k | v | g in one launch that shares
       // the normalised rows, the core, the gate, the output GEMM accumulated into x
       const size_t e = 2, to = (size_t)row0 * Hd * e;
       char* xr = (char*)zx + (size_t)row0 * c * e;
@@ -325,12 +326,13 @@ static nt_status attn_generic(const nt_layout* L, const Totals& tot, nt_order or
         xh = (char*)w.o + to;
         if ((r = fast_ln_rows(xr, W->ln_gamma, W->ln_beta, eps, c, rows, xh, st, "tok_attn_ln")) != NT_OK) return r;
       }
-      if ((r = fast_token_gemm(xh, rows, c, W->W_q, Hd, (char*)w.q + to, W->W_k, Hd, (char*)w.k + to, 0, 0, "tok_attn_in_qk", st)) != NT_OK) return r;
-      if ((r = fast_token_gemm(xh, rows, c, W->W_v, Hd, (char*)w.v + to, W->W_g, W->W_g ? Hd : 0, W->W_g ? (char*)w.g + to : nullptr, 0, 0,
-                               "tok_attn_in_vg", st)) != NT_OK) return r;
+      const TokSeg seg[4] = {{xh, rows, W->W_q, Hd, (char*)w.q + to}, {xh, rows, W->W_k, Hd, (char*)w.k + to}, {xh, rows, W->W_v, Hd, (char*)w.v + to},
+                             {xh, rows, W->W_g, Hd, W->W_g ? (char*)w.g + to : nullptr}};
+      if ((r = fast_token_gemm(seg, 4, c, 0, 0, "tok_attn_in", st)) != NT_OK) return r;
       if ((r = fast_attn_core_fr(w.q, w.k, w.v, nullptr, w.o, H, d, FR_MODE_TOKEN, m, L->status_d, st)) != NT_OK) return r;
       if (W->W_g && (r = fast_gate_mul((char*)w.g + to, (char*)w.o + to, rows * Hd, st, "tok_attn_gate")) != NT_OK) return r;
-      if ((r = fast_token_gemm((char*)w.o + to, rows, Hd, W->W_o, c, xr, nullptr, 0, nullptr, 0, 1, "tok_attn_out", st)) != NT_OK) return r;
+      const TokSeg so = {(char*)w.o + to, rows, W->W_o, c, xr};
+      if ((r = fast_token_gemm(&so, 1, Hd, 0, 1, "tok_attn_out", st)) != NT_OK) return r;
       continue;
     }
     ProjArgs pa{};
@@ -435,12 +437,14 @@ static nt_status single_attn_impl(const nt_layout* L, const Totals& tot, int c_s
       char* xh = (char*)w.xh + (size_t)trow0 * c_s * e;
       const size_t to = (size_t)trow0 * Hd * e;
       if ((r = fast_ln_rows(xr, W->ln_gamma, W->ln_beta, eps, c_s, trows, xh, st)) != NT_OK) return r;
-      if ((r = fast_token_gemm(xh, trows, c_s, W->W_q, Hd, (char*)w.q + to, W->W_k, Hd, (char*)w.k + to, 0, 0, "single_attn_in_qk", st)) != NT_OK) return r;
-      if ((r = fast_token_gemm(xh, trows, c_s, W->W_v, Hd, (char*)w.v + to, W->W_g, Hd, (char*)w.g + to, 0, 0, "single_attn_in_vg", st)) != NT_OK) return r;
+      const TokSeg seg[4] = {{xh, trows, W->W_q, Hd, (char*)w.q + to}, {xh, trows, W->W_k, Hd, (char*)w.k + to},
+                             {xh, trows, W->W_v, Hd, (char*)w.v + to}, {xh, trows, W->W_g, Hd, (char*)w.g + to}};
+      if ((r = fast_token_gemm(seg, 4, c_s, 0, 0, "single_attn_in", st)) != NT_OK) return r;
       if ((r = fast_single_bias(z, W->ln_z_gamma, W->ln_z_beta, W->W_b, eps, c_z, H, sqrtf((float)d), m, w.bias, st)) != NT_OK) return r;
       if ((r = fast_attn_core_fr(w.q, w.k, w.v, w.bias, w.o, H, d, FR_MODE_TOKEN, m, L->status_d, st)) != NT_OK) return r;
       if ((r = fast_gate_mul((char*)w.g + to, (char*)w.o + to, trows * Hd, st)) != NT_OK) return r;
-      if ((r = fast_token_gemm((char*)w.o + to, trows, Hd, W->W_o, c_s, xr, nullptr, 0, nullptr, 0, 1, "single_attn_out", st)) != NT_OK) return r;
+      const TokSeg so = {(char*)w.o + to, trows, W->W_o, c_s, xr};
+      if ((r = fast_token_gemm(&so, 1, Hd, 0, 1, "single_attn_out", st)) != NT_OK) return r;
       continue;
     }
     ProjArgs pa{};
@@ -668,8 +672,10 @@ nt_status nt_token_update(nt_dtype dt, int32_t c_s, int32_t c_z, int64_t T1, con
   pa.add(W_r, nullptr, c_s, ACT_NONE, x, O_ACCUM);
   cudaStream_t st = (cudaStream_t)stream;
   if (dt == NT_F32) return launch_proj<float>(pa, dummy, st, "token_update");
-  if (!g_force_generic && fast_token_gemm_supported(c_z, c_s, 0))
-    return fast_token_gemm(mvals, T1, c_z, W_r, c_s, x, nullptr, 0, nullptr, 0, 1, "token_update", st);
+  if (!g_force_generic && fast_token_gemm_supported(c_z, c_s, 0)) {
+    const TokSeg seg = {mvals, T1, W_r, c_s, x};
+    return fast_token_gemm(&seg, 1, c_z, 0, 1, "token_update", st);
+  }
   return launch_proj<__nv_bfloat16>(pa, dummy, st, "token_update");
 }
 

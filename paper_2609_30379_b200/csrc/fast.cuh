@@ -39,15 +39,16 @@ bool fast_segment_reduce_supported(int C);
 nt_status fast_segment_reduce(const void* v, void* out, const int64_t* splits, long long G, int C, int mean,
                               cudaStream_t st);
 
-// token-side projections: out[r][n] (+)= sum_k A[r][k] W[n][k] for up to two (W, out) pairs sharing A
+// token-side projections: out[r][n] (+)= sum_k A[r][k] W[n][k] for up to four segments in one launch
+constexpr int TOK_SEGS = 4;
+struct TokSeg { const void* A; long long rows; const void* W; int N; void* out; };
 bool fast_token_gemm_supported(int K, int N0, int N1);
-nt_status fast_token_gemm(const void* A, long long rows, int K, const void* W0, int N0, void* out0, const void* W1,
-                          int N1, void* out1, int out_f32, int accumulate, const char* name, cudaStream_t st);
+nt_status fast_token_gemm(const TokSeg* seg, int n, int K, int out_f32, int accumulate, const char* name, cudaStream_t st);
 
-// the same on tcgen05 (persistent 128 x 256 tiles), for token axes long enough to fill the GPU with tiles
-bool fast_token_gemm_tc_supported(long long rows, int K, int N0, int N1);
-nt_status fast_token_gemm_tc(const void* A, long long rows, int K, const void* W0, int N0, void* out0, const void* W1, int N1,
-                             void* out1, int out_f32, int accumulate, int* status, const char* name, cudaStream_t st);
+// the same on tcgen05 (persistent 128 x 256 tiles), for token axes long enough to fill the GPU with tiles; the segments
+// share A
+bool fast_token_gemm_tc_supported(const TokSeg* seg, int n, int K);
+nt_status fast_token_gemm_tc(const TokSeg* seg, int n, int K, int out_f32, int accumulate, int* status, const char* name, cudaStream_t st);
 
 // pair-biased single attention: LayerNorm of the token rows (bf16 out), o <- sigmoid(g) * o, and the bias planes
 // bias[s][h][i][j] = scale * (LN(z_ij) W_b^T)[h] in the head-major padded layout of the attention core

@@ -91,17 +91,17 @@ namespace ntp {
 
 // ------------------------------------------------------------------------------------------
 // Token-side projection (a few thousand rows, so a fraction of a percent of a block's work):
-//   out[r][n] (+)= sum_k A[r][k] W[n][k]   for up to two weight / output pairs sharing A.
+//   out[r][n] (+)= sum_k A[r][k] W[n][k]   for up to four segments (rows, weight, output), one after the other in grid.y.
 // 32 x 32 output tiles so that even T1 ~ 1.7k rows give several hundred CTAs; the A and W tiles are
 // staged whole in shared memory (K <= 1024).
 // ------------------------------------------------------------------------------------------
 struct TokGemmArgs {
-  const __nv_bfloat16* A;
-  long long rows;
+  const __nv_bfloat16* A[TOK_SEGS];
+  long long rows[TOK_SEGS];
   int K;
-  const __nv_bfloat16* W[2];
-  int N[2];
-  void* out[2];
+  const __nv_bfloat16* W[TOK_SEGS];
+  int N[TOK_SEGS];
+  void* out[TOK_SEGS];
   int out_f32;       // outputs are float (store) instead of bf16
   int accumulate;    // bf16 outputs: out += result
 };
@@ -114,14 +114,16 @@ __global__ void __launch_bounds__(256) token_gemm_kernel(TokGemmArgs a) {
   __nv_bfloat16* Ws = As + 32 * ldk;
   const long long r0 = (long long)blockIdx.x * 32;
   int n0 = blockIdx.y * 32, which = 0;
-  if (n0 >= a.N[0]) { n0 -= a.N[0]; which = 1; }
-  const __nv_bfloat16* W = a.W[which];
+  while (n0 >= a.N[which]) n0 -= a.N[which++];
+  const __nv_bfloat16 *A = a.A[which], *W = a.W[which];
+  const long long rows = a.rows[which];
+  if (r0 >= rows) return;
   const int N = a.N[which];
   const int t = threadIdx.x, kv = K / 8;
   for (int idx = t; idx < 32 * kv; idx += 256) {
     const int r = idx / kv, c = idx - r * kv;
     uint4 va = make_uint4(0, 0, 0, 0), vw = make_uint4(0, 0, 0, 0);
-    if (r0 + r < a.rows) va = *reinterpret_cast<const uint4*>(a.A + (r0 + r) * K + c * 8);
+    if (r0 + r < rows) va = *reinterpret_cast<const uint4*>(A + (r0 + r) * K + c * 8);
     if (n0 + r < N) vw = *reinterpret_cast<const uint4*>(W + (long long)(n0 + r) * K + c * 8);
     *reinterpret_cast<uint4*>(As + r * ldk + c * 8) = va;
     *reinterpret_cast<uint4*>(Ws + r * ldk + c * 8) = vw;
@@ -157,7 +159,7 @@ __global__ void __launch_bounds__(256) token_gemm_kernel(TokGemmArgs a) {
     for (int j = 0; j < 2; ++j) {
       const long long r = r0 + ty + 16 * i;
       const int n = n0 + tx + 16 * j;
-      if (r >= a.rows || n >= N) continue;
+      if (r >= rows || n >= N) continue;
       if (a.out_f32) {
         reinterpret_cast<float*>(a.out[which])[r * N + n] = acc[i][j];
       } else {
@@ -188,16 +190,18 @@ __global__ void __launch_bounds__(256) token_gemm_mma_kernel(TokGemmArgs a) {
   __nv_bfloat16* Ws = As + 64 * ldk;
   const long long r0 = (long long)blockIdx.x * 64;
   int n0 = blockIdx.y * 64, which = 0;
-  if (n0 >= a.N[0]) { n0 -= a.N[0]; which = 1; }
-  const __nv_bfloat16* W = a.W[which];
+  while (n0 >= a.N[which]) n0 -= a.N[which++];
+  const __nv_bfloat16 *A = a.A[which], *W = a.W[which];
+  const long long rows = a.rows[which];
+  if (r0 >= rows) return;
   const int N = a.N[which];
   const int t = threadIdx.x, kv = K / 8;
   // both panels with asynchronous 16-byte copies: every load of the CTA is in flight at once
   for (int idx = t; idx < 64 * kv; idx += 256) {
     const int r = idx / kv, c = idx - r * kv;
-    const bool ok = r0 + r < a.rows;
+    const bool ok = r0 + r < rows;
     const unsigned da = (unsigned)__cvta_generic_to_shared(As + r * ldk + c * 8), dw = (unsigned)__cvta_generic_to_shared(Ws + r * ldk + c * 8);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(da), "l"(a.A + (ok ? r0 + r : 0) * K + c * 8), "r"(ok ? 16 : 0));
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(da), "l"(A + (ok ? r0 + r : 0) * K + c * 8), "r"(ok ? 16 : 0));
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dw), "l"(W + (long long)(n0 + r) * K + c * 8));
   }
   asm volatile("cp.async.wait_all;\n" ::: "memory");
@@ -224,7 +228,7 @@ __global__ void __launch_bounds__(256) token_gemm_mma_kernel(TokGemmArgs a) {
     for (int hh = 0; hh < 2; ++hh) {
       const long long r = r0 + wr + g + hh * 8;
       const int n = n0 + wc + nt * 8 + 2 * tq;
-      if (r >= a.rows) continue;
+      if (r >= rows) continue;
       const float x0 = acc[nt][hh * 2], x1 = acc[nt][hh * 2 + 1];
       if (a.out_f32) {
         *reinterpret_cast<float2*>(reinterpret_cast<float*>(a.out[which]) + r * N + n) = make_float2(x0, x1);
@@ -241,24 +245,44 @@ bool fast_token_gemm_supported(int K, int N0, int N1) {
   return K % 8 == 0 && K >= 8 && K <= 1024 && N0 % 32 == 0 && N1 % 32 == 0;
 }
 
-nt_status fast_token_gemm(const void* A, long long rows, int K, const void* W0, int N0, void* out0, const void* W1,
-                          int N1, void* out1, int out_f32, int accumulate, const char* name, cudaStream_t st) {
-  if (rows <= 0) return NT_OK;
-  if (fast_token_gemm_tc_supported(rows, K, N0, W1 ? N1 : 0))     // a token axis long enough for persistent tcgen05 tiles
-    return fast_token_gemm_tc(A, rows, K, W0, N0, out0, W1, N1, out1, out_f32, accumulate, nullptr, name, st);
+nt_status fast_token_gemm(const TokSeg* seg, int n, int K, int out_f32, int accumulate, const char* name, cudaStream_t st) {
   TokGemmArgs a{};
-  a.A = (const __nv_bfloat16*)A;
-  a.rows = rows;
+  long long rows = 0;
+  int cols = 0, m = 0;
+  bool by64 = K % 16 == 0, shared = true;
+  TokSeg used[TOK_SEGS];
+  for (int i = 0; i < n; ++i) {
+    if (!seg[i].W || seg[i].N == 0 || seg[i].rows <= 0) continue;
+    if (m == TOK_SEGS) return NT_ERR_UNSUPPORTED;
+    shared = shared && (m == 0 || (seg[i].A == used[0].A && seg[i].rows == used[0].rows));
+    by64 = by64 && seg[i].N % 64 == 0;
+    rows = rows > seg[i].rows ? rows : seg[i].rows;
+    cols += seg[i].N;
+    a.A[m] = (const __nv_bfloat16*)seg[i].A;
+    a.rows[m] = seg[i].rows;
+    a.W[m] = (const __nv_bfloat16*)seg[i].W;
+    a.N[m] = seg[i].N;
+    a.out[m] = seg[i].out;
+    used[m++] = seg[i];
+  }
+  if (m == 0) return NT_OK;
+  if (shared && fast_token_gemm_tc_supported(used, m, K))         // a token axis long enough for persistent tcgen05 tiles
+    return fast_token_gemm_tc(used, m, K, out_f32, accumulate, nullptr, name, st);
+  if (!shared) {                                                  // any segment that is long enough for them goes by itself
+    bool lone = false;
+    for (int i = 0; i < m; ++i) lone = lone || fast_token_gemm_tc_supported(used + i, 1, K);
+    if (lone) {
+      for (int i = 0; i < m; ++i) {
+        nt_status r = fast_token_gemm(used + i, 1, K, out_f32, accumulate, name, st);
+        if (r != NT_OK) return r;
+      }
+      return NT_OK;
+    }
+  }
   a.K = K;
-  a.W[0] = (const __nv_bfloat16*)W0;
-  a.W[1] = (const __nv_bfloat16*)W1;
-  a.N[0] = N0;
-  a.N[1] = N1;
-  a.out[0] = out0;
-  a.out[1] = out1;
   a.out_f32 = out_f32;
   a.accumulate = accumulate;
-  if (K % 16 == 0 && N0 % 64 == 0 && N1 % 64 == 0) {
+  if (by64) {
     const size_t smem64 = (size_t)2 * 64 * (K + 8) * 2;
     static bool attr64_dev[64] = {};
     int attr_dev = 0;
@@ -272,7 +296,7 @@ nt_status fast_token_gemm(const void* A, long long rows, int K, const void* W0, 
     if (smem64 <= 200 * 1024) {
       const long long bx64 = (rows + 63) / 64;
       if (bx64 > 0x7FFFFFFFll) return NT_ERR_UNSUPPORTED;
-      dim3 grid64((unsigned)bx64, (unsigned)((N0 + N1) / 64));
+      dim3 grid64((unsigned)bx64, (unsigned)(cols / 64));
       {
         LaunchScope ls(name, st);
         launch_kernel(token_gemm_mma_kernel, grid64, 256, smem64, st, a);
@@ -292,7 +316,7 @@ nt_status fast_token_gemm(const void* A, long long rows, int K, const void* W0, 
   }
   const long long bx = (rows + 31) / 32;
   if (bx > 0x7FFFFFFFll) return NT_ERR_UNSUPPORTED;
-  dim3 grid((unsigned)bx, (unsigned)((N0 + N1) / 32));
+  dim3 grid((unsigned)bx, (unsigned)(cols / 32));
   {
     LaunchScope ls(name, st);
     launch_kernel(token_gemm_kernel, grid, 256, smem, st, a);

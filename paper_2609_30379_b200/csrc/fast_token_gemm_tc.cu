@@ -23,12 +23,13 @@ constexpr int TG_THREADS = 64 + 256;
 
 struct TokGemmTcParams {
   CUtensorMap amap;        // {K, rows}, box {64, 128}
-  CUtensorMap wmap[2];     // {K, N_i}, box {64, BN}
-  void* out[2];
-  int N[2];
+  CUtensorMap wmap[TOK_SEGS];   // {K, N_i}, box {64, BN}
+  void* out[TOK_SEGS];
+  int N[TOK_SEGS];
   long long rows;
   int K, BN, out_f32, accumulate;
-  int ntile[2];            // column tiles of each output
+  int ntile[TOK_SEGS];     // column tiles of each output
+  int ncol;                // of all of them
   int* status;
 };
 
@@ -60,7 +61,7 @@ __global__ void __launch_bounds__(TG_THREADS, 1) token_gemm_tc_kernel(const __gr
   pdl_begin();
   const unsigned tmem_base = tmem_base_s;
   AbortCtx ab{p.status, &abort_flag};
-  const int ncol = p.ntile[0] + p.ntile[1];
+  const int ncol = p.ncol;
   const long long nrow = (p.rows + 127) / 128;
   const long long njobs = nrow * ncol;
   const int nkc = (p.K + 63) / 64;
@@ -73,8 +74,8 @@ __global__ void __launch_bounds__(TG_THREADS, 1) token_gemm_tc_kernel(const __gr
     unsigned phase = 0;
     for (long long job = blockIdx.x; job < njobs; job += gridDim.x) {
       const long long rb = job / ncol;
-      const int ct = (int)(job - rb * ncol);
-      const int which = ct >= p.ntile[0] ? 1 : 0, cb = which ? ct - p.ntile[0] : ct;
+      int cb = (int)(job - rb * ncol), which = 0;
+      while (cb >= p.ntile[which]) cb -= p.ntile[which++];
       for (int kc = 0; kc < nkc; ++kc) {
         mbar_wait(&empty[stage], phase ^ 1, ab);
         unsigned char* As = smem + stage * STAGE_BYTES;
@@ -125,8 +126,8 @@ __global__ void __launch_bounds__(TG_THREADS, 1) token_gemm_tc_kernel(const __gr
     long long n = 0;
     for (long long job = blockIdx.x; job < njobs; job += gridDim.x, ++n) {
       const long long rb = job / ncol;
-      const int ct = (int)(job - rb * ncol);
-      const int which = ct >= p.ntile[0] ? 1 : 0, cb = which ? ct - p.ntile[0] : ct;
+      int cb = (int)(job - rb * ncol), which = 0;
+      while (cb >= p.ntile[which]) cb -= p.ntile[which++];
       const int buf = (int)(n & 1);
       mbar_wait(&tfull[buf], tph[buf], ab);
       tph[buf] ^= 1;
@@ -141,41 +142,39 @@ __global__ void __launch_bounds__(TG_THREADS, 1) token_gemm_tc_kernel(const __gr
         tmem_ld_wait();
         if (r < p.rows && NT_IN(cb * BN + cg * 64 + 63, Nout, NT_SITE_TOKEN_GEMM_OUT)) {
           const long long off = r * Nout + cb * BN + cg * 64;
+          // 32-byte stores: a thread's columns are whole sectors, which 16-byte stores each write in part
+          const bool wide = ((unsigned long long)p.out[which] & 31) == 0;
           if (p.out_f32) {
-            float4* o = reinterpret_cast<float4*>((float*)p.out[which] + off);
-#pragma unroll
-            for (int e = 0; e < 16; ++e) {
-              const unsigned* src = e < 8 ? r0 + e * 4 : r1 + (e - 8) * 4;
-              float4 v = make_float4(__uint_as_float(src[0]), __uint_as_float(src[1]), __uint_as_float(src[2]), __uint_as_float(src[3]));
-              if (p.accumulate) {
-                const float4 old = o[e];
-                v.x += old.x; v.y += old.y; v.z += old.z; v.w += old.w;
-              }
-              o[e] = v;
-            }
-          } else {
-            uint4* o = reinterpret_cast<uint4*>((__nv_bfloat16*)p.out[which] + off);
+            float* o = (float*)p.out[which] + off;
 #pragma unroll
             for (int e = 0; e < 8; ++e) {
               const unsigned* src = e < 4 ? r0 + e * 8 : r1 + (e - 4) * 8;
-              float f[8];
+              unsigned v[8];
 #pragma unroll
-              for (int q = 0; q < 8; ++q) f[q] = __uint_as_float(src[q]);
+              for (int q = 0; q < 8; ++q) v[q] = __float_as_uint(__uint_as_float(src[q]) + (p.accumulate ? o[e * 8 + q] : 0.f));
+              store_32b(o + e * 8, v, wide);
+            }
+          } else {
+            __nv_bfloat16* o = (__nv_bfloat16*)p.out[which] + off;
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              const unsigned* src = e < 2 ? r0 + e * 16 : r1 + (e - 2) * 16;
+              float f[16];
+#pragma unroll
+              for (int q = 0; q < 16; ++q) f[q] = __uint_as_float(src[q]);
               if (p.accumulate) {
-                const uint4 old = o[e];
-                const unsigned ow[4] = {old.x, old.y, old.z, old.w};
+                const uint4 x = *reinterpret_cast<const uint4*>(o + e * 16), y = *reinterpret_cast<const uint4*>(o + e * 16 + 8);
+                const unsigned ow[8] = {x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w};
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
+                for (int q = 0; q < 8; ++q) {
                   f[2 * q] += __uint_as_float(ow[q] << 16);
                   f[2 * q + 1] += __uint_as_float(ow[q] & 0xffff0000u);
                 }
               }
-              uint4 v;
-              v.x = pack2(__float_as_uint(f[0]), __float_as_uint(f[1]));
-              v.y = pack2(__float_as_uint(f[2]), __float_as_uint(f[3]));
-              v.z = pack2(__float_as_uint(f[4]), __float_as_uint(f[5]));
-              v.w = pack2(__float_as_uint(f[6]), __float_as_uint(f[7]));
-              o[e] = v;
+              unsigned v[8];
+#pragma unroll
+              for (int q = 0; q < 8; ++q) v[q] = pack2(__float_as_uint(f[2 * q]), __float_as_uint(f[2 * q + 1]));
+              store_32b(o + e * 16, v, wide);
             }
           }
         }
@@ -192,11 +191,13 @@ __global__ void __launch_bounds__(TG_THREADS, 1) token_gemm_tc_kernel(const __gr
   if (warp == 1) tmem_dealloc(tmem_base, 512);
 }
 
-bool fast_token_gemm_tc_supported(long long rows, int K, int N0, int N1) {
+bool fast_token_gemm_tc_supported(const TokSeg* seg, int n, int K) {
   // worth a persistent tensor-core launch only when there are enough tiles; shapes: K a multiple of 64 (full
   // swizzled slabs), outputs a multiple of 128 columns
-  if (K % 64 != 0 || K < 64 || N0 % 128 != 0 || N0 < 128 || (N1 % 128 != 0)) return false;
-  return rows >= 2048 && rows <= 0x7FFFFF00ll;
+  if (K % 64 != 0 || K < 64) return false;
+  for (int i = 0; i < n; ++i)
+    if (seg[i].N % 128 != 0 || seg[i].N < 128) return false;
+  return seg[0].rows >= 2048 && seg[0].rows <= 0x7FFFFF00ll;
 }
 
 template <int BN>
@@ -211,7 +212,7 @@ static nt_status launch_tg(TokGemmTcParams& p, const char* name, cudaStream_t st
       return cuda_fail("token gemm tc smem attribute");
     attr_set[dev] = true;
   }
-  const long long njobs = ((p.rows + 127) / 128) * (p.ntile[0] + p.ntile[1]);
+  const long long njobs = ((p.rows + 127) / 128) * p.ncol;
   const int sms = sm_count();
   {
     LaunchScope ls(name, st);
@@ -220,44 +221,45 @@ static nt_status launch_tg(TokGemmTcParams& p, const char* name, cudaStream_t st
   return cuda_ok(name);
 }
 
-nt_status fast_token_gemm_tc(const void* A, long long rows, int K, const void* W0, int N0, void* out0, const void* W1, int N1,
-                             void* out1, int out_f32, int accumulate, int* status, const char* name, cudaStream_t st) {
-  if (rows <= 0) return NT_OK;
-  if (!fast_token_gemm_tc_supported(rows, K, N0, W1 ? N1 : 0)) return NT_ERR_UNSUPPORTED;
+nt_status fast_token_gemm_tc(const TokSeg* seg, int n, int K, int out_f32, int accumulate, int* status, const char* name, cudaStream_t st) {
+  if (!fast_token_gemm_tc_supported(seg, n, K)) return NT_ERR_UNSUPPORTED;
+  const long long rows = seg[0].rows;
   TokGemmTcParams p;
   memset(&p, 0, sizeof(p));
   p.rows = rows;
   p.K = K;
-  p.out[0] = out0;
-  p.out[1] = out1;
-  p.N[0] = N0;
-  p.N[1] = W1 ? N1 : 0;
   p.out_f32 = out_f32;
   p.accumulate = accumulate;
   p.status = status;
+  int cols = 0;
+  bool by256 = true;
+  for (int i = 0; i < n; ++i) {
+    p.out[i] = seg[i].out;
+    p.N[i] = seg[i].N;
+    cols += seg[i].N;
+    by256 = by256 && seg[i].N % 256 == 0;
+  }
   // tile width by wave quantisation: the width whose tile count leaves the shorter tail on this many SMs
   int BN = 128;
-  if (N0 % 256 == 0 && p.N[1] % 256 == 0) {
+  if (by256) {
     const long long rb = (rows + 127) / 128, sms = sm_count();
-    const long long j256 = rb * ((N0 + p.N[1]) / 256), j128 = rb * ((N0 + p.N[1]) / 128);
+    const long long j256 = rb * (cols / 256), j128 = rb * (cols / 128);
     if (((j256 + sms - 1) / sms) * 256 <= ((j128 + sms - 1) / sms) * 128) BN = 256;
   }
   p.BN = BN;
-  p.ntile[0] = N0 / BN;
-  p.ntile[1] = p.N[1] / BN;
+  p.ncol = cols / BN;
   {
     const unsigned long long dims[2] = {(unsigned long long)K, (unsigned long long)rows};
     const unsigned long long strides[1] = {(unsigned long long)K * 2};
     const unsigned box[2] = {64, 128};
-    if (!make_tmap_bf16(&p.amap, A, 2, dims, strides, box)) return cuda_fail("token gemm tc A map");
+    if (!make_tmap_bf16(&p.amap, seg[0].A, 2, dims, strides, box)) return cuda_fail("token gemm tc A map");
   }
-  const void* Ws[2] = {W0, W1};
-  for (int i = 0; i < 2; ++i) {
-    if (p.N[i] == 0) continue;
+  for (int i = 0; i < n; ++i) {
+    p.ntile[i] = p.N[i] / BN;
     const unsigned long long dims[2] = {(unsigned long long)K, (unsigned long long)p.N[i]};
     const unsigned long long strides[1] = {(unsigned long long)K * 2};
     const unsigned box[2] = {64, (unsigned)BN};
-    if (!make_tmap_bf16(&p.wmap[i], Ws[i], 2, dims, strides, box)) return cuda_fail("token gemm tc W map");
+    if (!make_tmap_bf16(&p.wmap[i], seg[i].W, 2, dims, strides, box)) return cuda_fail("token gemm tc W map");
   }
   return BN == 256 ? launch_tg<256>(p, name, st) : launch_tg<128>(p, name, st);
 }

@@ -166,8 +166,8 @@ static nt_status rect_broadcast_impl(nt_dtype dt, int B, const int64_t* ln, cons
   BatchMeta dummy;
   fill_meta(dummy, nullptr, 0, 0, 0, 0, 0);
   if (fast && fast_token_gemm_supported(c_s, c_z, 0)) {
-    if ((r = fast_token_gemm(x, t1n, c_s, W_a, c_z, u, nullptr, 0, nullptr, 1, 0, "rect_tok_proj_u", st)) != NT_OK) return r;
-    if ((r = fast_token_gemm(y, t1m, c_s, W_b, c_z, v, nullptr, 0, nullptr, 1, 0, "rect_tok_proj_v", st)) != NT_OK) return r;
+    const TokSeg seg[2] = {{x, t1n, W_a, c_z, u}, {y, t1m, W_b, c_z, v}};      // rows and columns in one launch
+    if ((r = fast_token_gemm(seg, 2, c_s, 1, 0, "rect_tok_proj", st)) != NT_OK) return r;
   } else {
     ProjArgs pa{};
     pa.a_mode = A_ROWMAJOR; pa.row0 = 0; pa.K = c_s;

@@ -369,6 +369,18 @@ __device__ inline void convert_row_bf16_to_f16(unsigned char* tile, int nslab, i
   sq = (q4[0] + q4[1]) + (q4[2] + q4[3]);
 }
 
+// 32 bytes of one row to global memory.  `wide`: the buffer is aligned to 32 bytes (callers guarantee 16); one store then
+// fills a sector that two 16-byte stores would each write in part.
+__device__ inline void store_32b(void* to, const unsigned (&w)[8], bool wide) {
+  if (wide) {
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};\n" ::"l"(to), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]),
+                 "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7]) : "memory");
+  } else {
+    *reinterpret_cast<uint4*>(to) = make_uint4(w[0], w[1], w[2], w[3]);
+    *(reinterpret_cast<uint4*>(to) + 1) = make_uint4(w[4], w[5], w[6], w[7]);
+  }
+}
+
 // LayerNorm folded into the MMA for a tile that stays as it is.  One more K step adds s c0 - mean c1 to the raw product,
 // s = 1 / rstd, so that rstd times the accumulator is the normalised projection and a reader of the accumulator needs no
 // tables.  Both sides are split into fp16 parts: the row side is (-m_hi, -m_lo, -m_hi, s_hi, s_hi, s_lo, 4096 s_rest,
