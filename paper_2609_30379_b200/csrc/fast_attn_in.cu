@@ -184,7 +184,8 @@ __global__ void __launch_bounds__(AI_THREADS, 1) attn_in_kernel(const __grid_con
     unsigned tph[2] = {0, 0};
     long long unit = 0;
     bool store_pending = false;
-    for (long long t = blockIdx.x; t < ntiles; t += gridDim.x) {
+    int tn = 0;
+    for (long long t = blockIdx.x; t < ntiles; t += gridDim.x, ++tn) {
       for (int u = 0; u < nunits; ++u, ++unit) {
         const int buf = (int)(unit & 1);
         mbar_wait(&tfull[buf], tph[buf], ab);
@@ -245,7 +246,7 @@ __global__ void __launch_bounds__(AI_THREADS, 1) attn_in_kernel(const __grid_con
             }
             store_pending = true;
           }
-        } else if (half == 0) {
+        } else if (half == (tn & 1)) {                       // the two halves take the bias in turn
           // bias: H values per position, written head-major / channel-major
           unsigned r[16];
           tmem_ld16(taddr, r);
