@@ -40,6 +40,7 @@ struct AttnInParams {
   int bias_tr_above;             // samples longer than this get their bias planes transposed ([h][j][i]: column-wise attention)
 };
 
+template <bool SPLIT>   // a parameter of the code: with the units of a tile known, the loops over them keep their constants
 __global__ void __launch_bounds__(AI_THREADS, 1) attn_in_kernel(const __grid_constant__ AttnInParams p) {
   extern __shared__ unsigned char smem_raw[];
   __shared__ __align__(8) unsigned long long bars[11];
@@ -95,28 +96,29 @@ __global__ void __launch_bounds__(AI_THREADS, 1) attn_in_kernel(const __grid_con
   AbortCtx ab{p.status, &abort_flag};
   const long long ntiles = (p.rows + 127) / 128;
   const int nunits = p.bias ? 3 : 2;
+  // split: a CTA takes q | k of a tile or v and the bias, and fetches only those weights
+  const int u0 = SPLIT ? (int)(blockIdx.x & 1) : 0, u1 = SPLIT && u0 == 0 ? 1 : nunits;
+  const long long t0 = SPLIT ? blockIdx.x >> 1 : blockIdx.x, tstep = SPLIT ? gridDim.x >> 1 : gridDim.x;
   // unit u: weight row offset and accumulator width
   const int u_row[3] = {0, 2 * Hd, 3 * Hd};
   const int u_n[3] = {2 * Hd, Hd, 16};
 
   if (warp == 0 && lane == 0) {
     // ------------------------------------------------------------------ producer
-    mbar_expect_tx(wfull, nslab * w_slab + 2 * wx_region);
+    const int row0 = u0 == 0 ? 0 : 2 * Hd, row1 = u1 == 1 ? 2 * Hd : wrows;      // weight rows of this CTA's units
+    mbar_expect_tx(wfull, (row1 - row0) * (nslab * 128 + 2 * 16));
     for (int reg = 0; reg < 2; ++reg)
-      for (int r16 = 0; r16 < wrows; r16 += 16)
+      for (int r16 = row0; r16 < row1; r16 += 16)
         tma_load_2d(sWx + reg * wx_region + r16 * 16, &p.xmap, wfull, 0, reg * p.aug_rows + r16);
-    for (int sl = 0; sl < nslab; ++sl) {
-      for (int rb = 0; rb < 3 * Hd / 128; ++rb)
-        tma_load_2d(sW + sl * w_slab + rb * 128 * 128, &p.wmap, wfull, sl * 64, rb * 128);
-      if ((3 * Hd) % 128) {   // H d = 64: rows 128..191 via a second 128-row box would overrun; use 16-row boxes
-        for (int r16 = (3 * Hd / 128) * 128; r16 < 3 * Hd; r16 += 16)
-          tma_load_2d(sW + sl * w_slab + r16 * 128, &p.wbmap, wfull, sl * 64, r16);
+    for (int sl = 0; sl < nslab; ++sl)
+      for (int r = row0; r < row1;) {
+        const bool big = r + 128 <= 3 * Hd && r + 128 <= row1;   // 128-row boxes where they fit, 16-row boxes for the rest
+        tma_load_2d(sW + sl * w_slab + r * 128, big ? &p.wmap : &p.wbmap, wfull, sl * 64, r);
+        r += big ? 128 : 16;
       }
-      tma_load_2d(sW + sl * w_slab + 3 * Hd * 128, &p.wbmap, wfull, sl * 64, 3 * Hd);
-    }
     int stage = 0;
     unsigned phase = 0;
-    for (long long t = blockIdx.x; t < ntiles; t += gridDim.x) {
+    for (long long t = t0; t < ntiles; t += tstep) {
       mbar_wait(&aempty[stage], phase ^ 1, ab);
       mbar_expect_tx(&afull[stage], a_stage);
       for (int sl = 0; sl < nslab; ++sl)
@@ -132,12 +134,12 @@ __global__ void __launch_bounds__(AI_THREADS, 1) attn_in_kernel(const __grid_con
     const unsigned long long w_desc = desc_kmajor_sw128(smem_u32(sW));
     const unsigned w16 = (unsigned)w_slab >> 4, a16 = (unsigned)a_slab >> 4;
     const unsigned long long wx_desc = desc_kmajor_nosw(smem_u32(sWx), wx_region, 128);
-    for (long long t = blockIdx.x; t < ntiles; t += gridDim.x) {
+    for (long long t = t0; t < ntiles; t += tstep) {
       mbar_wait(&aconv[stage], phase, ab);
       tc_fence_after();
       const unsigned long long a_desc = desc_kmajor_sw128(smem_u32(sA + stage * a_stage));
       const unsigned long long ax_desc = desc_kmajor_nosw(smem_u32(sAx + stage * 2 * zx_region), zx_region, 128);
-      for (int u = 0; u < nunits; ++u, ++unit) {
+      for (int u = u0; u < u1; ++u, ++unit) {
         const unsigned buf = unit & 1;
         if (buf == 0) { mbar_wait(&tempty[0], tph0 ^ 1, ab); tph0 ^= 1; }
         else { mbar_wait(&tempty[1], tph1 ^ 1, ab); tph1 ^= 1; }
@@ -165,10 +167,10 @@ __global__ void __launch_bounds__(AI_THREADS, 1) attn_in_kernel(const __grid_con
     const int row = (warp - 2) * 16 + (lane >> 1), hf = lane & 1;
     int stage = 0;
     unsigned phase = 0;
-    for (long long t = blockIdx.x; t < ntiles; t += gridDim.x) {
+    for (long long t = t0; t < ntiles; t += tstep) {
       mbar_wait(&afull[stage], phase, ab);
       convert_row_ln_fp16(sA + stage * a_stage, nslab, a_slab, sAx + stage * 2 * zx_region + row * 16, row, hf, c, p.eps,
-                          p.zstats && t * 128 + row < p.rows ? p.zstats + t * 128 + row : nullptr);
+                          p.zstats && u0 == 0 && t * 128 + row < p.rows ? p.zstats + t * 128 + row : nullptr);
       fence_proxy_async_smem();
       __syncwarp();
       if (lane == 0) mbar_arrive(&aconv[stage]);
@@ -185,8 +187,8 @@ __global__ void __launch_bounds__(AI_THREADS, 1) attn_in_kernel(const __grid_con
     long long unit = 0;
     bool store_pending = false;
     int tn = 0;
-    for (long long t = blockIdx.x; t < ntiles; t += gridDim.x, ++tn) {
-      for (int u = 0; u < nunits; ++u, ++unit) {
+    for (long long t = t0; t < ntiles; t += tstep, ++tn) {
+      for (int u = u0; u < u1; ++u, ++unit) {
         const int buf = (int)(unit & 1);
         mbar_wait(&tfull[buf], tph[buf], ab);
         tph[buf] ^= 1;
@@ -303,7 +305,8 @@ nt_status fast_attn_in(const void* z, const AttnPrep& ap, float eps, int c, int 
   cudaGetDevice(&attr_dev);
   bool& attr_set = attr_set_dev[attr_dev & 63];
   if (!attr_set) {
-    if (cudaFuncSetAttribute(attn_in_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024) != cudaSuccess)
+    if (cudaFuncSetAttribute(attn_in_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024) != cudaSuccess ||
+        cudaFuncSetAttribute(attn_in_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024) != cudaSuccess)
       return cuda_fail("attn_in smem attribute");
     attr_set = true;
   }
@@ -355,10 +358,14 @@ nt_status fast_attn_in(const void* z, const AttnPrep& ap, float eps, int c, int 
           return cuda_fail("attn_in out map");
     }
     const long long ntiles = (p.rows + 127) / 128;
-    const unsigned grid = (unsigned)(ntiles < sm_count() ? ntiles : sm_count());
+    // few tiles: an SM for q | k and one for v and the bias of each halve the weights to wait for and the units to go through
+    // (as in the triangle's input projection)
+    const bool split = 2 * ntiles <= sm_count();
+    const long long nwork = split ? 2 * ntiles : ntiles;
+    const unsigned grid = (unsigned)(nwork < sm_count() ? nwork : sm_count());
     {
       LaunchScope ls("attn_in", st);
-      launch_kernel(attn_in_kernel, grid, AI_THREADS, smem, st, p);
+      launch_kernel(split ? attn_in_kernel<true> : attn_in_kernel<false>, grid, AI_THREADS, smem, st, p);
     }
     if (cudaPeekAtLastError() != cudaSuccess) return cuda_fail("attn_in launch");
   }

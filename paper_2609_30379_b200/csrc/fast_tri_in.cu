@@ -40,6 +40,7 @@ struct TriInParams {
   long long cm_off[TI_MAXB];
   int N[TI_MAXB];
   int B, c_z, c_h, aug_rows;
+  int split;                               // CTAs 2 k and 2 k + 1 share tile k, one unit each
   float eps;
   int* status;
   float2* zstats;                          // nullable: (mean, rstd) of every row of z, by packed position, for the output stage
@@ -121,19 +122,22 @@ __global__ void __launch_bounds__(TI_THREADS, 1) tri_in_kernel(const __grid_cons
   const long long nchunks = p.chunk_off[p.B];
   const long long ntiles = (nchunks + 3) / 4;
   const int nunits = c_h == 128 ? 2 : 1;           // accumulator units per tile: (gate rows | value rows) of 128 each
+  // split: a CTA takes one unit of a tile and fetches only that unit's weights
+  const int u0 = p.split ? (int)(blockIdx.x & 1) : 0, u1 = p.split ? u0 + 1 : nunits;
+  const long long t0 = p.split ? blockIdx.x >> 1 : blockIdx.x, tstep = p.split ? gridDim.x >> 1 : gridDim.x;
 
   if (warp == 0) {
     // ------------------------------------------------------------------ producer (lane q decodes and loads chunk q)
     if (lane == 0) {
-      mbar_expect_tx(wfull, w_bytes + wx_region);
+      mbar_expect_tx(wfull, (u1 - u0) * 256 * (nslab * 128 + 16));
       for (int sl = 0; sl < nslab; ++sl)
-        for (int rb = 0; rb < wrows / 128; ++rb)
+        for (int rb = 2 * u0; rb < 2 * u1; ++rb)
           tma_load_2d(sW + sl * w_slab_bytes + rb * 128 * 128, &p.wmap, wfull, sl * 64, rb * 128);
-      for (int rb = 0; rb < wrows / 256; ++rb) tma_load_2d(sWx + rb * 256 * 16, &p.xmap, wfull, 0, rb * 256);
+      for (int rb = u0; rb < u1; ++rb) tma_load_2d(sWx + rb * 256 * 16, &p.xmap, wfull, 0, rb * 256);
     }
     int stage = 0, tn = 0;
     unsigned phase = 0;
-    for (long long t = blockIdx.x; t < ntiles; t += gridDim.x, ++tn) {
+    for (long long t = t0; t < ntiles; t += tstep, ++tn) {
       int s = 0, i = 0, jc = 0;
       bool valid = false;
       if (lane < 4) {
@@ -165,13 +169,13 @@ __global__ void __launch_bounds__(TI_THREADS, 1) tri_in_kernel(const __grid_cons
     const unsigned long long w_desc = desc_kmajor_sw128(smem_u32(sW));
     const unsigned wx_addr = smem_u32(sWx), zero_addr = smem_u32(sZero);   // columns 8-15 of both operands: the zero region
     const unsigned w_slab16 = (unsigned)w_slab_bytes >> 4, z_slab16 = (unsigned)z_slab_bytes >> 4;
-    for (long long t = blockIdx.x; t < ntiles; t += gridDim.x) {
+    for (long long t = t0; t < ntiles; t += tstep) {
       mbar_wait(&aconv[stage], phase, ab);
       tc_fence_after();
       const unsigned long long z_desc = desc_kmajor_sw128(smem_u32(sZ + stage * z_stage_bytes));
       const unsigned zx_addr = smem_u32(sZx + stage * zx_region);
       const unsigned long long zx_desc = desc_kmajor_nosw(zx_addr, zero_addr - zx_addr, 128);
-      for (int u = 0; u < nunits; ++u, ++unit) {
+      for (int u = u0; u < u1; ++u, ++unit) {
         const unsigned buf = unit & 1;
         if (buf == 0) { mbar_wait(&tempty[0], tph0 ^ 1, ab); tph0 ^= 1; }
         else { mbar_wait(&tempty[1], tph1 ^ 1, ab); tph1 ^= 1; }
@@ -201,7 +205,7 @@ __global__ void __launch_bounds__(TI_THREADS, 1) tri_in_kernel(const __grid_cons
     const int row = (warp - 2) * 16 + (lane >> 1), hf = lane & 1;
     int stage = 0, tn = 0;
     unsigned phase = 0;
-    for (long long t = blockIdx.x; t < ntiles; t += gridDim.x, ++tn) {
+    for (long long t = t0; t < ntiles; t += tstep, ++tn) {
       mbar_wait(&afull[stage], phase, ab);
       unsigned char* tile = sZ + stage * z_stage_bytes;
       uint4 raw[2][4];
@@ -246,7 +250,7 @@ __global__ void __launch_bounds__(TI_THREADS, 1) tri_in_kernel(const __grid_cons
                 make_uint4(w[0], w[1], w[2], w[3]);
           }
         }
-      if (p.zstats && hf == 0) {             // the output stage normalises the same rows: hand the statistics over
+      if (p.zstats && hf == 0 && u0 == 0) {             // the output stage normalises the same rows: hand the statistics over
         const int4 info = tinfo[tn & 7][row / TI_CH];
         const int j = info.z + (row % TI_CH);
         if (info.w && j < p.N[info.x])
@@ -275,8 +279,8 @@ __global__ void __launch_bounds__(TI_THREADS, 1) tri_in_kernel(const __grid_cons
     unsigned tph[2] = {0, 0};
     long long unit = 0;
     int tn = 0;
-    for (long long t = blockIdx.x; t < ntiles; t += gridDim.x, ++tn) {
-      for (int u = 0; u < nunits; ++u, ++unit) {
+    for (long long t = t0; t < ntiles; t += tstep, ++tn) {
+      for (int u = u0; u < u1; ++u, ++unit) {
         const int buf = (int)(unit & 1);
         mbar_wait(&tfull[buf], tph[buf], ab);
         tph[buf] ^= 1;
@@ -412,7 +416,11 @@ nt_status fast_tri_in(const void* z, const TriPrep& tp, float eps, int c_z, int 
     }
     const long long ntiles = (p.chunk_off[p.B] + 3) / 4;
     if (ntiles == 0) continue;
-    const unsigned grid = (unsigned)(ntiles < sm_count() ? ntiles : sm_count());
+    // Few tiles leave most SMs idle and the launch is one tile's latency: 128 KB of weights, then two units one after the other.
+    // With an SM for either unit both parts halve (the line is where a CTA would have to come back for a second tile).
+    p.split = c_h == 128 && 2 * ntiles <= sm_count();
+    const long long nwork = p.split ? 2 * ntiles : ntiles;
+    const unsigned grid = (unsigned)(nwork < sm_count() ? nwork : sm_count());
     {
       LaunchScope ls("tri_in", st);
       launch_kernel(tri_in_kernel, grid, TI_THREADS, smem, st, p);
