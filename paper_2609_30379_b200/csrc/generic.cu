@@ -347,10 +347,20 @@ nt_status launch_proj(const ProjArgs& args, const BatchMeta& m, cudaStream_t st,
   if (a.rows <= 0 || tiles <= 0) return NT_OK;
   long long bx = (a.rows + PBM - 1) / PBM;
   if (bx > 0x7FFFFFFFll || tiles > 65535) return NT_ERR_UNSUPPORTED;
-  // one column tile per block while that leaves SMs without a block, all of them once the rows alone fill the GPU
-  const long long want = 2 * sm_count();
-  const long long split = bx >= want ? 1 : bx * tiles <= want ? tiles : (want + bx - 1) / bx;
-  const int tpb = (int)((tiles + split - 1) / split);
+  // One column tile per block while that leaves SMs without a block.  Once the rows fill the GPU, all of them where the rows
+  // come in many rounds, and fewer where a part of a round would be left over: the number per block for which rounds x
+  // (rows once + tiles) is smallest, a block's rows and their LayerNorm costing about half a tile (three blocks fit an SM).  Lengths
+  // 24-110, 32 k rows: 365.6 -> 351.6 us per float block.
+  const long long want = 2 * sm_count(), fit = 3 * sm_count();
+  const long long split = bx * tiles <= want ? tiles : (want + bx - 1) / bx;
+  int tpb = (int)((tiles + split - 1) / split);
+  if (bx >= want) {
+    double best = 1e300;
+    for (int k = 1; k <= tiles; ++k) {
+      const double cost = (double)((bx * ((tiles + k - 1) / k) + fit - 1) / fit) * (0.5 + k);
+      if (cost <= best) { best = cost; tpb = k; }
+    }
+  }
   const dim3 grid((unsigned)bx, (unsigned)((tiles + tpb - 1) / tpb));
   const bool vec = (a.K & 3) == 0 && (low & 15) == 0;      // (not every entry point asks for aligned weights)
   nt_status r;
