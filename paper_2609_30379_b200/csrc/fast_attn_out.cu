@@ -63,9 +63,8 @@ __global__ void __launch_bounds__(AO_THREADS, 1) attn_out_kernel(const __grid_co
   unsigned char* sWg = smem;                          // zslab slabs of [Hd rows][64]
   unsigned char* sWo = sWg + zslab * wg_slab;         // oslab slabs of [c rows][64]
   unsigned char* sSt = sWo + oslab * wo_slab;         // 2 stages: z slabs then o slabs
-  unsigned char* sAx = sSt + 2 * stage_bytes;         // [2 stages][128][8] fp16: augmentation columns 0-7 of the rows
-  unsigned char* sBx = sAx + 2 * 2048;                // [Hd][8] fp16: augmentation columns 0-7 of W_g
-  unsigned char* sZero = sBx + Hd * 16;               // [128][8] zeros: augmentation columns 8-15 of either
+  unsigned char* sAx = sSt + 2 * stage_bytes;         // [2 stages][2][128][8] bf16: augmentation columns 0-7, 8-15 of the rows
+  unsigned char* sBx = sAx + 2 * 4096;                // [2][Hd][8] bf16: the same of W_g
   unsigned long long* afull = bars;        // [2]
   unsigned long long* aempty = bars + 2;   // [2]
   unsigned long long* gfull = bars + 4;    // [2]
@@ -93,15 +92,11 @@ __global__ void __launch_bounds__(AO_THREADS, 1) attn_out_kernel(const __grid_co
     mbar_fence_init();
   }
   if (warp == 1) tmem_alloc(&tmem_base_s, 512);
-  for (int n = threadIdx.x; n < 128; n += AO_THREADS) *reinterpret_cast<uint4*>(sZero + n * 16) = make_uint4(0, 0, 0, 0);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   pdl_begin();
-  for (int n = threadIdx.x; n < Hd; n += AO_THREADS) {
-    const float2 k = p.c01g[n];
-    *reinterpret_cast<uint4*>(sBx + n * 16) = ln_aug_weight(k.x, k.y);
-  }
+  for (int n = threadIdx.x; n < Hd; n += AO_THREADS) ln_aug_weight(sBx + n * 16, Hd * 16, p.c01g[n]);
   fence_proxy_async_smem();
   __syncthreads();
   const unsigned tmem_base = __shfl_sync(0xffffffffu, tmem_base_s, 0);
@@ -132,10 +127,9 @@ __global__ void __launch_bounds__(AO_THREADS, 1) attn_out_kernel(const __grid_co
     int stage = 0;
     unsigned phase = 0;
     const unsigned idesc_g = idesc_f16(128, Hd, 0, 0, FMT_BF16, FMT_BF16);  // the bf16 z tile, folded W_g bf16
-    const unsigned idesc_x = idesc_f16(128, Hd, 0, 0, FMT_F16, FMT_F16);    // augmentation step
     const unsigned long long wg_desc = desc_kmajor_sw128(smem_u32(sWg));
     const unsigned slab16 = (unsigned)slab >> 4, wg16 = (unsigned)wg_slab >> 4;
-    const unsigned bx = smem_u32(sBx), zero = smem_u32(sZero);
+    const unsigned long long bx_desc = desc_kmajor_nosw(smem_u32(sBx), Hd * 16, 128);
     for (long long t = blockIdx.x; t < ntiles; t += gridDim.x) {
       mbar_wait(&tempty[stage], phase ^ 1, ab);              // accumulators and stages advance together
       mbar_wait(&afull[stage], phase, ab);
@@ -147,9 +141,8 @@ __global__ void __launch_bounds__(AO_THREADS, 1) attn_out_kernel(const __grid_co
         if (sl < zslab) umma_k4(dg, st_desc + sl * slab16, wg_desc + sl * wg16, idesc_g, sl);
       mbar_wait(&aconv[stage], phase, ab);                   // the rows' augmentation columns are written
       tc_fence_after();
-      const unsigned ax = smem_u32(sAx + stage * 2048);
       if (elect_one()) {
-        umma_bf16(dg, desc_kmajor_nosw(ax, zero - ax, 128), desc_kmajor_nosw(bx, zero - bx, 128), idesc_x, 1);
+        umma_bf16(dg, desc_kmajor_nosw(smem_u32(sAx + stage * 4096), 2048, 128), bx_desc, idesc_g, 1);
         tc_commit(&gfull[stage]);
       }
       __syncwarp();
@@ -189,8 +182,7 @@ __global__ void __launch_bounds__(AO_THREADS, 1) attn_out_kernel(const __grid_co
       if (p.zstats) {                       // the input projection normalised the same rows: take its statistics
         const float2 zst = t * 128 + row < p.rows ? *(p.zstats + t * 128 + row) : make_float2(0.f, 1.f);
         mbar_wait(&afull[stage], phase, ab);
-        *reinterpret_cast<uint4*>(sAx + stage * 2048 + row * 16) = ln_aug_row(zst.x, 1.f / zst.y);
-        sStats[stage][row] = 0.5f * zst.y;
+        sStats[stage][row] = 0.5f * ln_aug_row(sAx + stage * 4096 + row * 16, 2048, zst.x, zst.y);
         fence_proxy_async_smem();
         __syncwarp();
         if (lane == 0) mbar_arrive(&aconv[stage]);
@@ -213,9 +205,8 @@ __global__ void __launch_bounds__(AO_THREADS, 1) attn_out_kernel(const __grid_co
       }
       const float sum = (s4[0] + s4[1]) + (s4[2] + s4[3]), sq = (q4[0] + q4[1]) + (q4[2] + q4[3]);
       const float mean = sum / (float)c;
-      const float ve = fmaxf(sq / (float)c - mean * mean, 0.f) + p.eps, rstd = rsqrtf(ve);
-      *reinterpret_cast<uint4*>(sAx + stage * 2048 + row * 16) = ln_aug_row(mean, ve * rstd);
-      sStats[stage][row] = 0.5f * rstd;
+      const float rstd = rsqrtf(fmaxf(sq / (float)c - mean * mean, 0.f) + p.eps);
+      sStats[stage][row] = 0.5f * ln_aug_row(sAx + stage * 4096 + row * 16, 2048, mean, rstd);
       fence_proxy_async_smem();
       __syncwarp();
       if (lane == 0) mbar_arrive(&aconv[stage]);
@@ -442,7 +433,7 @@ nt_status fast_attn_out(void* z, const void* o, const void* W_o, const AttnPrep&
   const float2* c01g = (const float2*)ap.c01g;
   const int zslab = c / 64, oslab = Hd / 64;
   const size_t smem = (size_t)zslab * Hd * 128 + (size_t)oslab * c * 128 + 2 * (size_t)(zslab + oslab) * 128 * 128 +
-                      3 * 2048 + (size_t)Hd * 16 + 1024;
+                      2 * 4096 + (size_t)Hd * 32 + 1024;
   // the attribute belongs to a (kernel, device) pair: one flag per device
   static bool attr_set_dev[64] = {};
   int attr_dev = 0;

@@ -84,9 +84,8 @@ __global__ void __launch_bounds__(TO_THREADS, 1) tri_out_kernel(const __grid_con
   unsigned char* sWg = sWo + wo_bytes;
   unsigned char* sT = sWg + wg_bytes;                        // 2 stages of the two t chunks
   unsigned char* sZ = sT + 2 * t_stage;                      // 2 stages of the z tile
-  unsigned char* sAx = sZ + 2 * z_stage;                     // [2 stages][t | z][128][8] fp16: augmentation columns 0-7 of the rows
-  unsigned char* sBx = sAx + 4 * 2048;                       // [W_o | W_g][c_z][8] fp16: augmentation columns 0-7 of the weights
-  unsigned char* sZero = sBx + 2 * c_z * 16;                 // [128][8] zeros: augmentation columns 8-15 of all of them
+  unsigned char* sAx = sZ + 2 * z_stage;                     // [2 stages][t | z][2][128][8] bf16: augmentation columns 0-7, 8-15 of the rows
+  unsigned char* sBx = sAx + 4 * 4096;                       // [W_o | W_g][2][c_z][8] bf16: the same of the weights
   unsigned long long* tfullb = bars;        // [2] t chunks landed
   unsigned long long* tfree = bars + 2;     // [2] MMAs and statistics have read them
   unsigned long long* zfullb = bars + 4;    // [2] z tile landed
@@ -114,14 +113,13 @@ __global__ void __launch_bounds__(TO_THREADS, 1) tri_out_kernel(const __grid_con
     mbar_fence_init();
   }
   if (warp == 1) tmem_alloc(&tmem_base_s, 512);
-  for (int n = threadIdx.x; n < 128; n += TO_THREADS) *reinterpret_cast<uint4*>(sZero + n * 16) = make_uint4(0, 0, 0, 0);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   pdl_begin();
   for (int n = threadIdx.x; n < 2 * c_z; n += TO_THREADS) {
-    const float2 k = n < c_z ? p.c01o[n] : p.c01g[n - c_z];
-    *reinterpret_cast<uint4*>(sBx + n * 16) = ln_aug_weight(k.x, k.y);
+    const int g = n >= c_z ? 1 : 0, r = n - g * c_z;
+    ln_aug_weight(sBx + g * c_z * 32 + r * 16, c_z * 16, g ? p.c01g[r] : p.c01o[r]);
   }
   fence_proxy_async_smem();
   __syncthreads();
@@ -169,8 +167,9 @@ __global__ void __launch_bounds__(TO_THREADS, 1) tri_out_kernel(const __grid_con
     unsigned n = 0;
     const unsigned idesc_t = idesc_f16(128, c_z, 1, 0, FMT_F16, FMT_F16);     // A = t (fp16, MN-major), W_o' fp16
     const unsigned idesc_z = idesc_f16(128, c_z, 0, 0, FMT_BF16, FMT_BF16);   // A = the bf16 z tile, W_g' bf16
-    const unsigned idesc_x = idesc_f16(128, c_z, 0, 0, FMT_F16, FMT_F16);     // augmentation step
     const unsigned long long wo_desc = desc_kmajor_sw128(smem_u32(sWo)), wg_desc = desc_kmajor_sw128(smem_u32(sWg));
+    const unsigned long long bxo_desc = desc_kmajor_nosw(smem_u32(sBx), c_z * 16, 128);
+    const unsigned long long bxg_desc = desc_kmajor_nosw(smem_u32(sBx + c_z * 32), c_z * 16, 128);
     const unsigned wo16 = (unsigned)wo_slab >> 4, wg16 = (unsigned)wg_slab >> 4, z16 = (unsigned)z_slab >> 4;
     for (long long t = blockIdx.x; t < ntiles; t += gridDim.x, ++n) {
       const unsigned buf = n & 1;
@@ -194,10 +193,8 @@ __global__ void __launch_bounds__(TO_THREADS, 1) tri_out_kernel(const __grid_con
         if (sl < zslab) umma_k4(d2, z_desc + sl * z16, wg_desc + sl * wg16, idesc_z, sl);
       mbar_wait(&sconv[stage], phase, ab);                 // the rows' augmentation columns are written
       tc_fence_after();
-      const unsigned ax = smem_u32(sAx + stage * 4096), bx = smem_u32(sBx), zero = smem_u32(sZero);
-      if (elect_one()) umma_bf16(d1, desc_kmajor_nosw(ax, zero - ax, 128), desc_kmajor_nosw(bx, zero - bx, 128), idesc_x, 1);
-      if (elect_one())
-        umma_bf16(d2, desc_kmajor_nosw(ax + 2048, zero - ax - 2048, 128), desc_kmajor_nosw(bx + c_z * 16, zero - bx - c_z * 16, 128), idesc_x, 1);
+      if (elect_one()) umma_bf16(d1, desc_kmajor_nosw(smem_u32(sAx + stage * 8192), 2048, 128), bxo_desc, idesc_z, 1);
+      if (elect_one()) umma_bf16(d2, desc_kmajor_nosw(smem_u32(sAx + stage * 8192 + 4096), 2048, 128), bxg_desc, idesc_z, 1);
       if (elect_one()) {
         tc_commit(&tfull[buf]);
         tc_commit(&zfree[stage]);
@@ -275,7 +272,7 @@ __global__ void __launch_bounds__(TO_THREADS, 1) tri_out_kernel(const __grid_con
       if (lane == 0) mbar_arrive(&tfree[stage]);
       // t arrives scaled by 1 / N_s (see the contraction); LayerNorm is scale-free once eps is scaled alike
       const float tmean = ts / (float)c_h;
-      const float tve = fmaxf(tq / (float)c_h - tmean * tmean, 0.f) + eps_t, trstd = rsqrtf(tve);
+      const float trstd = rsqrtf(fmaxf(tq / (float)c_h - tmean * tmean, 0.f) + eps_t);
       // z row: statistics of the bf16 tile (read only)
       mbar_wait(&zfullb[stage], phase, ab);
       float zs = 0.f, zq = 0.f;
@@ -299,9 +296,9 @@ __global__ void __launch_bounds__(TO_THREADS, 1) tri_out_kernel(const __grid_con
       const float zmean = p.zstats ? zst.x : zs / (float)c_z;
       const float zrstd = p.zstats ? zst.y : rsqrtf(fmaxf(zq / (float)c_z - zmean * zmean, 0.f) + p.eps);
       // (the z tile has landed, so the MMAs that read this stage's columns for the tile before are complete)
-      *reinterpret_cast<uint4*>(sAx + stage * 4096 + row * 16) = ln_aug_row(tmean, tve * trstd);
-      *reinterpret_cast<uint4*>(sAx + stage * 4096 + 2048 + row * 16) = ln_aug_row(zmean, 1.f / zrstd);
-      sStats[stage][row] = make_float2(0.5f * trstd, 0.5f * zrstd);
+      unsigned char* ax = sAx + stage * 8192 + row * 16;
+      const float tr = ln_aug_row(ax, 2048, tmean, trstd), zr = ln_aug_row(ax + 4096, 2048, zmean, zrstd);
+      sStats[stage][row] = make_float2(0.5f * tr, 0.5f * zr);
       fence_proxy_async_smem();
       __syncwarp();
       if (lane == 0) {
@@ -397,7 +394,7 @@ nt_status fast_tri_out(void* z, const void* t, const TriPrep& tp, float eps, int
   const float2* c01g = (const float2*)tp.c01g;
   const int zslab = c_z / 64, hslab = c_h / 64;
   const size_t smem = (size_t)hslab * c_z * 128 + (size_t)zslab * c_z * 128 +
-                      2 * ((size_t)2 * c_h * 128 + (size_t)zslab * 128 * 128) + 5 * 2048 + 2 * (size_t)c_z * 16 + 1024;
+                      2 * ((size_t)2 * c_h * 128 + (size_t)zslab * 128 * 128) + 4 * 4096 + (size_t)c_z * 64 + 1024;
   // the attribute belongs to a (kernel, device) pair: one flag per device
   static bool attr_set_dev[64] = {};
   int attr_dev = 0;

@@ -383,23 +383,39 @@ __device__ inline void store_32b(void* to, const unsigned (&w)[8], bool wide) {
 
 // LayerNorm folded into the MMA for a tile that stays as it is.  One more K step adds s c0 - mean c1 to the raw product,
 // s = 1 / rstd, so that rstd times the accumulator is the normalised projection and a reader of the accumulator needs no
-// tables.  Both sides are split into fp16 parts: the row side is (-m_hi, -m_lo, -m_hi, s_hi, s_hi, s_lo, 4096 s_rest,
-// -4096 m_rest), the weight side (c1_hi, c1_hi, c1_lo, c0_hi, c0_lo, c0_hi, c0_hi / 4096, c1_hi / 4096).
-__device__ inline uint4 ln_aug_row(float mean, float s) {
-  s = fminf(s, 65504.f);                              // above that the tile's own fp16 values have overflowed
-  const __half mh = __float2half_rn(-mean), sh = __float2half_rn(s);
-  const float m1 = -mean - __half2float(mh), s1 = s - __half2float(sh);
-  const __half ml = __float2half_rn(m1), sl = __float2half_rn(s1);
-  const __half mr = __float2half_rn((m1 - __half2float(ml)) * 4096.f), sr = __float2half_rn((s1 - __half2float(sl)) * 4096.f);
-  __half2 a[4] = {__halves2half2(mh, ml), __halves2half2(mh, sh), __halves2half2(sh, sl), __halves2half2(sr, mr)};
-  return *reinterpret_cast<const uint4*>(a);
+// tables.  The step multiplies bf16 whatever the tile holds: a bf16 state reaches far beyond fp16, and so do its means and
+// spreads.  Three bf16 parts carry the 24 bits of a float; of the nine products of two such triples eight fit the columns
+// (0-7 mean and c1, 8-15 s and c0), and the one left out, third part times third part, is 2^-34 of the whole or less.
+__device__ inline void bf16_parts(float x, unsigned (&p)[3]) {
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    const __nv_bfloat16 h = __float2bfloat16_rn(x);
+    p[i] = __bfloat16_as_ushort(h);
+    x -= __bfloat162float(h);
+  }
 }
-__device__ inline uint4 ln_aug_weight(float c0, float c1) {
-  const __half c1h = __float2half_rn(c1), c1l = __float2half_rn(c1 - __half2float(c1h));
-  const __half c0h = __float2half_rn(c0), c0l = __float2half_rn(c0 - __half2float(c0h));
-  const __half c0s = __float2half_rn(__half2float(c0h) * (1.f / 4096.f)), c1s = __float2half_rn(__half2float(c1h) * (1.f / 4096.f));
-  __half2 a[4] = {__halves2half2(c1h, c1h), __halves2half2(c1l, c0h), __halves2half2(c0l, c0h), __halves2half2(c0s, c1s)};
-  return *reinterpret_cast<const uint4*>(a);
+__device__ inline uint4 ln_aug_row_cols(float x) {
+  unsigned p[3];
+  bf16_parts(x, p);
+  return make_uint4(p[0] | p[0] << 16, p[1] | p[1] << 16, p[0] | p[2] << 16, p[1] | p[2] << 16);
+}
+__device__ inline uint4 ln_aug_weight_cols(float x) {
+  unsigned p[3];
+  bf16_parts(x, p);
+  return make_uint4(p[0] | p[1] << 16, p[0] | p[1] << 16, p[2] | p[0] << 16, p[2] | p[1] << 16);
+}
+// The row's columns 0-7 to `at`, 8-15 `region` bytes further on; returns the rstd to apply to the accumulator.  rstd = 0 (the
+// row's sum of squares passed the float range): the offset alone, at a scale that no product reaches.
+__device__ inline float ln_aug_row(unsigned char* at, int region, float mean, float rstd) {
+  const bool none = rstd == 0.f;
+  rstd = none ? 7.8886091e-31f : rstd;                   // 2^-100
+  *reinterpret_cast<uint4*>(at) = ln_aug_row_cols(none ? 0.f : -mean);
+  *reinterpret_cast<uint4*>(at + region) = ln_aug_row_cols(1.f / rstd);
+  return rstd;
+}
+__device__ inline void ln_aug_weight(unsigned char* at, int region, float2 c01) {
+  *reinterpret_cast<uint4*>(at) = ln_aug_weight_cols(c01.y);
+  *reinterpret_cast<uint4*>(at + region) = ln_aug_weight_cols(c01.x);
 }
 
 // LayerNorm folded into the MMA, activation side.  Two threads per tile row (hf = 0 / 1), each owning four of the
