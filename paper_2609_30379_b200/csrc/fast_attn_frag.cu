@@ -486,8 +486,10 @@ __global__ void __launch_bounds__(128 + 128 * NT, 1) attn_fr_kernel(const __grid
         fr_wait_idle(&qfull[qb], qph, ab);
         const unsigned long long qd = fr_desc(q_base + qb * NT * Q_BYTES, SPAN);
         for (int k0 = 0; k0 < it.N; k0 += FR_KEYS) {
+          // every block, also of an item in which this tile has no row: a parity wait tells one phase from the next only,
+          // and a warp that left blocks out could take a slot's load of one ring turn ago, still in flight, for its own
+          fr_wait_idle(&full[st], ph, ab);
           if (valid) {
-            fr_wait_idle(&full[st], ph, ab);
             const unsigned b = cnt & 1, bph = (cnt >> 1) & 1;
             fr_wait_idle(&sempty[t * 2 + b], bph ^ 1, ab);
             tc_fence_after();
