@@ -396,6 +396,12 @@ nt_status nt_debug_bounds_report(int32_t *out_h, int32_t reset);
  * `stream`.  Returns NT_ERR_INVALID_ARG (nothing launched) for a null status_d or a limit out of range. */
 nt_status nt_debug_expire_wait(int32_t *status_d, int64_t limit_clocks, int32_t *observed_d, nt_stream stream);
 
+/* Testing aid for the failure path of the register-fragment attention core: from now on each of its CTAs requests only
+ * `blocks` blocks of 64 keys and then stops, so that the waits for the next one run out (about a second), the status word
+ * receives NT_ERR_TIMEOUT and the kernel ends without storing what it could not compute.  Negative (the default): all
+ * blocks.  Returns the previous value. */
+int32_t nt_debug_attn_drop(int32_t blocks);
+
 /* Testing aid: the bf16 pair-order attention uses two tensor-core kernels, one that holds a whole score row
  * on chip (samples of up to 224 tokens) and one that walks the keys in blocks (longer samples).  mode 1 sends every
  * sample to the second kernel, mode 0 restores the split by length.  Returns the previous mode. */

@@ -30,7 +30,7 @@ EXPORTS = ("nt_offsets_build", "nt_pair_broadcast", "nt_pair_broadcast_add", "nt
            "nt_single_attn_workspace_bytes", "nt_rect_offsets_build", "nt_rect_pair_broadcast",
            "nt_rect_broadcast_workspace_bytes", "nt_segment_reduce", "nt_pair_transition", "nt_transition_workspace_bytes", "nt_token_update",
            "nt_workspace_bytes", "nt_status_string",
-           "nt_prepare_trimul_weights", "nt_prepare_attn_weights", "nt_launch_count", "nt_force_generic", "nt_debug_bounds_report", "nt_attn_core_mode", "nt_debug_expire_wait", "nt_bench_exp_rate", "nt_profile_begin", "nt_profile_end")
+           "nt_prepare_trimul_weights", "nt_prepare_attn_weights", "nt_launch_count", "nt_force_generic", "nt_debug_bounds_report", "nt_attn_core_mode", "nt_debug_attn_drop", "nt_debug_expire_wait", "nt_bench_exp_rate", "nt_profile_begin", "nt_profile_end")
 
 
 class NtError(RuntimeError):
@@ -121,6 +121,8 @@ def _load() -> C.CDLL:
     lib.nt_debug_bounds_report.restype = i32
     lib.nt_attn_core_mode.argtypes = [i32]
     lib.nt_attn_core_mode.restype = i32
+    lib.nt_debug_attn_drop.argtypes = [i32]
+    lib.nt_debug_attn_drop.restype = i32
     lib.nt_profile_begin.argtypes = []
     lib.nt_profile_begin.restype = i32
     lib.nt_profile_end.argtypes = [vp, sz, vp, vp, i32]
@@ -439,6 +441,10 @@ def nt_debug_bounds_report(reset: bool = False):
     out = (C.c_int32 * 4)()
     _check(lib.nt_debug_bounds_report(out, 1 if reset else 0), "nt_debug_bounds_report")
     return int(out[0]), int(out[1]), (int(out[3]) << 32) | (int(out[2]) & 0xFFFFFFFF)
+
+
+def nt_debug_attn_drop(blocks: int) -> int:
+    return int(lib.nt_debug_attn_drop(int(blocks)))
 
 
 def nt_attn_core_mode(mode: int) -> int:

@@ -18,6 +18,7 @@ __device__ int g_nt_bounds[4] = {0, 0, 0, 0};
 
 std::atomic<long long> g_launches{0};
 int g_force_generic = 0;
+int g_fr_drop = -1; // testing aid (nt_debug_attn_drop): key blocks a CTA of that core requests before it stops
 int g_fr_all = 0;   // testing aid (nt_attn_core_mode): the register-fragment attention core for every sample length
 
 // ---- per-kernel event timing (off unless nt_profile_begin was called) ----------------------
@@ -851,6 +852,12 @@ nt_status nt_debug_bounds_report(int32_t* out_h, int32_t reset) {
   (void)reset;
   return NT_ERR_UNSUPPORTED;
 #endif
+}
+
+int32_t nt_debug_attn_drop(int32_t blocks) {
+  int32_t prev = g_fr_drop;
+  g_fr_drop = blocks;
+  return prev;
 }
 
 int32_t nt_attn_core_mode(int32_t mode) {

@@ -69,6 +69,7 @@ nt_status fast_attn_core_tc(const void* q, const void* k, const void* v, const v
 // pair order (rows or columns; one bias plane per (sample, head), stored times sqrt(d), for columns stored transposed)
 // or token order (rows = samples; the bias planes, if any, belong to the sample's own queries).  Samples with N <= n_min
 // are left out (they belong to another kernel).
+extern int g_fr_drop;
 enum { FR_MODE_PAIR_ROW = 0, FR_MODE_TOKEN = 1, FR_MODE_PAIR_COL = 2 };
 bool fast_attn_fr_supported(int H, int d);
 nt_status fast_attn_core_fr(const void* q, const void* k, const void* v, const void* bias, void* o, int H, int d,

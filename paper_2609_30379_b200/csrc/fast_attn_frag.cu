@@ -56,6 +56,7 @@ struct AttnFrParams {
   long long rows;                 // rows the flat maps (and the output) cover from row0 on
   int H, mode, nstage, single_tile;
   float sc2;                      // log2(e) / sqrt(d)
+  int drop;                       // testing aid: a CTA requests only this many key blocks (< 0: all)
   int* status;
 };
 
@@ -216,6 +217,9 @@ __device__ inline void fr_wait_idle(void* bar, unsigned parity, const AbortCtx& 
     if (ab.status) atomicCAS(ab.status, 0, (int)NT_ERR_TIMEOUT);
   }
 }
+// Whether a wait of the CTA has run out, the same answer for the whole warp.  Asked after every wait that shared memory is
+// trusted on: what a wait that gave up was for may not be there.
+__device__ inline bool fr_gone(const AbortCtx& ab) { return __any_sync(0xffffffffu, *ab.flag != 0); }
 // swizzled operand descriptor for a K-major tile whose rows are `span` = 32, 64 or 128 bytes
 __device__ inline unsigned long long fr_desc(unsigned saddr, int span) {
   unsigned long long d = 0;
@@ -423,13 +427,15 @@ __global__ void __launch_bounds__(128 + 128 * NT, 1) attn_fr_kernel(const __grid
       const int t = lane >> 1, part = lane & 1;      // Q: tile and 64-query half; keys: tile and K / V
       FrItem<NT> it;
       if (count > 0) it.seek(p, g0);
-      for (int n = 0; n < count; ++n, it.next(p)) {
+      int blocks = 0;
+      bool gone = false;
+      for (int n = 0; n < count && !gone; ++n, it.next(p)) {
         const unsigned qb = n & 1, qph = (n >> 1) & 1;
         const int tiles = it.tiles(p);
-        if (lane == 0) {
-          fr_wait_idle(&qempty[qb], qph ^ 1, ab);
-          mbar_expect_tx(&qfull[qb], tiles * Q_BYTES);
-        }
+        if (lane == 0) fr_wait_idle(&qempty[qb], qph ^ 1, ab);
+        gone = fr_gone(ab);
+        if (gone) break;
+        if (lane == 0) mbar_expect_tx(&qfull[qb], tiles * Q_BYTES);
         __syncwarp();
         const bool mine = t < tiles;
         const int x = it.head(p, t) * D, row = it.kvrow(p, t), col = it.g * NT + t;
@@ -443,8 +449,12 @@ __global__ void __launch_bounds__(128 + 128 * NT, 1) attn_fr_kernel(const __grid
         }
         for (int k0 = 0; k0 < it.N; k0 += FR_KEYS) {
           unsigned char* stg = sStage + st * STAGE_BYTES;
+          if (lane == 0) fr_wait_idle(&empty[st], ph ^ 1, ab);
+          // (after a wait that ran out nothing is written any more: the softmax warps may still be at the slot's item)
+          gone = fr_gone(ab) || blocks == p.drop;
+          if (gone) break;
+          ++blocks;
           if (lane == 0) {
-            fr_wait_idle(&empty[st], ph ^ 1, ab);
             if (k0 == 0) {
               FrInfo& f = info[n % FR_MAXSTAGE];
               f.N = it.N;
@@ -480,7 +490,8 @@ __global__ void __launch_bounds__(128 + 128 * NT, 1) attn_fr_kernel(const __grid
       unsigned cnt = 0;
       FrItem<NT> it;
       if (count > 0) it.seek(p, g0);
-      for (int n = 0; n < count; ++n, it.next(p)) {
+      bool gone = false;
+      for (int n = 0; n < count && !gone; ++n, it.next(p)) {
         const unsigned qb = n & 1, qph = (n >> 1) & 1;
         const bool valid = t < it.tiles(p);
         fr_wait_idle(&qfull[qb], qph, ab);
@@ -492,6 +503,8 @@ __global__ void __launch_bounds__(128 + 128 * NT, 1) attn_fr_kernel(const __grid
           if (valid) {
             const unsigned b = cnt & 1, bph = (cnt >> 1) & 1;
             fr_wait_idle(&sempty[t * 2 + b], bph ^ 1, ab);
+            gone = fr_gone(ab);
+            if (gone) break;
             tc_fence_after();
             const unsigned long long kd = fr_desc(k_base + st * STAGE_BYTES, SPAN);
             if (elect_one()) {
@@ -504,6 +517,7 @@ __global__ void __launch_bounds__(128 + 128 * NT, 1) attn_fr_kernel(const __grid
           }
           if (++st == nstage) { st = 0; ph ^= 1; }
         }
+        if (gone || fr_gone(ab)) break;
         if (valid) {
           if (elect_one()) tc_commit(&qempty[qb]);
         } else if (lane == 0) {
@@ -530,7 +544,8 @@ __global__ void __launch_bounds__(128 + 128 * NT, 1) attn_fr_kernel(const __grid
     unsigned cnt = 0;                                // blocks of this tile so far
 #pragma unroll 1
     for (int n = 0; n < count; ++n) {
-      mbar_wait(&full[st], ph, ab);                  // the item's first stage: its description is there too
+      mbar_wait(&full[st], ph, ab);                  // the item's first stage: its description is there too,
+      if (fr_gone(ab)) break;                        // unless the wait ran out
       const FrInfo& inf = info[n % FR_MAXSTAGE];
       const int N = __shfl_sync(0xffffffffu, inf.N, 0), q0 = __shfl_sync(0xffffffffu, inf.q0, 0) + quarter * 32;
       const bool valid = t < __shfl_sync(0xffffffffu, inf.tiles, 0);
@@ -637,6 +652,7 @@ __global__ void __launch_bounds__(128 + 128 * NT, 1) attn_fr_kernel(const __grid
         off |= bad & (q < N);
         nref[r] -= bad ? 0.f : (float)((int)(__float_as_uint(x) >> 23) - 127) + FR_MARGIN;
       }
+      if (fr_gone(ab)) break;                        // scores that never came: nothing to store, nothing to compute again
       const bool again = __any_sync(0xffffffffu, off);
       if (again) {
         const float lse = fr_exact_row<D, HAS_BIAS>(p, inf, t, quarter, lane);
@@ -750,6 +766,7 @@ nt_status fast_attn_core_fr(const void* q, const void* k, const void* v, const v
   p.status = status;
   p.sc2 = FR_LOG2E / sqrtf((float)d);
   p.nstage = fr_pick_stages(d, bias != nullptr);
+  p.drop = g_fr_drop;
   const bool token = mode == FR_MODE_TOKEN;
   p.single_tile = token && bias != nullptr;   // every head has bias planes of its own: nothing to share between two rows
   p.row0 = token ? m.tok_off[0] : m.pair_off[0];
