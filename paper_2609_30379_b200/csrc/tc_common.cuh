@@ -410,7 +410,9 @@ __device__ inline float ln_aug_row(unsigned char* at, int region, float mean, fl
   const bool none = rstd == 0.f;
   rstd = none ? 7.8886091e-31f : rstd;                   // 2^-100
   *reinterpret_cast<uint4*>(at) = ln_aug_row_cols(none ? 0.f : -mean);
-  *reinterpret_cast<uint4*>(at + region) = ln_aug_row_cols(1.f / rstd);
+  float s;
+  asm("rcp.approx.ftz.f32 %0, %1;\n" : "=f"(s) : "f"(rstd));
+  *reinterpret_cast<uint4*>(at + region) = ln_aug_row_cols(s);
   return rstd;
 }
 __device__ inline void ln_aug_weight(unsigned char* at, int region, float2 c01) {
