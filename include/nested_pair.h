@@ -398,8 +398,8 @@ nt_status nt_debug_expire_wait(int32_t *status_d, int64_t limit_clocks, int32_t 
 
 /* Testing aid for the failure path of the register-fragment attention core: from now on each of its CTAs requests only
  * `blocks` blocks of 64 keys and then stops, so that the waits for the next one run out (about a second), the status word
- * receives NT_ERR_TIMEOUT and the kernel ends without storing what it could not compute.  Negative (the default): all
- * blocks.  Returns the previous value. */
+ * receives NT_ERR_TIMEOUT and the kernel ends (the call's output is then undefined).  Negative (the default): all blocks.
+ *  Returns the previous value. */
 int32_t nt_debug_attn_drop(int32_t blocks);
 
 /* Testing aid: the bf16 pair-order attention uses two tensor-core kernels, one that holds a whole score row

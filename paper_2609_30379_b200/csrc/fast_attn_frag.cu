@@ -204,22 +204,23 @@ __device__ inline bool fr_ready(void* bar, unsigned parity) {
 }
 // The auxiliary warps' wait: they have a block's time in hand, and a warp that probes a barrier all the time takes issue
 // slots from the exponentials (a parked try_wait came back so often that the four warps took a tenth of the slots).
-__device__ inline void fr_wait_idle(void* bar, unsigned parity, const AbortCtx& ab) {
-  if (fr_ready(bar, parity)) return;
+// False: the wait ran out (as with mbar_wait).  A warp of this kernel then works through no further item, because what it
+// waited for may not be there, and because its later waits mean nothing: a barrier that has stopped satisfies every other
+// parity wait at once.
+__device__ inline bool fr_wait_idle(void* bar, unsigned parity, const AbortCtx& ab) {
+  if (fr_ready(bar, parity)) return true;
   const long long t0 = clock64();
   for (unsigned it = 0; it < WAIT_PROBES; ++it) {
     __nanosleep(200);
-    if (fr_ready(bar, parity)) return;
+    if (fr_ready(bar, parity)) return true;
     if ((it & 15u) == 15u && (clock64() - t0 > (*ab.flag ? WAIT_CLOCKS_ABORTED : WAIT_CLOCKS) || *ab.flag)) break;
   }
   if (!*ab.flag) {
     *ab.flag = 1;
     if (ab.status) atomicCAS(ab.status, 0, (int)NT_ERR_TIMEOUT);
   }
+  return false;
 }
-// Whether a wait of the CTA has run out, the same answer for the whole warp.  Asked after every wait that shared memory is
-// trusted on: what a wait that gave up was for may not be there.
-__device__ inline bool fr_gone(const AbortCtx& ab) { return __any_sync(0xffffffffu, *ab.flag != 0); }
 // swizzled operand descriptor for a K-major tile whose rows are `span` = 32, 64 or 128 bytes
 __device__ inline unsigned long long fr_desc(unsigned saddr, int span) {
   unsigned long long d = 0;
@@ -428,15 +429,16 @@ __global__ void __launch_bounds__(128 + 128 * NT, 1) attn_fr_kernel(const __grid
       FrItem<NT> it;
       if (count > 0) it.seek(p, g0);
       int blocks = 0;
-      bool gone = false;
-      for (int n = 0; n < count && !gone; ++n, it.next(p)) {
+      bool ok = true;
+      for (int n = 0; n < count && ok; ++n, it.next(p)) {
         const unsigned qb = n & 1, qph = (n >> 1) & 1;
         const int tiles = it.tiles(p);
-        if (lane == 0) fr_wait_idle(&qempty[qb], qph ^ 1, ab);
-        gone = fr_gone(ab);
-        if (gone) break;
-        if (lane == 0) mbar_expect_tx(&qfull[qb], tiles * Q_BYTES);
-        __syncwarp();
+        if (lane == 0) {
+          ok = fr_wait_idle(&qempty[qb], qph ^ 1, ab);
+          mbar_expect_tx(&qfull[qb], tiles * Q_BYTES);
+        }
+        ok = __shfl_sync(0xffffffffu, ok, 0);
+        if (!ok) break;
         const bool mine = t < tiles;
         const int x = it.head(p, t) * D, row = it.kvrow(p, t), col = it.g * NT + t;
         const CUtensorMap* cmap = &p.cmap[it.s];
@@ -449,13 +451,9 @@ __global__ void __launch_bounds__(128 + 128 * NT, 1) attn_fr_kernel(const __grid
         }
         for (int k0 = 0; k0 < it.N; k0 += FR_KEYS) {
           unsigned char* stg = sStage + st * STAGE_BYTES;
-          if (lane == 0) fr_wait_idle(&empty[st], ph ^ 1, ab);
-          // (after a wait that ran out nothing is written any more: the softmax warps may still be at the slot's item)
-          gone = fr_gone(ab) || blocks == p.drop;
-          if (gone) break;
-          ++blocks;
           if (lane == 0) {
-            if (k0 == 0) {
+            ok = blocks++ != p.drop && fr_wait_idle(&empty[st], ph ^ 1, ab);
+            if (ok && k0 == 0) {    // (after a wait that ran out nothing is written: the softmax warps may still be at an older item)
               FrInfo& f = info[n % FR_MAXSTAGE];
               f.N = it.N;
               f.q0 = it.jb * 128;
@@ -468,9 +466,10 @@ __global__ void __launch_bounds__(128 + 128 * NT, 1) attn_fr_kernel(const __grid
               f.ld = round_up8(it.N);
               f.bias_plane = (long long)p.H * p.m.cm_off[it.s] + (long long)f.head * it.N * f.ld;
             }
-            mbar_expect_tx(&full[st], BIAS_BYTES + tiles * 2 * KV_BYTES);
+            if (ok) mbar_expect_tx(&full[st], BIAS_BYTES + tiles * 2 * KV_BYTES);
           }
-          __syncwarp();
+          ok = __shfl_sync(0xffffffffu, ok, 0);
+          if (!ok) break;
           if (mine) {
             unsigned char* dst = stg + BIAS_BYTES + (t * 2 + part) * KV_BYTES;
             if (colmode) tma_load_4d(dst, cmap, &full[st], x, k0, col, 1 + part);
@@ -490,23 +489,22 @@ __global__ void __launch_bounds__(128 + 128 * NT, 1) attn_fr_kernel(const __grid
       unsigned cnt = 0;
       FrItem<NT> it;
       if (count > 0) it.seek(p, g0);
-      bool gone = false;
-      for (int n = 0; n < count && !gone; ++n, it.next(p)) {
+      bool ok = true;                                // false once a wait has run out
+      for (int n = 0; n < count; ++n, it.next(p)) {
         const unsigned qb = n & 1, qph = (n >> 1) & 1;
         const bool valid = t < it.tiles(p);
-        fr_wait_idle(&qfull[qb], qph, ab);
+        ok = fr_wait_idle(&qfull[qb], qph, ab);
         const unsigned long long qd = fr_desc(q_base + qb * NT * Q_BYTES, SPAN);
         for (int k0 = 0; k0 < it.N; k0 += FR_KEYS) {
           // every block, also of an item in which this tile has no row: a parity wait tells one phase from the next only,
           // and a warp that left blocks out could take a slot's load of one ring turn ago, still in flight, for its own
-          fr_wait_idle(&full[st], ph, ab);
+          ok &= fr_wait_idle(&full[st], ph, ab);
           if (valid) {
             const unsigned b = cnt & 1, bph = (cnt >> 1) & 1;
-            fr_wait_idle(&sempty[t * 2 + b], bph ^ 1, ab);
-            gone = fr_gone(ab);
-            if (gone) break;
+            ok &= fr_wait_idle(&sempty[t * 2 + b], bph ^ 1, ab);
             tc_fence_after();
             const unsigned long long kd = fr_desc(k_base + st * STAGE_BYTES, SPAN);
+            if (!__all_sync(0xffffffffu, ok)) break;
             if (elect_one()) {
 #pragma unroll
               for (int ks = 0; ks < D / 16; ++ks) umma_bf16(d_base + b * FR_KEYS, qd + ks * 2, kd + ks * 2, idesc, ks ? 1u : 0u);
@@ -517,7 +515,7 @@ __global__ void __launch_bounds__(128 + 128 * NT, 1) attn_fr_kernel(const __grid
           }
           if (++st == nstage) { st = 0; ph ^= 1; }
         }
-        if (gone || fr_gone(ab)) break;
+        if (!__all_sync(0xffffffffu, ok)) break;
         if (valid) {
           if (elect_one()) tc_commit(&qempty[qb]);
         } else if (lane == 0) {
@@ -544,17 +542,15 @@ __global__ void __launch_bounds__(128 + 128 * NT, 1) attn_fr_kernel(const __grid
     unsigned cnt = 0;                                // blocks of this tile so far
 #pragma unroll 1
     for (int n = 0; n < count; ++n) {
-      mbar_wait(&full[st], ph, ab);                  // the item's first stage: its description is there too,
-      if (fr_gone(ab)) break;                        // unless the wait ran out
+      if (!__all_sync(0xffffffffu, mbar_wait(&full[st], ph, ab))) break;   // the item's first stage: its description is there too
       const FrInfo& inf = info[n % FR_MAXSTAGE];
       const int N = __shfl_sync(0xffffffffu, inf.N, 0), q0 = __shfl_sync(0xffffffffu, inf.q0, 0) + quarter * 32;
       const bool valid = t < __shfl_sync(0xffffffffu, inf.tiles, 0);
       if (!valid || q0 >= N) {    // no row, or no query in this warp's quarter: follow the barriers only
         for (int k0 = 0; k0 < N; k0 += FR_KEYS) {
-          mbar_wait(&full[st], ph, ab);
+          if (!__all_sync(0xffffffffu, mbar_wait(&full[st], ph, ab))) goto gone;
           if (valid) {
-            mbar_wait(&sfull_t[cnt & 1], (cnt >> 1) & 1, ab);
-            __syncwarp();
+            if (!__all_sync(0xffffffffu, mbar_wait(&sfull_t[cnt & 1], (cnt >> 1) & 1, ab))) goto gone;
             fr_arrive(sempty_bar + (cnt & 1) * 8, lane);
             ++cnt;
           }
@@ -583,8 +579,7 @@ __global__ void __launch_bounds__(128 + 128 * NT, 1) attn_fr_kernel(const __grid
       unsigned stage = stage_base + st * STAGE_BYTES, v_prev = stage + v_off, s_addr = s_base + (cnt & 1) * FR_KEYS;
       int left = N;                                  // keys left in the row
       unsigned held = 0;                             // empty barrier of the stage whose last product is pending
-      mbar_wait(&sfull_t[cnt & 1], (cnt >> 1) & 1, ab);
-      __syncwarp();
+      if (!__all_sync(0xffffffffu, mbar_wait(&sfull_t[cnt & 1], (cnt >> 1) & 1, ab))) break;
       tc_fence_after();
       fr_request_scores(s_addr, sa);
       tmem_ld_wait2(sa[0], sa[1]);
@@ -612,9 +607,8 @@ __global__ void __launch_bounds__(128 + 128 * NT, 1) attn_fr_kernel(const __grid
         const unsigned bias_odd = stage + bias_off, v_odd = stage + v_off, buf = sempty_bar + (cnt & 1) * 8;
         if (more) {
           if (!__all_sync(0xffffffffu, ready)) {
-            mbar_wait(&full[nst], nph, ab);
-            mbar_wait(&sfull_t[ncnt & 1], (ncnt >> 1) & 1, ab);
-            __syncwarp();
+            const bool there = mbar_wait(&full[nst], nph, ab) & mbar_wait(&sfull_t[ncnt & 1], (ncnt >> 1) & 1, ab);
+            if (!__all_sync(0xffffffffu, there)) goto gone;
           }
           tc_fence_after();
           held = empty_bar + st * 8;
@@ -652,7 +646,6 @@ __global__ void __launch_bounds__(128 + 128 * NT, 1) attn_fr_kernel(const __grid
         off |= bad & (q < N);
         nref[r] -= bad ? 0.f : (float)((int)(__float_as_uint(x) >> 23) - 127) + FR_MARGIN;
       }
-      if (fr_gone(ab)) break;                        // scores that never came: nothing to store, nothing to compute again
       const bool again = __any_sync(0xffffffffu, off);
       if (again) {
         const float lse = fr_exact_row<D, HAS_BIAS>(p, inf, t, quarter, lane);
@@ -694,6 +687,7 @@ __global__ void __launch_bounds__(128 + 128 * NT, 1) attn_fr_kernel(const __grid
       if (++st == nstage) { st = 0; ph ^= 1; }
     }
   }
+gone:
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
