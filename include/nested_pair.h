@@ -177,9 +177,11 @@ nt_status nt_tri_mul_in(const nt_layout *L, nt_dtype dt, int32_t c_z, int32_t c_
  *     row maximum.  Samples of up to 224 tokens use the bound max_k(q.k)/sqrt(d) + max_k(bias) of the
  *     query (the first maximum also runs over the up to 15 keys of the next pair row that pad the
  *     last group of 16); a row whose true maximum lies more than about 80 nats below that bound
- *     loses its weights to underflow (its output row is then not finite).  Longer samples, token order and d = 64 use a
- *     running reference that follows the data and have no such limit.  Activations that have
- *     passed a LayerNorm and projections of O(1) norm stay far inside either range.
+ *     loses its weights to underflow (its output row is then not finite).  Longer samples, token order and d = 64 have no
+ *     such limit: their reference is guessed from the query's previous row, and a row whose log-sum lies more than 42 nats
+ *     below or 97 above that row's is computed a second time with a running maximum (a call in which nearly every row does
+ *     so takes two to three times as long).  Activations that have passed a LayerNorm and projections of O(1) norm stay far inside
+ *     either range.
  */
 nt_status nt_row_attn_pairbias(const nt_layout *L, nt_order order, nt_dtype dt,
                                int32_t c, int32_t H, int32_t d,
