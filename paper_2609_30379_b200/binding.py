@@ -177,19 +177,22 @@ class Layout:
         self.T1 = int(self.lengths_h.sum())
         self.T2 = int(np.dot(self.lengths_h, self.lengths_h))
         dev = torch.device(device)
-        # one allocation for all offset arrays; the lengths and the zeroed status word in front of it arrive in one copy,
-        # which is enqueued like the kernels that read it (a blocking copy would drain the stream for every new batch)
-        sizes = (self.B, 1, self.B + 1, self.B + 1, self.T1 + 1)
+        # one allocation for all offset arrays, each on a multiple of 16 bytes; the zeroed status word and the lengths in
+        # front of it arrive in one copy
+        sizes = [n + (n & 1) for n in (1, self.B, self.B + 1, self.B + 1, self.T1 + 1)]
         buf = torch.empty(sum(sizes), dtype=torch.int64, device=dev)
-        self.lengths_d, status, self.tok_off, self.pair_off, self.row_splits = buf.split(sizes)
+        status, lengths, tok_off, pair_off, row_splits = buf.split(sizes)
         self.status = status.view(torch.int32)[:1]
-        head = np.zeros(self.B + 1, dtype=np.int64)
-        head[:self.B] = self.lengths_h
+        self.lengths_d, self.tok_off, self.pair_off = lengths[:self.B], tok_off[:self.B + 1], pair_off[:self.B + 1]
+        self.row_splits = row_splits[:self.T1 + 1]
+        head = np.zeros(2 + self.B, dtype=np.int64)
+        head[2:] = self.lengths_h
+        # (enqueued like the kernels that read it: a blocking copy would drain the stream for every new batch)
         if stream is None:
-            buf[:self.B + 1].copy_(torch.from_numpy(head), non_blocking=True)
+            buf[:2 + self.B].copy_(torch.from_numpy(head), non_blocking=True)
         else:
             with torch.cuda.stream(stream):
-                buf[:self.B + 1].copy_(torch.from_numpy(head), non_blocking=True)
+                buf[:2 + self.B].copy_(torch.from_numpy(head), non_blocking=True)
         self.pos_sample = self.pos_i = self.pos_j = self.gather_rows = self.gather_cols = None
         if with_maps:
             self.pos_sample = torch.empty(self.T2, dtype=torch.int32, device=dev)
