@@ -187,12 +187,10 @@ class Layout:
         self.row_splits = row_splits[:self.T1 + 1]
         head = np.zeros(2 + self.B, dtype=np.int64)
         head[2:] = self.lengths_h
-        # (enqueued like the kernels that read it: a blocking copy would drain the stream for every new batch)
-        if stream is None:
-            buf[:2 + self.B].copy_(torch.from_numpy(head), non_blocking=True)
-        else:
-            with torch.cuda.stream(stream):
-                buf[:2 + self.B].copy_(torch.from_numpy(head), non_blocking=True)
+        # On the caller's own stream the copy is enqueued like the kernels that read it (a blocking copy would drain the
+        # stream for every new batch).  Kernels on another stream must not start before the current one is through with
+        # whatever had this memory, so there the copy blocks.
+        buf[:2 + self.B].copy_(torch.from_numpy(head), non_blocking=stream is None)
         self.pos_sample = self.pos_i = self.pos_j = self.gather_rows = self.gather_cols = None
         if with_maps:
             self.pos_sample = torch.empty(self.T2, dtype=torch.int32, device=dev)
@@ -203,6 +201,11 @@ class Layout:
         nt_offsets_build(self.lengths_d, self.B, self.T1, self.T2, self.tok_off, self.pair_off, self.row_splits,
                          self.pos_sample, self.pos_i, self.pos_j, self.gather_rows, self.gather_cols,
                          self.status, stream)
+        if stream is not None:      # dropping the Layout must not hand its memory out before that stream is done with it
+            user = stream if isinstance(stream, torch.cuda.Stream) else torch.cuda.ExternalStream(stream.cuda_stream, device=dev)
+            for t in (buf, self.pos_sample, self.pos_i, self.pos_j, self.gather_rows, self.gather_cols):
+                if t is not None:
+                    t.record_stream(user)
         self.c = nt_layout(self.B, self.T1, self.T2, self.lengths_h.ctypes.data if self.B else None,
                            _ptr(self.lengths_d) if self.B else None, _ptr(self.tok_off), _ptr(self.pair_off),
                            _ptr(self.row_splits), _ptr(self.status))
@@ -214,8 +217,8 @@ class Layout:
         if new.shape != self.lengths_h.shape or int(new.sum()) != self.T1 or int((new * new).sum()) != self.T2:
             raise ValueError("Layout.rebuild needs the same B, T1 and T2; build a new Layout instead")
         np.copyto(self.lengths_h, new)
-        if self.B:
-            self.lengths_d.copy_(torch.from_numpy(self.lengths_h), non_blocking=True)
+        if self.B:      # (blocking for kernels on another stream, as above)
+            self.lengths_d.copy_(torch.from_numpy(self.lengths_h), non_blocking=stream is None)
         nt_offsets_build(self.lengths_d, self.B, self.T1, self.T2, self.tok_off, self.pair_off, self.row_splits,
                          self.pos_sample, self.pos_i, self.pos_j, self.gather_rows, self.gather_cols,
                          self.status, stream)

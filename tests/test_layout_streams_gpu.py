@@ -1,4 +1,4 @@
-"""Layout: alignment of its arrays."""
+"""Layout on streams: memory that work on the current stream still reads, offsets built on another stream, alignment."""
 import numpy as np
 import pytest
 import torch
@@ -29,3 +29,36 @@ def test_every_array_is_aligned(nt, B):
     L = nt.Layout(lengths)
     assert all(t.data_ptr() % 16 == 0 for t in (L.status, L.lengths_d, L.tok_off, L.pair_off, L.row_splits) if t.numel())
     _same(L, lengths)
+
+
+def test_side_stream_waits_for_the_memory_it_gets(nt):
+    """A block of the allocator is freed while a copy from it is queued behind a long sleep; the Layout built on a side stream
+    gets that block."""
+    lengths = (5, 9, 30)
+    side = torch.cuda.Stream()
+    probe = nt.Layout(lengths, stream=side)
+    torch.cuda.synchronize()
+    n = probe.status.untyped_storage().nbytes() // 8
+    del probe
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    old = torch.full((n,), 7, dtype=torch.int64, device="cuda")
+    torch.cuda.synchronize()
+    torch.cuda._sleep(200_000_000)
+    seen = old.clone()
+    where = old.data_ptr()
+    del old
+    L = nt.Layout(lengths, stream=side)
+    assert L.status.data_ptr() == where      # or the test shows nothing
+    torch.cuda.synchronize()
+    assert bool((seen == 7).all())
+    _same(L, lengths)
+
+
+def test_rebuild_on_a_side_stream(nt):
+    side = torch.cuda.Stream()
+    L = nt.Layout((5, 9, 30), stream=side)
+    torch.cuda._sleep(50_000_000)
+    L.rebuild((30, 5, 9), stream=side)
+    torch.cuda.synchronize()
+    _same(L, (30, 5, 9))
