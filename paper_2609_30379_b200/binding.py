@@ -177,6 +177,8 @@ class Layout:
         self.T1 = int(self.lengths_h.sum())
         self.T2 = int(np.dot(self.lengths_h, self.lengths_h))
         dev = torch.device(device)
+        if torch.cuda.is_current_stream_capturing():
+            raise RuntimeError("a Layout uploads its lengths: build it before the capture begins")
         # one allocation for all offset arrays, each on a multiple of 16 bytes; the zeroed status word and the lengths in
         # front of it arrive in one copy
         sizes = [n + (n & 1) for n in (1, self.B, self.B + 1, self.B + 1, self.T1 + 1)]

@@ -1,4 +1,4 @@
-"""Layout on streams: memory that work on the current stream still reads, offsets built on another stream, alignment."""
+"""Layout on streams: memory that work on the current stream still reads, offsets built on another stream, capture, alignment."""
 import numpy as np
 import pytest
 import torch
@@ -62,3 +62,16 @@ def test_rebuild_on_a_side_stream(nt):
     L.rebuild((30, 5, 9), stream=side)
     torch.cuda.synchronize()
     _same(L, (30, 5, 9))
+
+
+def test_not_during_a_capture(nt):
+    x = torch.zeros(4, device="cuda")
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        x.add_(1)
+        with pytest.raises(RuntimeError):
+            nt.Layout((5, 9))
+    g.replay()
+    torch.cuda.synchronize()
+    assert float(x[0]) == 1.0
+    _same(nt.Layout((5, 9)), (5, 9))
