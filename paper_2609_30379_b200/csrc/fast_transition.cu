@@ -13,10 +13,12 @@
 // weights at 128 bytes per clock and needs N / 2 clocks of the tensor pipe, so N = 64 runs at two thirds of the
 // tensor rate (measured 48 clocks for 32) and leaves no bandwidth for anything else, while N = 128 runs at the full
 // rate (64 clocks).  Hence one GEMM 1 of 128 columns per tile rather than two accumulator buffers of 64; while one tile
-// is in its gate stage the other tile's MMAs fill the tensor pipe.  The tensor pipe runs one issuer's MMAs in order,
-// which lets GEMM 1 of the next chunk overwrite the columns right behind GEMM 2 without a barrier.  TMEM columns:
+// is in its gate stage the other tile's MMAs fill the tensor pipe.  GEMM 1 of the next chunk overwrites the columns that
+// GEMM 2 has just read and waits for it to be complete: the order in which MMAs are issued is only guaranteed to be
+// kept between those of one shape into one accumulator.  TMEM columns:
 // [0, 256) two tiles x two halves x (32 gate | 32 value), [256, 512) two output accumulators.
-// Measured (256,653 rows, c = 128, hidden 512): 143 us with two buffers of 64 columns, 116 us so.
+// Measured (256,653 rows, c = 128, hidden 512): 155 us with two buffers of 64 columns, 107 us so (99 without the wait for
+// GEMM 2); c = 64, hidden 256: 71 and 50 us.
 // LayerNorm is folded into the weights (W' = W gamma, fp16); its mean and offset ride in GEMM 1 as one more K step:
 // (-mean_hi, -mean_lo, -mean_hi, s_hi, s_hi, s_lo, 4096 s_rest, 0) per row, s = 1 / rstd split into fp16 parts, against
 // (c1_hi, c1_hi, c1_lo, c0_hi, c0_lo, c0_hi, c0_hi / 4096, 0) per weight row, so that rstd times the accumulator is
@@ -71,7 +73,7 @@ __device__ inline unsigned long long tr_desc_sw64(unsigned saddr) {
 
 __global__ void __launch_bounds__(TR_THREADS, 1) transition_kernel(const __grid_constant__ TransParams p) {
   extern __shared__ unsigned char smem_raw[];
-  __shared__ __align__(8) unsigned long long bars[28];
+  __shared__ __align__(8) unsigned long long bars[30];
   __shared__ float sRstd[4][128];
   __shared__ unsigned tmem_base_s;
   __shared__ int abort_flag;
@@ -101,6 +103,7 @@ __global__ void __launch_bounds__(TR_THREADS, 1) transition_kernel(const __grid_
   unsigned long long* oempty = bars + 22;   // [2]
   unsigned long long* gvfull = bars + 24;   // [2] gate | value accumulators of a tile complete
   unsigned long long* hfull = bars + 26;    // [2] hidden slices of a tile stored over them
+  unsigned long long* hread = bars + 28;    // [2] GEMM 2 has read them
 
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;   // warp-uniform for the compiler too
   if (threadIdx.x == 0) {
@@ -113,6 +116,7 @@ __global__ void __launch_bounds__(TR_THREADS, 1) transition_kernel(const __grid_
     for (int s = 0; s < 2; ++s) {
       mbar_init(&gvfull[s], 1);
       mbar_init(&hfull[s], 8);
+      mbar_init(&hread[s], 1);
       mbar_init(&ofull[s], 1);
       mbar_init(&oempty[s], 8);
     }
@@ -246,6 +250,7 @@ __global__ void __launch_bounds__(TR_THREADS, 1) transition_kernel(const __grid_
           }
           if (++st == TR_WST) { st = 0; ph ^= 1; }
         }
+      if (elect_one()) tc_commit(&hread[r]);
       if (q2 == nchunk - 1) {
         if (elect_one()) tc_commit(&ofull[r]);
       }
@@ -264,7 +269,10 @@ __global__ void __launch_bounds__(TR_THREADS, 1) transition_kernel(const __grid_
 #pragma unroll
       for (int r = 0; r < 2; ++r) {
         gemm2(r, g & 1);
-        if (g + 1 < total) gemm1(r);
+        if (g + 1 < total) {
+          mbar_wait(&hread[r], g & 1, ab);                 // the next chunk's accumulators go over the slices just read
+          gemm1(r);
+        }
       }
   } else if (warp < 6) {
     // ------------------------------------------------------------------ converters (4 warps, one row per thread)
