@@ -772,9 +772,19 @@ __global__ void __launch_bounds__(256) segment_reduce_kernel(const T* v, T* out,
   const int t = threadIdx.x;
   if (C >= 256) {
     for (int c = t; c < C; c += 256) {
+      // (eight loads in flight, one sum in order: a loop left to the compiler's unrolling kept one in flight, 210 us for twelve
+      // groups of 512 rows of 768 floats, 35 so)
+      const T* col = v + c;
       float acc = 0.f;
-#pragma unroll 8
-      for (long long r = lo; r < hi; ++r) acc += Cvt<T>::ld(v + r * C + c);
+      long long r = lo;
+      for (; r + 7 < hi; r += 8) {
+        float x[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) x[u] = Cvt<T>::ld(col + (r + u) * C);
+#pragma unroll
+        for (int u = 0; u < 8; ++u) acc += x[u];
+      }
+      for (; r < hi; ++r) acc += Cvt<T>::ld(col + r * C);
       Cvt<T>::st(out + g * C + c, acc * sc);
     }
     return;

@@ -1,0 +1,43 @@
+"""Shape-generic reduction at the edges of its loop: groups around multiples of the eight rows that are in flight, against the CPU
+oracle."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import nested_pair_oracle as orc
+from paper_2609_30379_b200 import workloads as wl
+from tests.parity_utils import check
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def nt():
+    from paper_2609_30379_b200 import binding
+    return binding
+
+
+def _dev(a, dtype):
+    return torch.from_numpy(np.ascontiguousarray(a)).to("cuda", torch.float32 if dtype == "f32" else torch.bfloat16)
+
+
+def _host(t):
+    return t.detach().to(torch.float32).cpu().numpy().astype(np.float64)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("C", [256, 260, 300, 1030])
+@pytest.mark.parametrize("op", ["mean", "sum"])
+def test_wide_groups(nt, dtype, C, op):
+    sizes = (0, 1, 7, 8, 9, 0, 15, 16, 17, 40)
+    splits = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int64)
+    v = np.random.default_rng(C).standard_normal((int(splits[-1]), C)).astype(np.float32)
+    if dtype == "bf16":
+        v = wl.round_to_bf16(v)
+    out = torch.full((len(sizes), C), 3.0, dtype=torch.float32 if dtype == "f32" else torch.bfloat16, device="cuda")
+    nt.nt_segment_reduce(nt.NT_REDUCE_MEAN if op == "mean" else nt.NT_REDUCE_SUM, torch.from_numpy(splits).cuda(), _dev(v, dtype), out)
+    ref = orc.segment_reduce(v.astype(np.float64), splits, op)
+    if dtype == "f32":
+        check("f32", _host(out), ref, f"{op} C={C}")
+    else:      # one rounding of a float sum
+        assert (np.abs(_host(out) - ref) <= 2.0 ** -8 * np.abs(ref) + 1e-5).all()
