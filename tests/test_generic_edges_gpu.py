@@ -1,5 +1,5 @@
-"""Shape-generic reduction at the edges of its loop: groups around multiples of the eight rows that are in flight, against the CPU
-oracle."""
+"""Shape-generic reduction and accumulated projection at the edges of their loops: groups around multiples of the eight rows that
+are in flight, outputs around multiples of the 64 columns of a tile, one row more or less than a block, against the CPU oracle."""
 import numpy as np
 import pytest
 import torch
@@ -41,3 +41,16 @@ def test_wide_groups(nt, dtype, C, op):
         check("f32", _host(out), ref, f"{op} C={C}")
     else:      # one rounding of a float sum
         assert (np.abs(_host(out) - ref) <= 2.0 ** -8 * np.abs(ref) + 1e-5).all()
+
+
+@pytest.mark.parametrize("rows", [1, 63, 64, 65, 200])
+@pytest.mark.parametrize("c_z,c_s", [(16, 32), (19, 33), (64, 64), (96, 100), (5, 1), (130, 65)])
+def test_accumulated_projection(nt, rows, c_z, c_s):
+    rng = np.random.default_rng(rows + c_s)
+    m, W, x = (rng.standard_normal(s).astype(np.float32) for s in ((rows, c_z), (c_s, c_z), (rows, c_s)))
+    buf = torch.full((rows * c_s + 64,), 7.0, device="cuda")
+    xd = buf[32:32 + rows * c_s].view(rows, c_s)
+    xd.copy_(_dev(x, "f32"))
+    nt.nt_token_update(_dev(m, "f32"), _dev(W, "f32"), xd)
+    check("f32", _host(xd), orc.token_update(x.astype(np.float64), m.astype(np.float64), W), f"{rows} rows, {c_z} -> {c_s}")
+    assert bool((buf[:32] == 7.0).all()) and bool((buf[32 + rows * c_s:] == 7.0).all())
