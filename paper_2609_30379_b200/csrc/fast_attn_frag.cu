@@ -320,7 +320,7 @@ __device__ inline void fr_first_reference(const unsigned (&s)[2][16], unsigned b
 // rows; of 977, 5.3 against 1.6, and 3.7 against 1.2 with 2 heads of 32.  With a query per lane and scalar loads the
 // sample of 400 took 114 ms.
 template <int D, bool HAS_BIAS>
-__device__ __noinline__ float4 fr_exact_row(const AttnFrParams& p, const FrInfo& inf, int t, int quarter, int lane) {
+static __device__ __noinline__ float4 fr_exact_row(const AttnFrParams& p, const FrInfo& inf, int t, int quarter, int lane) {
   const int N = inf.N, q0 = inf.q0 + quarter * 32, gr = lane >> 2, c2 = 2 * (lane & 3);
   const long long pitch = (long long)p.H * D * inf.step;                        // elements between consecutive queries / keys
   const long long key0 = (p.row0 + inf.orow + (long long)t * inf.tile_row - (long long)inf.q0 * inf.step) * p.H * D +
