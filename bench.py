@@ -267,7 +267,7 @@ def exp_rate_table(nt, torch):
              7: "ex2.approx.ftz.f32, results packed to bf16 pairs with cvt.rn.bf16x2.f32",
              8: "ex2.approx.ftz.f32, results packed to bf16 pairs with integer add + prmt",
              9: "the attention cores' softmax inner loop, registers only (bias unpack, add, fma, 2 ex2, sum, pack per pair)",
-             10: "the same loop with 8 warps per SM instead of 16 (the key-blocked core's softmax warps)"}
+             10: "the same loop with 8 warps per SM instead of 16 (two warps to a scheduler)"}
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     sink = torch.empty(4096 * 512, dtype=torch.float32, device="cuda")
     clocks = torch.zeros(4096, dtype=torch.int64, device="cuda")
@@ -373,8 +373,8 @@ def main():
                     help="nt_row_attn_pairbias + nt_segment_reduce instead of the fused nt_row_attn_pairbias_mean")
     ap.add_argument("--no-graph", action="store_true",
                     help="launch every kernel of the timed steps from the host instead of replaying the captured step")
-    ap.add_argument("--key-blocked-attention", action="store_true",
-                    help="send every sample length to the key-blocked attention core (default: split by length)")
+    ap.add_argument("--fragment-attention", "--key-blocked-attention", action="store_true", dest="fragment_attention",
+                    help="send every sample length to the register-fragment attention core (default: split by length)")
     ap.add_argument("--exp-rate", action="store_true",
                     help="run the exponential-rate microbenchmark (the attention core's third ceiling) and print its table")
     ap.add_argument("--write-rate", action="store_true",
@@ -433,7 +433,7 @@ def main():
         return
     if args.force_generic:
         nt.nt_force_generic(True)
-    if args.key_blocked_attention:
+    if args.fragment_attention:
         nt.nt_attn_core_mode(1)
     cfg = wl.CONFIGS[args.config]
     inp = wl.make_inputs(cfg)

@@ -235,7 +235,7 @@ static nt_status tri_mul_generic(const nt_layout* L, const Totals& tot, int c_z,
   // The tensor-core stages exchange a, b (fp16) and t (fp16, scaled by 1 / N): all three or none.
   // (the tensor-core kernels index positions inside a sample with 32 bits: N below 2^16)
   const bool tc = dt == NT_BF16 && !g_force_generic && tot.nmax < 60000 && fast_tri_in_supported(c_z, c_h) &&
-                  fast_contract_supported(c_h) && fast_tri_out_supported(c_z, c_h);
+                  fast_tri_out_supported(c_z, c_h);
   TriPrep tprep{};
   if (tc) {
     // folded weights: the caller's, prepared ahead of time, or built now into the workspace
@@ -815,7 +815,7 @@ nt_status nt_prepare_trimul_weights(nt_dtype dt, int32_t c_z, int32_t c_h, const
   if (!W->ln_in_gamma || !W->ln_in_beta || !W->W_ap || !W->W_ag || !W->W_bp || !W->W_bg || !W->W_g || !W->ln_out_gamma ||
       !W->ln_out_beta || !W->W_o)
     return NT_ERR_INVALID_ARG;
-  if (dt != NT_BF16 || !fast_tri_in_supported(c_z, c_h) || !fast_contract_supported(c_h) || !fast_tri_out_supported(c_z, c_h))
+  if (dt != NT_BF16 || !fast_tri_in_supported(c_z, c_h) || !fast_tri_out_supported(c_z, c_h))
     return NT_ERR_UNSUPPORTED;
   TriPrep tp{};
   return fast_tri_prep(W, c_z, c_h, prepared_out, tp, (cudaStream_t)stream);

@@ -60,7 +60,7 @@ template <> struct Cvt<__nv_bfloat16> {
 // the constant true and costs nothing.  nt_debug_bounds_report reads the record.
 enum NtBoundSite {
   NT_SITE_DECODE = 1, NT_SITE_PROJ_OUT, NT_SITE_CONTRACT_OUT, NT_SITE_BROADCAST_OUT, NT_SITE_ATTN_OUT, NT_SITE_SEGMENT_OUT,
-  NT_SITE_FAST_BROADCAST, NT_SITE_FAST_SEGMENT, NT_SITE_KB_ATTN_OUT, NT_SITE_ROW_ATTN_OUT, NT_SITE_ATTN_IN_BIAS,
+  NT_SITE_FAST_BROADCAST, NT_SITE_FAST_SEGMENT, NT_SITE_FRAG_ATTN_OUT, NT_SITE_ROW_ATTN_OUT, NT_SITE_ATTN_IN_BIAS,
   NT_SITE_TOKEN_GEMM_OUT, NT_SITE_RECT_BROADCAST
 };
 #ifdef NT_DEBUG_BOUNDS

@@ -418,7 +418,7 @@ static __device__ __noinline__ float4 fr_exact_row(const AttnFrParams& p, const 
     const float inv = 1.0f / l[r];
     const int q = q0 + (r >> 1) * 16 + (r & 1) * 8 + gr;
     lse[r] = mx[r] + log2f(l[r]);
-    if (q < N && NT_IN(inf.orow + (long long)t * inf.tile_row + (long long)(q - inf.q0) * inf.step, p.rows, NT_SITE_KB_ATTN_OUT)) {
+    if (q < N && NT_IN(inf.orow + (long long)t * inf.tile_row + (long long)(q - inf.q0) * inf.step, p.rows, NT_SITE_FRAG_ATTN_OUT)) {
 #pragma unroll
       for (int k = 0; k < D / 8; ++k)
         *reinterpret_cast<unsigned*>(p.o + key0 + q * pitch + k * 8 + c2) =
@@ -752,7 +752,7 @@ __global__ void __launch_bounds__(128 + 128 * NT, 1) attn_fr_kernel(const __grid
             const int q = (rr >> 1) * 16 + (rr & 1) * 8 + (lane >> 2);
             const int ch = D == 16 ? (lane & 1) * 8 : (k + (lane & 3)) * 8;
             const long long orow = orow0 + (long long)q * step;
-            if (q0 + q < N && NT_IN(orow, p.rows, NT_SITE_KB_ATTN_OUT)) *reinterpret_cast<uint4*>(op + orow * Hd + ch) = v;
+            if (q0 + q < N && NT_IN(orow, p.rows, NT_SITE_FRAG_ATTN_OUT)) *reinterpret_cast<uint4*>(op + orow * Hd + ch) = v;
           }
         }
       }

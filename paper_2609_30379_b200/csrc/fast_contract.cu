@@ -220,7 +220,6 @@ __global__ void __launch_bounds__(CT_THREADS, 1) tri_contract_kernel(const __gri
   if (warp == 1) tmem_dealloc(tmem_base, 512);
 }
 
-bool fast_contract_supported(int C) { return C >= 1; }
 
 nt_status fast_contract(const void* a, size_t buf_stride_bytes, int C, const BatchMeta& m, int* status,
                         cudaStream_t st, bool incoming) {

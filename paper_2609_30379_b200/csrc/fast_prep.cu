@@ -17,7 +17,7 @@ struct PrepJob {
   const __nv_bfloat16* gamma;
   const __nv_bfloat16* beta;
   __half* out;
-  float2* c01;
+  float2* c01;      // nullable
   __half* aug;      // nullable: [2][total][8] fp16 augmentation columns (see below)
 };
 struct PrepArgs { PrepJob job[2]; int njobs; };
@@ -88,7 +88,7 @@ __global__ void __launch_bounds__(256) ln_fold_prep_kernel(PrepArgs a) {
     c1 += __shfl_xor_sync(0xffffffffu, c1, o);
   }
   if (lane == 0) {
-    J.c01[n] = make_float2(c0, c1);
+    if (J.c01) J.c01[n] = make_float2(c0, c1);
     if (J.aug) {
       // Extra K columns that make the MMA itself apply the LayerNorm correction: against activation columns
       // (m_hi, m_lo, m_hi, 1, 1) with m = -mean * rstd they contribute m * c1 + c0 (hi/lo split keeps ~22 bits).  The
@@ -199,15 +199,13 @@ nt_status fast_transition_prep(const nt_transition_weights* W, int c, int hidden
   char* p = (char*)prep;
   out.w1 = p;
   p += align_up((size_t)rows * c * 2, 256);
-  out.c01 = p;
-  p += align_up((size_t)rows * sizeof(float2), 256);
-  out.aug = p;                          // [2][rows][8] fp16
+  out.aug = p;                          // [2][rows][8] fp16; the kernel needs no (c0, c1) beside it
   out.rows = rows;
   PrepArgs a{};
   const void* s0[2] = {W->W_a, W->W_b};
   const int r0[2] = {hidden, hidden};
   const float sc[2] = {0.5f, 1.0f};
-  add_job(a, s0, r0, 2, c, W->ln_gamma, W->ln_beta, out.w1, out.c01, sc, out.aug);
+  add_job(a, s0, r0, 2, c, W->ln_gamma, W->ln_beta, out.w1, nullptr, sc, out.aug);
   return run_prep(a, st);
 }
 

@@ -89,32 +89,6 @@ __device__ inline bool mbar_wait(void* bar, unsigned parity, const AbortCtx& ab,
   return false;
 }
 
-// The same wait with a long suspend-time hint on every probe (the warp is parked until the phase completes or the
-// hint runs out), for roles that spend most of their life waiting: far fewer probe loops compete for issue slots.
-__device__ inline bool mbar_try_park(void* bar, unsigned parity) {
-  unsigned ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
-      "selp.b32 %0, 1, 0, p;\n\t}\n"
-      : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity), "r"(20000u) : "memory");
-  return ok != 0;
-}
-__device__ inline bool mbar_wait_park(void* bar, unsigned parity, const AbortCtx& ab) {
-  if (mbar_try(bar, parity)) return true;
-  const long long t0 = clock64();
-  const long long limit = *ab.flag ? WAIT_CLOCKS_ABORTED : WAIT_CLOCKS;
-  for (unsigned it = 0; it < WAIT_PROBES; ++it) {
-    if (mbar_try_park(bar, parity)) return true;
-    if (clock64() - t0 > limit || *ab.flag) break;
-  }
-  if (!*ab.flag) {
-    *ab.flag = 1;
-    if (ab.status) atomicCAS(ab.status, 0, (int)NT_ERR_TIMEOUT);
-  }
-  return false;
-}
-
 __device__ inline void fence_proxy_async_smem() { asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory"); }
 
 __device__ inline void tma_load_2d(void* dst, const CUtensorMap* map, void* bar, int c0, int c1) {
@@ -142,11 +116,7 @@ __device__ inline void tma_store_4d(const CUtensorMap* map, const void* src, int
 }
 __device__ inline void tma_store_commit() { asm volatile("cp.async.bulk.commit_group;\n" ::: "memory"); }
 __device__ inline void tma_store_wait_read0() { asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory"); }
-__device__ inline void tma_store_wait_read1() { asm volatile("cp.async.bulk.wait_group.read 1;\n" ::: "memory"); }
 __device__ inline void tma_store_wait_all0() { asm volatile("cp.async.bulk.wait_group 0;\n" ::: "memory"); }
-__device__ inline void tma_prefetch_map(const CUtensorMap* map) {
-  asm volatile("prefetch.tensormap [%0];\n" ::"l"(map) : "memory");
-}
 
 // ---- TMEM
 __device__ inline void tmem_alloc(unsigned* dst_smem, unsigned ncols) {   // whole warp
@@ -188,27 +158,7 @@ __device__ inline void tmem_ld16(unsigned taddr, unsigned (&r)[16]) {
 }
 
 // 32 lanes x 8 / 2 consecutive columns
-__device__ inline void tmem_ld8(unsigned taddr, unsigned (&r)[8]) {
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];\n"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-               : "r"(taddr) : "memory");
-}
-__device__ inline void tmem_ld2(unsigned taddr, unsigned& r0, unsigned& r1) {
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0,%1}, [%2];\n" : "=r"(r0), "=r"(r1) : "r"(taddr) : "memory");
-}
-__device__ inline void tmem_st2(unsigned taddr, unsigned r0, unsigned r1) {
-  asm volatile("tcgen05.st.sync.aligned.32x32b.x2.b32 [%0], {%1,%2};\n" ::"r"(taddr), "r"(r0), "r"(r1) : "memory");
-}
-__device__ inline void tmem_ld1(unsigned taddr, unsigned& r) {
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];\n" : "=r"(r) : "r"(taddr) : "memory");
-}
 // registers -> TMEM: thread t writes row (lane base + t), 16 or 8 consecutive columns
-__device__ inline void tmem_st16(unsigned taddr, const unsigned (&r)[16]) {
-  asm volatile(
-      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};\n"
-      ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]),
-        "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]) : "memory");
-}
 __device__ inline void tmem_st8(unsigned taddr, const unsigned (&r)[8]) {
   asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};\n"
                ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]) : "memory");
@@ -328,12 +278,6 @@ __device__ inline unsigned pack2(unsigned lo, unsigned hi) {
 }
 
 // two floats (bit patterns) scaled and packed as fp16x2 (saturating), first in the low half
-__device__ inline unsigned pack2h(unsigned lo, unsigned hi, float scale) {
-  const float a = fminf(fmaxf(__uint_as_float(lo) * scale, -65504.f), 65504.f);
-  const float b = fminf(fmaxf(__uint_as_float(hi) * scale, -65504.f), 65504.f);
-  __half2 h = __floats2half2_rn(a, b);
-  return *reinterpret_cast<unsigned*>(&h);
-}
 
 // byte offset of 16-byte chunk `chunk` of row `row` inside a 128-byte-swizzled tile
 __device__ inline unsigned sw128_off(int row, int chunk) { return row * 128 + ((chunk ^ (row & 7)) << 4); }
