@@ -670,7 +670,7 @@ nt_status fast_single_bias(const void* z, const void* g, const void* b, const vo
   if (rows <= 0) return NT_OK;
   const long long nblk = (rows + 31) / 32;
   const long long want = (nblk + 7) / 8;
-  const unsigned grid = (unsigned)(want < 148 * 3 ? want : 148 * 3);      // 3 blocks of 256 threads fit an SM at 79 registers
+  const unsigned grid = (unsigned)(want < sm_count() * 3 ? want : sm_count() * 3);      // 3 blocks of 256 threads fit an SM at 79 registers
   if (H <= 4 && (C == 128 || C == 64)) {
     const long long ntile = (rows + 15) / 16, wantb = (ntile + 7) / 8;
     const unsigned gridm = (unsigned)(wantb < sm_count() * 3 ? wantb : sm_count() * 3);      // what is resident at 80 registers
