@@ -15,7 +15,8 @@
  *     accumulation, float LayerNorm / softmax statistics.  Intermediates that never leave the workspace are bf16
  *     (q, k, v, o, bias) or, on the tensor-core path, fp16 where three more significant bits pay: the
  *     LayerNorm-folded weights, the triangle update's a, b (gated projections of a normalised row) and t / N_s.
- *     fp16 ends at 65504: the folded input weights and their offsets W beta have to lie below; a, b and t / N_s are clamped to its finite range when they are written, so a state with
+ *     fp16 ends at 65504: the folded weights and the offsets W beta of the input projections and of the transition have
+ *     to lie below; a, b and t / N_s are clamped to its finite range when they are written, so a state with
  *     absurdly large projections saturates instead of producing infinities.
  *   - A process may drive several devices: per-kernel launch attributes are kept per device.
  *   - The caller owns every buffer.  No call allocates, frees or synchronises; all work is
