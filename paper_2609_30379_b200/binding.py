@@ -181,12 +181,11 @@ class Layout:
             raise RuntimeError("a Layout uploads its lengths: build it before the capture begins")
         # one allocation for all offset arrays, each on a multiple of 16 bytes; the zeroed status word and the lengths in
         # front of it arrive in one copy
-        sizes = [n + (n & 1) for n in (1, self.B, self.B + 1, self.B + 1, self.T1 + 1)]
+        odd = self.B & 1
+        sizes = (1, 1, self.B, odd, self.B + 1, 1 - odd, self.B + 1, 1 - odd, self.T1 + 1)
         buf = torch.empty(sum(sizes), dtype=torch.int64, device=dev)
-        status, lengths, tok_off, pair_off, row_splits = buf.split(sizes)
+        status, _, self.lengths_d, _, self.tok_off, _, self.pair_off, _, self.row_splits = buf.split(sizes)
         self.status = status.view(torch.int32)[:1]
-        self.lengths_d, self.tok_off, self.pair_off = lengths[:self.B], tok_off[:self.B + 1], pair_off[:self.B + 1]
-        self.row_splits = row_splits[:self.T1 + 1]
         head = np.zeros(2 + self.B, dtype=np.int64)
         head[2:] = self.lengths_h
         # On the caller's own stream the copy is enqueued like the kernels that read it (a blocking copy would drain the
