@@ -366,19 +366,20 @@ nt_status launch_proj(const ProjArgs& args, const BatchMeta& m, cudaStream_t st,
   if (a.rows <= 0 || tiles <= 0) return NT_OK;
   long long bx = (a.rows + PBM - 1) / PBM;
   if (bx > 0x7FFFFFFFll || tiles > 65535) return NT_ERR_UNSUPPORTED;
-  // One column tile per block while that leaves SMs without a block.  Once the rows fill the GPU, all of them where the rows
-  // come in many rounds, and fewer where a part of a round would be left over: the number per block for which rounds x
-  // (rows once + tiles) is smallest, a block's rows and their LayerNorm costing about half a tile (three blocks fit an SM).  Lengths
-  // 24-110, 32 k rows: 365.6 -> 351.6 us per float block.
-  const long long want = 2 * sm_count(), fit = 3 * sm_count();
-  const long long split = bx * tiles <= want ? tiles : (want + bx - 1) / bx;
-  int tpb = (int)((tiles + split - 1) / split);
-  if (bx >= want) {
-    double best = 1e300;
-    for (int k = 1; k <= tiles; ++k) {
-      const double cost = (double)((bx * ((tiles + k - 1) / k) + fit - 1) / fit) * (0.5 + k);
-      if (cost <= best) { best = cost; tpb = k; }
-    }
+  // Column tiles per block: the number for which the blocks' rounds take least.  A block costs its tiles (between the most and
+  // the average, where they do not divide evenly) and a little for its rows and their LayerNorm; three blocks fit an SM, and
+  // an SM with one or two left works at 0.6 or 0.9 of its rate, so a last round of up to one, two or three blocks per SM
+  // takes 1.6, 2.3 or 3 block times.  Fitted to the times of every tile count (widths 40 to 256, 1 to 16 tiles, 256 to 160 k rows,
+  // float and bf16; 984 launches): 1.5 % from the best choice on average, 15 % at worst.  (One tile per block up to two blocks per
+  // SM and whole rounds beyond that: 6 %, 56 %, and 31 % slower than a block per tile for a hidden layer of 1024 on 14400 rows.)
+  const long long sms = sm_count();
+  int tpb = 1;
+  double best = 1e300;
+  for (int k = 1; k <= tiles; ++k) {
+    const long long y = (tiles + k - 1) / k, n = bx * y, rounds = n / (3 * sms), rest = n - rounds * 3 * sms;
+    const double last = rest == 0 ? 0.0 : rest <= sms ? 1.6 : rest <= 2 * sms ? 2.3 : 3.0;
+    const double cost = (3.0 * (double)rounds + last) * (0.15 + 0.75 * (double)tiles / (double)y + 0.25 * k);
+    if (cost < best) { best = cost; tpb = k; }
   }
   const dim3 grid((unsigned)bx, (unsigned)((tiles + tpb - 1) / tpb));
   const bool vec = (a.K & 3) == 0 && (low & 15) == 0;      // (not every entry point asks for aligned weights)
