@@ -292,47 +292,48 @@ __global__ void __launch_bounds__(PTHREADS, 3) proj_kernel(const __grid_constant
     __syncthreads();
     const int ncol = min(PBN, g.Nout - nt0);
     const int total = cm ? ncol * PBM : rows * PBN;
-    // An output that is added to costs a trip to memory before each store; four at a time in single precision (402 rows, 16 -> 32:
-    // 10.6 -> 7.6 us, 8.4 with everything unrolled; in bf16 the registers for it spill)
-    constexpr int AHEAD = sizeof(T) == 4 ? 4 : 1;
     const bool accum = g.out_mode == O_ACCUM;
-    float old[AHEAD] = {};                     // (stays zero where nothing is added to)
-#pragma unroll (AHEAD == 1 ? 2 : 1)
-    for (int idx0 = t; idx0 < total; idx0 += AHEAD * PTHREADS) {
-      if (AHEAD > 1 && accum) {
-#pragma unroll
-        for (int u = 0; u < AHEAD; ++u) {
-          const int idx = idx0 + u * PTHREADS, rl = idx >> 6, n = nt0 + (idx & 63);
-          if (rl < rows && n < g.Nout) {
-            const long long at = (r0 + rl) * g.Nout + n;
-            old[u] = g.out_f32 ? ((const float*)g.out)[at] : Cvt<T>::ld((const T*)g.out + at);
-          }
-        }
+    auto emit = [&](int idx, bool have, float old) {          // result idx; have: its old value has been fetched
+      const int hi = idx >> 6, lo = idx & 63, rl = cm ? lo : hi, n = nt0 + (cm ? hi : lo);
+      if (rl >= rows || n >= g.Nout) return;
+      const long long p = r0 + rl;
+      float v = Ws[hi * PPITCH + lo];
+      if (gated) v = (g.act == ACT_SILU ? v * sigmoidf_acc(v) : sigmoidf_acc(v)) * Gs[hi * PPITCH + lo];
+      else if (g.act == ACT_SIGMOID) v = sigmoidf_acc(v);
+      if (cm) {
+        const long long at = (long long)g.Nout * cmbase[rl] + (long long)n * plane[rl] + inpl[rl];
+        if (NT_IN(at, (long long)g.Nout * m.cm_off[m.B], NT_SITE_PROJ_OUT)) Cvt<T>::st((T*)g.out + at, v);
+        return;
       }
-#pragma unroll
-      for (int u = 0; u < AHEAD; ++u) {
-        const int idx = idx0 + u * PTHREADS;
-        const int hi = idx >> 6, lo = idx & 63, rl = cm ? lo : hi, n = nt0 + (cm ? hi : lo);
-        if ((AHEAD > 1 && idx >= total) || rl >= rows || n >= g.Nout) continue;
-        const long long p = r0 + rl;
-        float v = Ws[hi * PPITCH + lo];
-        if (gated) v = (g.act == ACT_SILU ? v * sigmoidf_acc(v) : sigmoidf_acc(v)) * Gs[hi * PPITCH + lo];
-        else if (g.act == ACT_SIGMOID) v = sigmoidf_acc(v);
-        if (cm) {
-          const long long at = (long long)g.Nout * cmbase[rl] + (long long)n * plane[rl] + inpl[rl];
-          if (NT_IN(at, (long long)g.Nout * m.cm_off[m.B], NT_SITE_PROJ_OUT)) Cvt<T>::st((T*)g.out + at, v);
-          continue;
-        }
-        if (!NT_IN(p, a.row0 + a.rows, NT_SITE_PROJ_OUT)) continue;
-        if (gO) v *= Cvt<T>::ld(gO + p * g.Nout + n);
-        if (g.out_f32) {
-          float* o = (float*)g.out + p * g.Nout + n;
-          *o = AHEAD > 1 ? v + old[u] : accum ? *o + v : v;
-        } else {
-          T* o = (T*)g.out + p * g.Nout + n;
-          Cvt<T>::st(o, AHEAD > 1 ? v + old[u] : accum ? v + Cvt<T>::ld(o) : v);
-        }
+      if (!NT_IN(p, a.row0 + a.rows, NT_SITE_PROJ_OUT)) return;
+      if (gO) v *= Cvt<T>::ld(gO + p * g.Nout + n);
+      if (g.out_f32) {
+        float* o = (float*)g.out + p * g.Nout + n;
+        *o = accum ? (have ? old : *o) + v : v;
+      } else {
+        T* o = (T*)g.out + p * g.Nout + n;
+        Cvt<T>::st(o, accum ? v + (have ? old : Cvt<T>::ld(o)) : v);
       }
+    };
+    // An output that is added to costs a trip to memory before each store; four are fetched at a time (402 float rows, 16 -> 32:
+    // 10.6 -> 7.4 us, 8.4 with everything unrolled; bf16, 96 -> 100: 17.5 -> 15.9 and 16.5).  In a loop of its own: outputs that are
+    // only stored lost 0.8 us to the longer code.
+    if (accum && !g.out_f32) {
+      float old[4] = {};
+#pragma unroll 1
+      for (int idx0 = t; idx0 < total; idx0 += 4 * PTHREADS) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int rl = (idx0 + u * PTHREADS) >> 6, n = nt0 + ((idx0 + u * PTHREADS) & 63);
+          if (rl < rows && n < g.Nout) old[u] = Cvt<T>::ld((const T*)g.out + (r0 + rl) * g.Nout + n);
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (idx0 + u * PTHREADS < total) emit(idx0 + u * PTHREADS, true, old[u]);
+      }
+    } else {
+#pragma unroll 2
+      for (int idx = t; idx < total; idx += PTHREADS) emit(idx, false, 0.f);
     }
     __syncthreads();
   }

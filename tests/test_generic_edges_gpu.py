@@ -54,3 +54,15 @@ def test_accumulated_projection(nt, rows, c_z, c_s):
     nt.nt_token_update(_dev(m, "f32"), _dev(W, "f32"), xd)
     check("f32", _host(xd), orc.token_update(x.astype(np.float64), m.astype(np.float64), W), f"{rows} rows, {c_z} -> {c_s}")
     assert bool((buf[:32] == 7.0).all()) and bool((buf[32 + rows * c_s:] == 7.0).all())
+
+
+@pytest.mark.parametrize("rows", [1, 65, 200])
+@pytest.mark.parametrize("c_z,c_s", [(19, 33), (96, 100), (5, 1), (130, 65)])      # widths that the shape-generic kernel takes
+def test_accumulated_projection_bf16(nt, rows, c_z, c_s):
+    rng = np.random.default_rng(rows + c_s)
+    m, W, x = (wl.round_to_bf16(rng.standard_normal(s).astype(np.float32)) for s in ((rows, c_z), (c_s, c_z), (rows, c_s)))
+    xd = _dev(x, "bf16")
+    nt.nt_token_update(_dev(m, "bf16"), _dev(W, "bf16"), xd)
+    ref = orc.token_update(x.astype(np.float64), m.astype(np.float64), W)
+    # float products and sums of bf16 values, rounded to bf16 once
+    assert (np.abs(_host(xd) - ref) <= 2.0 ** -8 * np.abs(ref) + 1e-4).all()
