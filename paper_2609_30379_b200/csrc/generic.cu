@@ -32,7 +32,7 @@ __device__ inline float4 ld4_row(const T* row, int k, int K, bool vec) {
 // ------------------------------------------------------------------------------------------
 // projection: 64 rows x 64 output columns at a time, K in panels of 32.  The column tiles of all outputs that share their
 // rows are one launch; a block takes one of them where there are few rows (the smallest states are latency and nothing
-// else) and all of them where the rows alone fill the GPU: the rows are then read and normalised once.  Rows of up to 64
+// else) and more where the rows alone fill the GPU: the rows are then read and normalised less often.  Rows of up to 64
 // elements are normalised in shared memory, the next panel is in registers while one is worked on, and results leave
 // through shared memory in a rolled loop.  The loops are rolled on purpose: on a state of 531 rows a fully unrolled
 // kernel spent its time fetching instructions (17 us a launch for 1500 to 2200 instructions per warp, two thirds of the
@@ -316,7 +316,7 @@ __global__ void __launch_bounds__(PTHREADS, 3) proj_kernel(const __grid_constant
       }
     };
     // An output that is added to costs a trip to memory before each store; four are fetched at a time (402 float rows, 16 -> 32:
-    // 10.6 -> 7.4 us, 8.4 with everything unrolled; bf16, 96 -> 100: 17.5 -> 15.9 and 16.5).  In a loop of its own: outputs that are
+    // 10.6 -> 7.4 us, 8.4 with everything unrolled; bf16, 96 -> 100: 17.5 -> 15.3, 16.5 unrolled).  In a loop of its own: outputs that are
     // only stored lost 0.8 us to the longer code.
     if (accum && !g.out_f32) {
       float old[4] = {};
